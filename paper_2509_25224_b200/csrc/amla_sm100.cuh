@@ -335,6 +335,36 @@ __device__ __forceinline__ void mma_commit_pair_multicast(uint32_t bar, uint16_t
                ::"r"(bar), "h"(cta_mask) : "memory");
 }
 
+// The pair forms issued by a whole converged warp, one lane of which is elected: addresses and descriptors stay in
+// uniform registers.  (Under a lane-0 branch every operand of every MMA is moved over from the vector registers first:
+// measured 50 clk of issue per MMA against 20, and 45 against next to nothing per commit; an MMA of 128 x 256 x 16
+// takes 64.)
+__device__ __forceinline__ void mma_ss_pair_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void mma_ts_pair_elect(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit_pair_multicast_elect(uint32_t bar, uint16_t cta_mask) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+      ::"r"(bar), "h"(cta_mask) : "memory");
+}
+
 // Asynchronous stores into the shared memory of a CTA of the cluster; each adds its size to the transaction
 // count of a barrier of that CTA.  Generic-proxy writes: a consumer that reads them through the async proxy
 // (TMA, tcgen05.mma) fences with fence.proxy.async after its wait.
