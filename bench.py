@@ -359,7 +359,7 @@ def run_gpu(args):
 
     if rank == 0:
         roof = roofline_of(w, dec_ms, peaks, peak_kind)
-        roof.update({"kernel": "decode_quad_kernel" if (Sq * H > 128 and not args.rows128) else "decode_tc_kernel",
+        roof.update({"kernel": "decode_quad_kernel" if (Sq * H > 128 and not args.rows128) else "decode_pair_kernel",
                      "schedule_ms": plan_ms, "combine_ms": comb_ms})
         roof["traffic"] = load_traffic().get(w.name)
         n_rows = {"tiny": 16, "dsv3": 4096, "mtp": 2048, "stress": 1024, "long": 256}[w.name]

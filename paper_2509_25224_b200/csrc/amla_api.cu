@@ -12,12 +12,12 @@ cudaError_t launch_plan(const DecodeParams& prm, int* prefix_out, cudaStream_t s
 cudaError_t launch_combine(const DecodeParams& prm, cudaStream_t stream);
 cudaError_t launch_decode_simt(const DecodeParams& prm, cudaStream_t stream);
 // Returns cudaSuccess, or an error; sets *unsupported when the device cannot run the kernel.
-cudaError_t launch_decode_tc(const DecodeParams& prm, cudaStream_t stream, int* unsupported);
+cudaError_t launch_decode_pair(const DecodeParams& prm, cudaStream_t stream, int* unsupported);
 cudaError_t launch_decode_quad(const DecodeParams& prm, cudaStream_t stream, int* unsupported);
 cudaError_t launch_wait_selftest(int* status, unsigned long long limit_ns, cudaStream_t stream);
 cudaError_t launch_widen_pages(const uint8_t* kv8, const int32_t* block_table, const int32_t* seqlens, int B, int num_blocks,
                                int max_blocks_per_seq, __nv_bfloat16* scratch, int32_t* table_out, cudaStream_t stream);
-int decode_tc_parts(int sm_count);
+int decode_pair_parts(int sm_count);
 int decode_quad_parts(int device, int sm_count);
 
 namespace {
@@ -105,7 +105,7 @@ int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
   prm.ovh = quad ? kQuadOverheadTiles : kUnitOverheadTiles;
   prm.nrb = (prm.R + prm.item_rows - 1) / prm.item_rows;
   prm.n_items = prm.B * prm.nrb;
-  prm.P = simt ? sms : quad ? quad_parts : decode_tc_parts(sms);
+  prm.P = simt ? sms : quad ? quad_parts : decode_pair_parts(sms);
   prm.fused_plan = (!simt && prm.n_items <= kFusedPlanMaxItems) ? 1 : 0;
   return AMLA_OK;
 }
@@ -124,7 +124,7 @@ int launch_decode_call(const DecodeParams& prm, int* prefix, cudaStream_t stream
   } else {
     int unsupported = 0;
     const cudaError_t err = prm.item_rows > kRowBlock ? launch_decode_quad(prm, stream, &unsupported)
-                                                      : launch_decode_tc(prm, stream, &unsupported);
+                                                      : launch_decode_pair(prm, stream, &unsupported);
     if (err != cudaSuccess) {
       cudaGetLastError();
       return unsupported ? AMLA_ERR_UNSUPPORTED : AMLA_ERR_CUDA;

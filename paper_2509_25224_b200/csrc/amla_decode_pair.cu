@@ -1,0 +1,737 @@
+// Tensor-core MLA decode kernel for sequences of up to 128 query rows, sm_100a.
+//
+// A cluster of two CTAs works on one 128-row block of query rows and a range of 64-key cache pages.  Both CTAs do the
+// same work on 64 rows each; every matrix product is an MMA over the pair (tcgen05.mma.cta_group::2, M = 128, N up to
+// 256), so each CTA supplies its own 64 rows of A and HALF of the B operand:
+//
+//   S = Q K^T     A = Q (64 rows x 576, shared memory), B = K: CTA j loads keys 32 j .. 32 j + 31 of every page
+//   O += P~ V     A = P~ (64 rows x 64 keys per page, shared memory), B = V: CTA j loads columns 256 j .. 256 j + 255
+//
+// With M = 128 over two CTAs the accumulators use all 128 tensor-memory lanes of either CTA: lanes 0-63 hold the CTA's
+// 64 rows for the first half of the N columns, lanes 64-127 the same rows for the second half.  S of four pages
+// (256 keys) takes 128 columns, O (512 columns of V) takes 256, so S is double buffered and Q need not go into tensor
+// memory: it is an operand as soon as TMA has delivered it.
+//
+// Warps 0-7 run Algorithm 2's recurrence (lines 5-12; four threads share a query row: lane half = key half of a page,
+// warp group = even / odd pages), write P~ = bf16(P * S16) into the P buffer of their own CTA, apply the integer N to
+// the bit patterns of O when the row's reference moved (lines 13-16; Lemma 3.1) and run the epilogue (line 20).  They
+// never hand data to the other CTA.  Warps 8 and 10 load (TMA), warp 9 of the even CTA issues the MMAs for both.
+// Order on the tensor pipe: QK^T(i + 1) before P~V(i), across units too (the paper's [C1, C2, V1] order, Section 4.1).
+//
+// Why this split.  The kernel before it gave one CTA of the pair Q K^T and the other P~ V (M = 128 on one SM each): P~
+// crossed to the other SM by remote stores, Q went through shared memory into tensor memory and the score CTA had to be
+// drained before the next unit's Q could follow.  Here nothing but MMA operands crosses, Q is an operand as it lands, and
+// the tile is 256 keys.  192 sequences of 1-512 keys: 62.0 -> 50.0 us; one sequence of 2531: 34.3 -> 31.7; 16 x 16384 with
+// rising logits: 103.8 -> 101.5; 96 x 2048: 88.4 -> 85.5; 32 x 4096: 58.4 both (sustained, at the power cap).
+// What bounds it: a tile of 256 keys takes 8200-8700 clk against 4350 of MMAs and 6000 of HBM at its full rate.  A CTA
+// takes 275 KB per tile through a ring of 112 KB, whose slots turn around in ~2700 clk (load 1500-2000, MMA, commit,
+// next load).  With the MMAs left out the tile still takes 7400.
+//
+// All waits are bounded; on expiry the kernel records kStatusTimeout and unwinds.
+#include <atomic>
+#include <type_traits>
+
+#include "amla_common.cuh"
+#include "amla_sm100.cuh"
+#include "amla_epilogue.cuh"
+#include "amla_units.cuh"
+
+namespace amla {
+
+using namespace sm100;
+
+namespace {
+
+constexpr int kSoftmaxWarps = 8;
+constexpr int kLoaders = 2;                             // warps 8 and 10
+constexpr int kThreads = 32 * (kSoftmaxWarps + kLoaders + 1);
+constexpr int kTilePages = 4;                           // pages of a score tile: N = 256, the widest MMA
+constexpr int kCtaRows = kRowBlock / 2;                 // query rows per CTA
+constexpr int kQBlocks = kDqk / 64;                     // 64-column blocks of Q and K
+constexpr uint32_t kQBlockBytes = kCtaRows * 128;       // [64 rows][128 B], 128-byte swizzle
+constexpr uint32_t kQBytes = kQBlocks * kQBlockBytes;
+constexpr uint32_t kPPageBytes = kCtaRows * 128;        // P~ of one page: [64 rows][64 keys]
+constexpr uint32_t kKBoxBytes = 32 * 128;               // this CTA's half of a page x one 64-column block
+constexpr uint32_t kSlotBytes = 128 * 128;              // K: 4 pages x 32 keys x 64 columns; V: 64 keys x 128 columns
+constexpr uint32_t kVBlockBytes = 64 * 128;             // 64 keys x 64 columns
+constexpr int kSlots = 7;
+
+constexpr uint32_t kOffQ = 0;
+constexpr uint32_t kOffP = kOffQ + kQBytes;
+constexpr uint32_t kOffRing = kOffP + kTilePages * kPPageBytes;
+constexpr uint32_t kOffXchg = kOffRing + kSlots * kSlotBytes;      // float [2][4 threads of a row][64 rows]
+constexpr uint32_t kOffBars = kOffXchg + 2 * 4 * kCtaRows * 4;
+constexpr uint32_t kBarBytes = 256;
+// a copy of the schedule prefix and of the sequence lengths for batches of up to kSmemPlanItems items, so that the
+// roles' schedule look-ups (a dozen dependent loads per unit) stay on chip
+constexpr int kSmemPlanItems = 512;
+constexpr uint32_t kOffPlan = kOffBars + kBarBytes;
+constexpr uint32_t kOffSeqlens = kOffPlan + ((kSmemPlanItems + 1) * 4 + 15) / 16 * 16;
+constexpr uint32_t kSmemBytes = kOffSeqlens + kSmemPlanItems * 4;
+static_assert(kSmemBytes <= 232448, "exceeds the shared memory a block can opt in to");
+static_assert(kOffP % 1024 == 0 && kOffRing % 1024 == 0, "swizzled tiles need 1024-byte alignment");
+
+// tensor-memory columns
+constexpr uint32_t kTmemCols = 512;
+constexpr uint32_t kOCol = 0;            // 256 columns
+constexpr uint32_t kSCol = 256;          // 2 x 128 columns
+
+// Barriers.  (L): the copy in the even CTA is the one that counts; both CTAs arrive there.  The others exist in both
+// CTAs and complete by multicast commits of the even CTA's MMA warp, except X_XCHG, which is local.
+enum { X_FULL = 0 /*L*/, X_EMPTY = X_FULL + kSlots, X_QFULL = X_EMPTY + kSlots /*L*/, X_QFREE, X_SFULL, X_SEMPTY = X_SFULL + 2 /*L*/,
+       X_PREADY = X_SEMPTY + 2 /*L*/, X_PVDONE, X_XCHG, X_NUM = X_XCHG + 2 };
+constexpr uint32_t kTmemSlotOff = kBarBytes - 8;
+static_assert(X_NUM * 8 + 8 <= kBarBytes, "barrier area too small");
+
+__device__ __forceinline__ void report_timeout(int* status) { atomicExch(status, kStatusTimeout); }
+
+// Wait whose verdict is the same in every lane of the warp, so that the warp-collective tensor-memory instructions
+// that follow are never executed by a part of it.
+template <bool kClusterAcquire = false>
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait<kClusterAcquire>(bar, parity));
+}
+
+// What the loader keeps of a score tile: the page of lane l (pages [t, t + np) of the item), the Q row of its unit.
+struct TileRef {
+  int np, page, qrow;
+  bool first, last, valid;
+};
+
+using Tiles = TileIter<kTilePages>;
+
+}  // namespace
+
+template <int kMode, bool kGuard>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap q_map,
+                   const DecodeParams prm) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const uint32_t smem_base = smem_u32(smem_raw);
+  const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+  const int rank = static_cast<int>(cluster_ctarank());
+  const bool leader = rank == 0;
+  const int part = blockIdx.x >> 1;
+  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 0);
+  if (smem_base & 1023u) {   // the swizzled tiles assume a 1024-byte aligned window; identical in both CTAs
+    if (tid == 0) report_timeout(prm.status);
+    return;
+  }
+  const uint32_t bars = smem_base + kOffBars;
+  auto bar = [&](int i) { return bars + 8u * i; };
+  const uint32_t tmem_slot = bars + kTmemSlotOff;
+  const uint32_t lead_bars = map_to_cta(bars, 0);
+
+  // The lengths of the first 32 items are requested before anything else, so that their latency runs under the set-up
+  // below (they are inputs of the call: no kernel that this one may overlap with writes them).
+  int early_len = 0;
+  if (wid == 0 && prm.fused_plan && lane < prm.n_items) early_len = prm.seqlens[lane / prm.nrb];
+  if (tid == 32 * 8) {
+    for (int i = 0; i < kSlots; ++i) { mbar_init(bar(X_FULL + i), 1); mbar_init(bar(X_EMPTY + i), 1); }
+    mbar_init(bar(X_QFULL), 1);
+    mbar_init(bar(X_QFREE), 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar(X_SFULL + i), 1);
+      mbar_init(bar(X_SEMPTY + i), 2 * kSoftmaxWarps);
+      mbar_init(bar(X_XCHG + i), kSoftmaxWarps / 2);
+    }
+    mbar_init(bar(X_PREADY), 2 * kSoftmaxWarps);
+    mbar_init(bar(X_PVDONE), 1);
+    fence_mbar_init();
+    prefetch_tensormap(&k_map);
+    prefetch_tensormap(&v_map);
+    prefetch_tensormap(&q_map);
+  }
+  if (wid == 9) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
+  tc_fence_before_sync();
+  __syncthreads();
+  cluster_arrive();
+  cluster_wait();          // the peer's barriers are initialised before anyone signals them
+  tc_fence_after_sync();
+  const uint32_t tbase = ld_shared_b32(tmem_slot);
+
+  // Launched with programmatic stream serialization: everything above ran while the kernel before this one on the
+  // stream was still going; its results (the schedule kernel's prefix array, or the previous call's reads of the
+  // workspace) are complete after this wait.
+  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 3);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 4);
+  const int* prefix = prm.prefix;
+  const int* seqlens = prm.seqlens;
+  if (prm.fused_plan) {
+    // Few items: every CTA computes the schedule prefix itself instead of waiting for a one-block kernel (the combine
+    // kernel reads the copy that the first CTA leaves in the workspace).  A small batch's prefix and sequence lengths
+    // stay in shared memory; of a larger one every CTA writes the same values to the workspace.
+    int* ps = prm.n_items <= kSmemPlanItems ? reinterpret_cast<int*>(smem_raw + kOffPlan) : nullptr;
+    if (wid == 0) {
+      int* pw = !ps || blockIdx.x == 0 ? const_cast<int*>(prm.prefix) : nullptr;
+      int carry = 0;
+      for (int base = 0; base < prm.n_items; base += 32) {
+        const int it = base + lane;
+        const int n_seq = it >= prm.n_items ? 0 : base == 0 ? early_len : prm.seqlens[it / prm.nrb];
+        if (ps && it < prm.n_items) reinterpret_cast<int*>(smem_raw + kOffSeqlens)[it / prm.nrb] = n_seq;   // same value from every row block
+        const int v = it < prm.n_items ? schedule_length(n_seq, it, prm.tile_keys, prm.ovh) : 0;
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        if (it < prm.n_items) {
+          if (pw) pw[it] = carry + x - v;
+          if (ps) ps[it] = carry + x - v;
+        }
+        carry += __shfl_sync(0xffffffffu, x, 31);
+      }
+      if (lane == 0) {
+        if (pw) pw[prm.n_items] = carry;
+        if (ps) ps[prm.n_items] = carry;
+        if (blockIdx.x == 0) *prm.status = kStatusOk;
+      }
+      __threadfence_block();
+    }
+    __syncthreads();
+    if (ps) { prefix = ps; seqlens = reinterpret_cast<const int*>(smem_raw + kOffSeqlens); }
+  }
+
+  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 1);
+  bool ok = true;
+  Tiles tile(UnitIter(prm, prefix, seqlens, part));
+  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 5);
+
+  if (wid < kSoftmaxWarps) {
+    // ======================================================== softmax, correction, epilogue
+    const int quarter = wid & 3, grp = wid >> 2;
+    const int khalf = quarter >> 1;                      // S: key half of every page; O: which 256 columns
+    const int r = (quarter & 1) * 32 + lane;             // query row within this CTA's 64
+    const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
+    const bool scale_nonneg = prm.scale_log2 >= 0.f;
+    const uint32_t mask_fill = __float_as_uint(scale_nonneg ? -INFINITY : INFINITY);
+    const uint32_t xbar = bar(X_XCHG + (quarter & 1));
+    const uint32_t prow_smem = smem_base + kOffP + r * 128;
+    const uint32_t o_addr = tbase + lane_base + kOCol + 128 * grp;     // this thread's 128 of the row's 512 columns
+    uint32_t gs = 0, xc = 0;                             // score tiles and exchanges so far
+    // tells the row's other three threads `mine`; v[0..3] = what the four told
+    auto exchange = [&](float mine, float (&v)[4]) {
+      const uint32_t buf = smem_base + kOffXchg + (xc & 1) * (4 * kCtaRows * 4) + r * 4;
+      st_shared_b32(buf + (2 * khalf + grp) * (kCtaRows * 4), __float_as_uint(mine));
+      __syncwarp();
+      if (lane == 0) mbar_arrive(xbar);
+      ok = warp_wait(xbar, xc & 1);
+      ++xc;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(ld_shared_b32(buf + i * (kCtaRows * 4)));
+    };
+
+    while (ok && tile.valid) {
+      const Unit u = tile.u;
+      const int row = u.r0 + rank * kCtaRows + r;        // row within the sequence
+      const int tok = row / prm.H;
+      const int visible = min(u.n_b, u.n_b - prm.Sq + tok + 1);        // keys 0..visible-1 are seen by this row
+      const int first_masked = max(u.n_b - prm.Sq + 1, 0) / kPage;     // pages from here on may hold hidden keys
+      RowState st;
+      row_state_init(st);
+      bool more = true;
+      while (more) {
+        const uint32_t sb = gs & 1;
+        const int t = tile.t, np = tile.np;
+        ok = warp_wait(bar(X_SFULL + sb), (gs >> 1) & 1);
+        if (!ok) break;
+        tc_fence_after_sync();
+        if (tid == 0 && leader) AMLA_STAMP(prm, part, 8, gs);
+        // this group's pages of the tile: t + grp and t + grp + 2 (32 columns each, 32 keys per lane half)
+        const uint32_t scol = tbase + lane_base + kSCol + 128 * sb + 32 * grp;
+        const bool has0 = grp < np, has1 = grp + 2 < np;
+        const int nvis0 = has0 ? visible - (t + grp) * kPage - 32 * khalf : 0;
+        const int nvis1 = has1 ? visible - (t + grp + 2) * kPage - 32 * khalf : 0;
+        uint32_t b0[32], b1[32];
+        tmem_ld_32x32b_x32(scol, b0);
+        tmem_ld_32x32b_x32(scol + 64, b1);
+        tmem_wait_ld();
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) { if (leader) mbar_arrive(bar(X_SEMPTY + sb)); else mbar_arrive_cluster_relaxed(lead_bars + 8u * (X_SEMPTY + sb)); }
+
+        // Two compilations of the tile: the plain one (both pages there, every key visible, non-negative scale) and the
+        // general one with the visibility masks and the sign of the scale.
+        auto tile_body = [&](auto general_c) {
+          constexpr bool kGeneral = decltype(general_c)::value;
+          const bool scale_nn = kGeneral ? scale_nonneg : true;
+          // lines 5-6: running max on the raw scores (the scale is folded into the FMA below)
+          float ext = scale_nn ? -INFINITY : INFINITY, ext_b = ext;
+          auto chunk_max = [&](uint32_t (&v)[32], int nvis) {
+            if (kGeneral) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) v[i] = (i < nvis) ? v[i] : mask_fill;
+            }
+            if (scale_nn) {
+#pragma unroll
+              for (int i = 0; i < 32; i += 4) {
+                ext = fmax3(ext, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+                ext_b = fmax3(ext_b, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
+              }
+            } else {
+#pragma unroll
+              for (int i = 0; i < 32; i += 4) {
+                ext = fminf(ext, fminf(__uint_as_float(v[i]), __uint_as_float(v[i + 1])));
+                ext_b = fminf(ext_b, fminf(__uint_as_float(v[i + 2]), __uint_as_float(v[i + 3])));
+              }
+            }
+          };
+          chunk_max(b0, nvis0);
+          chunk_max(b1, nvis1);
+          ext = scale_nn ? fmaxf(ext, ext_b) : fminf(ext, ext_b);
+          const float mine = (nvis0 > 0 || nvis1 > 0) ? ext * prm.scale_log2 : -INFINITY;
+          float m4[4];
+          exchange(mine, m4);
+          if (!ok) return;
+          if (tid == 0 && leader) AMLA_STAMP(prm, part, 9, gs);
+          const float tmax = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+          // Lazy reference: a row must move when its maximum exceeds the reference by more than tau.  The four warps of
+          // these 32 rows pay for a rescale as soon as one row moves, so when one must, every row of the warp whose
+          // maximum rose moves with it (moving early is always allowed: tau = 0 moves at every rise); the rows then tend
+          // to stay in step and O is rescaled on far fewer tiles.  The four warps see the same maxima and agree.
+          const bool must = tmax > st.m2 + prm.tau;
+          const RowStep sp = row_step<kMode>(st, tmax, __any_sync(0xffffffffu, must) ? 0.f : prm.tau);
+          // Line 10's factor S16 goes into the exponential's argument (the remark after Algorithm 2).  The row sum of
+          // line 6 is the sum of the same FP32 values, taken before the bf16 cast and divided by S16 once per tile.
+          const float nsub = log2f_approx(sp.p_scale) - sp.m2_sub;
+          float rs0 = 0.f, rs1 = 0.f;
+          const uint64_t sc2 = pack_f32x2(prm.scale_log2, prm.scale_log2), ns2 = pack_f32x2(nsub, nsub);
+          uint64_t rsa = pack_f32x2(0.f, 0.f), rsb = rsa;
+          uint32_t pk[32];
+          auto chunk_exp = [&](const uint32_t (&v)[32], int nvis, int k0) {
+            if (kGeneral) {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                float p0 = ex2_approx(fmaf(__uint_as_float(v[2 * i]), prm.scale_log2, nsub));
+                float p1 = ex2_approx(fmaf(__uint_as_float(v[2 * i + 1]), prm.scale_log2, nsub));
+                p0 = (2 * i < nvis) ? p0 : 0.f;
+                p1 = (2 * i + 1 < nvis) ? p1 : 0.f;
+                rs0 += p0; rs1 += p1;
+                pk[k0 + i] = pack_bf16x2(p0, p1);
+              }
+            } else {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                float x0, x1;
+                unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), sc2, ns2), x0, x1);
+                const float q0 = ex2_approx(x0), q1 = ex2_approx(x1);
+                const uint64_t pp = pack_f32x2(q0, q1);
+                if (i & 1) rsb = add_f32x2(rsb, pp); else rsa = add_f32x2(rsa, pp);
+                pk[k0 + i] = pack_bf16x2(q0, q1);
+              }
+            }
+          };
+          chunk_exp(b0, nvis0, 0);
+          chunk_exp(b1, nvis1, 16);
+          {
+            float s0, s1;
+            unpack_f32x2(add_f32x2(rsa, rsb), s0, s1);
+            st.l = st.l * sp.l_up + __fdividef((rs0 + s0) + (rs1 + s1), sp.p_scale);   // this thread's share of the row sum
+          }
+          if (tid == 0 && leader) AMLA_STAMP(prm, part, 10, gs);
+          if (!tile.first) {
+            // the P~V of the tile before: it has read the P buffer, and O holds its sum
+            ok = warp_wait(bar(X_PVDONE), (gs - 1) & 1);
+            if (!ok) return;
+            const uint32_t nword = (kMode == 2) ? __float_as_uint(sp.l_up) : static_cast<uint32_t>(sp.n_bits);
+            const bool mine_moved = (kMode == 2) ? (sp.l_up != 1.f) : (sp.n_bits != 0);
+            if (__any_sync(0xffffffffu, mine_moved)) {
+              // lines 13-16: O <- AS_FP32(AS_INT32(O) + N).  The guarded add costs four integer operations per element,
+              // the FP32 multiply it replaces one.  The guard only matters for an element whose magnitude bits plus N
+              // would not stay positive (an exact zero, a value about to leave the normal range); so the smallest
+              // magnitude of the chunk is taken first (half an operation per element), and where it is safe the chunk
+              // gets the plain one-instruction add of Lemma 3.1.
+              tc_fence_after_sync();
+              auto apply = [&](uint32_t (&o)[32]) {
+                if (kMode == 2) {
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * __uint_as_float(nword));
+                } else if (!kGuard) {
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_raw(__uint_as_float(o[i]), static_cast<int>(nword)));
+                } else {
+                  float lo = fmin3_abs(__uint_as_float(o[0]), __uint_as_float(o[1]), __uint_as_float(o[2]));
+#pragma unroll
+                  for (int i = 3; i + 1 < 32; i += 2) lo = fmin3_abs(lo, __uint_as_float(o[i]), __uint_as_float(o[i + 1]));
+                  lo = fminf(lo, fabsf(__uint_as_float(o[31])));
+                  // NaN magnitudes compare as large numbers and take the plain add, like every other normal pattern
+                  if (__float_as_int(lo) + static_cast<int>(nword) > 0) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_raw(__uint_as_float(o[i]), static_cast<int>(nword)));
+                  } else {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_guarded(__uint_as_float(o[i]), static_cast<int>(nword)));
+                  }
+                }
+              };
+#pragma unroll 1
+              for (int c = 0; c < 4; ++c) {
+                uint32_t o[32];
+                tmem_ld_32x32b_x32(o_addr + 32 * c, o);
+                tmem_wait_ld();
+                apply(o);
+                tmem_st_32x32b_x32(o_addr + 32 * c, o);
+              }
+              tmem_wait_st();
+              tc_fence_before_sync();
+            }
+          }
+          if (tid == 0 && leader) AMLA_STAMP(prm, part, 11, gs);
+          if (has0) {
+            const uint32_t dst = prow_smem + grp * kPPageBytes;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              st_shared_v4(dst + (((4 * khalf + c) ^ (r & 7)) << 4), pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+          }
+          if (has1) {
+            const uint32_t dst = prow_smem + (grp + 2) * kPPageBytes;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              st_shared_v4(dst + (((4 * khalf + c) ^ (r & 7)) << 4), pk[16 + 4 * c], pk[16 + 4 * c + 1], pk[16 + 4 * c + 2], pk[16 + 4 * c + 3]);
+          }
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) { if (leader) mbar_arrive(bar(X_PREADY)); else mbar_arrive_cluster_relaxed(lead_bars + 8u * X_PREADY); }
+          if (tid == 0 && leader) AMLA_STAMP(prm, part, 12, gs);
+        };
+        if (!has1 || t + np > first_masked || !scale_nonneg) tile_body(std::true_type{});
+        else tile_body(std::false_type{});
+        if (!ok) break;
+        ++gs;
+        more = !tile.last();
+        if (more) tile.next();
+      }
+      if (!ok) break;
+      // ---- epilogue (line 20): out = O / (l * S16), lse = m + ln l.  Thread = row; the four threads of a row take 128
+      // of its 512 columns each and store them from registers with 256-bit stores (a full 32-byte sector per lane).
+      int2 info;
+      const int slot = tile.units.slot_of(u, &info);
+      if (tid == 0 && leader) prm.item_info[u.it] = info;
+      float l4[4];
+      exchange(st.l, l4);
+      if (!ok) break;
+      const float l_all = (l4[0] + l4[1]) + (l4[2] + l4[3]);
+      const bool live = l_all > 0.f;
+      const float inv = live ? prm.out_scale / (l_all * st.s_out) : 0.f;
+      const float lse = live ? (st.m2 + log2f(l_all)) * kLn2 : -INFINITY;
+      ok = warp_wait(bar(X_PVDONE), (gs - 1) & 1);
+      if (!ok) break;
+      tc_fence_after_sync();
+      if (tid == 0 && leader) AMLA_STAMP(prm, part, 13, gs - 1);
+      const bool valid = row < prm.R;
+      const int col0 = 256 * khalf + 128 * grp;
+      const size_t prow = static_cast<size_t>(slot < 0 ? 0 : slot) * kRowBlock + rank * kCtaRows + r;   // row of the partial arrays
+      uint16_t* dst = slot < 0 ? reinterpret_cast<uint16_t*>(prm.out) + (static_cast<size_t>(u.b) * prm.R + (valid ? row : 0)) * kDv + col0
+                               : partial_halves(prm) + prow * kDv + col0;
+      uint32_t sc = 0;                                    // this thread's four scale bytes
+      uint32_t o[2][32];
+      tmem_ld_32x32b_x32(o_addr, o[0]);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        tmem_wait_ld();
+        if (c + 1 < 4) tmem_ld_32x32b_x32(o_addr + 32 * (c + 1), o[(c + 1) & 1]);
+        uint32_t w[16];
+        if (slot < 0) epilogue_chunk_bf16(o[c & 1], inv, w);
+        else sc |= epilogue_chunk_partial(o[c & 1], inv, w) << (8 * c);
+        if (valid) {
+          stg_256(dst + 32 * c, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+          stg_256(dst + 32 * c + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+        }
+      }
+      tc_fence_before_sync();      // O has been read: this warp's next PREADY arrival lets the next unit overwrite it
+      if (valid) {
+        if (slot >= 0) *reinterpret_cast<uint32_t*>(partial_scales(prm) + prow * 16 + col0 / 32) = sc;
+        if (khalf == 0 && grp == 0) {
+          if (slot < 0) prm.lse[static_cast<size_t>(u.b) * prm.R + row] = lse;
+          else prm.part_lse[prow] = lse;
+        }
+      }
+      if (tid == 0 && leader) AMLA_STAMP(prm, part, 14, gs - 1);
+      tile.next();
+    }
+    if (!ok && lane == 0) report_timeout(prm.status);
+  } else if (wid == 8 || wid == 10) {
+    // ======================================================== TMA loads, in the order in which the MMAs use them:
+    // Q, K(0), K(1), V(0), K(2), V(1), ..., K(n-1), V(n-2), V(n-1), next unit.  One ring of 16 KB slots carries K (one
+    // 64-column block of the tile's keys, one box per page, each issued by its own lane) and V (one page x 128
+    // columns).  The two loader warps walk the same sequence and issue every second load of it.  Q is the first's: it is
+    // requested as soon as the QK^T of the unit before have let go of the buffer, if need be between the V loads of that
+    // unit's last tile.
+    const uint32_t mine = wid == 8 ? 0u : 1u;
+    const uint64_t keep = l2_policy_evict_normal(), last_use = l2_policy_evict_first();   // K: V follows a tile later; V: done with
+    uint32_t slot = 0, par = 1;
+    uint32_t n_issued = 0;
+    uint32_t un = 0;                                      // units whose Q has been requested
+    auto take = [&]() -> TileRef {
+      TileRef x;
+      x.valid = tile.valid;
+      x.np = 0; x.page = 0; x.qrow = 0; x.first = x.last = false;
+      if (x.valid) {
+        x.np = tile.np; x.first = tile.first; x.last = tile.last();
+        x.qrow = tile.u.b * prm.R + tile.u.r0 + rank * kCtaRows;
+        if (lane < x.np) x.page = __ldg(prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t + lane);
+        tile.next();
+      }
+      return x;
+    };
+    auto advance = [&]() { if (++slot == kSlots) { slot = 0; par ^= 1; } ++n_issued; };
+    auto issue_q = [&](int qrow) {
+      if (leader) mbar_arrive_expect_tx_elect(bar(X_QFULL), 2 * kQBytes);
+#pragma unroll
+      for (int c = 0; c < kQBlocks; c += 3)
+        tma_load_3d_pair_elect(smem_base + kOffQ + c * kQBlockBytes, &q_map, 0, qrow, c, lead_bars + 8u * X_QFULL, last_use);
+      ++un;
+    };
+    // What a load needs is at hand before its slot is waited for: the slot's turn-around is on the critical path of a
+    // ring that holds little more than the latency of memory.
+    auto issue_v = [&](int np, int page, int nxt_qrow, bool q_wanted, bool& q_out) {
+#pragma unroll 1
+      for (int i = 0; i < 2 * np; ++i) {
+        if ((n_issued & 1) == mine) {
+          if (q_wanted && !q_out && __all_sync(0xffffffffu, mbar_probe(bar(X_QFREE), (un - 1) & 1))) { issue_q(nxt_qrow); q_out = true; }
+          const int row = __shfl_sync(0xffffffffu, page, i >> 1) * kPage;
+          const uint32_t dst = smem_base + kOffRing + slot * kSlotBytes, full = bar(X_FULL + slot), lead_full = lead_bars + 8u * (X_FULL + slot);
+          ok = warp_wait(bar(X_EMPTY + slot), par);
+          if (!ok) return;
+          if (leader) mbar_arrive_expect_tx_elect(full, 2 * kSlotBytes);
+          tma_load_3d_pair_elect(dst, &v_map, 0, row, 4 * rank + 2 * (i & 1), lead_full, last_use);
+        }
+        advance();
+      }
+    };
+    TileRef cur = take(), nxt = take();
+    int np_prev = 0;
+    int page_prev = 0;
+    bool q_out = false;                                   // the Q of the unit that starts next has been requested
+    uint32_t pt = 0;
+    while (ok && cur.valid) {
+      if (cur.first && mine == 0) {
+        if (!q_out) {
+          if (un > 0) ok = warp_wait(bar(X_QFREE), (un - 1) & 1);
+          if (!ok) break;
+          issue_q(cur.qrow);
+        }
+        q_out = false;
+      }
+      int row[kTilePages];                                // first key row of the tile's pages
+#pragma unroll
+      for (int p = 0; p < kTilePages; ++p) row[p] = __shfl_sync(0xffffffffu, cur.page, p) * kPage;
+      const TileRef nn = take();
+#pragma unroll 1
+      for (int c = 0; c < kQBlocks; ++c) {
+        if ((n_issued & 1) == mine) {
+          const uint32_t dst = smem_base + kOffRing + slot * kSlotBytes, full = bar(X_FULL + slot), lead_full = lead_bars + 8u * (X_FULL + slot);
+          ok = warp_wait(bar(X_EMPTY + slot), par);
+          if (!ok) break;
+          if (lane == 0 && leader && (c <= 1 || c >= 7)) AMLA_STAMP(prm, part, c <= 1 ? 16 : 17, pt);
+          if (leader) mbar_arrive_expect_tx_elect(full, 2 * cur.np * kKBoxBytes);
+#pragma unroll
+          for (int p = 0; p < kTilePages; ++p)
+            if (p < cur.np) tma_load_3d_pair_elect(dst + p * kKBoxBytes, &k_map, 0, row[p] + 32 * rank, c, lead_full, keep);
+        }
+        advance();
+      }
+      if (!ok) break;
+      if (!cur.first) issue_v(np_prev, page_prev, 0, false, q_out);
+      if (ok && cur.last) issue_v(cur.np, cur.page, nxt.qrow, mine == 0 && nxt.valid, q_out);
+      np_prev = cur.np;
+      page_prev = cur.page;
+      cur = nxt;
+      nxt = nn;
+      ++pt;
+    }
+    if (!ok) {
+      if (lane == 0) report_timeout(prm.status);
+      // let the copies that may still be in flight land before the CTA exits
+      if (leader) {
+        for (uint32_t i = 0; i < kSlots && i < n_issued; ++i) {
+          const uint32_t k = n_issued - 1 - i;
+          if ((k & 1) == mine) mbar_wait(bar(X_FULL + k % kSlots), (k / kSlots) & 1);
+        }
+        if (un > 0) mbar_wait(bar(X_QFULL), (un - 1) & 1);
+      }
+    }
+  } else if (leader && wid == 9) {
+    // ======================================================== MMA issuer (even CTA, for the pair)
+    constexpr uint32_t idesc_pv = make_idesc_bf16(128, 256, false, true);
+    constexpr uint32_t idesc_qk1 = make_idesc_bf16(128, 64, false, false);     // N = 64 per page
+    constexpr uint32_t idesc_step = make_idesc_bf16(128, 128, false, false) - idesc_qk1;
+    constexpr uint32_t dhi = smem_desc_hi_sw128(1024);
+    const uint32_t qlo = smem_desc_lo(smem_base + kOffQ, 16);
+    const uint32_t plo = smem_desc_lo(smem_base + kOffP, 16);
+    const uint32_t klo = smem_desc_lo(smem_base + kOffRing, 16);
+    const uint32_t vlo = smem_desc_lo(smem_base + kOffRing, kVBlockBytes);
+    uint32_t slot = 0, par = 0;
+    uint32_t gs = 0, gp = 0, un = 0;                      // score tiles, P~V tiles, units so far
+    auto advance = [&]() { if (++slot == kSlots) { slot = 0; par ^= 1; } };
+    // O (+)= P~ V of one tile: per page two N = 256 products (128 columns from either CTA)
+    auto pv = [&](int np, bool fresh) {
+      if (lane == 0) AMLA_STAMP(prm, part, 4, gp);
+      ok = warp_wait<true>(bar(X_PREADY), gp & 1);
+      if (!ok) return;
+      if (lane == 0) AMLA_STAMP(prm, part, 5, gp);
+      tc_fence_after_sync();               // the softmax warps may have rewritten O (tcgen05.st) before arriving
+      for (int p = 0; p < np; ++p) {
+        const uint32_t pl = plo + p * (kPPageBytes >> 4);
+#pragma unroll
+        for (int nh = 0; nh < 2; ++nh) {
+          ok = ok && warp_wait(bar(X_FULL) + 8 * slot, par);
+          if (!ok) return;
+          if (p == 0 && nh == 0 && lane == 0) AMLA_STAMP(prm, part, 6, gp);
+          const uint32_t vl = vlo + slot * (kSlotBytes >> 4);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            mma_ss_pair_elect(tbase + kOCol + 128 * nh, smem_desc_join(pl + 2 * kk, dhi), smem_desc_join(vl + 128 * kk, dhi), idesc_pv,
+                        (kk == 0 && p == 0 && fresh) ? 0u : 1u);
+          mma_commit_pair_multicast_elect(bar(X_EMPTY) + 8 * slot, 3);
+          advance();
+        }
+      }
+      mma_commit_pair_multicast_elect(bar(X_PVDONE), 3);
+      if (lane == 0) AMLA_STAMP(prm, part, 7, gp);
+      ++gp;
+    };
+    int np_prev = 0;
+    bool fresh = true;
+    while (ok && tile.valid) {
+      if (tile.first) {
+        ok = warp_wait(bar(X_QFULL), un & 1);
+        if (!ok) break;
+        ++un;
+      }
+      {
+        const uint32_t sb = gs & 1;
+        if (lane == 0) AMLA_STAMP(prm, part, 0, gs);
+        ok = warp_wait<true>(bar(X_SEMPTY + sb), ((gs >> 1) & 1) ^ 1);
+        if (!ok) break;
+        tc_fence_after_sync();
+        if (lane == 0) AMLA_STAMP(prm, part, 1, gs);
+        const uint32_t d = tbase + kSCol + 128 * sb;
+        const uint32_t idesc = idesc_qk1 + (tile.np - 1) * idesc_step;
+#pragma unroll
+        for (int c = 0; c < kQBlocks; ++c) {
+          ok = ok && warp_wait(bar(X_FULL) + 8 * slot, par);    // TMA data -> MMA operand: both async proxy, no fence needed
+          if (ok) {
+            if (c == 0 && lane == 0) AMLA_STAMP(prm, part, 2, gs);
+            const uint32_t kl = klo + slot * (kSlotBytes >> 4);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              mma_ss_pair_elect(d, smem_desc_join(qlo + c * (kQBlockBytes >> 4) + 2 * kk, dhi), smem_desc_join(kl + 2 * kk, dhi), idesc, (c | kk) != 0 ? 1u : 0u);
+            mma_commit_pair_multicast_elect(bar(X_EMPTY) + 8 * slot, 3);
+          }
+          advance();
+        }
+        if (!ok) break;
+        mma_commit_pair_multicast_elect(bar(X_SFULL + sb), 3);
+        if (tile.last()) mma_commit_pair_multicast_elect(bar(X_QFREE), 3);
+        if (lane == 0) AMLA_STAMP(prm, part, 3, gs);
+        ++gs;
+      }
+      const int np = tile.np;
+      const bool first = tile.first, last = tile.last();
+      if (!first) { pv(np_prev, fresh); fresh = false; }
+      if (last) { if (ok) pv(np, first); fresh = true; }
+      np_prev = np;
+      if (ok) tile.next();
+    }
+    if (!ok && lane == 0) report_timeout(prm.status);
+  }
+
+  if (tid == 0 && leader) if (lane == 0) AMLA_STAMP(prm, part, 20, 2);
+  // teardown: nobody may still be signalling a CTA that has exited, and both CTAs must be done with tensor memory
+  tc_fence_before_sync();
+  __syncthreads();
+  cluster_arrive();
+  cluster_wait();
+  if (wid == 9) tmem_dealloc_pair(tbase, kTmemCols);
+}
+
+// ---------------------------------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------------------------------
+namespace {
+
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeTiledFn get_encode_fn() {
+  static std::atomic<EncodeTiledFn> fn{nullptr};
+  EncodeTiledFn f = fn.load(std::memory_order_acquire);
+  if (!f) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
+        qres == cudaDriverEntryPointSuccess) {
+      f = reinterpret_cast<EncodeTiledFn>(p);
+      fn.store(f, std::memory_order_release);
+    }
+  }
+  return f;
+}
+
+// Rows of 576 bf16 seen as (64 columns, rows, 9 column blocks); a box is box_rows x box_blocks, laid out in shared
+// memory as [block][row][128 B] with the 128-byte swizzle.
+bool encode_rows(EncodeTiledFn encode, CUtensorMap* map, const void* base, cuuint64_t rows, cuuint32_t box_rows, cuuint32_t box_blocks) {
+  const cuuint64_t dims[3] = {64, rows, static_cast<cuuint64_t>(kQBlocks)};
+  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(kDqk) * 2, 128};
+  const cuuint32_t box[3] = {64, box_rows, box_blocks};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int kMode, bool kGuard>
+cudaError_t launch_variant(const CUtensorMap& kmap, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
+  auto kern = decode_pair_kernel<kMode, kGuard>;
+  // the opt-in to large dynamic shared memory is per device and per kernel; do it once each
+  static std::atomic<uint64_t> done{0};
+  int device = 0;
+  cudaError_t err = cudaGetDevice(&device);
+  if (err != cudaSuccess) return err;
+  const uint64_t bit = 1ull << (device & 63);
+  if (!(done.load(std::memory_order_acquire) & bit)) {
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
+    if (err != cudaSuccess) return err;
+    done.fetch_or(bit, std::memory_order_release);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * prm.P);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, kmap, vmap, qmap, prm);
+}
+
+}  // namespace
+
+// Number of two-CTA clusters the schedule is cut into: one per SM pair.
+int decode_pair_parts(int sm_count) { return sm_count / 2 > 0 ? sm_count / 2 : 1; }
+
+cudaError_t launch_decode_pair(const DecodeParams& prm, cudaStream_t stream, int* unsupported) {
+  *unsupported = 0;
+  EncodeTiledFn encode = get_encode_fn();
+  if (!encode) { *unsupported = 1; return cudaErrorNotSupported; }
+  // K: half a page (32 keys) x one column block; V: a page x two column blocks; Q: a CTA's 64 rows x three column
+  // blocks (rows past the end of the array read as zero, rows of a following sequence are computed and dropped)
+  CUtensorMap kmap, vmap, qmap;
+  const cuuint64_t keys = static_cast<cuuint64_t>(prm.num_blocks) * kPage;
+  if (!encode_rows(encode, &kmap, prm.kv, keys, 32, 1) || !encode_rows(encode, &vmap, prm.kv, keys, 64, 2) ||
+      !encode_rows(encode, &qmap, prm.q, static_cast<cuuint64_t>(prm.B) * prm.R, kCtaRows, 3))
+    return cudaErrorInvalidValue;
+  const int mode = prm.flags & 3;
+  const bool guard = !(prm.flags & 4);
+  if (mode == 0) return guard ? launch_variant<0, true>(kmap, vmap, qmap, prm, stream) : launch_variant<0, false>(kmap, vmap, qmap, prm, stream);
+  if (mode == 1) return guard ? launch_variant<1, true>(kmap, vmap, qmap, prm, stream) : launch_variant<1, false>(kmap, vmap, qmap, prm, stream);
+  return launch_variant<2, true>(kmap, vmap, qmap, prm, stream);
+}
+
+}  // namespace amla

@@ -115,6 +115,16 @@ def test_all_sequences_empty():
     assert np.all(out == 0) and np.all(np.isneginf(lse))
 
 
+@pytest.mark.parametrize("H", [64, 65, 127])
+@pytest.mark.parametrize("lens", [[255], [256], [257], [511, 320, 193], [1025, 31, 32, 33, 97]])
+def test_128_row_kernel_tile_and_row_edges(lens, H):
+    # score tiles of up to four pages whose keys the two CTAs of a cluster share page by page in halves of 32, and 64
+    # query rows per CTA: lengths around a tile, a page and half a page; rows that end in the first or the second CTA
+    w = synth.make_workload("edge128", len(lens), 1, H, lens, seed=450 + sum(lens) + H)
+    check_full(w)
+    check_full(w, binding.RESCALE_ALG2 | binding.lazy(0))
+
+
 def test_many_short_sequences_more_items_than_parts():
     rng = np.random.default_rng(9)
     w = synth.make_workload("m", 200, 1, 128, rng.integers(0, 200, 200), seed=8)
@@ -137,6 +147,13 @@ def test_items_around_the_on_chip_schedule_copy(B):
     # from the workspace
     rng = np.random.default_rng(12 + B)
     w = synth.make_workload("edge", B, 1, 16, rng.integers(0, 300, B), seed=13)
+    check_full(w)
+
+
+@pytest.mark.parametrize("B", [512, 513])
+def test_items_around_the_on_chip_schedule_copy_of_the_128_row_kernel(B):
+    rng = np.random.default_rng(12 + B)
+    w = synth.make_workload("edge", B, 1, 16, rng.integers(0, 200, B), seed=14)
     check_full(w)
 
 
