@@ -94,7 +94,7 @@ void profile_mark(int i, cudaStream_t stream) {
 // AMLA_FLAG_KERNEL_ROWS128 asks for the 128-row kernel.
 int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
   const bool simt = (flags & AMLA_FLAG_KERNEL_SIMT) != 0;
-  bool quad = !simt && !(flags & AMLA_FLAG_KERNEL_ROWS128) && prm.R > kRowBlock;
+  bool quad = !simt && !(flags & AMLA_FLAG_KERNEL_ROWS128) && prm.R > kRowBlock && prm.kv8 == nullptr;
   int quad_parts = 0;
   if (quad) {
     quad_parts = decode_quad_parts(device, sms);
@@ -170,12 +170,12 @@ extern "C" int amla_mla_decode_workspace_size(int B, int Sq, int H, int max_bloc
 
 namespace {
 
-// The decode call on a bf16 cache.  out_scale multiplies the normalised output (1 unless the cache was widened from
+// The decode call on a bf16 cache (kv_cache) or an E4M3 cache (kv8).  out_scale multiplies the normalised output (1 unless the cache was widened from
 // FP8 with a dequantisation scale); launches are added to g_last_launches.
-int decode_impl(const void* q, const void* kv_cache, const int32_t* block_table, const int32_t* seqlens,
+int decode_impl(const void* q, const void* kv_cache, const uint8_t* kv8, const int32_t* block_table, const int32_t* seqlens,
                 float softmax_scale, float out_scale, int B, int Sq, int H, int num_blocks, int max_blocks_per_seq,
                 void* out, float* lse, void* workspace, size_t workspace_bytes, void* cuda_stream, int flags) {
-  if (!q || !kv_cache || !block_table || !seqlens || !out || !lse || !workspace) return AMLA_ERR_INVALID_ARG;
+  if (!q || (!kv_cache && !kv8) || !block_table || !seqlens || !out || !lse || !workspace) return AMLA_ERR_INVALID_ARG;
   if (num_blocks <= 0 || !(softmax_scale == softmax_scale)) return AMLA_ERR_INVALID_ARG;
   int rc = check_shape(B, Sq, H, max_blocks_per_seq);
   if (rc != AMLA_OK) return rc;
@@ -202,6 +202,7 @@ int decode_impl(const void* q, const void* kv_cache, const int32_t* block_table,
   std::memset(&prm, 0, sizeof(prm));
   prm.q = static_cast<const __nv_bfloat16*>(q);
   prm.kv = static_cast<const __nv_bfloat16*>(kv_cache);
+  prm.kv8 = kv8;
   prm.block_table = block_table;
   prm.seqlens = seqlens;
   prm.out = static_cast<__nv_bfloat16*>(out);
@@ -239,7 +240,7 @@ extern "C" int amla_mla_decode_ex(const void* q, const void* kv_cache, const int
                                   int num_blocks, int max_blocks_per_seq, void* out, float* lse,
                                   void* workspace, size_t workspace_bytes, void* cuda_stream, int flags) {
   g_last_launches = 0;
-  return decode_impl(q, kv_cache, block_table, seqlens, softmax_scale, 1.f, B, Sq, H, num_blocks, max_blocks_per_seq, out, lse,
+  return decode_impl(q, kv_cache, nullptr, block_table, seqlens, softmax_scale, 1.f, B, Sq, H, num_blocks, max_blocks_per_seq, out, lse,
                      workspace, workspace_bytes, cuda_stream, flags);
 }
 
@@ -271,6 +272,11 @@ extern "C" int amla_mla_decode_fp8(const void* q, const void* kv_cache_e4m3, flo
   const size_t tbytes = fp8_table_bytes(B, max_blocks_per_seq), pbytes = fp8_pages_bytes(B, max_blocks_per_seq);
   if (workspace_bytes < base + tbytes + pbytes) return AMLA_ERR_WORKSPACE;
   if (static_cast<long long>(B) * max_blocks_per_seq > (1ll << 30)) return AMLA_ERR_UNSUPPORTED;
+  // logits: scale * q . (k8 * kv_scale); output: sum p * (v8 * kv_scale)
+  if (!(flags & AMLA_FLAG_KERNEL_SIMT))
+    return decode_impl(q, nullptr, static_cast<const uint8_t*>(kv_cache_e4m3), block_table, seqlens, softmax_scale * kv_scale, kv_scale, B, Sq, H,
+                       num_blocks, max_blocks_per_seq, out, lse, workspace, base, cuda_stream, flags);
+  // the scalar bring-up kernel reads bf16: the pages are widened first
   char* ws = static_cast<char*>(workspace);
   int32_t* table2 = reinterpret_cast<int32_t*>(ws + base);
   __nv_bfloat16* pages = reinterpret_cast<__nv_bfloat16*>(ws + base + tbytes);
@@ -281,8 +287,7 @@ extern "C" int amla_mla_decode_fp8(const void* q, const void* kv_cache_e4m3, flo
     return AMLA_ERR_CUDA;
   }
   ++g_last_launches;
-  // logits: scale * q . (k8 * kv_scale); output: sum p * (v8 * kv_scale)
-  return decode_impl(q, pages, table2, seqlens, softmax_scale * kv_scale, kv_scale, B, Sq, H, B * max_blocks_per_seq,
+  return decode_impl(q, pages, nullptr, table2, seqlens, softmax_scale * kv_scale, kv_scale, B, Sq, H, B * max_blocks_per_seq,
                      max_blocks_per_seq, out, lse, workspace, base, cuda_stream, flags);
 }
 

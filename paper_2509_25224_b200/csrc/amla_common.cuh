@@ -22,6 +22,7 @@ constexpr int kStatusTimeout = 1;
 struct DecodeParams {
   const __nv_bfloat16* q;        // [B, Sq, H, 576] == [B, R, 576]
   const __nv_bfloat16* kv;       // [num_blocks, 64, 576]
+  const uint8_t* kv8;            // an E4M3 cache [num_blocks, 64, 576] instead of kv (or nullptr)
   const int32_t* block_table;    // [B, max_blocks_per_seq]
   const int32_t* seqlens;        // [B]
   __nv_bfloat16* out;            // [B, R, 512]
@@ -77,7 +78,7 @@ constexpr int kTraceTiles = 96;
 // the pipeline fill, the epilogue) that is worth about kUnitOverheadTiles tiles, so the schedule
 // balances a linear range in which every non-empty item but the first is preceded by that many
 // overhead positions: prefix[it] is the position where item `it` begins (overhead first, then its tiles),
-// L = prefix[n_items] the total, and part p owns positions [p*L/P, (p+1)*L/P).  A part does the
+// L = prefix[n_items] the total, and part p owns positions [p*share, (p+1)*share) with share = ceil(L / P).  A part does the
 // tiles whose positions it owns; overhead positions carry no work.
 // ---------------------------------------------------------------------------------------------
 #ifndef AMLA_UNIT_OVERHEAD_TILES
@@ -100,41 +101,28 @@ __host__ __device__ inline int schedule_length(int seqlen, int it, int tile_keys
   return tiles > 0 ? tiles + item_overhead(it, ovh) : 0;
 }
 
+// (share = ceil(L / P) positions per part rather than parts of floor or ceil(L / P): the largest part is the same, no
+// part boundary needs a 64-bit product, a position's part is one 32-bit division, and a short range has fewer parts.)
 struct Plan {
   const int* prefix;
   int n_items;
   int L;
-  int P;
+  int P;         // parts that own positions
   int ovh;
-  bool wide;     // L * P does not fit 31 bits: the part arithmetic needs 64-bit division (slow on the device)
+  int share;     // positions per part (the last part may have fewer)
 
-  // With fewer positions than parts only the first L parts exist (one position each).
   __host__ __device__ static Plan make(const int* prefix, int n_items, int max_parts, int ovh) {
     Plan pl;
     pl.prefix = prefix;
     pl.ovh = ovh;
     pl.n_items = n_items;
     pl.L = prefix[n_items];
-    pl.P = pl.L < max_parts ? (pl.L > 0 ? pl.L : 1) : max_parts;
-    pl.wide = static_cast<long long>(pl.L) * pl.P >= (1ll << 31);
+    pl.share = pl.L > max_parts ? static_cast<int>((static_cast<unsigned>(pl.L) + max_parts - 1) / static_cast<unsigned>(max_parts)) : 1;
+    pl.P = pl.L > 0 ? static_cast<int>((static_cast<unsigned>(pl.L) + pl.share - 1) / static_cast<unsigned>(pl.share)) : 1;
     return pl;
   }
-  // floor(a * b / c) for 0 <= a <= c-ish operands of the schedule; 32-bit unless the product could overflow
-  __host__ __device__ int muldiv(int a, int b, int c) const {
-    if (!wide) return static_cast<int>(static_cast<unsigned>(a) * static_cast<unsigned>(b) / static_cast<unsigned>(c));
-    return static_cast<int>((static_cast<long long>(a) * b) / c);
-  }
-  __host__ __device__ int part_start(int p) const {
-    if (p >= P) return L;
-    return muldiv(p, L, P);
-  }
-  __host__ __device__ int part_of_tile(int g) const {
-    int p = muldiv(g, P, L);
-    if (p > P - 1) p = P - 1;
-    while (p + 1 < P && part_start(p + 1) <= g) ++p;
-    while (p > 0 && part_start(p) > g) --p;
-    return p;
-  }
+  __host__ __device__ int part_start(int p) const { return p >= P ? L : p * share; }
+  __host__ __device__ int part_of_tile(int g) const { return static_cast<int>(static_cast<unsigned>(g) / static_cast<unsigned>(share)); }
   // Largest item index whose first tile is <= g (zero-tile items are skipped automatically).
   __host__ __device__ int item_of_tile(int g) const {
     int lo = 0, hi = n_items - 1;
@@ -195,6 +183,18 @@ __device__ __forceinline__ float2 unpack_f16x2(uint32_t h2) {
   float lo, hi;
   asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\tcvt.f32.f16 %0, a;\n\tcvt.f32.f16 %1, b;\n\t}" : "=f"(lo), "=f"(hi) : "r"(h2));
   return make_float2(lo, hi);
+}
+
+// Two E4M3 bytes (low 16 bits of `pair`) -> two bf16 in one word.  E4M3 -> f16 is one hardware conversion and
+// exact; f16 -> f32 -> bf16 is exact for these values (at most four significant bits, exponents -9 .. 8).
+__device__ __forceinline__ uint32_t e4m3x2_to_bf16x2(uint32_t pair) {
+  uint32_t h2;
+  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"(static_cast<unsigned short>(pair & 0xffffu)));
+  float lo, hi;
+  asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\tcvt.f32.f16 %0, a;\n\tcvt.f32.f16 %1, b;\n\t}" : "=f"(lo), "=f"(hi) : "r"(h2));
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
 }
 
 // ---------------------------------------------------------------------------------------------

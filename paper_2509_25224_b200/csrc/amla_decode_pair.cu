@@ -43,8 +43,9 @@ using namespace sm100;
 namespace {
 
 constexpr int kSoftmaxWarps = 8;
-constexpr int kLoaders = 2;                             // warps 8 and 10
-constexpr int kThreads = 32 * (kSoftmaxWarps + kLoaders + 1);
+// bf16 cache: warps 8 and 10 load.  E4M3 cache: warp 8 loads, warps 10-15 widen, three pairs taking turns.
+constexpr int kWideners = 6;
+template <bool kFp8> constexpr int kThreads = 32 * (kFp8 ? kSoftmaxWarps + 2 + kWideners : kSoftmaxWarps + 3);
 constexpr int kTilePages = 4;                           // pages of a score tile: N = 256, the widest MMA
 constexpr int kCtaRows = kRowBlock / 2;                 // query rows per CTA
 constexpr int kQBlocks = kDqk / 64;                     // 64-column blocks of Q and K
@@ -54,14 +55,20 @@ constexpr uint32_t kPPageBytes = kCtaRows * 128;        // P~ of one page: [64 r
 constexpr uint32_t kKBoxBytes = 32 * 128;               // this CTA's half of a page x one 64-column block
 constexpr uint32_t kSlotBytes = 128 * 128;              // K: 4 pages x 32 keys x 64 columns; V: 64 keys x 128 columns
 constexpr uint32_t kVBlockBytes = 64 * 128;             // 64 keys x 64 columns
-constexpr int kSlots = 7;
+// The ring of operand slots, and for an E4M3 cache a ring of raw slots in front of it: K of 4 pages x 32 keys x 128 columns,
+// or V of 64 keys x 256 columns, two operand slots each.
+template <bool kFp8> constexpr int kSlots = kFp8 ? 4 : 7;
+constexpr int kRawSlots = 3;
+constexpr uint32_t kRawBytes = 128 * 128, kRawPageBytes = 32 * 128;
 
 constexpr uint32_t kOffQ = 0;
 constexpr uint32_t kOffP = kOffQ + kQBytes;
 constexpr uint32_t kOffRing = kOffP + kTilePages * kPPageBytes;
-constexpr uint32_t kOffXchg = kOffRing + kSlots * kSlotBytes;      // float [2][4 threads of a row][64 rows]
+constexpr uint32_t kOffRaw = kOffRing + kSlots<true> * kSlotBytes;
+constexpr uint32_t kOffXchg = kOffRing + 7 * kSlotBytes;           // float [2][4 threads of a row][64 rows]
+static_assert(kOffRaw + kRawSlots * kRawBytes <= kOffXchg && kSlots<false> <= 7, "the rings share one area");
 constexpr uint32_t kOffBars = kOffXchg + 2 * 4 * kCtaRows * 4;
-constexpr uint32_t kBarBytes = 256;
+constexpr uint32_t kBarBytes = 320;
 // a copy of the schedule prefix and of the sequence lengths for batches of up to kSmemPlanItems items, so that the
 // roles' schedule look-ups (a dozen dependent loads per unit) stay on chip
 constexpr int kSmemPlanItems = 512;
@@ -77,9 +84,10 @@ constexpr uint32_t kOCol = 0;            // 256 columns
 constexpr uint32_t kSCol = 256;          // 2 x 128 columns
 
 // Barriers.  (L): the copy in the even CTA is the one that counts; both CTAs arrive there.  The others exist in both
-// CTAs and complete by multicast commits of the even CTA's MMA warp, except X_XCHG, which is local.
-enum { X_FULL = 0 /*L*/, X_EMPTY = X_FULL + kSlots, X_QFULL = X_EMPTY + kSlots /*L*/, X_QFREE, X_SFULL, X_SEMPTY = X_SFULL + 2 /*L*/,
-       X_PREADY = X_SEMPTY + 2 /*L*/, X_PVDONE, X_XCHG, X_NUM = X_XCHG + 2 };
+// CTAs and complete by multicast commits of the even CTA's MMA warp, except X_XCHG and the raw ring's, which are local.
+enum { X_FULL = 0 /*L*/, X_EMPTY = X_FULL + 7, X_QFULL = X_EMPTY + 7 /*L*/, X_QFREE, X_SFULL, X_SEMPTY = X_SFULL + 2 /*L*/,
+       X_PREADY = X_SEMPTY + 2 /*L*/, X_PVDONE, X_XCHG, X_RAWFULL = X_XCHG + 2, X_RAWEMPTY = X_RAWFULL + kRawSlots,
+       X_NUM = X_RAWEMPTY + kRawSlots };
 constexpr uint32_t kTmemSlotOff = kBarBytes - 8;
 static_assert(X_NUM * 8 + 8 <= kBarBytes, "barrier area too small");
 
@@ -92,9 +100,10 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
   return __all_sync(0xffffffffu, mbar_wait<kClusterAcquire>(bar, parity));
 }
 
-// What the loader keeps of a score tile: the page of lane l (pages [t, t + np) of the item), the Q row of its unit.
+// What the loader keeps of a score tile: where its pages stand in the block table, how many, the Q row of its unit.
 struct TileRef {
-  int np, page, qrow;
+  const int32_t* bt;
+  int np, qrow;
   bool first, last, valid;
 };
 
@@ -102,8 +111,8 @@ using Tiles = TileIter<kTilePages>;
 
 }  // namespace
 
-template <int kMode, bool kGuard>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+template <int kMode, bool kGuard, bool kFp8>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads<kFp8>, 1)
 decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap q_map,
                    const DecodeParams prm) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -127,7 +136,13 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   int early_len = 0;
   if (wid == 0 && prm.fused_plan && lane < prm.n_items) early_len = prm.seqlens[lane / prm.nrb];
   if (tid == 32 * 8) {
-    for (int i = 0; i < kSlots; ++i) { mbar_init(bar(X_FULL + i), 1); mbar_init(bar(X_EMPTY + i), 1); }
+    for (int i = 0; i < kSlots<kFp8>; ++i) {
+      mbar_init(bar(X_FULL + i), kFp8 ? 4 : 1);          // E4M3: the two warps that fill the slot, in either CTA
+      mbar_init(bar(X_EMPTY + i), 1);
+    }
+    if (kFp8) {
+      for (int i = 0; i < kRawSlots; ++i) { mbar_init(bar(X_RAWFULL + i), 1); mbar_init(bar(X_RAWEMPTY + i), 4); }
+    }
     mbar_init(bar(X_QFULL), 1);
     mbar_init(bar(X_QFREE), 1);
     for (int i = 0; i < 2; ++i) {
@@ -207,7 +222,6 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     const int r = (quarter & 1) * 32 + lane;             // query row within this CTA's 64
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const bool scale_nonneg = prm.scale_log2 >= 0.f;
-    const uint32_t mask_fill = __float_as_uint(scale_nonneg ? -INFINITY : INFINITY);
     const uint32_t xbar = bar(X_XCHG + (quarter & 1));
     const uint32_t prow_smem = smem_base + kOffP + r * 128;
     const uint32_t o_addr = tbase + lane_base + kOCol + 128 * grp;     // this thread's 128 of the row's 512 columns
@@ -257,32 +271,23 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         // general one with the visibility masks and the sign of the scale.
         auto tile_body = [&](auto general_c) {
           constexpr bool kGeneral = decltype(general_c)::value;
-          const bool scale_nn = kGeneral ? scale_nonneg : true;
-          // lines 5-6: running max on the raw scores (the scale is folded into the FMA below)
-          float ext = scale_nn ? -INFINITY : INFINITY, ext_b = ext;
+          // lines 5-6: running max; the plain tile takes it on the raw scores (the scale is folded into the FMA below),
+          // the general one on the scaled ones
+          float ext = -INFINITY, ext_b = ext;
           auto chunk_max = [&](uint32_t (&v)[32], int nvis) {
             if (kGeneral) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) v[i] = (i < nvis) ? v[i] : mask_fill;
+              for (int i = 0; i < 32; ++i) v[i] = (i < nvis) ? __float_as_uint(__uint_as_float(v[i]) * prm.scale_log2) : 0xff800000u;
             }
-            if (scale_nn) {
 #pragma unroll
-              for (int i = 0; i < 32; i += 4) {
-                ext = fmax3(ext, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
-                ext_b = fmax3(ext_b, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
-              }
-            } else {
-#pragma unroll
-              for (int i = 0; i < 32; i += 4) {
-                ext = fminf(ext, fminf(__uint_as_float(v[i]), __uint_as_float(v[i + 1])));
-                ext_b = fminf(ext_b, fminf(__uint_as_float(v[i + 2]), __uint_as_float(v[i + 3])));
-              }
+            for (int i = 0; i < 32; i += 4) {
+              ext = fmax3(ext, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+              ext_b = fmax3(ext_b, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
             }
           };
           chunk_max(b0, nvis0);
           chunk_max(b1, nvis1);
-          ext = scale_nn ? fmaxf(ext, ext_b) : fminf(ext, ext_b);
-          const float mine = (nvis0 > 0 || nvis1 > 0) ? ext * prm.scale_log2 : -INFINITY;
+          const float mine = kGeneral ? fmaxf(ext, ext_b) : fmaxf(ext, ext_b) * prm.scale_log2;
           float m4[4];
           exchange(mine, m4);
           if (!ok) return;
@@ -301,14 +306,12 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           const uint64_t sc2 = pack_f32x2(prm.scale_log2, prm.scale_log2), ns2 = pack_f32x2(nsub, nsub);
           uint64_t rsa = pack_f32x2(0.f, 0.f), rsb = rsa;
           uint32_t pk[32];
-          auto chunk_exp = [&](const uint32_t (&v)[32], int nvis, int k0) {
+          auto chunk_exp = [&](const uint32_t (&v)[32], int k0) {
             if (kGeneral) {
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
-                float p0 = ex2_approx(fmaf(__uint_as_float(v[2 * i]), prm.scale_log2, nsub));
-                float p1 = ex2_approx(fmaf(__uint_as_float(v[2 * i + 1]), prm.scale_log2, nsub));
-                p0 = (2 * i < nvis) ? p0 : 0.f;
-                p1 = (2 * i + 1 < nvis) ? p1 : 0.f;
+                const float p0 = ex2_approx(__uint_as_float(v[2 * i]) + nsub);          // a hidden key: 2^-inf = 0
+                const float p1 = ex2_approx(__uint_as_float(v[2 * i + 1]) + nsub);
                 rs0 += p0; rs1 += p1;
                 pk[k0 + i] = pack_bf16x2(p0, p1);
               }
@@ -324,8 +327,8 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
               }
             }
           };
-          chunk_exp(b0, nvis0, 0);
-          chunk_exp(b1, nvis1, 16);
+          chunk_exp(b0, 0);
+          chunk_exp(b1, 16);
           {
             float s0, s1;
             unpack_f32x2(add_f32x2(rsa, rsb), s0, s1);
@@ -453,194 +456,295 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       tile.next();
     }
     if (!ok && lane == 0) report_timeout(prm.status);
-  } else if (wid == 8 || wid == 10) {
+  } else if (wid == 8 || (!kFp8 && wid == 10)) {
     // ======================================================== TMA loads, in the order in which the MMAs use them:
-    // Q, K(0), K(1), V(0), K(2), V(1), ..., K(n-1), V(n-2), V(n-1), next unit.  One ring of 16 KB slots carries K (one
-    // 64-column block of the tile's keys, one box per page, each issued by its own lane) and V (one page x 128
-    // columns).  The two loader warps walk the same sequence and issue every second load of it.  Q is the first's: it is
-    // requested as soon as the QK^T of the unit before have let go of the buffer, if need be between the V loads of that
-    // unit's last tile.
-    const uint32_t mine = wid == 8 ? 0u : 1u;
-    const uint64_t keep = l2_policy_evict_normal(), last_use = l2_policy_evict_first();   // K: V follows a tile later; V: done with
-    uint32_t slot = 0, par = 1;
-    uint32_t n_issued = 0;
-    uint32_t un = 0;                                      // units whose Q has been requested
-    auto take = [&]() -> TileRef {
-      TileRef x;
-      x.valid = tile.valid;
-      x.np = 0; x.page = 0; x.qrow = 0; x.first = x.last = false;
-      if (x.valid) {
-        x.np = tile.np; x.first = tile.first; x.last = tile.last();
-        x.qrow = tile.u.b * prm.R + tile.u.r0 + rank * kCtaRows;
-        if (lane < x.np) x.page = __ldg(prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t + lane);
-        tile.next();
-      }
-      return x;
-    };
-    auto advance = [&]() { if (++slot == kSlots) { slot = 0; par ^= 1; } ++n_issued; };
-    auto issue_q = [&](int qrow) {
-      if (leader) mbar_arrive_expect_tx_elect(bar(X_QFULL), 2 * kQBytes);
-#pragma unroll
-      for (int c = 0; c < kQBlocks; c += 3)
-        tma_load_3d_pair_elect(smem_base + kOffQ + c * kQBlockBytes, &q_map, 0, qrow, c, lead_bars + 8u * X_QFULL, last_use);
-      ++un;
-    };
-    // What a load needs is at hand before its slot is waited for: the slot's turn-around is on the critical path of a
-    // ring that holds little more than the latency of memory.
-    auto issue_v = [&](int np, int page, int nxt_qrow, bool q_wanted, bool& q_out) {
+    // Q, K(0), K(1), V(0), K(2), V(1), ..., K(n-1), V(n-2), V(n-1), next unit.
+    //   bf16: one ring of 16 KB slots carries K (one 64-column block of the tile's keys, one box per page) and V (one page
+    //     x 128 columns).  The two loader warps walk the same sequence and issue every second load of it.
+    //   E4M3: raw slots; K in five of 128 columns (the last one half outside the row: zeros), V in one per page.
+    // A unit's Q is requested (by the first loader) as soon as the QK^T of the unit before have let go of the buffer, if
+    // need be between the V loads of that unit's last tile.
+    if (elect_one()) {
+      const uint32_t mine = wid == 8 ? 0u : 1u;
+      constexpr uint32_t kRing = kFp8 ? kRawSlots : kSlots<kFp8>;
+      const uint32_t full0 = kFp8 ? bar(X_RAWFULL) : bar(X_FULL), empty0 = kFp8 ? bar(X_RAWEMPTY) : bar(X_EMPTY);
+      const uint32_t lead_full0 = lead_bars + 8u * X_FULL, ring0 = smem_base + (kFp8 ? kOffRaw : kOffRing);
+      const uint64_t keep = l2_policy_evict_normal(), last_use = l2_policy_evict_first();   // K: V follows a tile later; V: done with
+      uint32_t slot = 0, par = 1, n_issued = 0;
+      uint32_t un = 0;                                      // units whose Q has been requested
+      auto take = [&]() -> TileRef {
+        TileRef x;
+        x.valid = tile.valid;
+        x.np = 0; x.qrow = 0; x.first = x.last = false;
+        x.bt = prm.block_table;
+        if (x.valid) {
+          x.np = tile.np; x.first = tile.first; x.last = tile.last();
+          x.qrow = tile.u.b * prm.R + tile.u.r0 + rank * kCtaRows;
+          x.bt = prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t;
+          tile.next();
+        }
+        return x;
+      };
+      // first key row of a page; E4M3: a page outside the cache reads as zeros (rows behind the end of the tensor do)
+      auto row_of = [&](int page) { return (kFp8 && (page < 0 || page >= prm.num_blocks) ? prm.num_blocks : page) * kPage; };
+      auto advance = [&]() { if (++slot == kRing) { slot = 0; par ^= 1; } ++n_issued; };
+      auto my_turn = [&]() { return kFp8 || (n_issued & 1) == mine; };
+      auto issue_q = [&](int qrow) {
+        if (leader) mbar_arrive_expect_tx(bar(X_QFULL), 2 * kQBytes);
 #pragma unroll 1
-      for (int i = 0; i < 2 * np; ++i) {
-        if ((n_issued & 1) == mine) {
-          if (q_wanted && !q_out && __all_sync(0xffffffffu, mbar_probe(bar(X_QFREE), (un - 1) & 1))) { issue_q(nxt_qrow); q_out = true; }
-          const int row = __shfl_sync(0xffffffffu, page, i >> 1) * kPage;
-          const uint32_t dst = smem_base + kOffRing + slot * kSlotBytes, full = bar(X_FULL + slot), lead_full = lead_bars + 8u * (X_FULL + slot);
-          ok = warp_wait(bar(X_EMPTY + slot), par);
-          if (!ok) return;
-          if (leader) mbar_arrive_expect_tx_elect(full, 2 * kSlotBytes);
-          tma_load_3d_pair_elect(dst, &v_map, 0, row, 4 * rank + 2 * (i & 1), lead_full, last_use);
-        }
-        advance();
-      }
-    };
-    TileRef cur = take(), nxt = take();
-    int np_prev = 0;
-    int page_prev = 0;
-    bool q_out = false;                                   // the Q of the unit that starts next has been requested
-    uint32_t pt = 0;
-    while (ok && cur.valid) {
-      if (cur.first && mine == 0) {
-        if (!q_out) {
-          if (un > 0) ok = warp_wait(bar(X_QFREE), (un - 1) & 1);
-          if (!ok) break;
-          issue_q(cur.qrow);
-        }
-        q_out = false;
-      }
-      int row[kTilePages];                                // first key row of the tile's pages
-#pragma unroll
-      for (int p = 0; p < kTilePages; ++p) row[p] = __shfl_sync(0xffffffffu, cur.page, p) * kPage;
-      const TileRef nn = take();
+        for (int c = 0; c < kQBlocks; c += 3)
+          tma_load_3d_pair_hint(smem_base + kOffQ + c * kQBlockBytes, &q_map, 0, qrow, c, lead_bars + 8u * X_QFULL, last_use);
+        ++un;
+      };
+      auto issue_v = [&](const TileRef& x, int nxt_qrow, bool q_wanted, bool& q_out) {
+        int page = __ldg(x.bt);
 #pragma unroll 1
-      for (int c = 0; c < kQBlocks; ++c) {
-        if ((n_issued & 1) == mine) {
-          const uint32_t dst = smem_base + kOffRing + slot * kSlotBytes, full = bar(X_FULL + slot), lead_full = lead_bars + 8u * (X_FULL + slot);
-          ok = warp_wait(bar(X_EMPTY + slot), par);
-          if (!ok) break;
-          if (lane == 0 && leader && (c <= 1 || c >= 7)) AMLA_STAMP(prm, part, c <= 1 ? 16 : 17, pt);
-          if (leader) mbar_arrive_expect_tx_elect(full, 2 * cur.np * kKBoxBytes);
-#pragma unroll
-          for (int p = 0; p < kTilePages; ++p)
-            if (p < cur.np) tma_load_3d_pair_elect(dst + p * kKBoxBytes, &k_map, 0, row[p] + 32 * rank, c, lead_full, keep);
-        }
-        advance();
-      }
-      if (!ok) break;
-      if (!cur.first) issue_v(np_prev, page_prev, 0, false, q_out);
-      if (ok && cur.last) issue_v(cur.np, cur.page, nxt.qrow, mine == 0 && nxt.valid, q_out);
-      np_prev = cur.np;
-      page_prev = cur.page;
-      cur = nxt;
-      nxt = nn;
-      ++pt;
-    }
-    if (!ok) {
-      if (lane == 0) report_timeout(prm.status);
-      // let the copies that may still be in flight land before the CTA exits
-      if (leader) {
-        for (uint32_t i = 0; i < kSlots && i < n_issued; ++i) {
-          const uint32_t k = n_issued - 1 - i;
-          if ((k & 1) == mine) mbar_wait(bar(X_FULL + k % kSlots), (k / kSlots) & 1);
-        }
-        if (un > 0) mbar_wait(bar(X_QFULL), (un - 1) & 1);
-      }
-    }
-  } else if (leader && wid == 9) {
-    // ======================================================== MMA issuer (even CTA, for the pair)
-    constexpr uint32_t idesc_pv = make_idesc_bf16(128, 256, false, true);
-    constexpr uint32_t idesc_qk1 = make_idesc_bf16(128, 64, false, false);     // N = 64 per page
-    constexpr uint32_t idesc_step = make_idesc_bf16(128, 128, false, false) - idesc_qk1;
-    constexpr uint32_t dhi = smem_desc_hi_sw128(1024);
-    const uint32_t qlo = smem_desc_lo(smem_base + kOffQ, 16);
-    const uint32_t plo = smem_desc_lo(smem_base + kOffP, 16);
-    const uint32_t klo = smem_desc_lo(smem_base + kOffRing, 16);
-    const uint32_t vlo = smem_desc_lo(smem_base + kOffRing, kVBlockBytes);
-    uint32_t slot = 0, par = 0;
-    uint32_t gs = 0, gp = 0, un = 0;                      // score tiles, P~V tiles, units so far
-    auto advance = [&]() { if (++slot == kSlots) { slot = 0; par ^= 1; } };
-    // O (+)= P~ V of one tile: per page two N = 256 products (128 columns from either CTA)
-    auto pv = [&](int np, bool fresh) {
-      if (lane == 0) AMLA_STAMP(prm, part, 4, gp);
-      ok = warp_wait<true>(bar(X_PREADY), gp & 1);
-      if (!ok) return;
-      if (lane == 0) AMLA_STAMP(prm, part, 5, gp);
-      tc_fence_after_sync();               // the softmax warps may have rewritten O (tcgen05.st) before arriving
-      for (int p = 0; p < np; ++p) {
-        const uint32_t pl = plo + p * (kPPageBytes >> 4);
-#pragma unroll
-        for (int nh = 0; nh < 2; ++nh) {
-          ok = ok && warp_wait(bar(X_FULL) + 8 * slot, par);
-          if (!ok) return;
-          if (p == 0 && nh == 0 && lane == 0) AMLA_STAMP(prm, part, 6, gp);
-          const uint32_t vl = vlo + slot * (kSlotBytes >> 4);
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_ss_pair_elect(tbase + kOCol + 128 * nh, smem_desc_join(pl + 2 * kk, dhi), smem_desc_join(vl + 128 * kk, dhi), idesc_pv,
-                        (kk == 0 && p == 0 && fresh) ? 0u : 1u);
-          mma_commit_pair_multicast_elect(bar(X_EMPTY) + 8 * slot, 3);
+        for (int i = 0; i < (kFp8 ? x.np : 2 * x.np); ++i) {
+          const int row = row_of(page);
+          const int nh = kFp8 ? 0 : i & 1, p_next = min(kFp8 ? i + 1 : (i + 1) >> 1, x.np - 1);
+          page = __ldg(x.bt + p_next);
+          if (my_turn()) {
+            if (q_wanted && !q_out && mbar_probe(bar(X_QFREE), (un - 1) & 1)) { issue_q(nxt_qrow); q_out = true; }
+            const uint32_t dst = ring0 + slot * kSlotBytes;
+            ok = mbar_wait(empty0 + 8 * slot, par);
+            if (!ok) return;
+            if (kFp8) {
+              mbar_arrive_expect_tx(full0 + 8 * slot, kRawBytes);
+              tma_load_2d_hint(dst, &v_map, 256 * rank, row, full0 + 8 * slot, last_use);            // [2][64 keys][128 columns]
+              tma_load_2d_hint(dst + kRawBytes / 2, &v_map, 256 * rank + 128, row, full0 + 8 * slot, last_use);
+            } else {
+              if (leader) mbar_arrive_expect_tx(full0 + 8 * slot, 2 * kSlotBytes);
+              tma_load_3d_pair_hint(dst, &v_map, 0, row, 4 * rank + 2 * nh, lead_full0 + 8 * slot, last_use);
+            }
+          }
           advance();
         }
-      }
-      mma_commit_pair_multicast_elect(bar(X_PVDONE), 3);
-      if (lane == 0) AMLA_STAMP(prm, part, 7, gp);
-      ++gp;
-    };
-    int np_prev = 0;
-    bool fresh = true;
-    while (ok && tile.valid) {
-      if (tile.first) {
-        ok = warp_wait(bar(X_QFULL), un & 1);
-        if (!ok) break;
-        ++un;
-      }
-      {
-        const uint32_t sb = gs & 1;
-        if (lane == 0) AMLA_STAMP(prm, part, 0, gs);
-        ok = warp_wait<true>(bar(X_SEMPTY + sb), ((gs >> 1) & 1) ^ 1);
-        if (!ok) break;
-        tc_fence_after_sync();
-        if (lane == 0) AMLA_STAMP(prm, part, 1, gs);
-        const uint32_t d = tbase + kSCol + 128 * sb;
-        const uint32_t idesc = idesc_qk1 + (tile.np - 1) * idesc_step;
+      };
+      int page[kTilePages];
+      auto get_pages = [&](const TileRef& x) {
 #pragma unroll
-        for (int c = 0; c < kQBlocks; ++c) {
-          ok = ok && warp_wait(bar(X_FULL) + 8 * slot, par);    // TMA data -> MMA operand: both async proxy, no fence needed
-          if (ok) {
-            if (c == 0 && lane == 0) AMLA_STAMP(prm, part, 2, gs);
-            const uint32_t kl = klo + slot * (kSlotBytes >> 4);
+        for (int p = 0; p < kTilePages; ++p) page[p] = p < x.np ? __ldg(x.bt + p) : 0;
+      };
+      TileRef cur = take(), prev = cur;
+      get_pages(cur);
+      TileRef nxt = take();
+      bool q_out = false;                                   // the Q of the unit that starts next has been requested
+      uint32_t pt = 0;
+      while (ok && cur.valid) {
+        if (cur.first && mine == 0) {
+          if (!q_out) {
+            if (un > 0) ok = mbar_wait(bar(X_QFREE), (un - 1) & 1);
+            if (!ok) break;
+            issue_q(cur.qrow);
+          }
+          q_out = false;
+        }
+        int row[kTilePages];
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              mma_ss_pair_elect(d, smem_desc_join(qlo + c * (kQBlockBytes >> 4) + 2 * kk, dhi), smem_desc_join(kl + 2 * kk, dhi), idesc, (c | kk) != 0 ? 1u : 0u);
-            mma_commit_pair_multicast_elect(bar(X_EMPTY) + 8 * slot, 3);
+        for (int p = 0; p < kTilePages; ++p) row[p] = row_of(page[p]);
+        get_pages(nxt);
+#pragma unroll 1
+        for (int c = 0; c < (kFp8 ? (kQBlocks + 1) / 2 : kQBlocks); ++c) {
+          if (my_turn()) {
+            const uint32_t dst = ring0 + slot * kSlotBytes;
+            ok = mbar_wait(empty0 + 8 * slot, par);
+            if (!ok) break;
+            if (leader && (c <= 1 || c >= 7)) AMLA_STAMP(prm, part, c <= 1 ? 16 : 17, pt);
+            if (kFp8) {
+              mbar_arrive_expect_tx(full0 + 8 * slot, cur.np * kRawPageBytes);
+#pragma unroll
+              for (int p = 0; p < kTilePages; ++p)
+                if (p < cur.np) tma_load_2d_hint(dst + p * kRawPageBytes, &k_map, 128 * c, row[p] + 32 * rank, full0 + 8 * slot, keep);   // [32 keys][128 columns]
+            } else {
+              if (leader) mbar_arrive_expect_tx(full0 + 8 * slot, 2 * cur.np * kKBoxBytes);
+#pragma unroll
+              for (int p = 0; p < kTilePages; ++p)
+                if (p < cur.np) tma_load_3d_pair_hint(dst + p * kKBoxBytes, &k_map, 0, row[p] + 32 * rank, c, lead_full0 + 8 * slot, keep);
+            }
           }
           advance();
         }
         if (!ok) break;
-        mma_commit_pair_multicast_elect(bar(X_SFULL + sb), 3);
-        if (tile.last()) mma_commit_pair_multicast_elect(bar(X_QFREE), 3);
-        if (lane == 0) AMLA_STAMP(prm, part, 3, gs);
-        ++gs;
+        const TileRef nn = take();
+        // V of the tile before, and behind a unit's last K its own V
+        for (int k = cur.first ? 1 : 0; k < (cur.last ? 2 : 1) && ok; ++k)
+          issue_v(k == 0 ? prev : cur, nxt.qrow, k == 1 && mine == 0 && nxt.valid, q_out);
+        prev = cur;
+        cur = nxt;
+        nxt = nn;
+        ++pt;
       }
+      if (!ok) {
+        report_timeout(prm.status);
+        // let the copies that may still be in flight land before the CTA exits
+        for (uint32_t i = 0; i < kRing && i < n_issued; ++i) {
+          const uint32_t k = n_issued - 1 - i;
+          if (kFp8 || (leader && (k & 1) == mine)) mbar_wait(full0 + 8 * (k % kRing), (k / kRing) & 1);
+        }
+        if (leader && un > 0) mbar_wait(bar(X_QFULL), (un - 1) & 1);
+      }
+    }
+    __syncwarp();
+  } else if (kFp8 && wid >= 10) {
+    // ======================================================== E4M3 cache: raw slot -> operand slots.  The three pairs of
+    // warps take every third operand slot each; a thread widens 16 bytes at a time (exact: E4M3 values are bf16 values)
+    // and stores them where the 128-byte swizzle of the operand tiles puts them.
+    const uint32_t mine = (wid - 10) >> 1;
+    const int wt = ((wid - 10) & 1) * 32 + lane;
+    uint32_t turn = 0, slot = 0, par = 1, rslot = 0, rpar = 0;
+    // One operand slot: `half` of raw slot rslot; `is_k`: K, else V; `last`: nothing else of the raw slot.  A thread holds
+    // its eight 16-byte pieces in registers, widened, before it waits for the operand slot: the raw slot goes back to the
+    // loader at once, and the operand slot is refilled within the time of sixteen stores.
+    auto fill = [&](bool is_k, uint32_t half, bool last) {
+      if (turn == mine) {
+        ok = warp_wait(bar(X_RAWFULL + rslot), rpar);
+        if (!ok) return;
+        // K: row = page * 32 + key, four threads a row; 64 of its 128 raw bytes are this slot's 64 columns (rows of pages
+        // that the tile does not have hold older bytes; the MMA does not read them).  V: 64 keys x 128 columns -> two
+        // blocks of 64 columns, eight threads a row.
+        const uint32_t raw = smem_base + kOffRaw + rslot * kRawBytes, out = smem_base + kOffRing + slot * kSlotBytes;
+        const int r0 = is_k ? wt >> 2 : wt >> 3, rstep = is_k ? 16 : 8;
+        const uint32_t src = raw + (is_k ? 64 * half + 16 * (wt & 3) : half * (kRawBytes / 2) + 16 * (wt & 7)) + r0 * 128;
+        const uint32_t dst = out + (is_k ? 0 : ((wt & 7) >> 2) * kVBlockBytes) + r0 * 128;
+        uint32_t x[8][4], w[8][8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x[k][0]), "=r"(x[k][1]), "=r"(x[k][2]), "=r"(x[k][3]) : "r"(src + k * rstep * 128));
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) { w[k][2 * q] = e4m3x2_to_bf16x2(x[k][q]); w[k][2 * q + 1] = e4m3x2_to_bf16x2(x[k][q] >> 16); }
+        }
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(bar(X_RAWEMPTY + rslot));
+          if (last && half == 0) mbar_arrive(bar(X_RAWEMPTY + rslot));       // the other half has no reader
+        }
+        ok = warp_wait(bar(X_EMPTY + slot), par);
+        if (!ok) return;
+        const uint32_t ch = 2 * (wt & 3), sw = r0 & 7;      // rows of a thread differ by multiples of 8: the same swizzle
+        const uint32_t d0 = dst + ((ch ^ sw) << 4), d1 = dst + (((ch + 1) ^ sw) << 4);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          st_shared_v4(d0 + k * rstep * 128, w[k][0], w[k][1], w[k][2], w[k][3]);
+          st_shared_v4(d1 + k * rstep * 128, w[k][4], w[k][5], w[k][6], w[k][7]);
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) { if (leader) mbar_arrive(bar(X_FULL + slot)); else mbar_arrive_cluster_relaxed(lead_bars + 8u * (X_FULL + slot)); }
+      }
+      if (++turn == kWideners / 2) turn = 0;
+      if (++slot == kSlots<kFp8>) { slot = 0; par ^= 1; }
+      if (last && ++rslot == kRawSlots) { rslot = 0; rpar ^= 1; }
+    };
+    int np_prev = 0;
+    while (ok && tile.valid) {
       const int np = tile.np;
       const bool first = tile.first, last = tile.last();
-      if (!first) { pv(np_prev, fresh); fresh = false; }
-      if (last) { if (ok) pv(np, first); fresh = true; }
+#pragma unroll 1
+      for (int c = 0; c < kQBlocks && ok; ++c) fill(true, c & 1, (c & 1) != 0 || c == kQBlocks - 1);
+      if (!first) {
+#pragma unroll 1
+        for (int i = 0; i < 2 * np_prev && ok; ++i) fill(false, i & 1, (i & 1) != 0);
+      }
+      if (last) {
+#pragma unroll 1
+        for (int i = 0; i < 2 * np && ok; ++i) fill(false, i & 1, (i & 1) != 0);
+      }
       np_prev = np;
       if (ok) tile.next();
     }
     if (!ok && lane == 0) report_timeout(prm.status);
+  } else if (leader && wid == 9) {
+    // ======================================================== MMA issuer (even CTA, for the pair)
+    if (elect_one()) {
+      constexpr uint32_t idesc_pv = make_idesc_bf16(128, 256, false, true);
+      constexpr uint32_t idesc_qk1 = make_idesc_bf16(128, 64, false, false);     // N = 64 per page
+      constexpr uint32_t idesc_step = make_idesc_bf16(128, 128, false, false) - idesc_qk1;
+      constexpr uint32_t dhi = smem_desc_hi_sw128(1024);
+      const uint32_t qlo = smem_desc_lo(smem_base + kOffQ, 16);
+      const uint32_t plo = smem_desc_lo(smem_base + kOffP, 16);
+      const uint32_t klo = smem_desc_lo(smem_base + kOffRing, 16);
+      const uint32_t vlo = smem_desc_lo(smem_base + kOffRing, kVBlockBytes);
+      uint32_t slot = 0, par = 0;
+      uint32_t gs = 0, gp = 0, un = 0;                      // score tiles, P~V tiles, units so far
+      auto advance = [&]() { if (++slot == kSlots<kFp8>) { slot = 0; par ^= 1; } };
+      int np_prev = 0;
+      bool fresh_prev = false;
+      while (ok && tile.valid) {
+        if (tile.first) {
+          ok = mbar_wait(bar(X_QFULL), un & 1);
+          if (!ok) break;
+          ++un;
+        }
+        const int np = tile.np;
+        const bool first = tile.first, last = tile.last();
+        {
+          const uint32_t sb = gs & 1;
+          AMLA_STAMP(prm, part, 0, gs);
+          ok = mbar_wait<true>(bar(X_SEMPTY + sb), ((gs >> 1) & 1) ^ 1);
+          if (!ok) break;
+          tc_fence_after_sync();
+          AMLA_STAMP(prm, part, 1, gs);
+          const uint32_t d = tbase + kSCol + 128 * sb;
+          const uint32_t idesc = idesc_qk1 + (np - 1) * idesc_step;
+#pragma unroll 1
+          for (int c = 0; c < kQBlocks; ++c) {
+            // bf16: TMA data -> MMA operand, both async proxy, no fence needed; E4M3: the widening threads have fenced
+            ok = mbar_wait<kFp8>(bar(X_FULL) + 8 * slot, par);
+            if (!ok) break;
+            if (c == 0) AMLA_STAMP(prm, part, 2, gs);
+            const uint32_t kl = klo + slot * (kSlotBytes >> 4), ql = qlo + c * (kQBlockBytes >> 4);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              mma_ss_pair(d, smem_desc_join(ql + 2 * kk, dhi), smem_desc_join(kl + 2 * kk, dhi), idesc, (c | kk) != 0 ? 1u : 0u);
+            mma_commit_pair_multicast(bar(X_EMPTY) + 8 * slot, 3);
+            advance();
+          }
+          if (!ok) break;
+          mma_commit_pair_multicast(bar(X_SFULL + sb), 3);
+          if (last) mma_commit_pair_multicast(bar(X_QFREE), 3);
+          AMLA_STAMP(prm, part, 3, gs);
+          ++gs;
+        }
+        // O (+)= P~ V of the tile before, and behind a unit's last QK^T its own: per page two N = 256 products (128 columns
+        // from either CTA)
+        for (int k = first ? 1 : 0; k < (last ? 2 : 1) && ok; ++k) {
+          const int np_v = k == 0 ? np_prev : np;
+          uint32_t acc = (k == 0 ? fresh_prev : first) ? 0u : 1u;
+          AMLA_STAMP(prm, part, 4, gp);
+          ok = mbar_wait<true>(bar(X_PREADY), gp & 1);
+          if (!ok) break;
+          AMLA_STAMP(prm, part, 5, gp);
+          tc_fence_after_sync();               // the softmax warps may have rewritten O (tcgen05.st) before arriving
+#pragma unroll 1
+          for (int i = 0; i < 2 * np_v; ++i) {
+            ok = mbar_wait<kFp8>(bar(X_FULL) + 8 * slot, par);
+            if (!ok) break;
+            if (i == 0) AMLA_STAMP(prm, part, 6, gp);
+            const uint32_t pl = plo + (i >> 1) * (kPPageBytes >> 4), vl = vlo + slot * (kSlotBytes >> 4), d = tbase + kOCol + 128 * (i & 1);
+            if (i >= 2) acc = 1u;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              mma_ss_pair(d, smem_desc_join(pl + 2 * kk, dhi), smem_desc_join(vl + 128 * kk, dhi), idesc_pv, kk == 0 ? acc : 1u);
+            mma_commit_pair_multicast(bar(X_EMPTY) + 8 * slot, 3);
+            advance();
+          }
+          if (!ok) break;
+          mma_commit_pair_multicast(bar(X_PVDONE), 3);
+          AMLA_STAMP(prm, part, 7, gp);
+          ++gp;
+        }
+        np_prev = np;
+        fresh_prev = first;
+        if (ok) tile.next();
+      }
+      if (!ok) report_timeout(prm.status);
+    }
+    __syncwarp();
   }
 
-  if (tid == 0 && leader) if (lane == 0) AMLA_STAMP(prm, part, 20, 2);
+  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 2);
   // teardown: nobody may still be signalling a CTA that has exited, and both CTAs must be done with tensor memory
   tc_fence_before_sync();
   __syncthreads();
@@ -684,9 +788,9 @@ bool encode_rows(EncodeTiledFn encode, CUtensorMap* map, const void* base, cuuin
                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int kMode, bool kGuard>
+template <int kMode, bool kGuard, bool kFp8>
 cudaError_t launch_variant(const CUtensorMap& kmap, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
-  auto kern = decode_pair_kernel<kMode, kGuard>;
+  auto kern = decode_pair_kernel<kMode, kGuard, kFp8>;
   // the opt-in to large dynamic shared memory is per device and per kernel; do it once each
   static std::atomic<uint64_t> done{0};
   int device = 0;
@@ -700,7 +804,7 @@ cudaError_t launch_variant(const CUtensorMap& kmap, const CUtensorMap& vmap, con
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * prm.P);
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(kThreads<kFp8>);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -709,6 +813,25 @@ cudaError_t launch_variant(const CUtensorMap& kmap, const CUtensorMap& vmap, con
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, kmap, vmap, qmap, prm);
+}
+
+template <bool kFp8>
+cudaError_t launch_mode(const CUtensorMap& kmap, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
+  const int mode = prm.flags & 3;
+  const bool guard = !(prm.flags & 4);
+  if (mode == 0) return guard ? launch_variant<0, true, kFp8>(kmap, vmap, qmap, prm, stream) : launch_variant<0, false, kFp8>(kmap, vmap, qmap, prm, stream);
+  if (mode == 1) return guard ? launch_variant<1, true, kFp8>(kmap, vmap, qmap, prm, stream) : launch_variant<1, false, kFp8>(kmap, vmap, qmap, prm, stream);
+  return launch_variant<2, true, kFp8>(kmap, vmap, qmap, prm, stream);
+}
+
+// An E4M3 cache: rows of 576 bytes, boxes of 128 columns.
+bool encode_bytes(EncodeTiledFn encode, CUtensorMap* map, const void* base, cuuint64_t rows, cuuint32_t box_rows) {
+  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(kDqk), rows};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(kDqk)};
+  const cuuint32_t box[2] = {128, box_rows};
+  const cuuint32_t estr[2] = {1, 1};
+  return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace
@@ -724,14 +847,13 @@ cudaError_t launch_decode_pair(const DecodeParams& prm, cudaStream_t stream, int
   // blocks (rows past the end of the array read as zero, rows of a following sequence are computed and dropped)
   CUtensorMap kmap, vmap, qmap;
   const cuuint64_t keys = static_cast<cuuint64_t>(prm.num_blocks) * kPage;
-  if (!encode_rows(encode, &kmap, prm.kv, keys, 32, 1) || !encode_rows(encode, &vmap, prm.kv, keys, 64, 2) ||
-      !encode_rows(encode, &qmap, prm.q, static_cast<cuuint64_t>(prm.B) * prm.R, kCtaRows, 3))
-    return cudaErrorInvalidValue;
-  const int mode = prm.flags & 3;
-  const bool guard = !(prm.flags & 4);
-  if (mode == 0) return guard ? launch_variant<0, true>(kmap, vmap, qmap, prm, stream) : launch_variant<0, false>(kmap, vmap, qmap, prm, stream);
-  if (mode == 1) return guard ? launch_variant<1, true>(kmap, vmap, qmap, prm, stream) : launch_variant<1, false>(kmap, vmap, qmap, prm, stream);
-  return launch_variant<2, true>(kmap, vmap, qmap, prm, stream);
+  if (!encode_rows(encode, &qmap, prm.q, static_cast<cuuint64_t>(prm.B) * prm.R, kCtaRows, 3)) return cudaErrorInvalidValue;
+  if (prm.kv8 != nullptr) {
+    if (!encode_bytes(encode, &kmap, prm.kv8, keys, 32) || !encode_bytes(encode, &vmap, prm.kv8, keys, 64)) return cudaErrorInvalidValue;
+    return launch_mode<true>(kmap, vmap, qmap, prm, stream);
+  }
+  if (!encode_rows(encode, &kmap, prm.kv, keys, 32, 1) || !encode_rows(encode, &vmap, prm.kv, keys, 64, 2)) return cudaErrorInvalidValue;
+  return launch_mode<false>(kmap, vmap, qmap, prm, stream);
 }
 
 }  // namespace amla

@@ -25,6 +25,7 @@
 #include "amla_common.cuh"
 #include "amla_sm100.cuh"
 #include "amla_epilogue.cuh"
+#include "amla_units.cuh"
 
 namespace amla {
 
@@ -112,47 +113,6 @@ enum { A_KFULL = X_COMMON /* even CTA */, A_KEMPTY = A_KFULL + kNumKSlots, A_SFU
 enum { B_VFULL = X_COMMON /* even CTA */, B_VEMPTY = B_VFULL + kNumVSlots, B_PFULL = B_VEMPTY + kNumVSlots, B_OREADY = B_PFULL + kNumP /*R*/,
        B_NUM = B_OREADY + kNumP };
 static_assert(A_NUM * 8 + 8 <= kBarBytes && B_NUM * 8 + 8 <= kBarBytes, "barrier area too small");
-
-struct Unit {
-  int b, r0, n_b, t0, t1, it;      // r0: first row of the 256-row block; t0, t1: 128-key tiles; it: item index
-};
-
-struct UnitIter {
-  const DecodeParams& prm;
-  Plan plan;
-  int p, g, g1;
-  const int* seqlens;
-  __device__ UnitIter(const DecodeParams& prm_, const int* prefix, const int* seqlens_, int part)
-      : prm(prm_), plan(Plan::make(prefix, prm_.n_items, prm_.P, prm_.ovh)), p(part), seqlens(seqlens_) {
-    if (plan.L <= 0 || p >= plan.P) { g = g1 = 0; }
-    else { g = plan.part_start(p); g1 = plan.part_start(p + 1); }
-  }
-  __device__ bool next(Unit& u) {
-    int it, a;
-    while (true) {
-      if (g >= g1) return false;
-      it = plan.item_of_tile(g);
-      a = plan.first_tile(it);
-      const int e = plan.prefix[it + 1];
-      const int lo = max(g, a), hi = min(e, g1);
-      g = min(e, g1);
-      if (hi > lo) { u.t0 = lo - a; u.t1 = hi - a; break; }
-    }
-    u.it = it;
-    u.b = it / prm.nrb;
-    u.r0 = (it % prm.nrb) * kItemRows;
-    u.n_b = min(max(seqlens[u.b], 0), prm.max_blocks_per_seq * kPage);
-    return true;
-  }
-  // Partial slot of the unit, -1 if its item lies in one part (several divisions: only the epilogue asks);
-  // *info = what the combine needs to know about the item
-  __device__ int slot_of(const Unit& u, int2* info) const {
-    int p_first, p_last;
-    const int nsplit = plan.item_parts(u.it, &p_first, &p_last);
-    *info = make_int2(plan.slot_of(p_first, u.it, p_first), nsplit);
-    return nsplit == 1 ? -1 : plan.slot_of(p, u.it, p_first);
-  }
-};
 
 // Finds the unit that holds the k-th tile of this cluster's part; k never decreases between calls.
 struct Cursor {
@@ -681,6 +641,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       // sustained and 134.8 cool; elected: 150.5 and 128.1).  Written out per slot and column block for the same reason:
       // with a rolled loop over the slots the call takes 188.7 us.
       if (leader) {
+        if (elect_one()) {
         constexpr uint32_t idesc = make_idesc_bf16(256, 128, false, false);
         constexpr uint32_t dhi = smem_desc_hi_sw128(kKGroupStride);
         constexpr uint32_t qhi = smem_desc_hi_sw128(1024);
@@ -688,15 +649,15 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         const uint32_t qlo0 = smem_desc_lo(smem_base + kOffQRope, 16);
         uint32_t slot = 0, kpar = 0;
         while (ok && iter.next(u)) {
-          ok = warp_wait<true>(bar(A_QREADY), un & 1);
+          ok = mbar_wait<true>(bar(A_QREADY), un & 1);
           if (!ok) break;
           tc_fence_after_sync();
           for (int t = u.t0; t < u.t1 && ok; ++t, ++gs) {
             const uint32_t sb = gs & 1;
-            ok = warp_wait(bar(A_SEMPTY + sb), ((gs >> 1) & 1) ^ 1);
+            ok = mbar_wait(bar(A_SEMPTY + sb), ((gs >> 1) & 1) ^ 1);
             if (!ok) break;
             tc_fence_after_sync();
-            if (lane == 0) QSTAMP(smem_base, 0, gs);
+            QSTAMP(smem_base, 0, gs);
             const uint32_t d = tbase + kSCol + 128 * sb;
             // the three slots of the tile are probed together (their latencies overlap); the blocking wait runs
             // only for one that is not there yet
@@ -705,15 +666,15 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
               uint32_t s2 = slot, p2 = kpar;
 #pragma unroll
               for (int gg = 0; gg < 3; ++gg) {
-                have[gg] = __all_sync(0xffffffffu, mbar_probe(bar(A_KFULL) + 8 * s2, p2));
+                have[gg] = mbar_probe(bar(A_KFULL) + 8 * s2, p2);
                 if (++s2 == kNumKSlots) { s2 = 0; p2 ^= 1; }
               }
             }
 #pragma unroll
             for (int gg = 0; gg < 3; ++gg) {
-              ok = ok && (have[gg] || warp_wait(bar(A_KFULL) + 8 * slot, kpar));
+              ok = ok && (have[gg] || mbar_wait(bar(A_KFULL) + 8 * slot, kpar));
               if (ok) {
-                if (gg == 0 && lane == 0) QSTAMP(smem_base, 12, gs);
+                if (gg == 0) QSTAMP(smem_base, 12, gs);
                 const uint32_t klo = klo0 + slot * (kKSlotBytes >> 4);
 #pragma unroll
                 for (int cl = 0; cl < 3; ++cl) {
@@ -721,23 +682,25 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
 #pragma unroll
                   for (int kk = 0; kk < 4; ++kk) {
                     const uint64_t bd = smem_desc_join(klo + 64 * cl + 2 * kk, dhi);
-                    if (cb < 8) mma_ts_pair_elect(d, tbase + kQCol + 32 * cb + 8 * kk, bd, idesc, (cb | kk) != 0 ? 1u : 0u);
-                    else mma_ss_pair_elect(d, smem_desc_join(qlo0 + 2 * kk, qhi), bd, idesc, 1u);   // RoPE columns: Q from shared memory
+                    if (cb < 8) mma_ts_pair(d, tbase + kQCol + 32 * cb + 8 * kk, bd, idesc, (cb | kk) != 0 ? 1u : 0u);
+                    else mma_ss_pair(d, smem_desc_join(qlo0 + 2 * kk, qhi), bd, idesc, 1u);   // RoPE columns: Q from shared memory
                   }
                 }
-                mma_commit_pair_multicast_elect(bar(A_KEMPTY) + 8 * slot, kMaskScore);
+                mma_commit_pair_multicast(bar(A_KEMPTY) + 8 * slot, kMaskScore);
               }
               if (++slot == kNumKSlots) { slot = 0; kpar ^= 1; }
             }
             if (!ok) break;
-            mma_commit_pair_multicast_elect(bar(A_SFULL + sb), kMaskScore);
-            if (lane == 0) QSTAMP(smem_base, 1, gs);
+            mma_commit_pair_multicast(bar(A_SFULL + sb), kMaskScore);
+            QSTAMP(smem_base, 1, gs);
           }
           if (!ok) break;
-          mma_commit_pair_multicast_elect(bar(A_QFREE), kMaskScore);
+          mma_commit_pair_multicast(bar(A_QFREE), kMaskScore);
           ++un;
         }
-        if (!ok && lane == 0) report_timeout(prm.status);
+        if (!ok) report_timeout(prm.status);
+        }
+        __syncwarp();
       } else if (!leader) {
         // ---- relay (odd CTA): lanes 0, 1 pass on the completed phases of SEMPTY[lane] (the tiles with that buffer),
         // lane 2 those of QREADY (one per unit)
@@ -931,6 +894,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       // ---- MMA issuer (even CTA only): O (+)= P~ V for both CTAs' rows; per page two N = 256 halves of four
       // K = 16 steps
       if (leader) {
+        if (elect_one()) {
         constexpr uint32_t idesc = make_idesc_bf16(256, 256, false, true);
         constexpr uint32_t dhi = smem_desc_hi_sw128(1024);
         const uint32_t vlo0 = smem_desc_lo(smem_base + kOffV, kBoxBytes);
@@ -940,17 +904,17 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           const int npages = 2 * (u.t1 - u.t0);
           for (int pi = 0; pi < npages && ok; ++pi, ++gt) {
             const uint32_t s = gt % kNumP, k = gt / kNumP;
-            ok = warp_wait<true>(bar(B_PFULL + s), k & 1);
+            ok = mbar_wait<true>(bar(B_PFULL + s), k & 1);
             if (!ok) break;
-            if (lane == 0) QSTAMP(smem_base, 10, gt);
-            ok = warp_wait(bar(B_OREADY + s), k & 1);
+            QSTAMP(smem_base, 10, gt);
+            ok = mbar_wait(bar(B_OREADY + s), k & 1);
             if (!ok) break;
-            if (lane == 0) QSTAMP(smem_base, 11, gt);
+            QSTAMP(smem_base, 11, gt);
             tc_fence_after_sync();
             fence_proxy_async_smem();
-            ok = warp_wait(bar(B_VFULL) + 8 * slot, vpar);
+            ok = mbar_wait(bar(B_VFULL) + 8 * slot, vpar);
             if (!ok) break;
-            if (lane == 0) QSTAMP(smem_base, 8, gt);
+            QSTAMP(smem_base, 8, gt);
             const uint32_t plo = plo0 + s * (kPStride >> 4);
             const uint32_t vlo = vlo0 + slot * (kVSlotBytes >> 4);
             const uint32_t acc0 = pi > 0 ? 1u : 0u;
@@ -958,17 +922,19 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
             for (int nh = 0; nh < 2; ++nh) {
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk)
-                mma_ss_pair_elect(tbase + nh * 256, smem_desc_join(plo + 2 * kk, dhi), smem_desc_join(vlo + nh * (kVHalfBytes >> 4) + 128 * kk, dhi),
+                mma_ss_pair(tbase + nh * 256, smem_desc_join(plo + 2 * kk, dhi), smem_desc_join(vlo + nh * (kVHalfBytes >> 4) + 128 * kk, dhi),
                             idesc, kk == 0 ? acc0 : 1u);
             }
-            mma_commit_pair_multicast_elect(bar(B_VEMPTY) + 8 * slot, kMaskValue);
+            mma_commit_pair_multicast(bar(B_VEMPTY) + 8 * slot, kMaskValue);
             if (++slot == kNumVSlots) { slot = 0; vpar ^= 1; }
-            mma_commit_pair_multicast_elect(bar(X_PV + s), kMaskAll);   // PVDONE in the value CTAs, "P buffer free" in the score CTAs
-            if (lane == 0) QSTAMP(smem_base, 9, gt);
+            mma_commit_pair_multicast(bar(X_PV + s), kMaskAll);   // PVDONE in the value CTAs, "P buffer free" in the score CTAs
+            QSTAMP(smem_base, 9, gt);
           }
           if (!ok) break;
         }
-        if (!ok && lane == 0) report_timeout(prm.status);
+        if (!ok) report_timeout(prm.status);
+        }
+        __syncwarp();
       } else if (!leader) {
         // ---- relay (odd CTA): lane s passes on the completed phases of OREADY[s] (the pages in P buffer s).  The
         // page's P~ in this CTA (remote asynchronous stores, generic proxy) is about to be read by the pair MMA.

@@ -13,18 +13,6 @@ namespace amla {
 
 namespace {
 
-// Two E4M3 bytes (low 16 bits of `pair`) -> two bf16 in one word.  E4M3 -> f16 is one hardware conversion and
-// exact; f16 -> f32 -> bf16 is exact for these values (at most four significant bits, exponents -9 .. 8).
-__device__ __forceinline__ uint32_t e4m3x2_to_bf16x2(uint32_t pair) {
-  uint32_t h2;
-  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"(static_cast<unsigned short>(pair & 0xffffu)));
-  float lo, hi;
-  asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\tcvt.f32.f16 %0, a;\n\tcvt.f32.f16 %1, b;\n\t}" : "=f"(lo), "=f"(hi) : "r"(h2));
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-
 constexpr int kWidenThreads = 256;
 constexpr int kPageBytes8 = kPage * kDqk;            // 36 864 bytes of E4M3 per page
 

@@ -6,43 +6,67 @@
 namespace amla {
 
 struct Unit {
-  int b, r0, n_b, t0, t1, it;      // sequence, first row of the row block, keys, page range [t0, t1), item
+  int b, r0, n_b, t0, t1, it;      // sequence, first row of the row block, keys, tile range [t0, t1) of the schedule, item
 };
+
+// The next unit at or after position g of a range that ends at g1.  Not inlined: every role asks for units, but seldom,
+// and what a cluster executes over and over has to stay small (a kernel of 144 KB of code, with this walk written out at
+// a dozen places, spent hundreds of cycles per score tile on instruction fetches in every role).
+struct UnitFound {
+  Unit u;
+  int g;                           // position behind the unit
+};
+static __device__ __noinline__ UnitFound find_unit(const int* prefix, const int* seqlens, int n_items, int nrb, int item_rows, int max_keys, int ovh, int g, int g1) {
+  UnitFound f;
+  f.u.t0 = f.u.t1 = 0;
+  f.u.it = f.u.b = f.u.r0 = f.u.n_b = 0;
+  while (g < g1) {
+    int lo = 0, hi = n_items - 1;                 // the item that holds position g (zero-tile items are skipped automatically)
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (prefix[mid] <= g) lo = mid; else hi = mid - 1;
+    }
+    const int a = prefix[lo] + item_overhead(lo, ovh), e = prefix[lo + 1];
+    const int first = max(g, a), last = min(e, g1);
+    g = last;
+    if (last > first) {
+      f.u.it = lo; f.u.t0 = first - a; f.u.t1 = last - a;
+      f.u.b = nrb == 1 ? lo : static_cast<int>(static_cast<unsigned>(lo) / static_cast<unsigned>(nrb));
+      f.u.r0 = (lo - f.u.b * nrb) * item_rows;
+      f.u.n_b = min(max(seqlens[f.u.b], 0), max_keys);
+      break;
+    }                                             // else: only overhead positions of this item fell into the range
+  }
+  f.g = g;
+  return f;
+}
 
 struct UnitIter {
   const DecodeParams& prm;
-  Plan plan;
-  int p, g, g1;
+  const int* prefix;
   const int* seqlens;
-  __device__ UnitIter(const DecodeParams& prm_, const int* prefix, const int* seqlens_, int part)
-      : prm(prm_), plan(Plan::make(prefix, prm_.n_items, prm_.P, prm_.ovh)), p(part), seqlens(seqlens_) {
+  int p, g, g1, share, parts;
+  __device__ UnitIter(const DecodeParams& prm_, const int* prefix_, const int* seqlens_, int part) : prm(prm_), prefix(prefix_), seqlens(seqlens_), p(part) {
+    const Plan plan = Plan::make(prefix, prm.n_items, prm.P, prm.ovh);
+    share = plan.share; parts = plan.P;
     if (plan.L <= 0 || p >= plan.P) { g = g1 = 0; }
     else { g = plan.part_start(p); g1 = plan.part_start(p + 1); }
   }
   __device__ bool next(Unit& u) {
-    int it, a;
-    while (true) {
-      if (g >= g1) return false;
-      it = plan.item_of_tile(g);
-      a = plan.first_tile(it);
-      const int e = plan.prefix[it + 1];
-      const int lo = max(g, a), hi = min(e, g1);
-      g = min(e, g1);
-      if (hi > lo) { u.t0 = lo - a; u.t1 = hi - a; break; }   // else: only overhead positions of this item fell into the part
-    }
-    u.it = it;
-    u.b = it / prm.nrb;
-    u.r0 = (it - u.b * prm.nrb) * prm.item_rows;
-    u.n_b = min(max(seqlens[u.b], 0), prm.max_blocks_per_seq * kPage);
-    return true;
+    if (g >= g1) return false;
+    const UnitFound f = find_unit(prefix, seqlens, prm.n_items, prm.nrb, prm.item_rows, prm.max_blocks_per_seq * kPage, prm.ovh, g, g1);
+    u = f.u;
+    g = f.g;
+    return u.t1 > u.t0;
   }
-  // Partial slot of the unit, -1 if its item lies in one part (several divisions: only the epilogue asks);
-  // *info = what the combine needs to know about the item
+  // Partial slot of the unit, -1 if its item lies in one part; *info = what the combine needs to know about the item
   __device__ int slot_of(const Unit& u, int2* info) const {
-    int p_first, p_last;
-    const int nsplit = plan.item_parts(u.it, &p_first, &p_last);
-    *info = make_int2(plan.slot_of(p_first, u.it, p_first), nsplit);
-    return nsplit == 1 ? -1 : plan.slot_of(p, u.it, p_first);
+    const int begin = prefix[u.it];
+    const int p_first = static_cast<int>(static_cast<unsigned>(begin + item_overhead(u.it, prm.ovh)) / static_cast<unsigned>(share));
+    const int p_last = static_cast<int>(static_cast<unsigned>(prefix[u.it + 1] - 1) / static_cast<unsigned>(share));
+    const int slot_first = 2 * p_first + (begin > p_first * share ? 1 : 0);
+    *info = make_int2(slot_first, p_last - p_first + 1);
+    return p_first == p_last ? -1 : p == p_first ? slot_first : 2 * p;
   }
 };
 
@@ -62,7 +86,7 @@ struct TileIter {
     valid = units.next(u);
     if (!valid) return;
     const int n = u.t1 - u.t0, nt = (n + kMaxPages - 1) / kMaxPages;
-    base = n / nt; rem = n - base * nt;
+    base = static_cast<int>(static_cast<unsigned>(n) / static_cast<unsigned>(nt)); rem = n - base * nt;
     left = nt; first = true;
     t = u.t0; np = 0;
     step();
