@@ -88,10 +88,18 @@ constexpr uint32_t kSCol = 256;          // 2 x 128 columns
 enum { X_FULL = 0 /*L*/, X_EMPTY = X_FULL + 7, X_QFULL = X_EMPTY + 7 /*L*/, X_QFREE, X_SFULL, X_SEMPTY = X_SFULL + 2 /*L*/,
        X_PREADY = X_SEMPTY + 2 /*L*/, X_PVDONE, X_XCHG, X_RAWFULL = X_XCHG + 2, X_RAWEMPTY = X_RAWFULL + kRawSlots,
        X_NUM = X_RAWEMPTY + kRawSlots };
-constexpr uint32_t kTmemSlotOff = kBarBytes - 8;
 static_assert(X_NUM * 8 + 8 <= kBarBytes, "barrier area too small");
 
 __device__ __forceinline__ void report_timeout(int* status) { atomicExch(status, kStatusTimeout); }
+
+__device__ __forceinline__ int warp_inclusive_scan(int v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  return v;
+}
 
 // Wait whose verdict is the same in every lane of the warp, so that the warp-collective tensor-memory instructions
 // that follow are never executed by a part of it.
@@ -128,14 +136,32 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   }
   const uint32_t bars = smem_base + kOffBars;
   auto bar = [&](int i) { return bars + 8u * i; };
-  const uint32_t tmem_slot = bars + kTmemSlotOff;
+  const uint32_t tmem_slot = bars + kBarBytes - 8;
   const uint32_t lead_bars = map_to_cta(bars, 0);
 
-  // The lengths of the first 32 items are requested before anything else, so that their latency runs under the set-up
-  // below (they are inputs of the call: no kernel that this one may overlap with writes them).
-  int early_len = 0;
-  if (wid == 0 && prm.fused_plan && lane < prm.n_items) early_len = prm.seqlens[lane / prm.nrb];
-  if (tid == 32 * 8) {
+  // Set-up, three things side by side: warp 8, which will need the result first, works out the schedule of a batch of up to
+  // kSmemPlanItems items (from the sequence lengths: inputs of the call, which no kernel that this one may overlap with
+  // writes), warp 9 allocates tensor memory, one thread of warp 10 initialises the barriers.
+  const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
+  int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
+  int* lens_smem = reinterpret_cast<int*>(smem_raw + kOffSeqlens);
+  if (wid == 8 && plan_here) {
+    int carry = 0;
+    for (int base = 0; base < prm.n_items; base += 32) {
+      const int it = base + lane;
+      const int b = prm.nrb == 1 ? it : it / prm.nrb;
+      const int n_seq = it < prm.n_items ? prm.seqlens[b] : 0;
+      const int v = it < prm.n_items ? schedule_length(n_seq, it, prm.tile_keys, prm.ovh) : 0;
+      const int x = warp_inclusive_scan(v, lane);
+      if (it < prm.n_items) {
+        lens_smem[b] = n_seq;                            // same value from every row block
+        plan_smem[it] = carry + x - v;
+      }
+      carry += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) plan_smem[prm.n_items] = carry;
+  }
+  if (tid == 32 * 10) {
     for (int i = 0; i < kSlots<kFp8>; ++i) {
       mbar_init(bar(X_FULL + i), kFp8 ? 4 : 1);          // E4M3: the two warps that fill the slot, in either CTA
       mbar_init(bar(X_EMPTY + i), 1);
@@ -158,62 +184,52 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     prefetch_tensormap(&q_map);
   }
   if (wid == 9) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
+  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 6);
   tc_fence_before_sync();
   __syncthreads();
-  cluster_arrive();
-  cluster_wait();          // the peer's barriers are initialised before anyone signals them
+  cluster_arrive();        // the peer's barriers are initialised before anyone signals them (waited for below)
   tc_fence_after_sync();
   const uint32_t tbase = ld_shared_b32(tmem_slot);
-
-  // Launched with programmatic stream serialization: everything above ran while the kernel before this one on the
-  // stream was still going; its results (the schedule kernel's prefix array, or the previous call's reads of the
-  // workspace) are complete after this wait.
   if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 3);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;");
-  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 4);
-  const int* prefix = prm.prefix;
-  const int* seqlens = prm.seqlens;
-  if (prm.fused_plan) {
-    // Few items: every CTA computes the schedule prefix itself instead of waiting for a one-block kernel (the combine
-    // kernel reads the copy that the first CTA leaves in the workspace).  A small batch's prefix and sequence lengths
-    // stay in shared memory; of a larger one every CTA writes the same values to the workspace.
-    int* ps = prm.n_items <= kSmemPlanItems ? reinterpret_cast<int*>(smem_raw + kOffPlan) : nullptr;
-    if (wid == 0) {
-      int* pw = !ps || blockIdx.x == 0 ? const_cast<int*>(prm.prefix) : nullptr;
-      int carry = 0;
-      for (int base = 0; base < prm.n_items; base += 32) {
-        const int it = base + lane;
-        const int n_seq = it >= prm.n_items ? 0 : base == 0 ? early_len : prm.seqlens[it / prm.nrb];
-        if (ps && it < prm.n_items) reinterpret_cast<int*>(smem_raw + kOffSeqlens)[it / prm.nrb] = n_seq;   // same value from every row block
-        const int v = it < prm.n_items ? schedule_length(n_seq, it, prm.tile_keys, prm.ovh) : 0;
-        int x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, x, o);
-          if (lane >= o) x += y;
-        }
-        if (it < prm.n_items) {
-          if (pw) pw[it] = carry + x - v;
-          if (ps) ps[it] = carry + x - v;
-        }
-        carry += __shfl_sync(0xffffffffu, x, 31);
-      }
-      if (lane == 0) {
-        if (pw) pw[prm.n_items] = carry;
-        if (ps) ps[prm.n_items] = carry;
-        if (blockIdx.x == 0) *prm.status = kStatusOk;
-      }
-      __threadfence_block();
-    }
-    __syncthreads();
-    if (ps) { prefix = ps; seqlens = reinterpret_cast<const int*>(smem_raw + kOffSeqlens); }
-  }
 
-  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 1);
+  const int* prefix = plan_here ? plan_smem : prm.prefix;
+  const int* seqlens = plan_here ? lens_smem : prm.seqlens;
+  if (!plan_here) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (prm.fused_plan) {      // (kSmemPlanItems, kFusedPlanMaxItems] items: every CTA writes the same prefix to the workspace
+      if (wid == 0) {
+        int* pw = const_cast<int*>(prm.prefix);
+        int carry = 0;
+        for (int base = 0; base < prm.n_items; base += 32) {
+          const int it = base + lane;
+          const int v = it < prm.n_items ? schedule_length(prm.seqlens[it / prm.nrb], it, prm.tile_keys, prm.ovh) : 0;
+          const int x = warp_inclusive_scan(v, lane);
+          if (it < prm.n_items) pw[it] = carry + x - v;
+          carry += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (lane == 0) pw[prm.n_items] = carry;
+        if (tid == 0 && blockIdx.x == 0) *prm.status = kStatusOk;
+        __threadfence_block();
+      }
+      __syncthreads();
+    }
+  }
   bool ok = true;
   Tiles tile(UnitIter(prm, prefix, seqlens, part));
   if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 5);
+  cluster_wait();
+  if (plan_here) {
+    // Launched with programmatic stream serialization: everything above ran while the kernel before this one on the stream
+    // was still going; its results (the previous call's reads of the workspace among them) are complete after this wait.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (blockIdx.x == 0 && wid == 0) {       // the combine kernel reads the prefix in the workspace
+      for (int it = lane; it <= prm.n_items; it += 32) const_cast<int*>(prm.prefix)[it] = plan_smem[it];
+      if (lane == 0) *prm.status = kStatusOk;
+    }
+  }
+  if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 4);
 
   if (wid < kSoftmaxWarps) {
     // ======================================================== softmax, correction, epilogue
@@ -526,7 +542,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         for (int p = 0; p < kTilePages; ++p) page[p] = p < x.np ? __ldg(x.bt + p) : 0;
       };
       TileRef cur = take(), prev = cur;
-      get_pages(cur);
+      get_pages(cur);                                       // on its way while Q is requested
       TileRef nxt = take();
       bool q_out = false;                                   // the Q of the unit that starts next has been requested
       uint32_t pt = 0;
