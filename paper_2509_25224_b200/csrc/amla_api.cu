@@ -28,15 +28,15 @@ constexpr int kMaxRows = 1024;   // Sq * H
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-  size_t status_off, prefix_off, info_off, part_lse_off, part_o_off, total;
+  size_t status_off, merge_off, prefix_off, part_lse_off, part_o_off, total;
 };
 
 Layout make_layout(int n_items, int max_parts) {
   Layout l;
   l.status_off = 0;
-  l.prefix_off = kAlign;
-  l.info_off = l.prefix_off + align_up(sizeof(int) * (static_cast<size_t>(n_items) + 1));
-  l.part_lse_off = l.info_off + align_up(sizeof(int2) * static_cast<size_t>(n_items));
+  l.merge_off = kAlign;
+  l.prefix_off = l.merge_off + align_up(sizeof(int4) * static_cast<size_t>(max_parts));
+  l.part_lse_off = l.prefix_off + align_up(sizeof(int) * (static_cast<size_t>(n_items) + 1));
   l.part_o_off = l.part_lse_off + align_up(sizeof(float) * 2 * static_cast<size_t>(max_parts) * kRowBlock);
   l.total = l.part_o_off + sizeof(float) * 2 * static_cast<size_t>(max_parts) * kRowBlock * kDv;
   return l;
@@ -103,6 +103,9 @@ int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
   prm.item_rows = quad ? 2 * kRowBlock : kRowBlock;
   prm.tile_keys = quad ? 2 * kPage : kPage;
   prm.ovh = quad ? kQuadOverheadTiles : kUnitOverheadTiles;
+  // (tau = 0 asks for Algorithm 2 to the letter: its parts stay as fine as the schedule's tiles, so that a short sequence
+  // is summed in blocks of 64 keys)
+  prm.min_share = simt || (flags & AMLA_LAZY_MASK) == 0 ? 1 : kMinPartKeys / prm.tile_keys;
   prm.nrb = (prm.R + prm.item_rows - 1) / prm.item_rows;
   prm.n_items = prm.B * prm.nrb;
   prm.P = simt ? sms : quad ? quad_parts : decode_pair_parts(sms);
@@ -210,7 +213,7 @@ int decode_impl(const void* q, const void* kv_cache, const uint8_t* kv8, const i
   prm.status = reinterpret_cast<int*>(ws + lay.status_off);
   int* prefix = reinterpret_cast<int*>(ws + lay.prefix_off);
   prm.prefix = prefix;
-  prm.item_info = reinterpret_cast<int2*>(ws + lay.info_off);
+  prm.merge_info = reinterpret_cast<int4*>(ws + lay.merge_off);
   prm.part_lse = reinterpret_cast<float*>(ws + lay.part_lse_off);
   prm.part_o = reinterpret_cast<float*>(ws + lay.part_o_off);
   prm.scale_log2 = softmax_scale * kLog2e;

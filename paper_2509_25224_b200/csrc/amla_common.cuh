@@ -32,8 +32,9 @@ struct DecodeParams {
   float* part_o;                 // normalised partial outputs of split items: [2 * P * item_rows][512] half precision, then
                                  // [2 * P * item_rows][16] scale bytes (see "Split partials" below)
   float* part_lse;               // [2 * P, 128]      partial lse (natural log)
-  int2* item_info;               // [n_items] (slot of the item's first partial, number of parts it is split over), written by
-                                 // the decode kernel for every item it touches, read by the combine
+  int4* merge_info;              // [min(n_items, P)] what the combine kernel has to merge: (item, slot of its first partial, number of
+                                 // partials, 0), number < 2: nothing.  Written by the decode kernel; indexed by item where there are no
+                                 // more items than parts, else by the part in which the item begins (one split item at most)
   float scale_log2;              // softmax_scale * log2(e)
   float tau;                     // lazy-reference threshold in octaves (0 = move the reference with every new maximum)
   float out_scale;               // factor on the normalised output (1; the dequantisation scale of an FP8 cache's V)
@@ -48,6 +49,7 @@ struct DecodeParams {
   int tile_keys;                 // keys per schedule tile: 64 (one page) or 128 (two pages, the 256-row kernel)
   int item_rows;                 // query rows per work item: 128, or 256 for the 256-row kernel (nrb counts these)
   int ovh;                       // schedule positions that stand for the cost of starting an item
+  int min_share;                 // a part is given at least this many positions
   unsigned long long* trace;     // timeline buffer of a -DAMLA_TRACE build, else unused (nullptr)
 };
 
@@ -89,6 +91,7 @@ constexpr int kUnitOverheadTiles = AMLA_UNIT_OVERHEAD_TILES;
 #define AMLA_QUAD_OVERHEAD_TILES 5            // 256-row kernel: in 128-key tiles (a build-time knob for tuning runs)
 #endif
 constexpr int kQuadOverheadTiles = AMLA_QUAD_OVERHEAD_TILES;
+constexpr int kMinPartKeys = 128;           // a part holds at least this many keys: a shorter one takes as long, and every part is a partial to merge
 constexpr int kFusedPlanMaxItems = 2048;   // up to this many items every decode CTA computes the prefix itself
 
 // Overhead positions in front of item `it`: none for the first item, which opens the first part anyway (every
@@ -111,13 +114,14 @@ struct Plan {
   int ovh;
   int share;     // positions per part (the last part may have fewer)
 
-  __host__ __device__ static Plan make(const int* prefix, int n_items, int max_parts, int ovh) {
+  __host__ __device__ static Plan make(const int* prefix, int n_items, int max_parts, int ovh, int min_share = 1) {
     Plan pl;
     pl.prefix = prefix;
     pl.ovh = ovh;
     pl.n_items = n_items;
     pl.L = prefix[n_items];
     pl.share = pl.L > max_parts ? static_cast<int>((static_cast<unsigned>(pl.L) + max_parts - 1) / static_cast<unsigned>(max_parts)) : 1;
+    if (pl.share < min_share) pl.share = min_share;
     pl.P = pl.L > 0 ? static_cast<int>((static_cast<unsigned>(pl.L) + pl.share - 1) / static_cast<unsigned>(pl.share)) : 1;
     return pl;
   }
@@ -148,9 +152,12 @@ struct Plan {
   __host__ __device__ int slot_of(int p, int it, int p_first) const {
     return 2 * p + ((p == p_first && prefix[it] > part_start(p)) ? 1 : 0);
   }
-  // The same from what item_info holds: slot of split s (0 = the part where the item begins) of an item
+  // The same from what merge_info holds: slot of split s (0 = the part where the item begins) of an item
   __host__ __device__ static int slot_of_split(int first_slot, int s) { return s == 0 ? first_slot : 2 * ((first_slot >> 1) + s); }
 };
+
+__host__ __device__ inline bool merge_by_item(const DecodeParams& prm) { return prm.n_items <= prm.P; }
+__host__ __device__ inline int merge_groups(const DecodeParams& prm) { return prm.n_items < prm.P ? prm.n_items : prm.P; }
 
 // ---------------------------------------------------------------------------------------------
 // Split partials.  A part that holds some of an item's tiles leaves the item's normalised output rows for the

@@ -254,6 +254,8 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(ld_shared_b32(buf + i * (kCtaRows * 4)));
     };
 
+    if (tid == 0 && leader) merge_begin(prm, part);
+    write_empty_items(prm, prefix, part, prm.P, rank * kCtaRows, kCtaRows, tid, 32 * kSoftmaxWarps);
     while (ok && tile.valid) {
       const Unit u = tile.u;
       const int row = u.r0 + rank * kCtaRows + r;        // row within the sequence
@@ -428,7 +430,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       // of its 512 columns each and store them from registers with 256-bit stores (a full 32-byte sector per lane).
       int2 info;
       const int slot = tile.units.slot_of(u, &info);
-      if (tid == 0 && leader) prm.item_info[u.it] = info;
+      if (tid == 0 && leader) merge_note(prm, part, u.it, info);
       float l4[4];
       exchange(st.l, l4);
       if (!ok) break;

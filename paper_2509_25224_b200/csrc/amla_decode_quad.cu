@@ -721,11 +721,13 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       const int r = (wid & 3) * 32 + lane;
       const uint32_t lane_base = static_cast<uint32_t>((wid & 3) * 32) << 16;
       const int c_first = partner ? 8 : 0;
+      if (tid == 0 && leader) merge_begin(prm, part);
+      write_empty_items(prm, prefix, part, prm.P, half * kRowBlock, kRowBlock, partner ? r + kRowBlock : r, 2 * kRowBlock);
       while (ok && iter.next(u)) {
         const int npages = 2 * (u.t1 - u.t0);
         int2 info;
         const int slot = iter.slot_of(u, &info);
-        if (tid == 0 && leader) prm.item_info[u.it] = info;
+        if (tid == 0 && leader) merge_note(prm, part, u.it, info);
         float inv = 0.f, lse = 0.f;
         for (int pi = 0; pi < npages && ok; ++pi, ++gt) {
           const uint32_t s = gt % kNumP, k = gt / kNumP;

@@ -3,6 +3,7 @@
 // tensor-core kernel, one warp per query row, and exists to validate those pieces; it is only
 // reachable through AMLA_FLAG_KERNEL_SIMT and is never chosen automatically.
 #include "amla_common.cuh"
+#include "amla_units.cuh"
 
 namespace amla {
 
@@ -22,9 +23,10 @@ __global__ void __launch_bounds__(kWarps * 32) decode_simt_kernel(DecodeParams p
 
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const Plan plan = Plan::make(prm.prefix, prm.n_items, prm.P, prm.ovh);
-  if (plan.L <= 0) return;
   const int p = blockIdx.x;
-  if (p >= plan.P) return;
+  if (tid == 0) merge_begin(prm, p);
+  write_empty_items(prm, prm.prefix, p, prm.P, 0, kRowBlock, tid, blockDim.x);
+  if (plan.L <= 0 || p >= plan.P) return;
   const int g0 = plan.part_start(p), g1 = plan.part_start(p + 1);
 
   int g = g0;
@@ -42,7 +44,7 @@ __global__ void __launch_bounds__(kWarps * 32) decode_simt_kernel(DecodeParams p
     int p_first, p_last;
     const int nsplit = plan.item_parts(it, &p_first, &p_last);
     const int slot = nsplit == 1 ? -1 : plan.slot_of(p, it, p_first);
-    if (tid == 0) prm.item_info[it] = make_int2(plan.slot_of(p_first, it, p_first), nsplit);
+    if (tid == 0) merge_note(prm, p, it, make_int2(plan.slot_of(p_first, it, p_first), nsplit));
     const int32_t* bt = prm.block_table + static_cast<size_t>(b) * prm.max_blocks_per_seq;
 
     for (int pass = 0; pass * kRowsPerPass < nrows; ++pass) {

@@ -46,51 +46,38 @@ __global__ void plan_kernel(const int32_t* __restrict__ seqlens, int nrb, int n_
   if (tid == 0) prefix[n_items] = carry;
 }
 
-// One warp per query row.  Items that one part covered entirely were written by the decode kernel and are skipped;
-// items without tiles get out = 0, lse = -inf; split items are merged:
-//   lse = ln sum_s exp(lse_s),  out = sum_s exp(lse_s - lse) * out_s.
-// What the row needs to know about its item (where its partials are) was left in item_info by the decode kernel, so
-// the warp's chain of dependent memory round trips is short: (prefix, item_info) -> (partial lse, partial rows).
-// Up to kFastSplits partials are fetched before any arithmetic.
+// The merge of split items,
+//   lse = ln sum_s exp(lse_s),  out = sum_s exp(lse_s - lse) * out_s,
+// one warp per query row.  The decode kernel left in merge_info which items are split, by item or, where there are more
+// items than parts, by the part in which a split item begins: the grid is min(items, parts) x rows of an item whatever
+// the batch (192 sequences, 74 parts: a grid over all rows cost the call 12 us; 32 sequences: a grid over parts 3 us more
+// than one over items), and a warp's chain of dependent memory round trips is merge_info -> (partial lse, partial rows).  Up to kFastSplits
+// partials are fetched before any arithmetic, of more than that eight at a time.
 constexpr int kFastSplits = 4;
+constexpr int kManyBatch = 8;
 
 __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
-#ifdef AMLA_TRACE
-  unsigned long long t_ns;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_ns));
-  if (prm.trace && blockIdx.x == 0 && threadIdx.x == 0) prm.trace[148 * 16 * 128 + 0] = t_ns & 0xffffffffull;
-#endif
   // A decode kernel that follows on the stream may set itself up beside this kernel (it writes nothing this kernel
   // reads before its own wait for this kernel's completion).
   asm volatile("griddepcontrol.launch_dependents;");
   const int warps_per_block = blockDim.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int row_global = blockIdx.x * warps_per_block + (threadIdx.x >> 5);
-  const int rows_padded = prm.nrb * prm.item_rows;
-  const int b = row_global / rows_padded;
-  const int rin = row_global - b * rows_padded;   // row within the sequence, padded to items
-  const bool live = b < prm.B && rin < prm.R;
-  const int rb = rin / prm.item_rows, rr = rin % prm.item_rows;   // item of the sequence, row within the item
-  const int it = b * prm.nrb + rb;
+  const int chunks = prm.item_rows / warps_per_block;
+  const int group = blockIdx.x / chunks;
+  const int rr = (blockIdx.x - group * chunks) * warps_per_block + (threadIdx.x >> 5);     // row within the item
   asm volatile("griddepcontrol.wait;" ::: "memory");   // launched early (programmatic dependent launch): the partials must be complete
-#ifdef AMLA_TRACE
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_ns));
-  if (prm.trace && blockIdx.x == 0 && threadIdx.x == 0) prm.trace[148 * 16 * 128 + 1] = t_ns & 0xffffffffull;
-  if (prm.trace && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) prm.trace[148 * 16 * 128 + 2] = t_ns & 0xffffffffull;
-#endif
-  if (!live) return;
-
-  const int pa = prm.prefix[it], pe = prm.prefix[it + 1];
-  const int2 info = prm.item_info[it];           // valid only for items with tiles
+  const int4 info = prm.merge_info[group];
+  const int nsplit = info.z;
+  if (nsplit < 2) return;
+  const int b = info.x / prm.nrb;
+  const int rin = (info.x - b * prm.nrb) * prm.item_rows + rr;                          // row within the sequence
+  if (rin >= prm.R) return;
   __nv_bfloat16* orow = prm.out + (static_cast<size_t>(b) * prm.R + rin) * kDv;
   float* lrow = prm.lse + static_cast<size_t>(b) * prm.R + rin;
   auto write_empty = [&]() {
     for (int c = lane * 8; c < kDv; c += 32 * 8) *reinterpret_cast<uint4*>(orow + c) = make_uint4(0, 0, 0, 0);
     if (lane == 0) *lrow = -INFINITY;
   };
-  if (pe <= pa) { write_empty(); return; }       // no tiles: no part ever saw this item
-  const int nsplit = info.y;
-  if (nsplit == 1) return;
 
   // a lane merges 16 consecutive columns (half of a 32-column chunk: one scale byte per split)
   const uint16_t* halves = partial_halves(prm);
@@ -116,7 +103,7 @@ __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
     for (int s = 0; s < kFastSplits; ++s) {
       ls[s] = -INFINITY;
       if (s < nsplit) {
-        const size_t prow = static_cast<size_t>(Plan::slot_of_split(info.x, s)) * prm.item_rows + rr;
+        const size_t prow = static_cast<size_t>(Plan::slot_of_split(info.y, s)) * prm.item_rows + rr;
         ls[s] = prm.part_lse[prow];
         sc[s] = scales[prow * 16 + (lane >> 1)];
         const uint4* src = reinterpret_cast<const uint4*>(halves + prow * kDv) + 2 * lane;
@@ -143,7 +130,7 @@ __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
     mx = -INFINITY;
     for (int base = 0; base < nsplit; base += 32) {
       const int sidx = base + lane;
-      if (sidx < nsplit) mx = fmaxf(mx, prm.part_lse[static_cast<size_t>(Plan::slot_of_split(info.x, sidx)) * prm.item_rows + rr]);
+      if (sidx < nsplit) mx = fmaxf(mx, prm.part_lse[static_cast<size_t>(Plan::slot_of_split(info.y, sidx)) * prm.item_rows + rr]);
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -155,18 +142,28 @@ __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
       int my_slot = 0;
       float my_w = 0.f;
       if (sidx < nsplit) {
-        my_slot = Plan::slot_of_split(info.x, sidx);
+        my_slot = Plan::slot_of_split(info.y, sidx);
         my_w = expf(prm.part_lse[static_cast<size_t>(my_slot) * prm.item_rows + rr] - mx);
       }
       const int n_here = min(32, nsplit - base);
-#pragma unroll 2
-      for (int j = 0; j < n_here; ++j) {
-        const float w = __shfl_sync(0xffffffffu, my_w, j);
-        const int slot = __shfl_sync(0xffffffffu, my_slot, j);
-        tot += w;
-        const size_t prow = static_cast<size_t>(slot) * prm.item_rows + rr;
-        const uint4* src = reinterpret_cast<const uint4*>(halves + prow * kDv) + 2 * lane;
-        accumulate(w, scales[prow * 16 + (lane >> 1)], src[0], src[1]);
+#pragma unroll 1
+      for (int j = 0; j < n_here; j += kManyBatch) {
+        uint4 va[kManyBatch], vb[kManyBatch];
+        uint32_t sc[kManyBatch];
+#pragma unroll
+        for (int k = 0; k < kManyBatch; ++k) {
+          const size_t prow = static_cast<size_t>(__shfl_sync(0xffffffffu, my_slot, min(j + k, n_here - 1))) * prm.item_rows + rr;
+          sc[k] = scales[prow * 16 + (lane >> 1)];
+          const uint4* src = reinterpret_cast<const uint4*>(halves + prow * kDv) + 2 * lane;
+          va[k] = src[0];
+          vb[k] = src[1];
+        }
+#pragma unroll
+        for (int k = 0; k < kManyBatch; ++k) {
+          const float w = j + k < n_here ? __shfl_sync(0xffffffffu, my_w, j + k) : 0.f;
+          tot += w;
+          accumulate(w, sc[k], va[k], vb[k]);
+        }
       }
     }
   }
@@ -181,10 +178,6 @@ __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
   dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
   dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
   if (lane == 0) *lrow = mx + logf(tot);
-#ifdef AMLA_TRACE
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_ns));
-  if (prm.trace && lane == 0) atomicMax(prm.trace + 148 * 16 * 128 + 3, t_ns & 0xffffffffull);
-#endif
 }
 
 cudaError_t launch_plan(const DecodeParams& prm, int* prefix_out, cudaStream_t stream) {
@@ -194,8 +187,7 @@ cudaError_t launch_plan(const DecodeParams& prm, int* prefix_out, cudaStream_t s
 
 cudaError_t launch_combine(const DecodeParams& prm, cudaStream_t stream) {
   const int warps_per_block = 4;   // small blocks: one fits beside a decode CTA (registers), so part of the grid is resident before the decode kernel ends
-  const long rows = static_cast<long>(prm.B) * prm.nrb * prm.item_rows;
-  const int blocks = static_cast<int>((rows + warps_per_block - 1) / warps_per_block);
+  const int blocks = merge_groups(prm) * (prm.item_rows / warps_per_block);
   // programmatic dependent launch: the blocks may be placed while the decode kernel drains; they wait inside
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);

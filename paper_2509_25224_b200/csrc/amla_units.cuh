@@ -47,7 +47,7 @@ struct UnitIter {
   const int* seqlens;
   int p, g, g1, share, parts;
   __device__ UnitIter(const DecodeParams& prm_, const int* prefix_, const int* seqlens_, int part) : prm(prm_), prefix(prefix_), seqlens(seqlens_), p(part) {
-    const Plan plan = Plan::make(prefix, prm.n_items, prm.P, prm.ovh);
+    const Plan plan = Plan::make(prefix, prm.n_items, prm.P, prm.ovh, prm.min_share);
     share = plan.share; parts = plan.P;
     if (plan.L <= 0 || p >= plan.P) { g = g1 = 0; }
     else { g = plan.part_start(p); g1 = plan.part_start(p + 1); }
@@ -59,7 +59,7 @@ struct UnitIter {
     g = f.g;
     return u.t1 > u.t0;
   }
-  // Partial slot of the unit, -1 if its item lies in one part; *info = what the combine needs to know about the item
+  // Partial slot of the unit, -1 if its item lies in one part; *info = (slot of the item's first partial, partials)
   __device__ int slot_of(const Unit& u, int2* info) const {
     const int begin = prefix[u.it];
     const int p_first = static_cast<int>(static_cast<unsigned>(begin + item_overhead(u.it, prm.ovh)) / static_cast<unsigned>(share));
@@ -69,6 +69,36 @@ struct UnitIter {
     return p_first == p_last ? -1 : p == p_first ? slot_first : 2 * p;
   }
 };
+
+// Items without tiles have no unit: their output is zero and their lse -inf.  `who` of `step` writers takes every step-th
+// item; within an item this writes rows [row0, row0 + nrows) of its block.
+// (The function takes values: a reference would make every caller keep the kernel's parameters in local memory.)
+static __device__ __noinline__ void write_empty_items_of(const int* prefix, int n_items, int nrb, int item_rows, int R, __nv_bfloat16* out, float* lse,
+                                                         int4* merge_info, int who, int step, int row0, int nrows, int tid, int threads) {
+  for (int it = who; it < n_items; it += step) {
+    if (prefix[it + 1] > prefix[it]) continue;
+    const int b = it / nrb, r0 = (it - b * nrb) * item_rows + row0;
+    const int rows = min(nrows, R - r0);
+    if (tid == 0 && row0 == 0 && merge_info != nullptr) merge_info[it] = make_int4(0, 0, 0, 0);
+    const size_t first = static_cast<size_t>(b) * R + r0;
+    uint4* dst = reinterpret_cast<uint4*>(out + first * kDv);
+    for (int i = tid; i < rows * (kDv / 8); i += threads) dst[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < rows; i += threads) lse[first + i] = -INFINITY;
+  }
+}
+__device__ __forceinline__ void write_empty_items(const DecodeParams& prm, const int* prefix, int who, int step, int row0, int nrows, int tid, int threads) {
+  write_empty_items_of(prefix, prm.n_items, prm.nrb, prm.item_rows, prm.R, prm.out, prm.lse, merge_by_item(prm) ? prm.merge_info : nullptr, who, step,
+                       row0, nrows, tid, threads);
+}
+
+// What a part leaves for the combine kernel, by one thread: begin() first, then note() once per unit with what slot_of said.
+__device__ __forceinline__ void merge_begin(const DecodeParams& prm, int part) {
+  if (!merge_by_item(prm)) prm.merge_info[part] = make_int4(0, 0, 0, 0);
+}
+__device__ __forceinline__ void merge_note(const DecodeParams& prm, int part, int it, int2 info) {
+  if ((info.x >> 1) == part && (merge_by_item(prm) || info.y > 1))      // the part in which the item begins speaks for it
+    prm.merge_info[merge_by_item(prm) ? it : part] = make_int4(it, info.x, info.y, 0);
+}
 
 // The score tiles of a unit: its n pages in ceil(n / kMaxPages) tiles of nearly equal size, so that no unit ends with
 // a one-page tile (an MMA of 64 keys takes two thirds of the time of one of 256).
