@@ -44,7 +44,8 @@ namespace {
 
 constexpr int kSoftmaxWarps = 8;
 // bf16 cache: warps 8 and 10 load.  E4M3 cache: warp 8 loads, warps 10-15 widen, three pairs taking turns.
-constexpr int kWideners = 6;
+constexpr int kWidenGroups = 3, kWidenWarps = 2;
+constexpr int kWideners = kWidenGroups * kWidenWarps;
 template <bool kFp8> constexpr int kThreads = 32 * (kFp8 ? kSoftmaxWarps + 2 + kWideners : kSoftmaxWarps + 3);
 constexpr int kTilePages = 4;                           // pages of a score tile: N = 256, the widest MMA
 constexpr int kCtaRows = kRowBlock / 2;                 // query rows per CTA
@@ -55,11 +56,16 @@ constexpr uint32_t kPPageBytes = kCtaRows * 128;        // P~ of one page: [64 r
 constexpr uint32_t kKBoxBytes = 32 * 128;               // this CTA's half of a page x one 64-column block
 constexpr uint32_t kSlotBytes = 128 * 128;              // K: 4 pages x 32 keys x 64 columns; V: 64 keys x 128 columns
 constexpr uint32_t kVBlockBytes = 64 * 128;             // 64 keys x 64 columns
-// The ring of operand slots, and for an E4M3 cache a ring of raw slots in front of it: K of 4 pages x 32 keys x 128 columns,
-// or V of 64 keys x 256 columns, two operand slots each.
+// The ring of operand slots, and for an E4M3 cache a ring of raw slots in front of it, one for every operand slot.
+// A rule that every user of a ring keeps: a thread waits only for slots that it fills or empties itself, and having waited
+// for number w (counted over the whole run; slots are released in order) next for one of w + 1 ... w + R, R being the number
+// of slots.  The barriers tell two successive phases apart, no more: a thread that asks for a phase further on is let
+// through by an older one, and one that comes to ask after the next phase has passed as well is held for good.  (So the
+// two loaders take every second of seven slots, and the three pairs that widen step by three through four operand slots,
+// and by three through six raw slots: raw slots fill out of order, and that makes each the business of one pair.)
 template <bool kFp8> constexpr int kSlots = kFp8 ? 4 : 7;
-constexpr int kRawSlots = 3;
-constexpr uint32_t kRawBytes = 128 * 128, kRawPageBytes = 32 * 128;
+constexpr int kRawSlots = 2 * kWidenGroups;
+constexpr uint32_t kRawBytes = kSlotBytes / 2;
 
 constexpr uint32_t kOffQ = 0;
 constexpr uint32_t kOffP = kOffQ + kQBytes;
@@ -68,7 +74,7 @@ constexpr uint32_t kOffRaw = kOffRing + kSlots<true> * kSlotBytes;
 constexpr uint32_t kOffXchg = kOffRing + 7 * kSlotBytes;           // float [2][4 threads of a row][64 rows]
 static_assert(kOffRaw + kRawSlots * kRawBytes <= kOffXchg && kSlots<false> <= 7, "the rings share one area");
 constexpr uint32_t kOffBars = kOffXchg + 2 * 4 * kCtaRows * 4;
-constexpr uint32_t kBarBytes = 320;
+constexpr uint32_t kBarBytes = 384;
 // a copy of the schedule prefix and of the sequence lengths for batches of up to kSmemPlanItems items, so that the
 // roles' schedule look-ups (a dozen dependent loads per unit) stay on chip
 constexpr int kSmemPlanItems = 512;
@@ -163,11 +169,11 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   }
   if (tid == 32 * 10) {
     for (int i = 0; i < kSlots<kFp8>; ++i) {
-      mbar_init(bar(X_FULL + i), kFp8 ? 4 : 1);          // E4M3: the two warps that fill the slot, in either CTA
+      mbar_init(bar(X_FULL + i), kFp8 ? 2 * kWidenWarps : 1);          // E4M3: the warps that fill the slot, in either CTA
       mbar_init(bar(X_EMPTY + i), 1);
     }
     if (kFp8) {
-      for (int i = 0; i < kRawSlots; ++i) { mbar_init(bar(X_RAWFULL + i), 1); mbar_init(bar(X_RAWEMPTY + i), 4); }
+      for (int i = 0; i < kRawSlots; ++i) { mbar_init(bar(X_RAWFULL + i), 1); mbar_init(bar(X_RAWEMPTY + i), kWidenWarps); }
     }
     mbar_init(bar(X_QFULL), 1);
     mbar_init(bar(X_QFREE), 1);
@@ -272,154 +278,135 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         if (!ok) break;
         tc_fence_after_sync();
         if (tid == 0 && leader) AMLA_STAMP(prm, part, 8, gs);
-        // this group's pages of the tile: t + grp and t + grp + 2 (32 columns each, 32 keys per lane half)
+        // This group's pages of the tile are t + grp and t + grp + 2 (32 columns each, 32 keys per lane half).  The scores are
+        // read from tensor memory twice, a page at a time: for the maximum, and for the exponentials once the P buffer is
+        // free.  (Held in registers in between they cost 64 more of them and twice the code.)
         const uint32_t scol = tbase + lane_base + kSCol + 128 * sb + 32 * grp;
-        const bool has0 = grp < np, has1 = grp + 2 < np;
-        const int nvis0 = has0 ? visible - (t + grp) * kPage - 32 * khalf : 0;
-        const int nvis1 = has1 ? visible - (t + grp + 2) * kPage - 32 * khalf : 0;
-        uint32_t b0[32], b1[32];
-        tmem_ld_32x32b_x32(scol, b0);
-        tmem_ld_32x32b_x32(scol + 64, b1);
-        tmem_wait_ld();
-        tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) { if (leader) mbar_arrive(bar(X_SEMPTY + sb)); else mbar_arrive_cluster_relaxed(lead_bars + 8u * (X_SEMPTY + sb)); }
-
-        // Two compilations of the tile: the plain one (both pages there, every key visible, non-negative scale) and the
-        // general one with the visibility masks and the sign of the scale.
-        auto tile_body = [&](auto general_c) {
-          constexpr bool kGeneral = decltype(general_c)::value;
-          // lines 5-6: running max; the plain tile takes it on the raw scores (the scale is folded into the FMA below),
-          // the general one on the scaled ones
-          float ext = -INFINITY, ext_b = ext;
-          auto chunk_max = [&](uint32_t (&v)[32], int nvis) {
-            if (kGeneral) {
-#pragma unroll
-              for (int i = 0; i < 32; ++i) v[i] = (i < nvis) ? __float_as_uint(__uint_as_float(v[i]) * prm.scale_log2) : 0xff800000u;
-            }
+        const int nvis0 = visible - (t + grp) * kPage - 32 * khalf;        // keys of the first page that the row sees (may be <= 0)
+        const bool plain = t + np <= first_masked && scale_nonneg;          // every key of the tile is visible
+        // lines 5-6: running max (the scale is folded into the FMA below)
+        float ext = -INFINITY;
+#pragma unroll 1
+        for (int h = 0; grp + 2 * h < np && h < 2; ++h) {
+          uint32_t v[32];
+          tmem_ld_32x32b_x32(scol + 64 * h, v);
+          tmem_wait_ld();
+          float a = -INFINITY, b = a;
+          if (plain) {
 #pragma unroll
             for (int i = 0; i < 32; i += 4) {
-              ext = fmax3(ext, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
-              ext_b = fmax3(ext_b, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
+              a = fmax3(a, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+              b = fmax3(b, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
             }
-          };
-          chunk_max(b0, nvis0);
-          chunk_max(b1, nvis1);
-          const float mine = kGeneral ? fmaxf(ext, ext_b) : fmaxf(ext, ext_b) * prm.scale_log2;
-          float m4[4];
-          exchange(mine, m4);
-          if (!ok) return;
-          if (tid == 0 && leader) AMLA_STAMP(prm, part, 9, gs);
-          const float tmax = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-          // Lazy reference: a row must move when its maximum exceeds the reference by more than tau.  The four warps of
-          // these 32 rows pay for a rescale as soon as one row moves, so when one must, every row of the warp whose
-          // maximum rose moves with it (moving early is always allowed: tau = 0 moves at every rise); the rows then tend
-          // to stay in step and O is rescaled on far fewer tiles.  The four warps see the same maxima and agree.
-          const bool must = tmax > st.m2 + prm.tau;
-          const RowStep sp = row_step<kMode>(st, tmax, __any_sync(0xffffffffu, must) ? 0.f : prm.tau);
-          // Line 10's factor S16 goes into the exponential's argument (the remark after Algorithm 2).  The row sum of
-          // line 6 is the sum of the same FP32 values, taken before the bf16 cast and divided by S16 once per tile.
-          const float nsub = log2f_approx(sp.p_scale) - sp.m2_sub;
-          float rs0 = 0.f, rs1 = 0.f;
-          const uint64_t sc2 = pack_f32x2(prm.scale_log2, prm.scale_log2), ns2 = pack_f32x2(nsub, nsub);
-          uint64_t rsa = pack_f32x2(0.f, 0.f), rsb = rsa;
-          uint32_t pk[32];
-          auto chunk_exp = [&](const uint32_t (&v)[32], int k0) {
-            if (kGeneral) {
+            a = fmaxf(a, b) * prm.scale_log2;
+          } else {
+            const int nvis = nvis0 - 2 * kPage * h;
 #pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                const float p0 = ex2_approx(__uint_as_float(v[2 * i]) + nsub);          // a hidden key: 2^-inf = 0
-                const float p1 = ex2_approx(__uint_as_float(v[2 * i + 1]) + nsub);
-                rs0 += p0; rs1 += p1;
-                pk[k0 + i] = pack_bf16x2(p0, p1);
-              }
-            } else {
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                float x0, x1;
-                unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), sc2, ns2), x0, x1);
-                const float q0 = ex2_approx(x0), q1 = ex2_approx(x1);
-                const uint64_t pp = pack_f32x2(q0, q1);
-                if (i & 1) rsb = add_f32x2(rsb, pp); else rsa = add_f32x2(rsa, pp);
-                pk[k0 + i] = pack_bf16x2(q0, q1);
-              }
-            }
-          };
-          chunk_exp(b0, 0);
-          chunk_exp(b1, 16);
-          {
-            float s0, s1;
-            unpack_f32x2(add_f32x2(rsa, rsb), s0, s1);
-            st.l = st.l * sp.l_up + __fdividef((rs0 + s0) + (rs1 + s1), sp.p_scale);   // this thread's share of the row sum
+            for (int i = 0; i < 32; ++i) a = fmaxf(a, i < nvis ? __uint_as_float(v[i]) * prm.scale_log2 : -INFINITY);
           }
-          if (tid == 0 && leader) AMLA_STAMP(prm, part, 10, gs);
-          if (!tile.first) {
-            // the P~V of the tile before: it has read the P buffer, and O holds its sum
-            ok = warp_wait(bar(X_PVDONE), (gs - 1) & 1);
-            if (!ok) return;
-            const uint32_t nword = (kMode == 2) ? __float_as_uint(sp.l_up) : static_cast<uint32_t>(sp.n_bits);
-            const bool mine_moved = (kMode == 2) ? (sp.l_up != 1.f) : (sp.n_bits != 0);
-            if (__any_sync(0xffffffffu, mine_moved)) {
-              // lines 13-16: O <- AS_FP32(AS_INT32(O) + N).  The guarded add costs four integer operations per element,
-              // the FP32 multiply it replaces one.  The guard only matters for an element whose magnitude bits plus N
-              // would not stay positive (an exact zero, a value about to leave the normal range); so the smallest
-              // magnitude of the chunk is taken first (half an operation per element), and where it is safe the chunk
-              // gets the plain one-instruction add of Lemma 3.1.
-              tc_fence_after_sync();
-              auto apply = [&](uint32_t (&o)[32]) {
-                if (kMode == 2) {
+          ext = fmaxf(ext, a);
+        }
+        float m4[4];
+        exchange(ext, m4);
+        if (!ok) break;
+        if (tid == 0 && leader) AMLA_STAMP(prm, part, 9, gs);
+        const float tmax = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+        // Lazy reference: a row must move when its maximum exceeds the reference by more than tau.  The four warps of these
+        // 32 rows pay for a rescale as soon as one row moves, so when one must, every row of the warp whose maximum rose
+        // moves with it (moving early is always allowed: tau = 0 moves at every rise); the rows then tend to stay in step and
+        // O is rescaled on far fewer tiles.  The four warps see the same maxima and agree.
+        const bool must = tmax > st.m2 + prm.tau;
+        const RowStep sp = row_step<kMode>(st, tmax, __any_sync(0xffffffffu, must) ? 0.f : prm.tau);
+        if (!tile.first) {
+          // the P~V of the tile before: it has read the P buffer, and O holds its sum
+          ok = warp_wait(bar(X_PVDONE), (gs - 1) & 1);
+          if (!ok) break;
+          const uint32_t nword = (kMode == 2) ? __float_as_uint(sp.l_up) : static_cast<uint32_t>(sp.n_bits);
+          const bool mine_moved = (kMode == 2) ? (sp.l_up != 1.f) : (sp.n_bits != 0);
+          if (__any_sync(0xffffffffu, mine_moved)) {
+            // lines 13-16: O <- AS_FP32(AS_INT32(O) + N).  The guarded add costs four integer operations per element, the
+            // FP32 multiply it replaces one.  The guard only matters for an element whose magnitude bits plus N would not
+            // stay positive (an exact zero, a value about to leave the normal range); so the smallest magnitude of the chunk
+            // is taken first (half an operation per element), and where it is safe the chunk gets the plain one-instruction
+            // add of Lemma 3.1.
+            tc_fence_after_sync();
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {
+              uint32_t o[32];
+              tmem_ld_32x32b_x32(o_addr + 32 * c, o);
+              tmem_wait_ld();
+              if (kMode == 2) {
 #pragma unroll
-                  for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * __uint_as_float(nword));
-                } else if (!kGuard) {
-#pragma unroll
-                  for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_raw(__uint_as_float(o[i]), static_cast<int>(nword)));
-                } else {
+                for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * __uint_as_float(nword));
+              } else {
+                bool safe = true;
+                if (kGuard) {
                   float lo = fmin3_abs(__uint_as_float(o[0]), __uint_as_float(o[1]), __uint_as_float(o[2]));
 #pragma unroll
                   for (int i = 3; i + 1 < 32; i += 2) lo = fmin3_abs(lo, __uint_as_float(o[i]), __uint_as_float(o[i + 1]));
                   lo = fminf(lo, fabsf(__uint_as_float(o[31])));
                   // NaN magnitudes compare as large numbers and take the plain add, like every other normal pattern
-                  if (__float_as_int(lo) + static_cast<int>(nword) > 0) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_raw(__uint_as_float(o[i]), static_cast<int>(nword)));
-                  } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_guarded(__uint_as_float(o[i]), static_cast<int>(nword)));
-                  }
+                  safe = __float_as_int(lo) + static_cast<int>(nword) > 0;
                 }
-              };
-#pragma unroll 1
-              for (int c = 0; c < 4; ++c) {
-                uint32_t o[32];
-                tmem_ld_32x32b_x32(o_addr + 32 * c, o);
-                tmem_wait_ld();
-                apply(o);
-                tmem_st_32x32b_x32(o_addr + 32 * c, o);
+                if (safe) {
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_raw(__uint_as_float(o[i]), static_cast<int>(nword)));
+                } else {
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_guarded(__uint_as_float(o[i]), static_cast<int>(nword)));
+                }
               }
-              tmem_wait_st();
-              tc_fence_before_sync();
+              tmem_st_32x32b_x32(o_addr + 32 * c, o);
             }
+            tmem_wait_st();
           }
-          if (tid == 0 && leader) AMLA_STAMP(prm, part, 11, gs);
-          if (has0) {
-            const uint32_t dst = prow_smem + grp * kPPageBytes;
+        }
+        if (tid == 0 && leader) AMLA_STAMP(prm, part, 11, gs);
+        // Line 10's factor S16 goes into the exponential's argument (the remark after Algorithm 2).  The row sum of line 6 is
+        // the sum of the same FP32 values, taken before the bf16 cast and divided by S16 once per tile.
+        const float nsub = log2f_approx(sp.p_scale) - sp.m2_sub;
+        const float sc = plain ? prm.scale_log2 : 1.f;
+        const uint64_t sc2 = pack_f32x2(sc, sc), ns2 = pack_f32x2(nsub, nsub);
+        uint64_t rsa = pack_f32x2(0.f, 0.f), rsb = rsa;
+#pragma unroll 1
+        for (int h = 0; grp + 2 * h < np && h < 2; ++h) {
+          uint32_t v[32];
+          tmem_ld_32x32b_x32(scol + 64 * h, v);
+          tmem_wait_ld();
+          if (!plain) {
+            const int nvis = nvis0 - 2 * kPage * h;        // scaled here; hidden keys become 2^-inf = 0
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-              st_shared_v4(dst + (((4 * khalf + c) ^ (r & 7)) << 4), pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+            for (int i = 0; i < 32; ++i) v[i] = i < nvis ? __float_as_uint(__uint_as_float(v[i]) * prm.scale_log2) : 0xff800000u;
           }
-          if (has1) {
-            const uint32_t dst = prow_smem + (grp + 2) * kPPageBytes;
+          const uint32_t dst = prow_smem + (grp + 2 * h) * kPPageBytes;
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-              st_shared_v4(dst + (((4 * khalf + c) ^ (r & 7)) << 4), pk[16 + 4 * c], pk[16 + 4 * c + 1], pk[16 + 4 * c + 2], pk[16 + 4 * c + 3]);
+          for (int c = 0; c < 4; ++c) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              float x0, x1;
+              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[8 * c + 2 * i]), __uint_as_float(v[8 * c + 2 * i + 1])), sc2, ns2), x0, x1);
+              const float q0 = ex2_approx(x0), q1 = ex2_approx(x1);
+              const uint64_t pp = pack_f32x2(q0, q1);
+              if (i & 1) rsb = add_f32x2(rsb, pp); else rsa = add_f32x2(rsa, pp);
+              pk[i] = pack_bf16x2(q0, q1);
+            }
+            st_shared_v4(dst + (((4 * khalf + c) ^ (r & 7)) << 4), pk[0], pk[1], pk[2], pk[3]);
           }
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) { if (leader) mbar_arrive(bar(X_PREADY)); else mbar_arrive_cluster_relaxed(lead_bars + 8u * X_PREADY); }
-          if (tid == 0 && leader) AMLA_STAMP(prm, part, 12, gs);
-        };
-        if (!has1 || t + np > first_masked || !scale_nonneg) tile_body(std::true_type{});
-        else tile_body(std::false_type{});
+        }
+        tc_fence_before_sync();            // S has been read, O (perhaps) rewritten
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          if (leader) { mbar_arrive(bar(X_SEMPTY + sb)); mbar_arrive(bar(X_PREADY)); }
+          else { mbar_arrive_cluster_relaxed(lead_bars + 8u * (X_SEMPTY + sb)); mbar_arrive_cluster_relaxed(lead_bars + 8u * X_PREADY); }
+        }
+        if (tid == 0 && leader) AMLA_STAMP(prm, part, 12, gs);
+        {
+          float s0, s1;
+          unpack_f32x2(add_f32x2(rsa, rsb), s0, s1);
+          st.l = st.l * sp.l_up + __fdividef(s0 + s1, sp.p_scale);   // this thread's share of the row sum
+        }
         if (!ok) break;
         ++gs;
         more = !tile.last();
@@ -479,13 +466,14 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     // Q, K(0), K(1), V(0), K(2), V(1), ..., K(n-1), V(n-2), V(n-1), next unit.
     //   bf16: one ring of 16 KB slots carries K (one 64-column block of the tile's keys, one box per page) and V (one page
     //     x 128 columns).  The two loader warps walk the same sequence and issue every second load of it.
-    //   E4M3: raw slots; K in five of 128 columns (the last one half outside the row: zeros), V in one per page.
+    //   E4M3: the same as raw slots of half the size, all by the first loader.
     // A unit's Q is requested (by the first loader) as soon as the QK^T of the unit before have let go of the buffer, if
     // need be between the V loads of that unit's last tile.
     if (elect_one()) {
       const uint32_t mine = wid == 8 ? 0u : 1u;
       constexpr uint32_t kRing = kFp8 ? kRawSlots : kSlots<kFp8>;
       const uint32_t full0 = kFp8 ? bar(X_RAWFULL) : bar(X_FULL), empty0 = kFp8 ? bar(X_RAWEMPTY) : bar(X_EMPTY);
+      constexpr uint32_t kBytes = kFp8 ? kRawBytes : kSlotBytes;
       const uint32_t lead_full0 = lead_bars + 8u * X_FULL, ring0 = smem_base + (kFp8 ? kOffRaw : kOffRing);
       const uint64_t keep = l2_policy_evict_normal(), last_use = l2_policy_evict_first();   // K: V follows a tile later; V: done with
       uint32_t slot = 0, par = 1, n_issued = 0;
@@ -517,19 +505,18 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       auto issue_v = [&](const TileRef& x, int nxt_qrow, bool q_wanted, bool& q_out) {
         int page = __ldg(x.bt);
 #pragma unroll 1
-        for (int i = 0; i < (kFp8 ? x.np : 2 * x.np); ++i) {
+        for (int i = 0; i < 2 * x.np; ++i) {
           const int row = row_of(page);
-          const int nh = kFp8 ? 0 : i & 1, p_next = min(kFp8 ? i + 1 : (i + 1) >> 1, x.np - 1);
+          const int nh = i & 1, p_next = min((i + 1) >> 1, x.np - 1);
           page = __ldg(x.bt + p_next);
           if (my_turn()) {
             if (q_wanted && !q_out && mbar_probe(bar(X_QFREE), (un - 1) & 1)) { issue_q(nxt_qrow); q_out = true; }
-            const uint32_t dst = ring0 + slot * kSlotBytes;
+            const uint32_t dst = ring0 + slot * kBytes;
             ok = mbar_wait(empty0 + 8 * slot, par);
             if (!ok) return;
             if (kFp8) {
               mbar_arrive_expect_tx(full0 + 8 * slot, kRawBytes);
-              tma_load_2d_hint(dst, &v_map, 256 * rank, row, full0 + 8 * slot, last_use);            // [2][64 keys][128 columns]
-              tma_load_2d_hint(dst + kRawBytes / 2, &v_map, 256 * rank + 128, row, full0 + 8 * slot, last_use);
+              tma_load_2d_hint(dst, &v_map, 256 * rank + 128 * nh, row, full0 + 8 * slot, last_use);            // [64 keys][128 columns]
             } else {
               if (leader) mbar_arrive_expect_tx(full0 + 8 * slot, 2 * kSlotBytes);
               tma_load_3d_pair_hint(dst, &v_map, 0, row, 4 * rank + 2 * nh, lead_full0 + 8 * slot, last_use);
@@ -562,17 +549,17 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         for (int p = 0; p < kTilePages; ++p) row[p] = row_of(page[p]);
         get_pages(nxt);
 #pragma unroll 1
-        for (int c = 0; c < (kFp8 ? (kQBlocks + 1) / 2 : kQBlocks); ++c) {
+        for (int c = 0; c < kQBlocks; ++c) {
           if (my_turn()) {
-            const uint32_t dst = ring0 + slot * kSlotBytes;
+            const uint32_t dst = ring0 + slot * kBytes;
             ok = mbar_wait(empty0 + 8 * slot, par);
             if (!ok) break;
             if (leader && (c <= 1 || c >= 7)) AMLA_STAMP(prm, part, c <= 1 ? 16 : 17, pt);
             if (kFp8) {
-              mbar_arrive_expect_tx(full0 + 8 * slot, cur.np * kRawPageBytes);
+              mbar_arrive_expect_tx(full0 + 8 * slot, cur.np * (kKBoxBytes / 2));
 #pragma unroll
               for (int p = 0; p < kTilePages; ++p)
-                if (p < cur.np) tma_load_2d_hint(dst + p * kRawPageBytes, &k_map, 128 * c, row[p] + 32 * rank, full0 + 8 * slot, keep);   // [32 keys][128 columns]
+                if (p < cur.np) tma_load_2d_hint(dst + p * (kKBoxBytes / 2), &k_map, 64 * c, row[p] + 32 * rank, full0 + 8 * slot, keep);   // [32 keys][64 columns]
             } else {
               if (leader) mbar_arrive_expect_tx(full0 + 8 * slot, 2 * cur.np * kKBoxBytes);
 #pragma unroll
@@ -607,70 +594,63 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     // ======================================================== E4M3 cache: raw slot -> operand slots.  The three pairs of
     // warps take every third operand slot each; a thread widens 16 bytes at a time (exact: E4M3 values are bf16 values)
     // and stores them where the 128-byte swizzle of the operand tiles puts them.
-    const uint32_t mine = (wid - 10) >> 1;
-    const int wt = ((wid - 10) & 1) * 32 + lane;
-    uint32_t turn = 0, slot = 0, par = 1, rslot = 0, rpar = 0;
-    // One operand slot: `half` of raw slot rslot; `is_k`: K, else V; `last`: nothing else of the raw slot.  A thread holds
-    // its eight 16-byte pieces in registers, widened, before it waits for the operand slot: the raw slot goes back to the
-    // loader at once, and the operand slot is refilled within the time of sixteen stores.
-    auto fill = [&](bool is_k, uint32_t half, bool last) {
-      if (turn == mine) {
-        ok = warp_wait(bar(X_RAWFULL + rslot), rpar);
-        if (!ok) return;
-        // K: row = page * 32 + key, four threads a row; 64 of its 128 raw bytes are this slot's 64 columns (rows of pages
-        // that the tile does not have hold older bytes; the MMA does not read them).  V: 64 keys x 128 columns -> two
-        // blocks of 64 columns, eight threads a row.
-        const uint32_t raw = smem_base + kOffRaw + rslot * kRawBytes, out = smem_base + kOffRing + slot * kSlotBytes;
-        const int r0 = is_k ? wt >> 2 : wt >> 3, rstep = is_k ? 16 : 8;
-        const uint32_t src = raw + (is_k ? 64 * half + 16 * (wt & 3) : half * (kRawBytes / 2) + 16 * (wt & 7)) + r0 * 128;
-        const uint32_t dst = out + (is_k ? 0 : ((wt & 7) >> 2) * kVBlockBytes) + r0 * 128;
-        uint32_t x[8][4], w[8][8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x[k][0]), "=r"(x[k][1]), "=r"(x[k][2]), "=r"(x[k][3]) : "r"(src + k * rstep * 128));
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) { w[k][2 * q] = e4m3x2_to_bf16x2(x[k][q]); w[k][2 * q + 1] = e4m3x2_to_bf16x2(x[k][q] >> 16); }
-        }
-        __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(bar(X_RAWEMPTY + rslot));
-          if (last && half == 0) mbar_arrive(bar(X_RAWEMPTY + rslot));       // the other half has no reader
-        }
-        ok = warp_wait(bar(X_EMPTY + slot), par);
-        if (!ok) return;
-        const uint32_t ch = 2 * (wt & 3), sw = r0 & 7;      // rows of a thread differ by multiples of 8: the same swizzle
-        const uint32_t d0 = dst + ((ch ^ sw) << 4), d1 = dst + (((ch + 1) ^ sw) << 4);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          st_shared_v4(d0 + k * rstep * 128, w[k][0], w[k][1], w[k][2], w[k][3]);
-          st_shared_v4(d1 + k * rstep * 128, w[k][4], w[k][5], w[k][6], w[k][7]);
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) { if (leader) mbar_arrive(bar(X_FULL + slot)); else mbar_arrive_cluster_relaxed(lead_bars + 8u * (X_FULL + slot)); }
-      }
-      if (++turn == kWideners / 2) turn = 0;
-      if (++slot == kSlots<kFp8>) { slot = 0; par ^= 1; }
-      if (last && ++rslot == kRawSlots) { rslot = 0; rpar ^= 1; }
-    };
+    const uint32_t mine = (wid - 10) / kWidenWarps;
+    const int wt = ((wid - 10) % kWidenWarps) * 32 + lane;
+    // `n` is the number of the slot, `pos` its place in the present phase (K of a tile: nine slots; V of one: two per page).
+    uint32_t n = mine, pos = mine, len = kQBlocks;
     int np_prev = 0;
+    int what = 0;                                        // 0: K of the tile, 1: V of the tile before, 2: V of the tile (unit's last)
     while (ok && tile.valid) {
-      const int np = tile.np;
-      const bool first = tile.first, last = tile.last();
-#pragma unroll 1
-      for (int c = 0; c < kQBlocks && ok; ++c) fill(true, c & 1, (c & 1) != 0 || c == kQBlocks - 1);
-      if (!first) {
-#pragma unroll 1
-        for (int i = 0; i < 2 * np_prev && ok; ++i) fill(false, i & 1, (i & 1) != 0);
+      while (pos >= len) {                               // next phase
+        pos -= len;
+        if (what == 0 && !tile.first) { what = 1; len = 2 * np_prev; }
+        else if (what != 2 && tile.last()) { what = 2; len = 2 * tile.np; }
+        else {
+          np_prev = tile.np;
+          tile.next();
+          what = 0; len = kQBlocks;
+          if (!tile.valid) break;
+        }
       }
-      if (last) {
-#pragma unroll 1
-        for (int i = 0; i < 2 * np && ok; ++i) fill(false, i & 1, (i & 1) != 0);
+      if (!tile.valid) break;
+      const bool is_k = what == 0;
+      const uint32_t rslot = n % kRawSlots, rpar = (n / kRawSlots) & 1;
+      const uint32_t slot = n % kSlots<kFp8>, par = ((n / kSlots<kFp8>) & 1) ^ 1;
+      ok = warp_wait(bar(X_RAWFULL + rslot), rpar);
+      if (ok) ok = warp_wait(bar(X_EMPTY + slot), par);
+      if (!ok) break;
+      // K: row = page * 32 + key, 64 bytes, four threads a row (rows of pages that the tile does not have hold older bytes; the
+      // MMA does not read them).  V: 64 keys x 128 columns -> two blocks of 64 columns, eight threads a row.
+      const uint32_t raw = smem_base + kOffRaw + rslot * kRawBytes, out = smem_base + kOffRing + slot * kSlotBytes;
+      const int r0 = is_k ? wt >> 2 : wt >> 3;
+      const uint32_t step = is_k ? 16 * 128 : 8 * 128;    // rows of a thread differ by multiples of 8: the same swizzle
+      const uint32_t src = raw + 16 * wt;                 // the pieces of a slot in order, 64 threads wide
+      const uint32_t ch = 2 * (wt & 3), sw = r0 & 7;
+      const uint32_t d0 = out + (is_k ? 0 : ((wt & 7) >> 2) * kVBlockBytes) + r0 * 128 + ((ch ^ sw) << 4);
+      const uint32_t d1 = (((ch + 1) ^ sw) << 4) - ((ch ^ sw) << 4);
+#pragma unroll
+      for (uint32_t h = 0; h < 8; h += 4) {               // eight pieces of 16 bytes, four requested at a time
+        uint32_t x[4][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x[k][0]), "=r"(x[k][1]), "=r"(x[k][2]), "=r"(x[k][3]) : "r"(src + (h + k) * 1024));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          uint32_t w[8];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) { w[2 * q] = e4m3x2_to_bf16x2(x[k][q]); w[2 * q + 1] = e4m3x2_to_bf16x2(x[k][q] >> 16); }
+          st_shared_v4(d0 + (h + k) * step, w[0], w[1], w[2], w[3]);
+          st_shared_v4(d0 + d1 + (h + k) * step, w[4], w[5], w[6], w[7]);
+        }
       }
-      np_prev = np;
-      if (ok) tile.next();
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        if (leader) mbar_arrive(bar(X_FULL + slot)); else mbar_arrive_cluster_relaxed(lead_bars + 8u * (X_FULL + slot));
+        mbar_arrive(bar(X_RAWEMPTY + rslot));
+      }
+      pos += kWidenGroups;
+      n += kWidenGroups;
     }
     if (!ok && lane == 0) report_timeout(prm.status);
   } else if (leader && wid == 9) {
@@ -842,11 +822,11 @@ cudaError_t launch_mode(const CUtensorMap& kmap, const CUtensorMap& vmap, const 
   return launch_variant<2, true, kFp8>(kmap, vmap, qmap, prm, stream);
 }
 
-// An E4M3 cache: rows of 576 bytes, boxes of 128 columns.
-bool encode_bytes(EncodeTiledFn encode, CUtensorMap* map, const void* base, cuuint64_t rows, cuuint32_t box_rows) {
+// An E4M3 cache: rows of 576 bytes.
+bool encode_bytes(EncodeTiledFn encode, CUtensorMap* map, const void* base, cuuint64_t rows, cuuint32_t box_rows, cuuint32_t box_cols) {
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(kDqk), rows};
   const cuuint64_t strides[1] = {static_cast<cuuint64_t>(kDqk)};
-  const cuuint32_t box[2] = {128, box_rows};
+  const cuuint32_t box[2] = {box_cols, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -867,7 +847,7 @@ cudaError_t launch_decode_pair(const DecodeParams& prm, cudaStream_t stream, int
   const cuuint64_t keys = static_cast<cuuint64_t>(prm.num_blocks) * kPage;
   if (!encode_rows(encode, &qmap, prm.q, static_cast<cuuint64_t>(prm.B) * prm.R, kCtaRows, 3)) return cudaErrorInvalidValue;
   if (prm.kv8 != nullptr) {
-    if (!encode_bytes(encode, &kmap, prm.kv8, keys, 32) || !encode_bytes(encode, &vmap, prm.kv8, keys, 64)) return cudaErrorInvalidValue;
+    if (!encode_bytes(encode, &kmap, prm.kv8, keys, 32, 64) || !encode_bytes(encode, &vmap, prm.kv8, keys, 64, 128)) return cudaErrorInvalidValue;
     return launch_mode<true>(kmap, vmap, qmap, prm, stream);
   }
   if (!encode_rows(encode, &kmap, prm.kv, keys, 32, 1) || !encode_rows(encode, &vmap, prm.kv, keys, 64, 2)) return cudaErrorInvalidValue;
