@@ -41,6 +41,7 @@ EXPORTS = [
 ]
 
 _lib = None
+_PAGE_SHAPE = (64, 576)
 
 
 class AmlaError(RuntimeError):
@@ -139,16 +140,12 @@ def mla_decode_static(q, kv_cache, block_table, seqlens, softmax_scale: float, o
     """amla_mla_decode_static on device tensors: the decode call that takes no workspace and allocates nothing
     (its scratch is a fixed array inside the library).  `out` and `lse` must be given -- this wrapper allocates
     nothing either.  Raises AmlaError(-6) when the problem exceeds the built-in scratch."""
-    import torch
-
     B, Sq, H, _ = q.shape
-    stream = torch.cuda.current_stream(q.device).cuda_stream
-    with torch.cuda.device(q.device):
-        rc = lib().amla_mla_decode_static(q.data_ptr(), kv_cache.data_ptr(), block_table.data_ptr(), seqlens.data_ptr(),
-                                          float(softmax_scale), B, Sq, H, kv_cache.shape[0], block_table.shape[1],
-                                          out.data_ptr(), lse.data_ptr(), stream)
-    if rc != AMLA_OK:
-        raise AmlaError(rc, "amla_mla_decode_static")
+    if _lib is None:
+        lib()
+    _on_device(q.device, _lib.amla_mla_decode_static,
+               (q.data_ptr(), kv_cache.data_ptr(), block_table.data_ptr(), seqlens.data_ptr(), float(softmax_scale), B, Sq, H, kv_cache.shape[0],
+                block_table.shape[1], out.data_ptr(), lse.data_ptr()), (), "amla_mla_decode_static")
 
 
 def fp8_workspace_size(B: int, Sq: int, H: int, max_blocks_per_seq: int, device: int = 0) -> int:
@@ -181,14 +178,12 @@ def mla_decode_fp8(q, kv_cache_e4m3, kv_scale: float, block_table, seqlens, soft
         lse = torch.empty((B, Sq, H), dtype=torch.float32, device=dev)
     if workspace is None:
         workspace = torch.empty(fp8_workspace_size(B, Sq, H, block_table.shape[1], dev.index or 0), dtype=torch.uint8, device=dev)
-    stream = torch.cuda.current_stream(dev).cuda_stream
-    with torch.cuda.device(dev):
-        rc = lib().amla_mla_decode_fp8(q.data_ptr(), kv_cache_e4m3.data_ptr(), float(kv_scale), block_table.data_ptr(),
-                                       seqlens.data_ptr(), float(softmax_scale), B, Sq, H, kv_cache_e4m3.shape[0],
-                                       block_table.shape[1], out.data_ptr(), lse.data_ptr(), workspace.data_ptr(),
-                                       workspace.numel(), stream, DEFAULT_FLAGS if flags is None else int(flags))
-    if rc != AMLA_OK:
-        raise AmlaError(rc, "amla_mla_decode_fp8")
+    if _lib is None:
+        lib()
+    _on_device(dev, _lib.amla_mla_decode_fp8,
+               (q.data_ptr(), kv_cache_e4m3.data_ptr(), float(kv_scale), block_table.data_ptr(), seqlens.data_ptr(), float(softmax_scale), B, Sq, H,
+                kv_cache_e4m3.shape[0], block_table.shape[1], out.data_ptr(), lse.data_ptr(), workspace.data_ptr(), workspace.numel()),
+               (DEFAULT_FLAGS if flags is None else int(flags),), "amla_mla_decode_fp8")
     return out, lse
 
 
@@ -220,6 +215,31 @@ def validate_paging_host(block_table, seqlens, num_blocks: int):
     if rc != -1:
         raise AmlaError(rc, "amla_validate_paging_host")
     return int(bs.value), int(bb.value)
+
+
+_raw_stream = None      # torch's accessors of the current device and stream, looked up once
+_current_device = None
+
+
+def _on_device(dev, call, args, tail, what):
+    """call(*args, stream, *tail) with `dev` current, on its current stream.  (The context manager and the stream object
+    of torch.cuda cost 3 us of a call that takes 8 in all; they are only needed when another device is current.)"""
+    global _raw_stream, _current_device
+    if _raw_stream is None:
+        import torch
+        _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
+    index = dev.index
+    now = _current_device()
+    if index is None:
+        index = now
+    if index == now:
+        rc = call(*args, _raw_stream(index), *tail)
+    else:
+        import torch
+        with torch.cuda.device(dev):
+            rc = call(*args, _raw_stream(index), *tail)
+    if rc != AMLA_OK:
+        raise AmlaError(rc, what)
 
 
 def last_launch_count() -> int:
@@ -258,15 +278,17 @@ def mla_decode(q, kv_cache, block_table, seqlens, softmax_scale: float, out=None
 
     if not (q.is_cuda and kv_cache.is_cuda and block_table.is_cuda and seqlens.is_cuda):
         raise ValueError("mla_decode needs CUDA tensors")
-    if q.dtype != torch.bfloat16 or kv_cache.dtype != torch.bfloat16:
+    if q.dtype is not torch.bfloat16 or kv_cache.dtype is not torch.bfloat16:
         raise ValueError("q and kv_cache must be bfloat16")
-    if block_table.dtype != torch.int32 or seqlens.dtype != torch.int32:
+    if block_table.dtype is not torch.int32 or seqlens.dtype is not torch.int32:
         raise ValueError("block_table and seqlens must be int32")
     if not (q.is_contiguous() and kv_cache.is_contiguous() and block_table.is_contiguous() and seqlens.is_contiguous()):
         raise ValueError("inputs must be contiguous")
     B, Sq, H, d = q.shape
-    if d != 576 or tuple(kv_cache.shape[1:]) != (64, 576) or block_table.shape[0] != B or seqlens.shape[0] != B:
+    if d != 576 or kv_cache.shape[1:] != _PAGE_SHAPE or block_table.shape[0] != B or seqlens.shape[0] != B:
         raise ValueError("shape mismatch")
+    if _lib is None:
+        lib()
     dev = q.device
     if out is None:
         out = torch.empty((B, Sq, H, 512), dtype=torch.bfloat16, device=dev)
@@ -275,11 +297,12 @@ def mla_decode(q, kv_cache, block_table, seqlens, softmax_scale: float, out=None
     if workspace is None:
         workspace = torch.empty(workspace_size(B, Sq, H, block_table.shape[1], dev.index or 0),
                                 dtype=torch.uint8, device=dev)
-    stream = torch.cuda.current_stream(dev).cuda_stream
-    with torch.cuda.device(dev):
-        mla_decode_raw(q.data_ptr(), kv_cache.data_ptr(), block_table.data_ptr(), seqlens.data_ptr(),
-                       softmax_scale, B, Sq, H, kv_cache.shape[0], block_table.shape[1], out.data_ptr(),
-                       lse.data_ptr(), workspace.data_ptr(), workspace.numel(), stream, flags)
+    args = (q.data_ptr(), kv_cache.data_ptr(), block_table.data_ptr(), seqlens.data_ptr(), float(softmax_scale), B, Sq, H, kv_cache.shape[0],
+            block_table.shape[1], out.data_ptr(), lse.data_ptr(), workspace.data_ptr(), workspace.numel())
+    if flags is None:
+        _on_device(dev, _lib.amla_mla_decode, args, (), "amla_mla_decode")
+    else:
+        _on_device(dev, _lib.amla_mla_decode_ex, args, (int(flags),), "amla_mla_decode")
     return out, lse
 
 

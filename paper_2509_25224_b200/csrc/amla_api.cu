@@ -1,5 +1,6 @@
 // C-ABI entry points of libamla: argument validation, workspace carving and the three launches
 // (schedule prefix, decode, combine) on the caller's stream.
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <new>
@@ -109,6 +110,14 @@ int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
   prm.nrb = (prm.R + prm.item_rows - 1) / prm.item_rows;
   prm.n_items = prm.B * prm.nrb;
   prm.P = simt ? sms : quad ? quad_parts : decode_pair_parts(sms);
+  // No more parts than the longest schedule that the block table's width allows can fill.  A schedule of one score tile at
+  // most is one part: nothing is split and no combine kernel runs.
+  if (!simt) {
+    const long long tiles = (static_cast<long long>(prm.max_blocks_per_seq) * kPage + prm.tile_keys - 1) / prm.tile_keys;
+    const long long longest = prm.n_items * tiles + (prm.n_items - 1ll) * prm.ovh;
+    if (longest * prm.tile_keys <= 256) prm.P = 1;
+    else prm.P = static_cast<int>(std::min<long long>(prm.P, (longest + prm.min_share - 1) / prm.min_share));
+  }
   prm.fused_plan = (!simt && prm.n_items <= kFusedPlanMaxItems) ? 1 : 0;
   return AMLA_OK;
 }
@@ -135,8 +144,10 @@ int launch_decode_call(const DecodeParams& prm, int* prefix, cudaStream_t stream
   }
   ++*launches;
   if (mark) mark(2, stream);
-  if (launch_combine(prm, stream) != cudaSuccess) { cudaGetLastError(); return AMLA_ERR_CUDA; }
-  ++*launches;
+  if (prm.P > 1) {
+    if (launch_combine(prm, stream) != cudaSuccess) { cudaGetLastError(); return AMLA_ERR_CUDA; }
+    ++*launches;
+  }
   if (mark) mark(3, stream);
   return AMLA_OK;
 }
