@@ -12,6 +12,7 @@ constexpr int kDqk = 576;      // K width: 512 latent + 64 RoPE columns (Section
 constexpr int kDv = 512;       // V width: the latent columns
 constexpr int kPage = 64;      // keys per cache page == keys per tile
 constexpr int kRowBlock = 128; // query rows per work item (= MMA M)
+constexpr int kFewRows = 32;   // most query rows per sequence that the kernel for few rows takes (tensor memory holds Q once in every 32 lanes)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -30,8 +31,8 @@ struct DecodeParams {
   int* status;                   // workspace status word
   const int* prefix;             // [n_items + 1] linear tile index of each item's first tile
   float* part_o;                 // normalised partial outputs of split items: [2 * P * item_rows][512] half precision, then
-                                 // [2 * P * item_rows][16] scale bytes (see "Split partials" below)
-  float* part_lse;               // [2 * P, 128]      partial lse (natural log)
+                                 // [2 * P * item_rows][16] scale bytes (see "Split partials" below); FP32 from the kernel for few rows
+  float* part_lse;               // [2 * P * item_rows] partial lse (natural log)
   int4* merge_info;              // [min(n_items, P)] what the combine kernel has to merge: (item, slot of its first partial, number of
                                  // partials, 0), number < 2: nothing.  Written by the decode kernel; indexed by item where there are no
                                  // more items than parts, else by the part in which the item begins (one split item at most)
@@ -40,14 +41,14 @@ struct DecodeParams {
   float out_scale;               // factor on the normalised output (1; the dequantisation scale of an FP8 cache's V)
   int B, Sq, H;
   int R;                         // Sq * H query rows per sequence
-  int nrb;                       // row blocks per sequence = ceil(R / 128)
+  int nrb;                       // row blocks per sequence = ceil(R / item_rows)
   int n_items;                   // B * nrb
   int num_blocks, max_blocks_per_seq;
   int P;                         // parts the linear tile range is cut into
   int fused_plan;                // the decode kernel computes `prefix` itself (few items), no schedule kernel
   int flags;
   int tile_keys;                 // keys per schedule tile: 64 (one page) or 128 (two pages, the 256-row kernel)
-  int item_rows;                 // query rows per work item: 128, or 256 for the 256-row kernel (nrb counts these)
+  int item_rows;                 // query rows per work item: 32, 128 or 256, after the kernel (nrb counts these)
   int ovh;                       // schedule positions that stand for the cost of starting an item
   int min_share;                 // a part is given at least this many positions
   unsigned long long* trace;     // timeline buffer of a -DAMLA_TRACE build, else unused (nullptr)
@@ -91,6 +92,10 @@ constexpr int kUnitOverheadTiles = AMLA_UNIT_OVERHEAD_TILES;
 #define AMLA_QUAD_OVERHEAD_TILES 5            // 256-row kernel: in 128-key tiles (a build-time knob for tuning runs)
 #endif
 constexpr int kQuadOverheadTiles = AMLA_QUAD_OVERHEAD_TILES;
+#ifndef AMLA_FEW_OVERHEAD_TILES
+#define AMLA_FEW_OVERHEAD_TILES 3             // kernel for few rows: in 64-key pages (a build-time knob; 2-4 measure alike, 1 and 6 worse)
+#endif
+constexpr int kFewOverheadTiles = AMLA_FEW_OVERHEAD_TILES;
 constexpr int kMinPartKeys = 128;           // a part holds at least this many keys: a shorter one takes as long, and every part is a partial to merge
 constexpr int kFusedPlanMaxItems = 2048;   // up to this many items every decode CTA computes the prefix itself
 
@@ -165,7 +170,9 @@ __host__ __device__ inline int merge_groups(const DecodeParams& prm) { return pr
 // more mantissa bits), each 32-column chunk of a row scaled by a power of two so that its largest magnitude lies in
 // [1, 2): the chunk's scale byte is the biased FP32 exponent of that magnitude, the stored halves are value *
 // 2^(127 - byte), and value = half * 2^(byte - 127) exactly (byte 0: a chunk of zeros).  Half the bytes of FP32
-// partials, whatever the range of V.
+// partials, whatever the range of V.  (The kernel for few rows leaves FP32 rows [2 * P * 32][512]: its partials are small,
+// and a thread of it holds a column, so that a chunk's largest magnitude would be a reduction over the warp for every row:
+// 10 K of an epilogue's 13 K clk.)
 // ---------------------------------------------------------------------------------------------
 __host__ __device__ inline size_t partial_rows(const DecodeParams& prm) { return static_cast<size_t>(2) * prm.P * prm.item_rows; }
 __device__ __forceinline__ uint16_t* partial_halves(const DecodeParams& prm) { return reinterpret_cast<uint16_t*>(prm.part_o); }

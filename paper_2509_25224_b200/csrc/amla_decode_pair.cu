@@ -28,10 +28,8 @@
 // next load).  With the MMAs left out the tile still takes 7400.
 //
 // All waits are bounded; on expiry the kernel records kStatusTimeout and unwinds.
-#include <atomic>
-#include <type_traits>
-
 #include "amla_common.cuh"
+#include "amla_host.cuh"
 #include "amla_sm100.cuh"
 #include "amla_epilogue.cuh"
 #include "amla_units.cuh"
@@ -98,15 +96,6 @@ static_assert(X_NUM * 8 + 8 <= kBarBytes, "barrier area too small");
 
 __device__ __forceinline__ void report_timeout(int* status) { atomicExch(status, kStatusTimeout); }
 
-__device__ __forceinline__ int warp_inclusive_scan(int v, int lane) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= o) v += y;
-  }
-  return v;
-}
-
 // Wait whose verdict is the same in every lane of the warp, so that the warp-collective tensor-memory instructions
 // that follow are never executed by a part of it.
 template <bool kClusterAcquire = false>
@@ -151,22 +140,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = reinterpret_cast<int*>(smem_raw + kOffSeqlens);
-  if (wid == 8 && plan_here) {
-    int carry = 0;
-    for (int base = 0; base < prm.n_items; base += 32) {
-      const int it = base + lane;
-      const int b = prm.nrb == 1 ? it : it / prm.nrb;
-      const int n_seq = it < prm.n_items ? prm.seqlens[b] : 0;
-      const int v = it < prm.n_items ? schedule_length(n_seq, it, prm.tile_keys, prm.ovh) : 0;
-      const int x = warp_inclusive_scan(v, lane);
-      if (it < prm.n_items) {
-        lens_smem[b] = n_seq;                            // same value from every row block
-        plan_smem[it] = carry + x - v;
-      }
-      carry += __shfl_sync(0xffffffffu, x, 31);
-    }
-    if (lane == 0) plan_smem[prm.n_items] = carry;
-  }
+  if (wid == 8 && plan_here) plan_on_chip(prm, plan_smem, lens_smem, lane);
   if (tid == 32 * 10) {
     for (int i = 0; i < kSlots<kFp8>; ++i) {
       mbar_init(bar(X_FULL + i), kFp8 ? 2 * kWidenWarps : 1);          // E4M3: the warps that fill the slot, in either CTA
@@ -205,16 +179,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     asm volatile("griddepcontrol.launch_dependents;");
     if (prm.fused_plan) {      // (kSmemPlanItems, kFusedPlanMaxItems] items: every CTA writes the same prefix to the workspace
       if (wid == 0) {
-        int* pw = const_cast<int*>(prm.prefix);
-        int carry = 0;
-        for (int base = 0; base < prm.n_items; base += 32) {
-          const int it = base + lane;
-          const int v = it < prm.n_items ? schedule_length(prm.seqlens[it / prm.nrb], it, prm.tile_keys, prm.ovh) : 0;
-          const int x = warp_inclusive_scan(v, lane);
-          if (it < prm.n_items) pw[it] = carry + x - v;
-          carry += __shfl_sync(0xffffffffu, x, 31);
-        }
-        if (lane == 0) pw[prm.n_items] = carry;
+        plan_in_workspace(prm, lane);
         if (tid == 0 && blockIdx.x == 0) *prm.status = kStatusOk;
         __threadfence_block();
       }
@@ -756,61 +721,10 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
 // ---------------------------------------------------------------------------------------------------
 namespace {
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn get_encode_fn() {
-  static std::atomic<EncodeTiledFn> fn{nullptr};
-  EncodeTiledFn f = fn.load(std::memory_order_acquire);
-  if (!f) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess) {
-      f = reinterpret_cast<EncodeTiledFn>(p);
-      fn.store(f, std::memory_order_release);
-    }
-  }
-  return f;
-}
-
-// Rows of 576 bf16 seen as (64 columns, rows, 9 column blocks); a box is box_rows x box_blocks, laid out in shared
-// memory as [block][row][128 B] with the 128-byte swizzle.
-bool encode_rows(EncodeTiledFn encode, CUtensorMap* map, const void* base, cuuint64_t rows, cuuint32_t box_rows, cuuint32_t box_blocks) {
-  const cuuint64_t dims[3] = {64, rows, static_cast<cuuint64_t>(kQBlocks)};
-  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(kDqk) * 2, 128};
-  const cuuint32_t box[3] = {64, box_rows, box_blocks};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int kMode, bool kGuard, bool kFp8>
 cudaError_t launch_variant(const CUtensorMap& kmap, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
-  auto kern = decode_pair_kernel<kMode, kGuard, kFp8>;
-  // the opt-in to large dynamic shared memory is per device and per kernel; do it once each
   static std::atomic<uint64_t> done{0};
-  int device = 0;
-  cudaError_t err = cudaGetDevice(&device);
-  if (err != cudaSuccess) return err;
-  const uint64_t bit = 1ull << (device & 63);
-  if (!(done.load(std::memory_order_acquire) & bit)) {
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
-    if (err != cudaSuccess) return err;
-    done.fetch_or(bit, std::memory_order_release);
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * prm.P);
-  cfg.blockDim = dim3(kThreads<kFp8>);
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, kmap, vmap, qmap, prm);
+  return launch_serialized(decode_pair_kernel<kMode, kGuard, kFp8>, done, 2 * prm.P, kThreads<kFp8>, kSmemBytes, stream, kmap, vmap, qmap, prm);
 }
 
 template <bool kFp8>

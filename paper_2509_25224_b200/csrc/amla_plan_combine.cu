@@ -56,6 +56,8 @@ __global__ void plan_kernel(const int32_t* __restrict__ seqlens, int nrb, int n_
 constexpr int kFastSplits = 4;
 constexpr int kManyBatch = 8;
 
+// kFloat: the partials are plain FP32 rows (the kernel for few rows).
+template <bool kFloat>
 __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
   // A decode kernel that follows on the stream may set itself up beside this kernel (it writes nothing this kernel
   // reads before its own wait for this kernel's completion).
@@ -82,10 +84,37 @@ __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
   // a lane merges 16 consecutive columns (half of a 32-column chunk: one scale byte per split)
   const uint16_t* halves = partial_halves(prm);
   const uint8_t* scales = partial_scales(prm);
+  constexpr int kBatch = kFloat ? kManyBatch / 2 : kManyBatch;
   float acc[16];
   float tot = 0.f, mx;
-  auto accumulate = [&](float w, uint32_t scale_byte, const uint4& a, const uint4& b) {
-    const float ws = w * partial_unscale(scale_byte);
+  struct Piece { uint4 v[kFloat ? 4 : 2]; uint32_t scale; };   // FP32: columns 128 i + 4 lane .. + 3, else 16 lane .. + 15
+  auto fetch = [&](size_t prow) {
+    Piece x;
+    if (kFloat) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x.v[i % (kFloat ? 4 : 2)] = reinterpret_cast<const uint4*>(prm.part_o + prow * kDv)[32 * i + lane];
+    } else {
+      x.scale = scales[prow * 16 + (lane >> 1)];
+      const uint4* src = reinterpret_cast<const uint4*>(halves + prow * kDv) + 2 * lane;
+      x.v[0] = src[0];
+      x.v[1] = src[1];
+    }
+    return x;
+  };
+  auto accumulate = [&](float w, const Piece& x) {
+    if (kFloat) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint4 q = x.v[i % (kFloat ? 4 : 2)];
+        acc[4 * i] += w * __uint_as_float(q.x);
+        acc[4 * i + 1] += w * __uint_as_float(q.y);
+        acc[4 * i + 2] += w * __uint_as_float(q.z);
+        acc[4 * i + 3] += w * __uint_as_float(q.w);
+      }
+      return;
+    }
+    const float ws = w * partial_unscale(x.scale);
+    const uint4 a = x.v[0], b = x.v[1];
     const uint32_t h[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -97,18 +126,14 @@ __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
   if (nsplit <= kFastSplits) {
     // everything is requested before anything is used
     float ls[kFastSplits];
-    uint4 va[kFastSplits], vb[kFastSplits];
-    uint32_t sc[kFastSplits];
+    Piece x[kFastSplits];
 #pragma unroll
     for (int s = 0; s < kFastSplits; ++s) {
       ls[s] = -INFINITY;
       if (s < nsplit) {
         const size_t prow = static_cast<size_t>(Plan::slot_of_split(info.y, s)) * prm.item_rows + rr;
         ls[s] = prm.part_lse[prow];
-        sc[s] = scales[prow * 16 + (lane >> 1)];
-        const uint4* src = reinterpret_cast<const uint4*>(halves + prow * kDv) + 2 * lane;
-        va[s] = src[0];
-        vb[s] = src[1];
+        x[s] = fetch(prow);
       }
     }
     mx = ls[0];
@@ -122,7 +147,7 @@ __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
       if (s < nsplit) {
         const float w = expf(ls[s] - mx);             // 0 for a split that saw nothing
         tot += w;
-        accumulate(w, sc[s], va[s], vb[s]);
+        accumulate(w, x[s]);
       }
     }
   } else {
@@ -147,22 +172,18 @@ __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
       }
       const int n_here = min(32, nsplit - base);
 #pragma unroll 1
-      for (int j = 0; j < n_here; j += kManyBatch) {
-        uint4 va[kManyBatch], vb[kManyBatch];
-        uint32_t sc[kManyBatch];
+      for (int j = 0; j < n_here; j += kBatch) {
+        Piece x[kBatch];
 #pragma unroll
-        for (int k = 0; k < kManyBatch; ++k) {
+        for (int k = 0; k < kBatch; ++k) {
           const size_t prow = static_cast<size_t>(__shfl_sync(0xffffffffu, my_slot, min(j + k, n_here - 1))) * prm.item_rows + rr;
-          sc[k] = scales[prow * 16 + (lane >> 1)];
-          const uint4* src = reinterpret_cast<const uint4*>(halves + prow * kDv) + 2 * lane;
-          va[k] = src[0];
-          vb[k] = src[1];
+          x[k] = fetch(prow);
         }
 #pragma unroll
-        for (int k = 0; k < kManyBatch; ++k) {
+        for (int k = 0; k < kBatch; ++k) {
           const float w = j + k < n_here ? __shfl_sync(0xffffffffu, my_w, j + k) : 0.f;
           tot += w;
-          accumulate(w, sc[k], va[k], vb[k]);
+          accumulate(w, x[k]);
         }
       }
     }
@@ -174,9 +195,14 @@ __global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
     __nv_bfloat162 v = __floats2bfloat162_rn(acc[2 * i] * inv, acc[2 * i + 1] * inv);
     pk[i] = *reinterpret_cast<uint32_t*>(&v);
   }
-  uint4* dst = reinterpret_cast<uint4*>(orow + 16 * lane);
-  dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-  dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+  if (kFloat) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) *reinterpret_cast<uint2*>(orow + 128 * i + 4 * lane) = make_uint2(pk[2 * i], pk[2 * i + 1]);
+  } else {
+    uint4* dst = reinterpret_cast<uint4*>(orow + 16 * lane);
+    dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+  }
   if (lane == 0) *lrow = mx + logf(tot);
 }
 
@@ -199,7 +225,7 @@ cudaError_t launch_combine(const DecodeParams& prm, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, combine_kernel, prm);
+  return cudaLaunchKernelEx(&cfg, prm.item_rows < kRowBlock ? combine_kernel<true> : combine_kernel<false>, prm);
 }
 
 }  // namespace amla

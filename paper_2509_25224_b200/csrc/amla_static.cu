@@ -25,12 +25,12 @@ constexpr size_t kAlign = 256;
 constexpr size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 constexpr int kMaxItems = AMLA_STATIC_MAX_ITEMS;      // (sequence, 128-row block) pairs
-constexpr int kMaxParts = AMLA_STATIC_MAX_SMS / 2;    // clusters
+constexpr int kMaxParts = AMLA_STATIC_MAX_SMS / 2;    // parts of 128 rows (the kernel for few rows: twice as many of 32)
 
-// status | merge info [parts] | prefix[kMaxItems + 1] | partial lse [2 * parts][128] | partial O [2 * parts][128][512]
+// status | merge info [SMs: the most parts of any kernel] | prefix[kMaxItems + 1] | partial lse [2 * parts][128] | partial O [2 * parts][128][512]
 constexpr size_t kStatusOff = 0;
 constexpr size_t kMergeOff = kAlign;
-constexpr size_t kPrefixOff = kMergeOff + align_up(sizeof(int4) * kMaxParts);
+constexpr size_t kPrefixOff = kMergeOff + align_up(sizeof(int4) * AMLA_STATIC_MAX_SMS);
 constexpr size_t kPartLseOff = kPrefixOff + align_up(sizeof(int) * (kMaxItems + 1));
 constexpr size_t kPartOOff = kPartLseOff + align_up(sizeof(float) * 2 * kMaxParts * amla::kRowBlock);
 constexpr size_t kScratchBytes = kPartOOff + sizeof(float) * 2 * kMaxParts * amla::kRowBlock * amla::kDv;

@@ -5,6 +5,45 @@
 
 namespace amla {
 
+__device__ __forceinline__ int warp_inclusive_scan(int v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  return v;
+}
+
+// The schedule prefix of the batch, by one warp: into shared memory together with the sequence lengths, or into the workspace.
+__device__ __forceinline__ void plan_on_chip(const DecodeParams& prm, int* prefix, int* lens, int lane) {
+  int carry = 0;
+  for (int base = 0; base < prm.n_items; base += 32) {
+    const int it = base + lane;
+    const int b = prm.nrb == 1 ? it : it / prm.nrb;
+    const int n_seq = it < prm.n_items ? prm.seqlens[b] : 0;
+    const int v = it < prm.n_items ? schedule_length(n_seq, it, prm.tile_keys, prm.ovh) : 0;
+    const int x = warp_inclusive_scan(v, lane);
+    if (it < prm.n_items) {
+      lens[b] = n_seq;                                   // same value from every row block
+      prefix[it] = carry + x - v;
+    }
+    carry += __shfl_sync(0xffffffffu, x, 31);
+  }
+  if (lane == 0) prefix[prm.n_items] = carry;
+}
+__device__ __forceinline__ void plan_in_workspace(const DecodeParams& prm, int lane) {
+  int* pw = const_cast<int*>(prm.prefix);
+  int carry = 0;
+  for (int base = 0; base < prm.n_items; base += 32) {
+    const int it = base + lane;
+    const int v = it < prm.n_items ? schedule_length(prm.seqlens[it / prm.nrb], it, prm.tile_keys, prm.ovh) : 0;
+    const int x = warp_inclusive_scan(v, lane);
+    if (it < prm.n_items) pw[it] = carry + x - v;
+    carry += __shfl_sync(0xffffffffu, x, 31);
+  }
+  if (lane == 0) pw[prm.n_items] = carry;
+}
+
 struct Unit {
   int b, r0, n_b, t0, t1, it;      // sequence, first row of the row block, keys, tile range [t0, t1) of the schedule, item
 };
