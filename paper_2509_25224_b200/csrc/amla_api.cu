@@ -91,17 +91,32 @@ void profile_mark(int i, cudaStream_t stream) {
 
 }  // namespace
 
-// Chooses the kernel for the shape and fills the schedule fields of prm (rows per item, keys per tile, parts).
-// Sequences with more than 128 query rows go to the 256-row kernel (four-CTA clusters, pair MMAs) unless
-// AMLA_FLAG_KERNEL_ROWS128 asks for the 128-row kernel; sequences with at most 32 rows of a bf16 cache to the kernel for
-// few rows, the rest to the 128-row kernel.
+// Sequences with more than 128 query rows: blocks of 256 rows on four SMs, or independent blocks of 128 rows on two?  The
+// 256-row kernel reads the cache once for 256 rows, but a call of it takes longer to start and to finish, and so does every
+// further item that a part begins.  What either takes was measured over 1-200 sequences of 64-60000 keys and 2-8 tokens:
+//   256 rows: 21.5 us + 2.08 us per 128-key tile of a part + 11 us per item of a part beyond the first
+//   128 rows: 13 us + 1.41 us per page of a part + 6 us per item of a part
+// e.g. (two tokens, 128 heads) 1 x 3000 keys 22.0 against 15.7 us, 32 x 256 23.4 / 21.8, 32 x 2000 49 / 57, 1 x 60000 47.9 / 48.8.
+// Lengths are not known here: the block table's width bounds them.
+static bool blocks_of_256(const DecodeParams& prm, int pair_parts, int quad_parts) {
+  const double pages = prm.max_blocks_per_seq, tiles = (prm.max_blocks_per_seq + 1) / 2;
+  const double items1 = static_cast<double>(prm.B) * ((prm.R + kRowBlock - 1) / kRowBlock) / pair_parts;
+  const double items2 = static_cast<double>(prm.B) * ((prm.R + 2 * kRowBlock - 1) / (2 * kRowBlock)) / quad_parts;
+  return 21.5 + 2.08 * items2 * tiles + 11. * std::max(items2 - 1., 0.) < 13. + 1.41 * items1 * pages + 6. * items1;
+}
+
+// Chooses the kernel for the shape and fills the schedule fields of prm (rows per item, keys per tile, parts):
+//   up to 32 query rows of a bf16 cache      the kernel for few rows
+//   more than 128 rows of a bf16 cache       the 256-row kernel (four-CTA clusters, pair MMAs) where it is the faster one
+//   everything else                          the 128-row kernel
+// AMLA_FLAG_KERNEL_ROWS128 asks for the 128-row kernel whatever the shape.
 int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
   const bool simt = (flags & AMLA_FLAG_KERNEL_SIMT) != 0;
   bool quad = !simt && !(flags & AMLA_FLAG_KERNEL_ROWS128) && prm.R > kRowBlock && prm.kv8 == nullptr;
   int quad_parts = 0;
   if (quad) {
     quad_parts = decode_quad_parts(device, sms);
-    if (quad_parts <= 0) quad = false;         // four-CTA clusters cannot be placed on this device
+    if (quad_parts <= 0 || !blocks_of_256(prm, decode_pair_parts(sms), quad_parts)) quad = false;   // (0: four-CTA clusters cannot be placed on this device)
   }
   // A single sequence of at most four pages is one score tile of the 128-row kernel, and the kernel for few rows would take
   // it a page at a time: 256 keys, 16 rows 8.4 us against 8.6, 32 rows 8.8 against 10.0 (64 keys 8.3 against 8.2).

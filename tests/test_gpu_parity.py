@@ -169,6 +169,25 @@ def test_few_row_kernel_row_and_page_edges(lens, Sq, H):
         check_full(w, mode | binding.lazy(0))
 
 
+def _wide_table(w, pages=4096):
+    # a block table of this width may hold sequences long enough for the 256-row kernel, whatever the lengths are
+    pad = np.full((w.B, pages - w.block_table.shape[1]), -1, np.int32)
+    w.block_table = np.ascontiguousarray(np.concatenate([w.block_table, pad], axis=1))
+    return w
+
+
+@pytest.mark.parametrize("lens", [[1], [64], [65], [128], [129], [191], [192], [193], [1000, 3, 0, 257, 64], "128 short", "300 short", "2100 short"])
+def test_256_row_kernel_on_short_sequences_in_a_wide_table(lens):
+    # short sequences of more than 128 rows are blocks of 128 rows where the table's width says that they are short, and
+    # 256-row items where it does not: tile tails, and items around its on-chip and in-kernel schedules
+    if isinstance(lens, str):
+        lens = np.random.default_rng(31).integers(0, 130, int(lens.split()[0]))
+    w = _wide_table(synth.make_workload("wide", len(lens), 2, 128 if len(lens) < 100 else 65, lens, seed=500 + int(np.sum(lens))))
+    check_full(w)
+    if len(lens) < 100:
+        check_full(w, binding.RESCALE_ALG2 | binding.lazy(0))
+
+
 def test_few_row_kernel_reruns_are_bit_identical():
     # the lanes without a row hold leftovers of other pages: they must not have a say in when the reference moves
     w = synth.make_workload("again", 6, 1, 8, [300, 0, 1, 65, 1000, 2], seed=13)
