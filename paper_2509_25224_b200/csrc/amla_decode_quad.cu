@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "amla_common.cuh"
+#include "amla_host.cuh"
 #include "amla_sm100.cuh"
 #include "amla_epilogue.cuh"
 #include "amla_units.cuh"
@@ -65,17 +66,19 @@ constexpr uint32_t kEndB = kOffP + kNumP * kPStride;
 constexpr uint32_t kOffBars = kEndA > kEndB ? kEndA : kEndB;
 constexpr uint32_t kBarBytes = 320;
 #ifdef AMLA_TRACE
-constexpr int kSmemPlanItems = 4;                    // trace builds: the room goes to the stamps
+constexpr int kSmemPlanItems = 4, kSmemLens = 4;     // trace builds: the room goes to the stamps
 #else
-constexpr int kSmemPlanItems = 64;
+// on-chip copies of the schedule prefix, and behind a short one of the sequence lengths: that is what room there is
+constexpr int kSmemPlanItems = 160, kSmemLens = 64;
 #endif
 constexpr uint32_t kOffPlan = kOffBars + kBarBytes;
-constexpr uint32_t kOffSeqlens = kOffPlan + ((kSmemPlanItems + 1) * 4 + 15) / 16 * 16;
+constexpr uint32_t kOffSeqlens = kOffPlan + (kSmemLens + 1) * 4;
+constexpr uint32_t kEndPlan = kOffPlan + 4 * (kSmemPlanItems + 1 > 2 * kSmemLens + 1 ? kSmemPlanItems + 1 : 2 * kSmemLens + 1);
 #ifdef AMLA_TRACE
 // trace builds: every CTA keeps its stamps (low 32 bits of its SM's cycle counter) in shared memory, so that taking
 // one does not put a global store in front of the role's next release, and dumps them when it is done
 constexpr int kQTraceEvents = 16, kQTraceIdx = 10;
-constexpr uint32_t kOffTrace = kOffSeqlens + kSmemPlanItems * 4;
+constexpr uint32_t kOffTrace = kEndPlan;
 constexpr uint32_t kSmemBytes = kOffTrace + kQTraceEvents * kQTraceIdx * 4;
 #define QSTAMP(smem_base_, ev, idx)                                                                          \
   do {                                                                                                       \
@@ -89,7 +92,7 @@ constexpr uint32_t kSmemBytes = kOffTrace + kQTraceEvents * kQTraceIdx * 4;
       st_shared_b32((smem_base_) + kOffTrace + (15 * kQTraceIdx + (idx)) * 4, static_cast<uint32_t>(global_timer_ns())); \
   } while (0)
 #else
-constexpr uint32_t kSmemBytes = kOffSeqlens + kSmemPlanItems * 4;
+constexpr uint32_t kSmemBytes = kEndPlan;
 #define QSTAMP(smem_base_, ev, idx) do { } while (0)
 #define QSTAMP_NS(smem_base_, idx) do { } while (0)
 #endif
@@ -414,10 +417,12 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   const uint32_t myV_base = map_to_cta(smem_base, 2 + half);           // score CTA j -> value CTA j
   const uint32_t myV_bars = map_to_cta(bars, 2 + half);
 
-  // The lengths of the first 32 items are requested before anything else, so that their latency runs under the set-up
-  // below (they are inputs of the call: no kernel that this one may overlap with writes them).
-  int early_len = 0;
-  if (wid == 6 && prm.fused_plan && lane < prm.n_items) early_len = prm.seqlens[lane / prm.nrb];
+  // Warp 6 works out the schedule of a batch of up to kSmemPlanItems items during the set-up (from the sequence lengths: inputs
+  // of the call, which no kernel that this one may overlap with writes).
+  const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
+  int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
+  int* lens_smem = prm.n_items <= kSmemLens ? reinterpret_cast<int*>(smem_raw + kOffSeqlens) : nullptr;
+  if (wid == 6 && plan_here) plan_on_chip(prm, plan_smem, lens_smem, lane);
   if (tid == 0) {
     for (int i = 0; i < kNumP; ++i) mbar_init(bar(X_PV + i), 1);
     if (is_score) {
@@ -450,48 +455,36 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   const uint32_t tbase = ld_shared_b32(tmem_slot);
 
   if (tid == 0) QSTAMP_NS(smem_base, 1);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;");
-  if (tid == 0) QSTAMP_NS(smem_base, 2);
-  const int* prefix = prm.prefix;
-  const int* seqlens = prm.seqlens;
-  if (prm.fused_plan) {
-    int* ps = prm.n_items <= kSmemPlanItems ? reinterpret_cast<int*>(smem_raw + kOffPlan) : nullptr;
-    if (wid == 6) {
-      int* pw = const_cast<int*>(prm.prefix);
-      int carry = 0;
-      for (int base = 0; base < prm.n_items; base += 32) {
-        const int it = base + lane;
-        const int n_seq = it >= prm.n_items ? 0 : base == 0 ? early_len : prm.seqlens[it / prm.nrb];
-        if (ps && it < prm.n_items) reinterpret_cast<int*>(smem_raw + kOffSeqlens)[it / prm.nrb] = n_seq;
-        const int v = it < prm.n_items ? schedule_length(n_seq, it, prm.tile_keys, prm.ovh) : 0;
-        int x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, x, o);
-          if (lane >= o) x += y;
-        }
-        if (it < prm.n_items) {
-          pw[it] = carry + x - v;
-          if (ps) ps[it] = carry + x - v;
-        }
-        carry += __shfl_sync(0xffffffffu, x, 31);
+  const int* prefix = plan_here ? plan_smem : prm.prefix;
+  const int* seqlens = plan_here && lens_smem ? lens_smem : prm.seqlens;
+  if (!plan_here) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (prm.fused_plan) {      // (kSmemPlanItems, kFusedPlanMaxItems] items: every CTA writes the same prefix to the workspace
+      if (wid == 6) {
+        plan_in_workspace(prm, lane);
+        if (lane == 0 && blockIdx.x == 0) *prm.status = kStatusOk;
+        __threadfence_block();
       }
-      if (lane == 0) {
-        pw[prm.n_items] = carry;
-        if (ps) ps[prm.n_items] = carry;
-        if (blockIdx.x == 0) *prm.status = kStatusOk;
-      }
-      __threadfence_block();
+      __syncthreads();
     }
-    __syncthreads();
-    if (ps) { prefix = ps; seqlens = reinterpret_cast<const int*>(smem_raw + kOffSeqlens); }
   }
-  if (is_score && tid < kNumKSlots) {   // the first unit's Q is requested before the roles start: one piece per lane
-    UnitIter first(prm, prefix, seqlens, part);
-    Unit fu;
-    if (first.next(fu)) issue_q_piece(&q_map, smem_base, bars, tid, fu.b * prm.R + fu.r0 + half * kRowBlock);
+  UnitIter first(prm, prefix, seqlens, part);
+  Unit fu;
+  const bool any = first.next(fu);
+  if (plan_here) {
+    // Launched with programmatic stream serialization: everything above ran while the kernel before this one on the stream
+    // was still going; its results (the previous call's reads of the workspace among them) are complete after this wait.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (blockIdx.x == 0 && wid == 6) {       // the prefix in the workspace is part of what a call leaves behind
+      for (int it = lane; it <= prm.n_items; it += 32) const_cast<int*>(prm.prefix)[it] = plan_smem[it];
+      if (lane == 0) *prm.status = kStatusOk;
+    }
   }
+  if (tid == 0) QSTAMP_NS(smem_base, 2);
+  // the first unit's Q is requested before the roles start: one piece per lane
+  if (is_score && tid < kNumKSlots && any) issue_q_piece(&q_map, smem_base, bars, tid, fu.b * prm.R + fu.r0 + half * kRowBlock);
 
   bool ok = true;
   UnitIter iter(prm, prefix, seqlens, part);
@@ -973,25 +966,6 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
 // ---------------------------------------------------------------------------------------------------
 namespace {
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn get_encode_fn() {
-  static std::atomic<EncodeTiledFn> fn{nullptr};
-  EncodeTiledFn f = fn.load(std::memory_order_acquire);
-  if (!f) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess) {
-      f = reinterpret_cast<EncodeTiledFn>(p);
-      fn.store(f, std::memory_order_release);
-    }
-  }
-  return f;
-}
-
 void fill_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int clusters, cudaStream_t stream) {
   cfg = cudaLaunchConfig_t{};
   cfg.gridDim = dim3(4 * clusters);
@@ -1068,33 +1042,13 @@ cudaError_t launch_decode_quad(const DecodeParams& prm, cudaStream_t stream, int
                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (cr != CUDA_SUCCESS) return cudaErrorInvalidValue;
   }
-  // V: the same rows seen as (64 columns, rows, column block); one box = 64 keys x 2 column blocks, laid out in
-  // shared memory as [column block][key][64 columns]: the MN-major B operand of 128 output columns.
-  CUtensorMap vmap;
-  {
-    const cuuint64_t vdims[3] = {64, static_cast<cuuint64_t>(prm.num_blocks) * kPage, static_cast<cuuint64_t>(kDqk / 64)};
-    const cuuint64_t vstrides[2] = {static_cast<cuuint64_t>(kDqk) * 2, 128};
-    const cuuint32_t vbox[3] = {64, 64, 2};
-    const cuuint32_t vestr[3] = {1, 1, 1};
-    const CUresult vr = encode(&vmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(prm.kv), vdims, vstrides,
-                               vbox, vestr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (vr != CUDA_SUCCESS) return cudaErrorInvalidValue;
-  }
-  // Q: (64 columns, rows of all sequences, 9 column blocks); one box = 64 rows x one column block, laid out
-  // [row][64 columns] like an operand tile.  Rows past the end of the array read as zero; rows of a following
-  // sequence that a short block's boxes cover are dropped by the kernel.
-  CUtensorMap qmap;
-  {
-    const cuuint64_t qdims[3] = {64, static_cast<cuuint64_t>(prm.B) * prm.R, static_cast<cuuint64_t>(kDqk / 64)};
-    const cuuint64_t qstrides[2] = {static_cast<cuuint64_t>(kDqk) * 2, 128};
-    const cuuint32_t qbox[3] = {64, 64, 1};
-    const cuuint32_t qestr[3] = {1, 1, 1};
-    const CUresult qr = encode(&qmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(prm.q), qdims, qstrides,
-                               qbox, qestr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (qr != CUDA_SUCCESS) return cudaErrorInvalidValue;
-  }
+  // V: a box is 64 keys x 2 column blocks, [column block][key][64 columns]: the MN-major B operand of 128 output columns.
+  // Q: a box is 64 rows x one column block, like an operand tile.  Rows past the end of the array read as zero; rows of a
+  // following sequence that a short block's boxes cover are dropped by the kernel.
+  CUtensorMap vmap, qmap;
+  if (!encode_rows(encode, &vmap, prm.kv, static_cast<cuuint64_t>(prm.num_blocks) * kPage, kPage, 2) ||
+      !encode_rows(encode, &qmap, prm.q, static_cast<cuuint64_t>(prm.B) * prm.R, 64, 1))
+    return cudaErrorInvalidValue;
   const int mode = prm.flags & 3;
   const bool guard = !(prm.flags & 4);
   if (mode == 0) return guard ? launch_variant<0, true>(kmap, vmap, qmap, prm, stream) : launch_variant<0, false>(kmap, vmap, qmap, prm, stream);

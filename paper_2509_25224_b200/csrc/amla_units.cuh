@@ -14,7 +14,8 @@ __device__ __forceinline__ int warp_inclusive_scan(int v, int lane) {
   return v;
 }
 
-// The schedule prefix of the batch, by one warp: into shared memory together with the sequence lengths, or into the workspace.
+// The schedule prefix of the batch, by one warp: into shared memory together with the sequence lengths (unless lens is null),
+// or into the workspace.
 __device__ __forceinline__ void plan_on_chip(const DecodeParams& prm, int* prefix, int* lens, int lane) {
   int carry = 0;
   for (int base = 0; base < prm.n_items; base += 32) {
@@ -24,7 +25,7 @@ __device__ __forceinline__ void plan_on_chip(const DecodeParams& prm, int* prefi
     const int v = it < prm.n_items ? schedule_length(n_seq, it, prm.tile_keys, prm.ovh) : 0;
     const int x = warp_inclusive_scan(v, lane);
     if (it < prm.n_items) {
-      lens[b] = n_seq;                                   // same value from every row block
+      if (lens) lens[b] = n_seq;                         // same value from every row block
       prefix[it] = carry + x - v;
     }
     carry += __shfl_sync(0xffffffffu, x, 31);

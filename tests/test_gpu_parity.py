@@ -176,7 +176,7 @@ def _wide_table(w, pages=4096):
     return w
 
 
-@pytest.mark.parametrize("lens", [[1], [64], [65], [128], [129], [191], [192], [193], [1000, 3, 0, 257, 64], "128 short", "300 short", "2100 short"])
+@pytest.mark.parametrize("lens", [[1], [64], [65], [128], [129], [191], [192], [193], [1000, 3, 0, 257, 64], "64 short", "65 short", "160 short", "161 short", "300 short", "2100 short"])
 def test_256_row_kernel_on_short_sequences_in_a_wide_table(lens):
     # short sequences of more than 128 rows are blocks of 128 rows where the table's width says that they are short, and
     # 256-row items where it does not: tile tails, and items around its on-chip and in-kernel schedules
