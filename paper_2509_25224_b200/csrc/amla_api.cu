@@ -111,6 +111,7 @@ static bool blocks_of_256(const DecodeParams& prm, int pair_parts, int quad_part
 //   everything else                          the 128-row kernel
 // AMLA_FLAG_KERNEL_ROWS128 asks for the 128-row kernel whatever the shape.
 int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
+  prm.sms = sms;
   const bool simt = (flags & AMLA_FLAG_KERNEL_SIMT) != 0;
   bool quad = !simt && !(flags & AMLA_FLAG_KERNEL_ROWS128) && prm.R > kRowBlock && prm.kv8 == nullptr;
   int quad_parts = 0;

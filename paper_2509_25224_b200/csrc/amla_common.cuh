@@ -44,6 +44,7 @@ struct DecodeParams {
   int nrb;                       // row blocks per sequence = ceil(R / item_rows)
   int n_items;                   // B * nrb
   int num_blocks, max_blocks_per_seq;
+  int sms;                       // SMs of the device
   int P;                         // parts the linear tile range is cut into
   int fused_plan;                // the decode kernel computes `prefix` itself (few items), no schedule kernel
   int flags;
@@ -162,6 +163,7 @@ struct Plan {
 };
 
 __host__ __device__ inline bool merge_by_item(const DecodeParams& prm) { return prm.n_items <= prm.P; }
+__host__ __device__ inline int merge_rows(const DecodeParams& prm) { return prm.nrb == 1 ? prm.R : prm.item_rows; }
 __host__ __device__ inline int merge_groups(const DecodeParams& prm) { return prm.n_items < prm.P ? prm.n_items : prm.P; }
 
 // ---------------------------------------------------------------------------------------------

@@ -47,163 +47,127 @@ __global__ void plan_kernel(const int32_t* __restrict__ seqlens, int nrb, int n_
 }
 
 // The merge of split items,
-//   lse = ln sum_s exp(lse_s),  out = sum_s exp(lse_s - lse) * out_s,
-// one warp per query row.  The decode kernel left in merge_info which items are split, by item or, where there are more
-// items than parts, by the part in which a split item begins: the grid is min(items, parts) x rows of an item whatever
-// the batch (192 sequences, 74 parts: a grid over all rows cost the call 12 us; 32 sequences: a grid over parts 3 us more
-// than one over items), and a warp's chain of dependent memory round trips is merge_info -> (partial lse, partial rows).  Up to kFastSplits
-// partials are fetched before any arithmetic, of more than that eight at a time.
-constexpr int kFastSplits = 4;
-constexpr int kManyBatch = 8;
-
-// kFloat: the partials are plain FP32 rows (the kernel for few rows).
-template <bool kFloat>
-__global__ void __launch_bounds__(128) combine_kernel(DecodeParams prm) {
+//   lse = ln sum_s exp(lse_s),  out = sum_s exp(lse_s - lse) * out_s.
+// The decode kernel left in merge_info which items are split, by item or, where there are more items than parts, by the part
+// in which a split item begins: the grid is min(items, parts) x query rows of an item whatever the batch.
+//
+// What bounds it is a chain of memory round trips, merge_info -> (partial lse, partial rows) -> store, how often the middle
+// is repeated, and how many blocks an SM can hold: the decode kernel of the next call is placed, and sets itself up, when
+// the last of these blocks has started.  So a warp is kept to few registers, and takes
+//   a row, up to four partials at a time, where there are many rows (more than eight per SM);
+//   a quarter of a row, eight at a time, where there are few rows, and those of many partials;
+//   half or a quarter of a row of FP32 partials (the kernel for few rows).
+// Against a whole row per warp in 126 registers, eight partials at a time, and a warp for every row that an item has room
+// for (the whole call): one sequence of 2531 keys 14.3 -> 13.2 us, of 60000 39.4 -> 35.1, of 3000 with 16 rows 12.4 -> 9.9;
+// 192 sequences of 1-512 keys 45.4 -> 44.2; 32 of 1-8 K with 16 rows 37.5 -> 36.4; 96 of 2048 73.1 -> 71.7 cool.
+// (One block per SM that walks over the rows and fits beside a decode CTA lets the next call's decode kernel in at once, but
+// takes 10 us where these take 4: 32 x 4096 keys 55.8 -> 61.5.)
+template <bool kFloat, int kCols>
+__global__ void __launch_bounds__(128, kCols == 16 ? 7 : kCols == 8 ? 8 : 5) combine_kernel(const __grid_constant__ DecodeParams prm) {
   // A decode kernel that follows on the stream may set itself up beside this kernel (it writes nothing this kernel
   // reads before its own wait for this kernel's completion).
   asm volatile("griddepcontrol.launch_dependents;");
-  const int warps_per_block = blockDim.x >> 5;
+  constexpr int kUnits = 16 / kCols;                       // warps per row
+  constexpr int kFast = 4, kBatch = kCols == 16 || (kFloat && kCols == 8) ? 4 : 8;
+  constexpr int kWords = kFloat ? kCols : kCols / 2;       // 32-bit words of a partial per lane
   const int lane = threadIdx.x & 31;
-  const int chunks = prm.item_rows / warps_per_block;
-  const int group = blockIdx.x / chunks;
-  const int rr = (blockIdx.x - group * chunks) * warps_per_block + (threadIdx.x >> 5);     // row within the item
+  const int unit = blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int row = unit / kUnits, group = row / merge_rows(prm);
+  const int rr = row - group * merge_rows(prm);            // row within the item
+  const int col = (unit - row * kUnits) * (kDv / kUnits) + lane * kCols;
   asm volatile("griddepcontrol.wait;" ::: "memory");   // launched early (programmatic dependent launch): the partials must be complete
+  if (group >= merge_groups(prm)) return;
   const int4 info = prm.merge_info[group];
   const int nsplit = info.z;
   if (nsplit < 2) return;
-  const int b = info.x / prm.nrb;
+  const int b = prm.nrb == 1 ? info.x : info.x / prm.nrb;
   const int rin = (info.x - b * prm.nrb) * prm.item_rows + rr;                          // row within the sequence
   if (rin >= prm.R) return;
-  __nv_bfloat16* orow = prm.out + (static_cast<size_t>(b) * prm.R + rin) * kDv;
-  float* lrow = prm.lse + static_cast<size_t>(b) * prm.R + rin;
-  auto write_empty = [&]() {
-    for (int c = lane * 8; c < kDv; c += 32 * 8) *reinterpret_cast<uint4*>(orow + c) = make_uint4(0, 0, 0, 0);
-    if (lane == 0) *lrow = -INFINITY;
-  };
 
-  // a lane merges 16 consecutive columns (half of a 32-column chunk: one scale byte per split)
-  const uint16_t* halves = partial_halves(prm);
-  const uint8_t* scales = partial_scales(prm);
-  constexpr int kBatch = kFloat ? kManyBatch / 2 : kManyBatch;
-  float acc[16];
-  float tot = 0.f, mx;
-  struct Piece { uint4 v[kFloat ? 4 : 2]; uint32_t scale; };   // FP32: columns 128 i + 4 lane .. + 3, else 16 lane .. + 15
-  auto fetch = [&](size_t prow) {
+  auto part_row = [&](int s) { return static_cast<size_t>(Plan::slot_of_split(info.y, s)) * prm.item_rows + rr; };
+  struct Piece { uint32_t w[kWords], scale; };
+  auto fetch = [&](int s) {
+    const size_t prow = part_row(s);
     Piece x;
-    if (kFloat) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) x.v[i % (kFloat ? 4 : 2)] = reinterpret_cast<const uint4*>(prm.part_o + prow * kDv)[32 * i + lane];
+    const uint32_t* src = kFloat ? reinterpret_cast<const uint32_t*>(prm.part_o + prow * kDv + col) : reinterpret_cast<const uint32_t*>(partial_halves(prm) + prow * kDv + col);
+    if constexpr (kWords == 2) {
+      *reinterpret_cast<uint2*>(x.w) = *reinterpret_cast<const uint2*>(src);
     } else {
-      x.scale = scales[prow * 16 + (lane >> 1)];
-      const uint4* src = reinterpret_cast<const uint4*>(halves + prow * kDv) + 2 * lane;
-      x.v[0] = src[0];
-      x.v[1] = src[1];
+#pragma unroll
+      for (int i = 0; i < kWords / 4; ++i) *reinterpret_cast<uint4*>(x.w + 4 * i) = reinterpret_cast<const uint4*>(src)[i];
     }
+    if (!kFloat) x.scale = partial_scales(prm)[prow * 16 + col / 32];
     return x;
   };
+  float acc[kCols], tot = 0.f;
+#pragma unroll
+  for (int i = 0; i < kCols; ++i) acc[i] = 0.f;
   auto accumulate = [&](float w, const Piece& x) {
-    if (kFloat) {
+    tot += w;
+    const float ws = kFloat ? w : w * partial_unscale(x.scale);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const uint4 q = x.v[i % (kFloat ? 4 : 2)];
-        acc[4 * i] += w * __uint_as_float(q.x);
-        acc[4 * i + 1] += w * __uint_as_float(q.y);
-        acc[4 * i + 2] += w * __uint_as_float(q.z);
-        acc[4 * i + 3] += w * __uint_as_float(q.w);
+    for (int i = 0; i < kWords; ++i) {
+      if (kFloat) {
+        acc[i] += ws * __uint_as_float(x.w[i]);
+      } else {
+        const float2 v = unpack_f16x2(x.w[i]);
+        acc[2 * i % kCols] += ws * v.x;
+        acc[(2 * i + 1) % kCols] += ws * v.y;
       }
-      return;
-    }
-    const float ws = w * partial_unscale(x.scale);
-    const uint4 a = x.v[0], b = x.v[1];
-    const uint32_t h[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float2 v = unpack_f16x2(h[i]);
-      acc[2 * i] += ws * v.x;
-      acc[2 * i + 1] += ws * v.y;
     }
   };
-  if (nsplit <= kFastSplits) {
-    // everything is requested before anything is used
-    float ls[kFastSplits];
-    Piece x[kFastSplits];
+  // the lse of 32 splits, one per lane, and the partials of a batch are on their way together
+  float ls = lane < nsplit ? prm.part_lse[part_row(lane)] : -INFINITY;
+  Piece x[kBatch];
+  if (nsplit <= kFast) {
 #pragma unroll
-    for (int s = 0; s < kFastSplits; ++s) {
-      ls[s] = -INFINITY;
-      if (s < nsplit) {
-        const size_t prow = static_cast<size_t>(Plan::slot_of_split(info.y, s)) * prm.item_rows + rr;
-        ls[s] = prm.part_lse[prow];
-        x[s] = fetch(prow);
-      }
-    }
-    mx = ls[0];
-#pragma unroll
-    for (int s = 1; s < kFastSplits; ++s) mx = fmaxf(mx, ls[s]);
-    if (mx == -INFINITY) { write_empty(); return; }   // no split saw a visible key for this row
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-#pragma unroll
-    for (int s = 0; s < kFastSplits; ++s) {
-      if (s < nsplit) {
-        const float w = expf(ls[s] - mx);             // 0 for a split that saw nothing
-        tot += w;
-        accumulate(w, x[s]);
-      }
-    }
+    for (int k = 0; k < kFast; ++k)
+      if (k < nsplit) x[k] = fetch(k);
   } else {
-    // lse of the splits: one split per lane (in rounds of 32), so that the loads overlap
-    mx = -INFINITY;
-    for (int base = 0; base < nsplit; base += 32) {
-      const int sidx = base + lane;
-      if (sidx < nsplit) mx = fmaxf(mx, prm.part_lse[static_cast<size_t>(Plan::slot_of_split(info.y, sidx)) * prm.item_rows + rr]);
-    }
 #pragma unroll
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (mx == -INFINITY) { write_empty(); return; }
+    for (int k = 0; k < kBatch; ++k) x[k] = fetch(min(k, nsplit - 1));
+  }
+  float mx = ls;
+  for (int s = lane + 32; s < nsplit; s += 32) mx = fmaxf(mx, prm.part_lse[part_row(s)]);
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-    for (int base = 0; base < nsplit; base += 32) {
-      const int sidx = base + lane;
-      int my_slot = 0;
-      float my_w = 0.f;
-      if (sidx < nsplit) {
-        my_slot = Plan::slot_of_split(info.y, sidx);
-        my_w = expf(prm.part_lse[static_cast<size_t>(my_slot) * prm.item_rows + rr] - mx);
-      }
-      const int n_here = min(32, nsplit - base);
+  for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (mx != -INFINITY) {                                   // else no split saw a visible key for this row: zeros
+    ls = expf(ls - mx);                                    // 0 for a split that saw nothing
+    if (nsplit <= kFast) {
+#pragma unroll
+      for (int k = 0; k < kFast; ++k)
+        if (k < nsplit) accumulate(__shfl_sync(0xffffffffu, ls, k), x[k]);
+    } else {
 #pragma unroll 1
-      for (int j = 0; j < n_here; j += kBatch) {
-        Piece x[kBatch];
+      for (int s0 = 0;;) {
 #pragma unroll
         for (int k = 0; k < kBatch; ++k) {
-          const size_t prow = static_cast<size_t>(__shfl_sync(0xffffffffu, my_slot, min(j + k, n_here - 1))) * prm.item_rows + rr;
-          x[k] = fetch(prow);
+          const float w = __shfl_sync(0xffffffffu, ls, (s0 + k) & 31);
+          if (s0 + k < nsplit) accumulate(w, x[k]);
         }
+        s0 += kBatch;
+        if (s0 >= nsplit) break;
 #pragma unroll
-        for (int k = 0; k < kBatch; ++k) {
-          const float w = j + k < n_here ? __shfl_sync(0xffffffffu, my_w, j + k) : 0.f;
-          tot += w;
-          accumulate(w, x[k]);
-        }
+        for (int k = 0; k < kBatch; ++k) x[k] = fetch(min(s0 + k, nsplit - 1));
+        if ((s0 & 31) == 0) ls = s0 + lane < nsplit ? expf(prm.part_lse[part_row(s0 + lane)] - mx) : 0.f;
       }
     }
   }
-  const float inv = 1.f / tot;
-  uint32_t pk[8];
+  const float inv = tot > 0.f ? 1.f / tot : 0.f;
+  uint32_t pk[kCols / 2];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    __nv_bfloat162 v = __floats2bfloat162_rn(acc[2 * i] * inv, acc[2 * i + 1] * inv);
-    pk[i] = *reinterpret_cast<uint32_t*>(&v);
+  for (int i = 0; i < kCols / 2; ++i) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(acc[2 * i] * inv, acc[2 * i + 1] * inv);
+    pk[i] = *reinterpret_cast<const uint32_t*>(&v);
   }
-  if (kFloat) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) *reinterpret_cast<uint2*>(orow + 128 * i + 4 * lane) = make_uint2(pk[2 * i], pk[2 * i + 1]);
+  __nv_bfloat16* dst = prm.out + (static_cast<size_t>(b) * prm.R + rin) * kDv + col;
+  if constexpr (kCols == 4) {
+    *reinterpret_cast<uint2*>(dst) = make_uint2(pk[0], pk[1]);
   } else {
-    uint4* dst = reinterpret_cast<uint4*>(orow + 16 * lane);
-    dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+#pragma unroll
+    for (int i = 0; i < kCols / 8; ++i) reinterpret_cast<uint4*>(dst)[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
   }
-  if (lane == 0) *lrow = mx + logf(tot);
+  if (lane == 0 && col == 0) prm.lse[static_cast<size_t>(b) * prm.R + rin] = tot > 0.f ? mx + logf(tot) : -INFINITY;
 }
 
 cudaError_t launch_plan(const DecodeParams& prm, int* prefix_out, cudaStream_t stream) {
@@ -212,12 +176,13 @@ cudaError_t launch_plan(const DecodeParams& prm, int* prefix_out, cudaStream_t s
 }
 
 cudaError_t launch_combine(const DecodeParams& prm, cudaStream_t stream) {
-  const int warps_per_block = 4;   // small blocks: one fits beside a decode CTA (registers), so part of the grid is resident before the decode kernel ends
-  const int blocks = merge_groups(prm) * (prm.item_rows / warps_per_block);
-  // programmatic dependent launch: the blocks may be placed while the decode kernel drains; they wait inside
+  const bool fp32 = prm.item_rows < kRowBlock;
+  const int rows = merge_groups(prm) * merge_rows(prm);
+  const bool few = rows <= 8 * prm.sms;
+  const int units = rows * (few ? 4 : fp32 ? 2 : 1);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(warps_per_block * 32);
+  cfg.gridDim = dim3((units + 3) / 4);
+  cfg.blockDim = dim3(128);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -225,7 +190,7 @@ cudaError_t launch_combine(const DecodeParams& prm, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, prm.item_rows < kRowBlock ? combine_kernel<true> : combine_kernel<false>, prm);
+  return cudaLaunchKernelEx(&cfg, fp32 ? (few ? combine_kernel<true, 4> : combine_kernel<true, 8>) : few ? combine_kernel<false, 4> : combine_kernel<false, 16>, prm);
 }
 
 }  // namespace amla

@@ -169,6 +169,17 @@ def test_few_row_kernel_row_and_page_edges(lens, Sq, H):
         check_full(w, mode | binding.lazy(0))
 
 
+@pytest.mark.parametrize("B,Sq,H,n", [(1, 1, 128, 400), (1, 1, 40, 4500), (1, 1, 128, 12000), (9, 1, 128, 1500), (11, 1, 128, 1500), (36, 1, 33, 700),
+                                      (1, 1, 16, 20000), (36, 2, 16, 900), (75, 1, 16, 700)])
+def test_merges_by_rows_and_by_quarters_of_rows(B, Sq, H, n):
+    # up to 8 rows per SM a warp merges a quarter of a row, above that a row (FP32 partials: half); 2 to over 32 partials
+    # per row, in one batch or several; by item and, with more items than parts, by part
+    rng = np.random.default_rng(B + n)
+    lens = np.maximum(1, n - rng.integers(0, n // 3, B))
+    w = synth.make_workload("merge", B, Sq, H, lens, seed=600 + B + n)
+    check_full(w)
+
+
 def _wide_table(w, pages=4096):
     # a block table of this width may hold sequences long enough for the 256-row kernel, whatever the lengths are
     pad = np.full((w.B, pages - w.block_table.shape[1]), -1, np.int32)
