@@ -4,7 +4,7 @@
 // same work on 64 rows each; every matrix product is an MMA over the pair (tcgen05.mma.cta_group::2, M = 128, N up to
 // 256), so each CTA supplies its own 64 rows of A and HALF of the B operand:
 //
-//   S = Q K^T     A = Q (64 rows x 576, shared memory), B = K: CTA j loads keys 32 j .. 32 j + 31 of every page
+//   S = Q K^T     A = Q (64 rows x 576, shared memory), B = K: CTA j loads the first or second half of a tile's keys
 //   O += P~ V     A = P~ (64 rows x 64 keys per page, shared memory), B = V: CTA j loads columns 256 j .. 256 j + 255
 //
 // With M = 128 over two CTAs the accumulators use all 128 tensor-memory lanes of either CTA: lanes 0-63 hold the CTA's
@@ -12,7 +12,7 @@
 // (256 keys) takes 128 columns, O (512 columns of V) takes 256, so S is double buffered and Q need not go into tensor
 // memory: it is an operand as soon as TMA has delivered it.
 //
-// Warps 0-7 run Algorithm 2's recurrence (lines 5-12; four threads share a query row: lane half = key half of a page,
+// Warps 0-7 run Algorithm 2's recurrence (lines 5-12; four threads share a query row: lane half = half of a tile's keys,
 // warp group = even / odd pages), write P~ = bf16(P * S16) into the P buffer of their own CTA, apply the integer N to
 // the bit patterns of O when the row's reference moved (lines 13-16; Lemma 3.1) and run the epilogue (line 20).  They
 // never hand data to the other CTA.  Warps 8 and 10 load (TMA), warp 9 of the even CTA issues the MMAs for both.
@@ -51,8 +51,8 @@ constexpr int kQBlocks = kDqk / 64;                     // 64-column blocks of Q
 constexpr uint32_t kQBlockBytes = kCtaRows * 128;       // [64 rows][128 B], 128-byte swizzle
 constexpr uint32_t kQBytes = kQBlocks * kQBlockBytes;
 constexpr uint32_t kPPageBytes = kCtaRows * 128;        // P~ of one page: [64 rows][64 keys]
-constexpr uint32_t kKBoxBytes = 32 * 128;               // this CTA's half of a page x one 64-column block
-constexpr uint32_t kSlotBytes = 128 * 128;              // K: 4 pages x 32 keys x 64 columns; V: 64 keys x 128 columns
+constexpr uint32_t kKBoxBytes = 32 * 128;               // half a page (32 keys) x one 64-column block
+constexpr uint32_t kSlotBytes = 128 * 128;              // K: half of 4 pages' keys x 64 columns; V: 64 keys x 128 columns
 constexpr uint32_t kVBlockBytes = 64 * 128;             // 64 keys x 64 columns
 // The ring of operand slots, and for an E4M3 cache a ring of raw slots in front of it, one for every operand slot.
 // A rule that every user of a ring keeps: a thread waits only for slots that it fills or empties itself, and having waited
@@ -116,7 +116,7 @@ using Tiles = TileIter<kTilePages>;
 
 template <int kMode, bool kGuard, bool kFp8>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads<kFp8>, 1)
-decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap q_map,
+decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap khalf_map, const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap q_map,
                    const DecodeParams prm) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t smem_base = smem_u32(smem_raw);
@@ -160,6 +160,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     mbar_init(bar(X_PVDONE), 1);
     fence_mbar_init();
     prefetch_tensormap(&k_map);
+    prefetch_tensormap(&khalf_map);
     prefetch_tensormap(&v_map);
     prefetch_tensormap(&q_map);
   }
@@ -243,11 +244,12 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         if (!ok) break;
         tc_fence_after_sync();
         if (tid == 0 && leader) AMLA_STAMP(prm, part, 8, gs);
-        // This group's pages of the tile are t + grp and t + grp + 2 (32 columns each, 32 keys per lane half).  The scores are
-        // read from tensor memory twice, a page at a time: for the maximum, and for the exponentials once the P buffer is
+        // A lane half holds 32 np neighbouring keys; this group takes its 32-key chunks grp and grp + 2.  The scores are
+        // read from tensor memory twice, a chunk at a time: for the maximum, and for the exponentials once the P buffer is
         // free.  (Held in registers in between they cost 64 more of them and twice the code.)
         const uint32_t scol = tbase + lane_base + kSCol + 128 * sb + 32 * grp;
-        const int nvis0 = visible - (t + grp) * kPage - 32 * khalf;        // keys of the first page that the row sees (may be <= 0)
+        const int chunk0 = np * khalf + grp;                                // of the tile's 2 np
+        const int nvis0 = visible - t * kPage - 32 * chunk0;                // keys of the first chunk that the row sees (may be <= 0)
         const bool plain = t + np <= first_masked && scale_nonneg;          // every key of the tile is visible
         // lines 5-6: running max (the scale is folded into the FMA below)
         float ext = -INFINITY;
@@ -265,7 +267,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
             }
             a = fmaxf(a, b) * prm.scale_log2;
           } else {
-            const int nvis = nvis0 - 2 * kPage * h;
+            const int nvis = nvis0 - 64 * h;
 #pragma unroll
             for (int i = 0; i < 32; ++i) a = fmaxf(a, i < nvis ? __uint_as_float(v[i]) * prm.scale_log2 : -INFINITY);
           }
@@ -339,11 +341,12 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           tmem_ld_32x32b_x32(scol + 64 * h, v);
           tmem_wait_ld();
           if (!plain) {
-            const int nvis = nvis0 - 2 * kPage * h;        // scaled here; hidden keys become 2^-inf = 0
+            const int nvis = nvis0 - 64 * h;        // scaled here; hidden keys become 2^-inf = 0
 #pragma unroll
             for (int i = 0; i < 32; ++i) v[i] = i < nvis ? __float_as_uint(__uint_as_float(v[i]) * prm.scale_log2) : 0xff800000u;
           }
-          const uint32_t dst = prow_smem + (grp + 2 * h) * kPPageBytes;
+          const int chunk = chunk0 + 2 * h;                // half (chunk & 1) of page chunk / 2
+          const uint32_t dst = prow_smem + (chunk >> 1) * kPPageBytes;
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             uint32_t pk[4];
@@ -356,7 +359,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
               if (i & 1) rsb = add_f32x2(rsb, pp); else rsa = add_f32x2(rsa, pp);
               pk[i] = pack_bf16x2(q0, q1);
             }
-            st_shared_v4(dst + (((4 * khalf + c) ^ (r & 7)) << 4), pk[0], pk[1], pk[2], pk[3]);
+            st_shared_v4(dst + (((4 * (chunk & 1) + c) ^ (r & 7)) << 4), pk[0], pk[1], pk[2], pk[3]);
           }
         }
         tc_fence_before_sync();            // S has been read, O (perhaps) rewritten
@@ -490,10 +493,14 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           advance();
         }
       };
-      int page[kTilePages];
+      // This CTA's half of the tile's keys, 32 np of them from key 32 np rank on, is at most two boxes: a page, or the half page
+      // in the middle of a tile of three pages or of one.  (With 32 keys of every page it was four boxes: E4M3, one loader:
+      // 62.6 -> 61.2 us for 32 x 4096 keys, 120.1 -> 116.4 for 32 x 512-8192, two tokens; bf16 494 -> 481 for 96 x 16384.)
+      int page[2];
       auto get_pages = [&](const TileRef& x) {
-#pragma unroll
-        for (int p = 0; p < kTilePages; ++p) page[p] = p < x.np ? __ldg(x.bt + p) : 0;
+        const int p0 = (x.np * rank) >> 1;
+        page[0] = x.np > 0 ? __ldg(x.bt + p0) : 0;
+        page[1] = p0 + 1 < x.np ? __ldg(x.bt + p0 + 1) : 0;
       };
       TileRef cur = take(), prev = cur;
       get_pages(cur);                                       // on its way while Q is requested
@@ -509,9 +516,11 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           }
           q_out = false;
         }
-        int row[kTilePages];
-#pragma unroll
-        for (int p = 0; p < kTilePages; ++p) row[p] = row_of(page[p]);
+        const bool odd = (cur.np * rank) & 1;                               // begins in the middle of a page
+        const int chunks0 = odd || cur.np == 1 ? 1 : 2, chunks1 = min(cur.np - chunks0, 2);
+        const int row0 = row_of(page[0]) + (odd ? 32 : 0), row1 = row_of(page[1]);
+        const CUtensorMap* const map0 = chunks0 == 2 ? &k_map : &khalf_map;
+        const CUtensorMap* const map1 = chunks1 == 2 ? &k_map : &khalf_map;
         get_pages(nxt);
 #pragma unroll 1
         for (int c = 0; c < kQBlocks; ++c) {
@@ -522,14 +531,12 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
             if (leader && (c <= 1 || c >= 7)) AMLA_STAMP(prm, part, c <= 1 ? 16 : 17, pt);
             if (kFp8) {
               mbar_arrive_expect_tx(full0 + 8 * slot, cur.np * (kKBoxBytes / 2));
-#pragma unroll
-              for (int p = 0; p < kTilePages; ++p)
-                if (p < cur.np) tma_load_2d_hint(dst + p * (kKBoxBytes / 2), &k_map, 64 * c, row[p] + 32 * rank, full0 + 8 * slot, keep);   // [32 keys][64 columns]
+              tma_load_2d_hint(dst, map0, 64 * c, row0, full0 + 8 * slot, keep);                                          // [64 or 32 keys][64 columns]
+              if (chunks1 > 0) tma_load_2d_hint(dst + chunks0 * (kKBoxBytes / 2), map1, 64 * c, row1, full0 + 8 * slot, keep);
             } else {
               if (leader) mbar_arrive_expect_tx(full0 + 8 * slot, 2 * cur.np * kKBoxBytes);
-#pragma unroll
-              for (int p = 0; p < kTilePages; ++p)
-                if (p < cur.np) tma_load_3d_pair_hint(dst + p * kKBoxBytes, &k_map, 0, row[p] + 32 * rank, c, lead_full0 + 8 * slot, keep);
+              tma_load_3d_pair_hint(dst, map0, 0, row0, c, lead_full0 + 8 * slot, keep);
+              if (chunks1 > 0) tma_load_3d_pair_hint(dst + chunks0 * kKBoxBytes, map1, 0, row1, c, lead_full0 + 8 * slot, keep);
             }
           }
           advance();
@@ -722,18 +729,18 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
 namespace {
 
 template <int kMode, bool kGuard, bool kFp8>
-cudaError_t launch_variant(const CUtensorMap& kmap, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
+cudaError_t launch_variant(const CUtensorMap& kmap, const CUtensorMap& khalf, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
   static std::atomic<uint64_t> done{0};
-  return launch_serialized(decode_pair_kernel<kMode, kGuard, kFp8>, done, 2 * prm.P, kThreads<kFp8>, kSmemBytes, stream, kmap, vmap, qmap, prm);
+  return launch_serialized(decode_pair_kernel<kMode, kGuard, kFp8>, done, 2 * prm.P, kThreads<kFp8>, kSmemBytes, stream, kmap, khalf, vmap, qmap, prm);
 }
 
 template <bool kFp8>
-cudaError_t launch_mode(const CUtensorMap& kmap, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
+cudaError_t launch_mode(const CUtensorMap& kmap, const CUtensorMap& khalf, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
   const int mode = prm.flags & 3;
   const bool guard = !(prm.flags & 4);
-  if (mode == 0) return guard ? launch_variant<0, true, kFp8>(kmap, vmap, qmap, prm, stream) : launch_variant<0, false, kFp8>(kmap, vmap, qmap, prm, stream);
-  if (mode == 1) return guard ? launch_variant<1, true, kFp8>(kmap, vmap, qmap, prm, stream) : launch_variant<1, false, kFp8>(kmap, vmap, qmap, prm, stream);
-  return launch_variant<2, true, kFp8>(kmap, vmap, qmap, prm, stream);
+  if (mode == 0) return guard ? launch_variant<0, true, kFp8>(kmap, khalf, vmap, qmap, prm, stream) : launch_variant<0, false, kFp8>(kmap, khalf, vmap, qmap, prm, stream);
+  if (mode == 1) return guard ? launch_variant<1, true, kFp8>(kmap, khalf, vmap, qmap, prm, stream) : launch_variant<1, false, kFp8>(kmap, khalf, vmap, qmap, prm, stream);
+  return launch_variant<2, true, kFp8>(kmap, khalf, vmap, qmap, prm, stream);
 }
 
 // An E4M3 cache: rows of 576 bytes.
@@ -755,17 +762,17 @@ cudaError_t launch_decode_pair(const DecodeParams& prm, cudaStream_t stream, int
   *unsupported = 0;
   EncodeTiledFn encode = get_encode_fn();
   if (!encode) { *unsupported = 1; return cudaErrorNotSupported; }
-  // K: half a page (32 keys) x one column block; V: a page x two column blocks; Q: a CTA's 64 rows x three column
+  // K: a page or half of one (32 keys) x one column block; V: a page x two column blocks; Q: a CTA's 64 rows x three column
   // blocks (rows past the end of the array read as zero, rows of a following sequence are computed and dropped)
-  CUtensorMap kmap, vmap, qmap;
+  CUtensorMap kmap, khalf, vmap, qmap;
   const cuuint64_t keys = static_cast<cuuint64_t>(prm.num_blocks) * kPage;
   if (!encode_rows(encode, &qmap, prm.q, static_cast<cuuint64_t>(prm.B) * prm.R, kCtaRows, 3)) return cudaErrorInvalidValue;
   if (prm.kv8 != nullptr) {
-    if (!encode_bytes(encode, &kmap, prm.kv8, keys, 32, 64) || !encode_bytes(encode, &vmap, prm.kv8, keys, 64, 128)) return cudaErrorInvalidValue;
-    return launch_mode<true>(kmap, vmap, qmap, prm, stream);
+    if (!encode_bytes(encode, &kmap, prm.kv8, keys, 64, 64) || !encode_bytes(encode, &khalf, prm.kv8, keys, 32, 64) || !encode_bytes(encode, &vmap, prm.kv8, keys, 64, 128)) return cudaErrorInvalidValue;
+    return launch_mode<true>(kmap, khalf, vmap, qmap, prm, stream);
   }
-  if (!encode_rows(encode, &kmap, prm.kv, keys, 32, 1) || !encode_rows(encode, &vmap, prm.kv, keys, 64, 2)) return cudaErrorInvalidValue;
-  return launch_mode<false>(kmap, vmap, qmap, prm, stream);
+  if (!encode_rows(encode, &kmap, prm.kv, keys, 64, 1) || !encode_rows(encode, &khalf, prm.kv, keys, 32, 1) || !encode_rows(encode, &vmap, prm.kv, keys, 64, 2)) return cudaErrorInvalidValue;
+  return launch_mode<false>(kmap, khalf, vmap, qmap, prm, stream);
 }
 
 }  // namespace amla
