@@ -56,13 +56,16 @@ __global__ void plan_kernel(const int32_t* __restrict__ seqlens, int nrb, int n_
 // the last of these blocks has started.  So a warp is kept to few registers, and takes
 //   a row, up to four partials at a time, where there are many rows (more than eight per SM);
 //   a quarter of a row, eight at a time, where there are few rows, and those of many partials;
-//   half or a quarter of a row of FP32 partials (the kernel for few rows).
+//   half or a quarter of a row of FP32 partials (the kernel for few rows);
+//   a quarter of a row and every fourth partial, the block's four warps adding up in shared memory, where a row has sixteen
+//   partials or more on average: one sequence of 20000 keys (74 partials, nine batches one behind the other took 8-14 us)
+//   22.0 -> 18.8 us, with 16 rows 17.7 -> 12.9; of 2531 keys 13.3 -> 12.6; of 6000 17.0 -> 15.1.
 // Against a whole row per warp in 126 registers, eight partials at a time, and a warp for every row that an item has room
 // for (the whole call): one sequence of 2531 keys 14.3 -> 13.2 us, of 60000 39.4 -> 35.1, of 3000 with 16 rows 12.4 -> 9.9;
 // 192 sequences of 1-512 keys 45.4 -> 44.2; 32 of 1-8 K with 16 rows 37.5 -> 36.4; 96 of 2048 73.1 -> 71.7 cool.
 // (One block per SM that walks over the rows and fits beside a decode CTA lets the next call's decode kernel in at once, but
 // takes 10 us where these take 4: 32 x 4096 keys 55.8 -> 61.5.)
-template <bool kFloat, int kCols>
+template <bool kFloat, int kCols, int kSplitWarps>
 __global__ void __launch_bounds__(128, kCols == 16 ? 7 : kCols == 8 ? 8 : 5) combine_kernel(const __grid_constant__ DecodeParams prm) {
   // A decode kernel that follows on the stream may set itself up beside this kernel (it writes nothing this kernel
   // reads before its own wait for this kernel's completion).
@@ -71,20 +74,21 @@ __global__ void __launch_bounds__(128, kCols == 16 ? 7 : kCols == 8 ? 8 : 5) com
   constexpr int kFast = 4, kBatch = kCols == 16 || (kFloat && kCols == 8) ? 4 : 8;
   constexpr int kWords = kFloat ? kCols : kCols / 2;       // 32-bit words of a partial per lane
   const int lane = threadIdx.x & 31;
-  const int unit = blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int sw = kSplitWarps == 1 ? 0 : threadIdx.x >> 5;  // takes the partials sw, sw + kSplitWarps, ...
+  const int unit = kSplitWarps == 1 ? blockIdx.x * 4 + (threadIdx.x >> 5) : blockIdx.x;
   const int row = unit / kUnits, group = row / merge_rows(prm);
   const int rr = row - group * merge_rows(prm);            // row within the item
   const int col = (unit - row * kUnits) * (kDv / kUnits) + lane * kCols;
   asm volatile("griddepcontrol.wait;" ::: "memory");   // launched early (programmatic dependent launch): the partials must be complete
   if (group >= merge_groups(prm)) return;
   const int4 info = prm.merge_info[group];
-  const int nsplit = info.z;
-  if (nsplit < 2) return;
+  if (info.z < 2) return;
+  const int nsplit = (info.z - sw + kSplitWarps - 1) / kSplitWarps;      // of this warp
   const int b = prm.nrb == 1 ? info.x : info.x / prm.nrb;
   const int rin = (info.x - b * prm.nrb) * prm.item_rows + rr;                          // row within the sequence
   if (rin >= prm.R) return;
 
-  auto part_row = [&](int s) { return static_cast<size_t>(Plan::slot_of_split(info.y, s)) * prm.item_rows + rr; };
+  auto part_row = [&](int s) { return static_cast<size_t>(Plan::slot_of_split(info.y, sw + kSplitWarps * s)) * prm.item_rows + rr; };
   struct Piece { uint32_t w[kWords], scale; };
   auto fetch = [&](int s) {
     const size_t prow = part_row(s);
@@ -153,6 +157,27 @@ __global__ void __launch_bounds__(128, kCols == 16 ? 7 : kCols == 8 ? 8 : 5) com
       }
     }
   }
+  if constexpr (kSplitWarps > 1) {
+    static_assert(kCols == 4, "a lane's columns travel as one float4");
+    __shared__ float4 s_acc[kSplitWarps][32];
+    __shared__ float2 s_lse[kSplitWarps];
+    s_acc[sw][lane] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    if (lane == 0) s_lse[sw] = make_float2(mx, tot);
+    __syncthreads();
+    if (sw != 0) return;
+#pragma unroll
+    for (int k = 1; k < kSplitWarps; ++k) mx = fmaxf(mx, s_lse[k].x);
+    acc[0] = acc[1] = acc[2] = acc[3] = tot = 0.f;
+    if (mx != -INFINITY) {
+#pragma unroll
+      for (int k = 0; k < kSplitWarps; ++k) {
+        const float w = expf(s_lse[k].x - mx);
+        const float4 v = s_acc[k][lane];
+        tot += w * s_lse[k].y;
+        acc[0] += w * v.x; acc[1] += w * v.y; acc[2] += w * v.z; acc[3] += w * v.w;
+      }
+    }
+  }
   const float inv = tot > 0.f ? 1.f / tot : 0.f;
   uint32_t pk[kCols / 2];
 #pragma unroll
@@ -180,8 +205,9 @@ cudaError_t launch_combine(const DecodeParams& prm, cudaStream_t stream) {
   const int rows = merge_groups(prm) * merge_rows(prm);
   const bool few = rows <= 8 * prm.sms;
   const int units = rows * (few ? 4 : fp32 ? 2 : 1);
+  const bool many = few && prm.P >= 16 * merge_groups(prm);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((units + 3) / 4);
+  cfg.gridDim = dim3(many ? units : (units + 3) / 4);
   cfg.blockDim = dim3(128);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = stream;
@@ -190,7 +216,9 @@ cudaError_t launch_combine(const DecodeParams& prm, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fp32 ? (few ? combine_kernel<true, 4> : combine_kernel<true, 8>) : few ? combine_kernel<false, 4> : combine_kernel<false, 16>, prm);
+  if (many) return cudaLaunchKernelEx(&cfg, fp32 ? combine_kernel<true, 4, 4> : combine_kernel<false, 4, 4>, prm);
+  if (few) return cudaLaunchKernelEx(&cfg, fp32 ? combine_kernel<true, 4, 1> : combine_kernel<false, 4, 1>, prm);
+  return cudaLaunchKernelEx(&cfg, fp32 ? combine_kernel<true, 8, 1> : combine_kernel<false, 16, 1>, prm);
 }
 
 }  // namespace amla
