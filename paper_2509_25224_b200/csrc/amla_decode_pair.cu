@@ -15,7 +15,7 @@
 // Warps 0-7 run Algorithm 2's recurrence (lines 5-12; four threads share a query row: lane half = half of a tile's keys,
 // warp group = even / odd pages), write P~ = bf16(P * S16) into the P buffer of their own CTA, apply the integer N to
 // the bit patterns of O when the row's reference moved (lines 13-16; Lemma 3.1) and run the epilogue (line 20).  They
-// never hand data to the other CTA.  Warps 8 and 10 load (TMA), warp 9 of the even CTA issues the MMAs for both.
+// never hand data to the other CTA.  Warps 8 and 10-12 load (TMA), warp 9 of the even CTA issues the MMAs for both.
 // Order on the tensor pipe: QK^T(i + 1) before P~V(i), across units too (the paper's [C1, C2, V1] order, Section 4.1).
 //
 // Why this split.  The kernel before it gave one CTA of the pair Q K^T and the other P~ V (M = 128 on one SM each): P~
@@ -41,10 +41,12 @@ using namespace sm100;
 namespace {
 
 constexpr int kSoftmaxWarps = 8;
-// bf16 cache: warps 8 and 10 load.  E4M3 cache: warp 8 loads, warps 10-15 widen, three pairs taking turns.
+// bf16 cache: warps 8 and 10-12 load.  E4M3 cache: warp 8 loads (more warps would leave too few registers), warps 10-15
+// widen, three pairs taking turns.
 constexpr int kWidenGroups = 3, kWidenWarps = 2;
 constexpr int kWideners = kWidenGroups * kWidenWarps;
-template <bool kFp8> constexpr int kThreads = 32 * (kFp8 ? kSoftmaxWarps + 2 + kWideners : kSoftmaxWarps + 3);
+template <bool kFp8> constexpr int kLoaders = kFp8 ? 1 : 4;
+template <bool kFp8> constexpr int kThreads = 32 * (kFp8 ? kSoftmaxWarps + 2 + kWideners : kSoftmaxWarps + 1 + kLoaders<false>);
 constexpr int kTilePages = 4;                           // pages of a score tile: N = 256, the widest MMA
 constexpr int kCtaRows = kRowBlock / 2;                 // query rows per CTA
 constexpr int kQBlocks = kDqk / 64;                     // 64-column blocks of Q and K
@@ -59,7 +61,7 @@ constexpr uint32_t kVBlockBytes = 64 * 128;             // 64 keys x 64 columns
 // for number w (counted over the whole run; slots are released in order) next for one of w + 1 ... w + R, R being the number
 // of slots.  The barriers tell two successive phases apart, no more: a thread that asks for a phase further on is let
 // through by an older one, and one that comes to ask after the next phase has passed as well is held for good.  (So the
-// two loaders take every second of seven slots, and the three pairs that widen step by three through four operand slots,
+// four loaders take every fourth number on a ring of seven slots, and the three pairs that widen step by three through four operand slots,
 // and by three through six raw slots: raw slots fill out of order, and that makes each the business of one pair.)
 template <bool kFp8> constexpr int kSlots = kFp8 ? 4 : 7;
 constexpr int kRawSlots = 2 * kWidenGroups;
@@ -429,22 +431,24 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       tile.next();
     }
     if (!ok && lane == 0) report_timeout(prm.status);
-  } else if (wid == 8 || (!kFp8 && wid == 10)) {
+  } else if (wid == 8 || (!kFp8 && wid >= 10)) {
     // ======================================================== TMA loads, in the order in which the MMAs use them:
     // Q, K(0), K(1), V(0), K(2), V(1), ..., K(n-1), V(n-2), V(n-1), next unit.
-    //   bf16: one ring of 16 KB slots carries K (one 64-column block of the tile's keys, one box per page) and V (one page
-    //     x 128 columns).  The two loader warps walk the same sequence and issue every second load of it.
+    //   bf16: one ring of 16 KB slots carries K (one 64-column block of half the tile's keys) and V (one page x 128 columns).
+    //     The loader warps walk the same sequence and issue every fourth load of it: a slot takes ~350 clk to issue, a warp by
+    //     itself never waits for a slot.  Two -> four loaders: 16 x 16384 keys, rising 85.7 -> 83.3 us cool, 96 x 16384 488 ->
+    //     478, 32 x 4096 50.9 -> 50.2; three or five are no better.
     //   E4M3: the same as raw slots of half the size, all by the first loader.
     // A unit's Q is requested (by the first loader) as soon as the QK^T of the unit before have let go of the buffer, if
     // need be between the V loads of that unit's last tile.
     if (elect_one()) {
-      const uint32_t mine = wid == 8 ? 0u : 1u;
+      const uint32_t mine = wid == 8 ? 0u : wid - 9u;
       constexpr uint32_t kRing = kFp8 ? kRawSlots : kSlots<kFp8>;
       const uint32_t full0 = kFp8 ? bar(X_RAWFULL) : bar(X_FULL), empty0 = kFp8 ? bar(X_RAWEMPTY) : bar(X_EMPTY);
       constexpr uint32_t kBytes = kFp8 ? kRawBytes : kSlotBytes;
       const uint32_t lead_full0 = lead_bars + 8u * X_FULL, ring0 = smem_base + (kFp8 ? kOffRaw : kOffRing);
       const uint64_t keep = l2_policy_evict_normal(), last_use = l2_policy_evict_first();   // K: V follows a tile later; V: done with
-      uint32_t slot = 0, par = 1, n_issued = 0;
+      uint32_t slot = 0, par = 1, n_issued = 0, turn = 0;
       uint32_t un = 0;                                      // units whose Q has been requested
       auto take = [&]() -> TileRef {
         TileRef x;
@@ -461,8 +465,8 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       };
       // first key row of a page; E4M3: a page outside the cache reads as zeros (rows behind the end of the tensor do)
       auto row_of = [&](int page) { return (kFp8 && (page < 0 || page >= prm.num_blocks) ? prm.num_blocks : page) * kPage; };
-      auto advance = [&]() { if (++slot == kRing) { slot = 0; par ^= 1; } ++n_issued; };
-      auto my_turn = [&]() { return kFp8 || (n_issued & 1) == mine; };
+      auto advance = [&]() { if (++slot == kRing) { slot = 0; par ^= 1; } ++n_issued; if (++turn == kLoaders<kFp8>) turn = 0; };
+      auto my_turn = [&]() { return kLoaders<kFp8> == 1 || turn == mine; };
       auto issue_q = [&](int qrow) {
         if (leader) mbar_arrive_expect_tx(bar(X_QFULL), 2 * kQBytes);
 #pragma unroll 1
@@ -470,16 +474,15 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           tma_load_3d_pair_hint(smem_base + kOffQ + c * kQBlockBytes, &q_map, 0, qrow, c, lead_bars + 8u * X_QFULL, last_use);
         ++un;
       };
-      auto issue_v = [&](const TileRef& x, int nxt_qrow, bool q_wanted, bool& q_out) {
-        int page = __ldg(x.bt);
+      struct Pages { int a, b, c, d; };                    // of a tile
+      auto issue_v = [&](int np, Pages pg, int nxt_qrow, bool q_wanted, bool& q_out) {
 #pragma unroll 1
-        for (int i = 0; i < 2 * x.np; ++i) {
-          const int row = row_of(page);
-          const int nh = i & 1, p_next = min((i + 1) >> 1, x.np - 1);
-          page = __ldg(x.bt + p_next);
+        for (int i = 0; i < 2 * np; ++i) {
+          const int nh = i & 1;
           if (my_turn()) {
             if (q_wanted && !q_out && mbar_probe(bar(X_QFREE), (un - 1) & 1)) { issue_q(nxt_qrow); q_out = true; }
             const uint32_t dst = ring0 + slot * kBytes;
+            const int row = row_of(pg.a);
             ok = mbar_wait(empty0 + 8 * slot, par);
             if (!ok) return;
             if (kFp8) {
@@ -490,20 +493,27 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
               tma_load_3d_pair_hint(dst, &v_map, 0, row, 4 * rank + 2 * nh, lead_full0 + 8 * slot, last_use);
             }
           }
+          if (nh) { pg.a = pg.b; pg.b = pg.c; pg.c = pg.d; }
           advance();
         }
       };
       // This CTA's half of the tile's keys, 32 np of them from key 32 np rank on, is at most two boxes: a page, or the half page
       // in the middle of a tile of three pages or of one.  (With 32 keys of every page it was four boxes: E4M3, one loader:
       // 62.6 -> 61.2 us for 32 x 4096 keys, 120.1 -> 116.4 for 32 x 512-8192, two tokens; bf16 494 -> 481 for 96 x 16384.)
-      int page[2];
+      // The page numbers of a tile are loaded once, a tile ahead, and kept for its V: a load of the block table in front of
+      // every V slot cost the loaders 500 clk there: a tile of the E4M3 cache took 11.9 K clk instead of 10.4 K.
+      static_assert(kTilePages == 4, "a tile's page numbers");
       auto get_pages = [&](const TileRef& x) {
-        const int p0 = (x.np * rank) >> 1;
-        page[0] = x.np > 0 ? __ldg(x.bt + p0) : 0;
-        page[1] = p0 + 1 < x.np ? __ldg(x.bt + p0 + 1) : 0;
+        Pages pg;
+        pg.a = x.np > 0 ? __ldg(x.bt) : 0;
+        pg.b = x.np > 1 ? __ldg(x.bt + 1) : 0;
+        pg.c = x.np > 2 ? __ldg(x.bt + 2) : 0;
+        pg.d = x.np > 3 ? __ldg(x.bt + 3) : 0;
+        return pg;
       };
-      TileRef cur = take(), prev = cur;
-      get_pages(cur);                                       // on its way while Q is requested
+      TileRef cur = take();
+      Pages pg = get_pages(cur), pg_prev = {};              // on its way while Q is requested
+      int np_prev = 0;
       TileRef nxt = take();
       bool q_out = false;                                   // the Q of the unit that starts next has been requested
       uint32_t pt = 0;
@@ -518,10 +528,11 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         }
         const bool odd = (cur.np * rank) & 1;                               // begins in the middle of a page
         const int chunks0 = odd || cur.np == 1 ? 1 : 2, chunks1 = min(cur.np - chunks0, 2);
-        const int row0 = row_of(page[0]) + (odd ? 32 : 0), row1 = row_of(page[1]);
+        const int row0 = row_of(rank == 0 || cur.np == 1 ? pg.a : cur.np == 4 ? pg.c : pg.b) + (odd ? 32 : 0);
+        const int row1 = row_of(rank == 0 ? pg.b : cur.np == 4 ? pg.d : pg.c);
         const CUtensorMap* const map0 = chunks0 == 2 ? &k_map : &khalf_map;
         const CUtensorMap* const map1 = chunks1 == 2 ? &k_map : &khalf_map;
-        get_pages(nxt);
+        const Pages pg_nxt = get_pages(nxt);
 #pragma unroll 1
         for (int c = 0; c < kQBlocks; ++c) {
           if (my_turn()) {
@@ -545,8 +556,10 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         const TileRef nn = take();
         // V of the tile before, and behind a unit's last K its own V
         for (int k = cur.first ? 1 : 0; k < (cur.last ? 2 : 1) && ok; ++k)
-          issue_v(k == 0 ? prev : cur, nxt.qrow, k == 1 && mine == 0 && nxt.valid, q_out);
-        prev = cur;
+          issue_v(k == 0 ? np_prev : cur.np, k == 0 ? pg_prev : pg, nxt.qrow, k == 1 && mine == 0 && nxt.valid, q_out);
+        np_prev = cur.np;
+        pg_prev = pg;
+        pg = pg_nxt;
         cur = nxt;
         nxt = nn;
         ++pt;
@@ -556,7 +569,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         // let the copies that may still be in flight land before the CTA exits
         for (uint32_t i = 0; i < kRing && i < n_issued; ++i) {
           const uint32_t k = n_issued - 1 - i;
-          if (kFp8 || (leader && (k & 1) == mine)) mbar_wait(full0 + 8 * (k % kRing), (k / kRing) & 1);
+          if (kFp8 || (leader && k % kLoaders<kFp8> == mine)) mbar_wait(full0 + 8 * (k % kRing), (k / kRing) & 1);
         }
         if (leader && un > 0) mbar_wait(bar(X_QFULL), (un - 1) & 1);
       }
