@@ -385,7 +385,7 @@ def run_gpu(args):
 
 
 def fp8_entry(w, dev, local, steps, barrier, peaks, peak_kind, kv_scale=1.0 / 64.0):
-    """The same workload with an E4M3 cache (amla_mla_decode_fp8: widen the used pages, then the bf16 kernels): whole
+    """The same workload with an E4M3 cache (amla_mla_decode_fp8: the decode kernel widens the bytes on chip): whole
     call, CUDA events; its algorithmic bytes count one byte per cache element."""
     import torch
     from paper_2509_25224_b200 import binding
@@ -416,7 +416,7 @@ def fp8_entry(w, dev, local, steps, barrier, peaks, peak_kind, kv_scale=1.0 / 64
     bound = "hbm" if t_b >= t_f else "tensor"
     frac = max(t_b, t_f) / (ms * 1e-3)
     return {"ms_per_step": ms, "median_step_ms": statistics.median(per), "tflops": flops / (ms * 1e-3) / 1e12, "bound": bound,
-            "frac": frac, "frac_of": "whole call (widen + decode + combine) against the " + peak_kind + " peak", "steps": steps,
+            "frac": frac, "frac_of": "whole call (decode + combine) against the " + peak_kind + " peak", "steps": steps,
             "algorithmic_bytes": alg_bytes, "launches_per_step": binding.last_launch_count(),
             "workload": workload_name(w).replace("bf16 paged-64", "bf16 q, E4M3 cache (scale 1/64) paged-64")}
 

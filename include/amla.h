@@ -96,9 +96,9 @@ int amla_mla_decode_workspace_size(int B, int Sq, int H, int max_blocks_per_seq,
  *                need not be preserved or initialised; calls that overlap in time need distinct ones
  *   cuda_stream  a cudaStream_t (NULL = default stream)
  *
- * Supported: 1 <= Sq <= 8, 1 <= H <= 128 (any Sq*H up to 1024 query rows per sequence; up to 128 rows are
- * processed as one block by a pair of SMs, more than 128 rows in blocks of 256 by four SMs that share every
- * cache tile they load); page size 64; sm_100 devices only (AMLA_ERR_UNSUPPORTED otherwise).
+ * Supported: 1 <= Sq <= 8, 1 <= H <= 128 (any Sq*H up to 1024 query rows per sequence; up to 32 rows are
+ * processed by one SM, up to 128 as one block by a pair of SMs, more than 128 rows in blocks of 256 by four SMs
+ * that share every cache tile they load, or, where that is faster, of 128); page size 64; sm_100 devices only (AMLA_ERR_UNSUPPORTED otherwise).
  * Argument errors are reported before anything is launched.
  */
 int amla_mla_decode(const void* q, const void* kv_cache, const int32_t* block_table,
@@ -156,11 +156,12 @@ int amla_mla_decode_ex(const void* q, const void* kv_cache, const int32_t* block
  *   workspace      at least amla_mla_decode_fp8_workspace_size() bytes, 256-byte aligned
  *   flags          as for amla_mla_decode_ex
  *
- * Two passes: the pages the batch uses are first widened, exactly, into a bf16 copy inside the workspace
- * (B * max_blocks_per_seq pages of 73 728 bytes), kv_scale is folded into the softmax scale and into the final
- * normalisation, and the bf16 kernels run on the copy.  The FP8 cache saves device memory, not traffic: a call reads
- * the FP8 pages and writes and reads their copy.  Everything else (visibility rule, outputs, errors) is as for
- * amla_mla_decode.  A block-table entry outside [0, num_blocks) of a used page reads as a page of zeros.
+ * The pages are widened, exactly, on their way into the tensor cores' operand tiles; kv_scale is folded into the
+ * softmax scale and into the final normalisation.  A call reads half the bytes of a bf16 cache.  (Only with
+ * AMLA_FLAG_KERNEL_SIMT are the used pages first widened into a bf16 copy inside the workspace: B *
+ * max_blocks_per_seq pages of 73 728 bytes, which the workspace has room for.)  Everything else (visibility rule,
+ * outputs, errors) is as for amla_mla_decode.  A block-table entry outside [0, num_blocks) of a used page reads as
+ * a page of zeros.
  */
 int amla_mla_decode_fp8_workspace_size(int B, int Sq, int H, int max_blocks_per_seq, int device, size_t* bytes_out);
 int amla_mla_decode_fp8(const void* q, const void* kv_cache_e4m3, float kv_scale, const int32_t* block_table,
@@ -210,10 +211,12 @@ int amla_profile_last_ms(float* ms3);
 /*
  * Host mirror of the device-side split-KV schedule (the plan is not in the paper; it exists because
  * B * ceil(Sq*H/128) work items are far fewer than the SMs).  For Sq*H <= 128 the items are (sequence, 128-row
- * block) pairs, their tiles 64-key pages, and every non-empty item but the first is preceded by 10 overhead
+ * block) pairs, their tiles 64-key pages, and every non-empty item but the first is preceded by 6 overhead
  * positions that stand for the cost of starting an item; for Sq*H > 128 the items are (sequence, 256-row block)
  * pairs, the tiles 128 keys (two pages) and the overhead 5 positions.  Items in order form one linear range
- * that is cut into num_parts equal parts.
+ * that is cut into parts of ceil(length / num_parts) positions.  (On the device a part also holds at least 128 keys
+ * unless tau is 0, sequences of up to 32 rows have a schedule of their own, with 32-row items and 3 overhead
+ * positions, and short sequences of more than 128 rows may run as 128-row items.)
  * For every (part, item) intersection ("unit") one record of 6 int32 is written:
  *   part, item, tile_begin, tile_end (within the item), slot (-1 = writes out/lse directly,
  *   otherwise index of its fp32 partial), n_split of the item.

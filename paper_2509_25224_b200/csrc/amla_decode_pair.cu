@@ -21,11 +21,12 @@
 // Why this split.  The kernel before it gave one CTA of the pair Q K^T and the other P~ V (M = 128 on one SM each): P~
 // crossed to the other SM by remote stores, Q went through shared memory into tensor memory and the score CTA had to be
 // drained before the next unit's Q could follow.  Here nothing but MMA operands crosses, Q is an operand as it lands, and
-// the tile is 256 keys.  192 sequences of 1-512 keys: 62.0 -> 50.0 us; one sequence of 2531: 34.3 -> 31.7; 16 x 16384 with
-// rising logits: 103.8 -> 101.5; 96 x 2048: 88.4 -> 85.5; 32 x 4096: 58.4 both (sustained, at the power cap).
-// What bounds it: a tile of 256 keys takes 8200-8700 clk against 4350 of MMAs and 6000 of HBM at its full rate.  A CTA
-// takes 275 KB per tile through a ring of 112 KB, whose slots turn around in ~2700 clk (load 1500-2000, MMA, commit,
-// next load).  With the MMAs left out the tile still takes 7400.
+// the tile is 256 keys.  Calls with it, from that kernel to this one as it stands (sustained): 192 sequences of 1-512 keys
+// 62.8 -> 43.9 us; one of 2531 33.8 -> 12.2; 16 x 16384 with rising logits 105.2 -> 93.0; 96 x 2048 88.4 -> 80.2; 32 x 4096
+// 59.3 -> 55.1; E4M3 32 x 4096 101.0 -> 61.8.
+// What bounds it: a tile of 256 keys takes ~7500 clk (E4M3 10.4 K) against 4350 of MMAs and 5900 of HBM at its full rate: a
+// CTA takes 278 KB per tile through a ring of 112 KB, whose slots turn around in ~2700 clk (load 1500-2000, MMA, commit,
+// next load), and every slot has to be issued.  Long calls run at the power limit: 32 x 4096 takes 50.2 us cool.
 //
 // All waits are bounded; on expiry the kernel records kStatusTimeout and unwinds.
 #include "amla_common.cuh"
