@@ -228,6 +228,8 @@ def _on_device(dev, call, args, tail, what):
     if _raw_stream is None:
         import torch
         _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
+    if dev.type != "cuda":
+        raise ValueError("the decode entries take CUDA tensors, not tensors on " + str(dev))
     index = dev.index
     now = _current_device()
     if index is None:
