@@ -227,7 +227,8 @@ def _on_device(dev, call, args, tail, what):
     global _raw_stream, _current_device
     if _raw_stream is None:
         import torch
-        _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
+        _current_device = torch.cuda.current_device
+        _raw_stream = torch._C._cuda_getCurrentRawStream     # last: it is what another thread's call looks for
     if dev.type != "cuda":
         raise ValueError("the decode entries take CUDA tensors, not tensors on " + str(dev))
     index = dev.index

@@ -1,4 +1,7 @@
 """CPU-side checks of the binding's argument marshalling: what it refuses, and what it hands to the library."""
+import sys
+import threading
+
 import pytest
 import torch
 
@@ -48,3 +51,45 @@ def test_host_tensors_never_reach_a_kernel(fake):
     with pytest.raises(ValueError):
         binding.mla_decode_fp8(q, kv, 1.0, bt, sl, 0.1, out, lse, torch.empty(1 << 20, dtype=torch.uint8))
     assert fake.calls == []
+
+
+def test_a_second_thread_may_come_in_anywhere_in_the_first_call(fake):
+    # whatever the first call keeps for later ones has to be complete whenever another thread can see it: the first call is
+    # held at each of its steps in turn while a second one runs
+    dev = torch.device("cuda", 0)
+
+    def held_at(step):
+        binding._raw_stream = binding._current_device = None
+        count, errors = [0], []
+
+        def second():
+            try:
+                binding._on_device(dev, fake.anything, (), (), "second")
+            except Exception as e:
+                errors.append(e)
+
+        def tracer(frame, event, arg):
+            if frame.f_code is not binding._on_device.__code__:
+                return None
+            frame.f_trace_opcodes = True
+            if event == "opcode":
+                if count[0] == step:
+                    t = threading.Thread(target=second)
+                    t.start()
+                    t.join()
+                count[0] += 1
+            return tracer
+
+        before = sys.gettrace()
+        sys.settrace(tracer)
+        try:
+            binding._on_device(dev, fake.anything, (), (), "first")
+        finally:
+            sys.settrace(before)
+        assert not errors, (step, errors)
+        return count[0]
+
+    steps = held_at(-1)
+    assert steps > 20
+    for step in range(steps):
+        held_at(step)
