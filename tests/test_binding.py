@@ -81,6 +81,7 @@ def test_a_second_thread_may_come_in_anywhere_in_the_first_call(fake):
             return tracer
 
         before = sys.gettrace()
+        sys._getframe().f_trace_opcodes = True          # Python 3.12: opcode events are on from settrace() if a frame wants them
         sys.settrace(tracer)
         try:
             binding._on_device(dev, fake.anything, (), (), "first")
