@@ -134,13 +134,14 @@ int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
   prm.P = simt || few ? sms : quad ? quad_parts : decode_pair_parts(sms);
   // No more parts than the longest schedule that the block table's width allows can fill.  A schedule of one score tile at
   // most is one part: nothing is split and no combine kernel runs.
+  const long long tiles = (static_cast<long long>(prm.max_blocks_per_seq) * kPage + prm.tile_keys - 1) / prm.tile_keys;
+  const long long longest = prm.n_items * tiles + (prm.n_items - 1ll) * prm.ovh;
   if (!simt) {
-    const long long tiles = (static_cast<long long>(prm.max_blocks_per_seq) * kPage + prm.tile_keys - 1) / prm.tile_keys;
-    const long long longest = prm.n_items * tiles + (prm.n_items - 1ll) * prm.ovh;
     if (longest * prm.tile_keys <= 256) prm.P = 1;
     else prm.P = static_cast<int>(std::min<long long>(prm.P, (longest + prm.min_share - 1) / prm.min_share));
   }
-  prm.fused_plan = (!simt && prm.n_items <= kFusedPlanMaxItems) ? 1 : 0;
+  // (a plan made in the decode kernel may begin as a guess: any lengths that the table has room for must add up)
+  prm.fused_plan = (!simt && prm.n_items <= kFusedPlanMaxItems && longest <= 0x7fffffff) ? 1 : 0;
   return AMLA_OK;
 }
 

@@ -90,9 +90,9 @@ decode_few_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_const
   auto bar = [&](int i) { return bars + 8u * i; };
   const uint32_t tmem_slot = bars + kBarBytes - 8;
 
-  // Set-up, three things side by side: the load warp, which needs the result first, works out the schedule (from the
-  // sequence lengths: inputs of the call, which no kernel that this one may overlap with writes), the MMA warp allocates
-  // tensor memory, one thread of a softmax warp initialises the barriers.
+  // Set-up, three things side by side: the load warp works out the schedule from the sequence lengths as they are found
+  // (held against the final ones after the wait below), the MMA warp allocates tensor memory, one thread of a softmax warp
+  // initialises the barriers.
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = reinterpret_cast<int*>(smem_raw + kOffSeqlens);
@@ -135,6 +135,13 @@ decode_few_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_const
     // was still going; its results (the previous call's reads of the workspace among them) are complete after this wait.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
+    if (wid == kLoadWarp && lane == 0 && tile.valid) prefetch_pages(prm, tile.u.b, tile.t);
+    if (plan_is_stale(prm, plan_smem, lens_smem, tid, kThreads)) {
+      if (wid == kLoadWarp) plan_on_chip(prm, plan_smem, lens_smem, lane);
+      __syncthreads();
+      tile.units.start();
+      tile.begin();
+    }
     if (blockIdx.x == 0 && wid == 0) {       // the prefix in the workspace is part of what a call leaves behind
       for (int it = lane; it <= prm.n_items; it += 32) const_cast<int*>(prm.prefix)[it] = plan_smem[it];
       if (lane == 0) *prm.status = kStatusOk;

@@ -137,9 +137,9 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   const uint32_t tmem_slot = bars + kBarBytes - 8;
   const uint32_t lead_bars = map_to_cta(bars, 0);
 
-  // Set-up, three things side by side: warp 8, which will need the result first, works out the schedule of a batch of up to
-  // kSmemPlanItems items (from the sequence lengths: inputs of the call, which no kernel that this one may overlap with
-  // writes), warp 9 allocates tensor memory, one thread of warp 10 initialises the barriers.
+  // Set-up, three things side by side: warp 8 works out the schedule of a batch of up to kSmemPlanItems items from the
+  // sequence lengths as they are found (held against the final ones after the wait below), warp 9 allocates tensor memory,
+  // one thread of warp 10 initialises the barriers.
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = reinterpret_cast<int*>(smem_raw + kOffSeqlens);
@@ -199,6 +199,13 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     // was still going; its results (the previous call's reads of the workspace among them) are complete after this wait.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
+    if (wid == 8 && lane == 0 && tile.valid) prefetch_pages(prm, tile.u.b, tile.t);
+    if (plan_is_stale(prm, plan_smem, lens_smem, tid, kThreads<kFp8>)) {     // (both CTAs see the same lengths)
+      if (wid == 8) plan_on_chip(prm, plan_smem, lens_smem, lane);
+      __syncthreads();
+      tile.units.start();
+      tile.begin();
+    }
     if (blockIdx.x == 0 && wid == 0) {       // the combine kernel reads the prefix in the workspace
       for (int it = lane; it <= prm.n_items; it += 32) const_cast<int*>(prm.prefix)[it] = plan_smem[it];
       if (lane == 0) *prm.status = kStatusOk;

@@ -417,8 +417,8 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   const uint32_t myV_base = map_to_cta(smem_base, 2 + half);           // score CTA j -> value CTA j
   const uint32_t myV_bars = map_to_cta(bars, 2 + half);
 
-  // Warp 6 works out the schedule of a batch of up to kSmemPlanItems items during the set-up (from the sequence lengths: inputs
-  // of the call, which no kernel that this one may overlap with writes).
+  // Warp 6 works out the schedule of a batch of up to kSmemPlanItems items during the set-up, from the sequence lengths as they
+  // are found (held against the final ones after the wait below).
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = prm.n_items <= kSmemLens ? reinterpret_cast<int*>(smem_raw + kOffSeqlens) : nullptr;
@@ -471,12 +471,19 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   }
   UnitIter first(prm, prefix, seqlens, part);
   Unit fu;
-  const bool any = first.next(fu);
+  bool any = first.next(fu);
   if (plan_here) {
     // Launched with programmatic stream serialization: everything above ran while the kernel before this one on the stream
     // was still going; its results (the previous call's reads of the workspace among them) are complete after this wait.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
+    if (wid == 4 && lane == 0 && any) prefetch_pages(prm, fu.b, fu.t0 * (kTileKeys / kPage));
+    if (plan_is_stale(prm, plan_smem, lens_smem, tid, kThreads)) {           // (all four CTAs see the same lengths)
+      if (wid == 6) plan_on_chip(prm, plan_smem, lens_smem, lane);
+      __syncthreads();
+      first.start();
+      any = first.next(fu);
+    }
     if (blockIdx.x == 0 && wid == 6) {       // the prefix in the workspace is part of what a call leaves behind
       for (int it = lane; it <= prm.n_items; it += 32) const_cast<int*>(prm.prefix)[it] = plan_smem[it];
       if (lane == 0) *prm.status = kStatusOk;

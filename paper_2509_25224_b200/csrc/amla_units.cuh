@@ -14,14 +14,30 @@ __device__ __forceinline__ int warp_inclusive_scan(int v, int lane) {
   return v;
 }
 
+// A sequence length as it stands in device memory (or the GPU's common cache) at this moment; the SM's own cache neither
+// answers nor keeps it.
+__device__ __forceinline__ int load_length(const DecodeParams& prm, int b) {
+  int n;
+  asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(n) : "l"(prm.seqlens + b) : "memory");
+  return min(max(n, 0), prm.max_blocks_per_seq * kPage);
+}
+
 // The schedule prefix of the batch, by one warp: into shared memory together with the sequence lengths (unless lens is null),
 // or into the workspace.
+//
+// plan_on_chip also runs ahead of griddepcontrol.wait, when a kernel in front that produces the lengths may not have written
+// them yet, or not so that this kernel sees it.  What it finds there is a guess, whatever it is: lengths are clamped to the
+// table's width, for which the schedule's positions fit their type (the launch sees to that).  After the wait
+// plan_is_stale() holds the guess against the lengths as they are; where they differ the plan is made again.
+// (The guess is right unless the kernel directly in front writes the lengths.  One sequence of 256 keys with 16 heads: planned
+// wholly behind the wait 8.5 us, guessed and checked 7.7, guessed and not checked 7.2; 32 x 4096 keys 51.7, 50.9 and 50.4,
+// calls replayed back to back.)
 __device__ __forceinline__ void plan_on_chip(const DecodeParams& prm, int* prefix, int* lens, int lane) {
   int carry = 0;
   for (int base = 0; base < prm.n_items; base += 32) {
     const int it = base + lane;
     const int b = prm.nrb == 1 ? it : it / prm.nrb;
-    const int n_seq = it < prm.n_items ? prm.seqlens[b] : 0;
+    const int n_seq = it < prm.n_items ? load_length(prm, b) : 0;
     const int v = it < prm.n_items ? schedule_length(n_seq, it, prm.tile_keys, prm.ovh) : 0;
     const int x = warp_inclusive_scan(v, lane);
     if (it < prm.n_items) {
@@ -31,6 +47,20 @@ __device__ __forceinline__ void plan_on_chip(const DecodeParams& prm, int* prefi
     carry += __shfl_sync(0xffffffffu, x, 31);
   }
   if (lane == 0) prefix[prm.n_items] = carry;
+}
+// Page numbers of the first unit, on their way while the lengths are (the guess's place in the table is inside the table).
+__device__ __forceinline__ void prefetch_pages(const DecodeParams& prm, int b, int page) {
+  asm volatile("{\n\t.reg .b32 x;\n\tld.global.b32 x, [%0];\n\t}" ::"l"(prm.block_table + static_cast<size_t>(b) * prm.max_blocks_per_seq + page));
+}
+// By all threads of the CTA, after griddepcontrol.wait: does the plan differ from what the lengths give?
+__device__ __forceinline__ bool plan_is_stale(const DecodeParams& prm, const int* prefix, const int* lens, int tid, int threads) {
+  bool stale = false;
+  for (int it = tid; it < prm.n_items; it += threads) {
+    const int b = prm.nrb == 1 ? it : it / prm.nrb;
+    const int n_seq = load_length(prm, b);
+    stale |= lens ? lens[b] != n_seq : prefix[it + 1] - prefix[it] != schedule_length(n_seq, it, prm.tile_keys, prm.ovh);
+  }
+  return __syncthreads_or(stale);
 }
 __device__ __forceinline__ void plan_in_workspace(const DecodeParams& prm, int lane) {
   int* pw = const_cast<int*>(prm.prefix);
@@ -87,6 +117,9 @@ struct UnitIter {
   const int* seqlens;
   int p, g, g1, share, parts;
   __device__ UnitIter(const DecodeParams& prm_, const int* prefix_, const int* seqlens_, int part) : prm(prm_), prefix(prefix_), seqlens(seqlens_), p(part) {
+    start();
+  }
+  __device__ void start() {
     const Plan plan = Plan::make(prefix, prm.n_items, prm.P, prm.ovh, prm.min_share);
     share = plan.share; parts = plan.P;
     if (plan.L <= 0 || p >= plan.P) { g = g1 = 0; }
