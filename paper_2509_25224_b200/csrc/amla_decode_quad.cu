@@ -375,6 +375,7 @@ __device__ __forceinline__ bool relay_phases(uint32_t bars, uint32_t lead_bars, 
     bool progress = false;
     if (k < phases && mbar_probe(lb, k & 1)) {
       if (kProxyFence) fence_proxy_async_smem();
+      release_shared_to_cluster();           // Q's RoPE columns, P~: what the phase stands for is in this CTA's shared memory
       mbar_arrive_cluster_relaxed(rb);
       ++k;
       progress = true;
@@ -909,7 +910,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
             ok = mbar_wait<true>(bar(B_PFULL + s), k & 1);
             if (!ok) break;
             QSTAMP(smem_base, 10, gt);
-            ok = mbar_wait(bar(B_OREADY + s), k & 1);
+            ok = mbar_wait<true>(bar(B_OREADY + s), k & 1);
             if (!ok) break;
             QSTAMP(smem_base, 11, gt);
             tc_fence_after_sync();

@@ -266,6 +266,31 @@ def test_rerun_is_bit_identical():
     assert torch.equal(o1.view(torch.int16), o2.view(torch.int16)) and torch.equal(l1, l2)
 
 
+@pytest.mark.parametrize("fp8", [False, True])
+def test_reruns_of_both_ctas_rows_are_bit_identical(fp8):
+    # the MMAs of a cluster read what the warps of its odd CTA have written (P~, widened keys and values) on the word of
+    # arrivals that cross to the even CTA: rising logits, so that O is rewritten too, and many units per cluster
+    import torch
+    w = synth.config_stress(B=20, N=1500)
+    q, kv, bt, sl = to_device(w)
+    if fp8:
+        kv = torch.from_numpy(synth.quantise_cache_e4m3(w, 1.0 / 8.0)).to(q.device)
+        ro, rl = R.decode_fp8(w.q, kv.cpu().numpy(), 1.0 / 8.0, w.block_table, w.seqlens, w.scale)
+    else:
+        ro, rl = R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)
+    runs = []
+    for _ in range(12):
+        if fp8:
+            runs.append(binding.mla_decode_fp8(q, kv, 1.0 / 8.0, bt, sl, w.scale))
+        else:
+            runs.append(binding.mla_decode(q, kv, bt, sl, w.scale))
+    torch.cuda.synchronize()
+    for o, l in runs[1:]:
+        assert torch.equal(o.view(torch.int16), runs[0][0].view(torch.int16)) and torch.equal(l, runs[0][1])
+    from tests._gpu_util import compare
+    compare(runs[0][0].float().cpu().numpy().astype(np.float64), runs[0][1].cpu().numpy().astype(np.float64), ro, rl, f"rerun fp8={fp8}")
+
+
 def test_matches_algorithm2_simulator_closely(capsys):
     # The CPU Algorithm-2 simulator uses the same readings; agreement should be far tighter than the oracle tolerance
     # (both round P to bf16 and accumulate in fp32).  The sequence is split over many SM groups here, and the partial
