@@ -156,9 +156,9 @@ int amla_mla_decode_ex(const void* q, const void* kv_cache, const int32_t* block
  *   flags          as for amla_mla_decode_ex
  *
  * The pages are widened, exactly, on their way into the tensor cores' operand tiles; kv_scale is folded into the
- * softmax scale and into the final normalisation.  A call reads half the bytes of a bf16 cache.  (Only with
- * AMLA_FLAG_KERNEL_SIMT are the used pages first widened into a bf16 copy inside the workspace: B *
- * max_blocks_per_seq pages of 73 728 bytes, which the workspace has room for.)  Everything else (visibility rule,
+ * softmax scale and into the final normalisation.  A call reads half the bytes of a bf16 cache.  (Large calls of more
+ * than 640 query rows per sequence, and AMLA_FLAG_KERNEL_SIMT, widen the used pages into a bf16 copy inside the
+ * workspace first: B * max_blocks_per_seq pages of 73 728 bytes.)  Everything else (visibility rule,
  * outputs, errors) is as for amla_mla_decode.  A block-table entry outside [0, num_blocks) of a used page reads as
  * a page of zeros.
  */

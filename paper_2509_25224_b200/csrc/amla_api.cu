@@ -267,6 +267,20 @@ int decode_impl(const void* q, const void* kv_cache, const uint8_t* kv8, const i
   return launch_decode_call(prm, prefix, static_cast<cudaStream_t>(cuda_stream), &g_last_launches, profile_mark);
 }
 
+// Are the pages of an E4M3 cache widened into a bf16 copy first, and the bf16 kernels run on that, or does the 128-row kernel
+// widen them on their way in?  On their way in they are widened once more for every 128 query rows, and for K and for V; the
+// copy costs its writing and reading once, and more than 128 rows then are blocks of 256.  Measured (on the way in / copy
+// first, 128 heads): eight tokens 32 x 4096 keys 381 / 326 us, 16 x 16384 734 / 599, 1 x 65536 183 / 150; six tokens 289 / 259,
+// 566 / 488; but five and less differ by little or the other way (1 x 4096 20.6 / 21.0, two tokens 32 x 4096 98 / 130), and so
+// do small calls (1 x 100, six tokens 12.1 / 13.6; 20 x 375-3000 79.7 / 81.0).  Lengths are not known here: the table's width
+// stands for them, unless the cache could not fill half of such a table (100 sequences of 300 keys, six tokens, a table of
+// 512 pages: 141 / 184).  (The scalar bring-up kernel reads bf16 only.)
+bool widen_first(int B, int rows, int num_blocks, int max_blocks_per_seq, int flags) {
+  if (flags & AMLA_FLAG_KERNEL_SIMT) return true;
+  const long long row_blocks = (rows + kRowBlock - 1) / kRowBlock, slots = static_cast<long long>(B) * max_blocks_per_seq;
+  return !(flags & AMLA_FLAG_KERNEL_ROWS128) && row_blocks > 5 && row_blocks * slots >= 8192 && slots <= 2ll * num_blocks;
+}
+
 // Bytes of the FP8 path's extra scratch behind the ordinary workspace: the new block table and the widened pages.
 size_t fp8_table_bytes(int B, int max_blocks_per_seq) { return align_up(sizeof(int32_t) * static_cast<size_t>(B) * max_blocks_per_seq); }
 size_t fp8_pages_bytes(int B, int max_blocks_per_seq) { return static_cast<size_t>(B) * max_blocks_per_seq * kPage * kDqk * sizeof(__nv_bfloat16); }
@@ -311,10 +325,9 @@ extern "C" int amla_mla_decode_fp8(const void* q, const void* kv_cache_e4m3, flo
   if (workspace_bytes < base + tbytes + pbytes) return AMLA_ERR_WORKSPACE;
   if (static_cast<long long>(B) * max_blocks_per_seq > (1ll << 30)) return AMLA_ERR_UNSUPPORTED;
   // logits: scale * q . (k8 * kv_scale); output: sum p * (v8 * kv_scale)
-  if (!(flags & AMLA_FLAG_KERNEL_SIMT))
+  if (!widen_first(B, Sq * H, num_blocks, max_blocks_per_seq, flags))
     return decode_impl(q, nullptr, static_cast<const uint8_t*>(kv_cache_e4m3), block_table, seqlens, softmax_scale * kv_scale, kv_scale, B, Sq, H,
                        num_blocks, max_blocks_per_seq, out, lse, workspace, base, cuda_stream, flags);
-  // the scalar bring-up kernel reads bf16: the pages are widened first
   char* ws = static_cast<char*>(workspace);
   int32_t* table2 = reinterpret_cast<int32_t*>(ws + base);
   __nv_bfloat16* pages = reinterpret_cast<__nv_bfloat16*>(ws + base + tbytes);

@@ -1,12 +1,12 @@
-// FP8 (E4M3) latent cache: widening of the pages a batch uses into a bf16 scratch cache, ahead of the scalar bring-up kernel
-// (the 128-row kernel reads the bytes itself).
+// FP8 (E4M3) latent cache: widening of the pages a batch uses into a bf16 scratch cache, ahead of the bf16 kernels, for large
+// calls of many query rows and for the scalar bring-up kernel (the 128-row kernel reads the bytes itself).
 //
 // The paper's remark after Lemma 3.1 notes that the exponent-add applies to other floating-point formats; what it
 // acts on here stays the FP32 accumulator.  An FP8 cache changes the inputs only: every cache byte is an OCP E4M3
 // number (1 sign, 4 exponent bits with bias 7, 3 mantissa bits, no infinities, S.1111.111 = NaN) and the stored
 // value is byte_value * kv_scale.  E4M3 values are exactly representable in bf16, so the pages are widened without
 // rounding, the per-tensor scale is folded into the softmax scale (for the logits) and into the final
-// normalisation (for V), and the scalar kernel runs unchanged on the widened copy.
+// normalisation (for V), and the bf16 kernels run unchanged on the widened copy.
 #include "amla_common.cuh"
 
 namespace amla {

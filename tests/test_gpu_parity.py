@@ -105,6 +105,16 @@ def test_fp8_cache_small_shapes():
     _check_fp8(synth.make_workload("f8s", 2, 1, 64, [500, 77], seed=603), kv_scale=0.0173)
 
 
+@pytest.mark.parametrize("Sq,width,launches", [(6, 342, 3), (6, 341, 2), (8, 256, 3), (8, 255, 2), (5, 410, 2)])
+def test_fp8_cache_widened_ahead_of_large_calls_of_many_rows(Sq, width, launches):
+    # from six blocks of 128 rows and 8192 blocks x pages of the table on the pages are widened into a bf16 copy first
+    # (a third launch); page indices outside the cache are pages of zeros on either way
+    lens = [300, 0, 65, 1000]
+    w = synth.make_workload("f8w", 4, Sq, 128, lens, seed=610 + Sq, spare_blocks=2 * width, max_blocks_per_seq=width)
+    _check_fp8(w)
+    assert binding.last_launch_count() == launches
+
+
 def test_fp8_cache_dsv3_shape_full():
     _check_fp8(synth.config_dsv3())
 
