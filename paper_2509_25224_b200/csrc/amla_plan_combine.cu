@@ -82,7 +82,8 @@ __global__ void __launch_bounds__(128, kCols == 16 ? 7 : kCols == 8 ? 8 : 5) com
   asm volatile("griddepcontrol.wait;" ::: "memory");   // launched early (programmatic dependent launch): the partials must be complete
   if (group >= merge_groups(prm)) return;
   const int4 info = prm.merge_info[group];
-  if (info.z < 2) return;
+  // (a decode kernel that gave up has perhaps not written it: what it names then need not exist)
+  if (*prm.status != kStatusOk || info.z < 2) return;
   const int nsplit = (info.z - sw + kSplitWarps - 1) / kSplitWarps;      // of this warp
   const int b = prm.nrb == 1 ? info.x : info.x / prm.nrb;
   const int rin = (info.x - b * prm.nrb) * prm.item_rows + rr;                          // row within the sequence
