@@ -287,6 +287,7 @@ def run_gpu(args):
         run.step(i)
     total_ms, per_step = run.timed(args.steps, barrier)
     launches = binding.last_launch_count() * args.steps
+    kernel = {32: "decode_few_kernel", 128: "decode_pair_kernel", 256: "decode_quad_kernel"}[binding.last_item_rows()]
     # ---- same K steps again with per-kernel events (decode kernel duration for the roofline)
     plan_ms, dec_ms, comb_ms = run.kernel_times(args.steps)
     clocks = sampler.stop() if rank == 0 else None
@@ -359,8 +360,7 @@ def run_gpu(args):
 
     if rank == 0:
         roof = roofline_of(w, dec_ms, peaks, peak_kind)
-        roof.update({"kernel": "decode_quad_kernel" if (Sq * H > 128 and not args.rows128) else "decode_pair_kernel",
-                     "schedule_ms": plan_ms, "combine_ms": comb_ms})
+        roof.update({"kernel": kernel, "schedule_ms": plan_ms, "combine_ms": comb_ms})
         roof["traffic"] = load_traffic().get(w.name)
         n_rows = {"tiny": 16, "dsv3": 4096, "mtp": 2048, "stress": 1024, "long": 256}[w.name]
         tf, dt, cores, sample = time_oracle(w, n_rows)

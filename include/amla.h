@@ -56,9 +56,10 @@ enum {
   AMLA_RESCALE_MASK = 3,
   AMLA_FLAG_UNGUARDED_ADD = 4,
   AMLA_FLAG_KERNEL_SIMT = 8,    /* run the scalar bring-up kernel instead of the tensor-core kernels */
-  AMLA_FLAG_KERNEL_ROWS128 = 16, /* A/B measurements: treat sequences with more than 128 query rows as independent
-                                    128-row blocks (each streams the cache on its own) instead of running the
-                                    256-row kernel, in which one load of a cache tile serves all 256 rows */
+  AMLA_FLAG_KERNEL_ROWS128 = 16, /* A/B measurements: run the 128-row kernel whatever the shape: sequences with more
+                                    query rows as independent 128-row blocks (each streams the cache on its own)
+                                    instead of 256-row items, sequences of up to 32 rows as one padded block, E4M3
+                                    pages widened on their way in */
   AMLA_LAZY_SHIFT = 8,
   AMLA_LAZY_MASK = 0xF00,
   AMLA_DEFAULT_TAU = 8
@@ -196,7 +197,11 @@ int amla_validate_paging_host(const int32_t* block_table, const int32_t* seqlens
 /* Number of kernels the most recent amla_mla_decode[_ex] call on this thread launched. */
 int amla_last_launch_count(void);
 
-/* Measurement aid (the one piece of per-thread state in the library): when enabled, every decode call
+/* Query rows per work item of the most recent decode call on this thread, which tells the kernel that ran: 32 (the kernel
+ * for few rows), 128 or 256.  0 before the first call. */
+int amla_last_item_rows(void);
+
+/* Measurement aid: when enabled, every decode call
  * on this thread records CUDA events on its stream around its launches: before the schedule kernel
  * (which only batches of more than 2048 items have; otherwise that interval is empty), between it and
  * the decode kernel, between decode and combine, and after.  The events are created on the first

@@ -37,7 +37,7 @@ EXPORTS = [
     "amla_status_string", "amla_mla_decode_workspace_size", "amla_mla_decode", "amla_mla_decode_ex",
     "amla_check_status", "amla_last_launch_count", "amla_plan_host", "amla_profile_enable",
     "amla_profile_last_ms", "amla_mla_decode_static", "amla_static_check_status", "amla_wait_selftest",
-    "amla_validate_paging_host", "amla_mla_decode_fp8", "amla_mla_decode_fp8_workspace_size",
+    "amla_last_item_rows", "amla_validate_paging_host", "amla_mla_decode_fp8", "amla_mla_decode_fp8_workspace_size",
 ]
 
 _lib = None
@@ -84,6 +84,8 @@ def lib() -> ctypes.CDLL:
         L.amla_check_status.restype = i32
         L.amla_last_launch_count.argtypes = []
         L.amla_last_launch_count.restype = i32
+        L.amla_last_item_rows.argtypes = []
+        L.amla_last_item_rows.restype = i32
         L.amla_plan_host.argtypes = [vp, i32, i32, i32, i32, vp, i32]
         L.amla_plan_host.restype = i32
         L.amla_profile_enable.argtypes = [i32]
@@ -247,6 +249,11 @@ def _on_device(dev, call, args, tail, what):
 
 def last_launch_count() -> int:
     return int(lib().amla_last_launch_count())
+
+
+def last_item_rows() -> int:
+    """Query rows per work item of this thread's last decode call: 32, 128 or 256, after the kernel that ran."""
+    return int(lib().amla_last_item_rows())
 
 
 def profile_enable(on: bool) -> None:

@@ -75,7 +75,7 @@ int sm_count_of(int device, int* sms, int* cc_major) {
   return AMLA_OK;
 }
 
-thread_local int g_last_launches = 0;
+thread_local int g_last_launches = 0, g_last_item_rows = 0;
 #ifdef AMLA_TRACE
 thread_local unsigned long long* g_trace = nullptr;
 #endif
@@ -148,6 +148,7 @@ int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
 // The launches of one decode call (schedule kernel for large batches, decode, combine) on `stream`.
 int launch_decode_call(const DecodeParams& prm, int* prefix, cudaStream_t stream, int* launches, void (*mark)(int, cudaStream_t)) {
   const bool simt = (prm.flags & AMLA_FLAG_KERNEL_SIMT) != 0;
+  g_last_item_rows = prm.item_rows;
   if (mark) mark(0, stream);
   if (!prm.fused_plan) {
     if (launch_plan(prm, prefix, stream) != cudaSuccess) { cudaGetLastError(); return AMLA_ERR_CUDA; }
@@ -364,6 +365,7 @@ extern "C" int amla_check_status(const void* workspace, void* cuda_stream) {
 }
 
 extern "C" int amla_last_launch_count(void) { return g_last_launches; }
+extern "C" int amla_last_item_rows(void) { return g_last_item_rows; }
 
 extern "C" int amla_wait_selftest(void* workspace, unsigned long long limit_ns, void* cuda_stream) {
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 3)) return AMLA_ERR_INVALID_ARG;

@@ -39,6 +39,23 @@ def run_gpu(w, flags=None, poison=True, dev_inputs=None):
     return out.float().cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64), (out, lse)
 
 
+def wide_table(w, pages=4096):
+    """The same workload in a block table that has room for sequences long enough for the 256-row kernel, whatever the
+    lengths are (in a table as narrow as its sequences, short ones of more than 128 query rows run as blocks of 128)."""
+    pad = np.full((w.B, max(0, pages - w.block_table.shape[1])), -1, np.int32)
+    w.block_table = np.ascontiguousarray(np.concatenate([w.block_table, pad], axis=1))
+    return w
+
+
+def repeated(w, times):
+    """The batch `times` times over, on the same pages: long units for every part of the schedule at the cost of one."""
+    w.B *= times
+    w.q = np.ascontiguousarray(np.tile(w.q, (times, 1, 1, 1)))
+    w.block_table = np.ascontiguousarray(np.tile(w.block_table, (times, 1)))
+    w.seqlens = np.ascontiguousarray(np.tile(w.seqlens, times))
+    return w
+
+
 def compare(out, lse, ref_out, ref_lse, what="", tol_abs=TOL_ABS):
     assert not np.isnan(out).any(), f"{what}: NaN in out"
     err = np.abs(out - ref_out)
@@ -53,9 +70,12 @@ def compare(out, lse, ref_out, ref_lse, what="", tol_abs=TOL_ABS):
     return float(err.max()), float(rel)
 
 
-def check_full(w, flags=None, what="", tol_abs=TOL_ABS):
+def check_full(w, flags=None, what="", tol_abs=TOL_ABS, kernel=None, ref=None):
+    """Every output element against the oracle (or `ref`, its results from an earlier call); `kernel`: query rows per work
+    item of the kernel that has to have run."""
     out, lse, _ = run_gpu(w, flags)
-    ro, rl = R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)
+    assert kernel is None or binding.last_item_rows() == kernel, (binding.last_item_rows(), kernel)
+    ro, rl = ref if ref is not None else R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)
     return compare(out, lse, ro, rl, what or w.name, tol_abs)
 
 

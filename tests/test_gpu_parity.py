@@ -6,7 +6,7 @@ import pytest
 from oracle import amla_sim as S
 from oracle import reference as R
 from paper_2509_25224_b200 import binding, synth
-from tests._gpu_util import check_full, check_sampled, run_gpu, to_device
+from tests._gpu_util import check_full, check_sampled, repeated, run_gpu, to_device, wide_table
 
 pytestmark = pytest.mark.gpu
 
@@ -38,33 +38,53 @@ def test_ragged_batch_all_rescale_modes(mode):
 def test_head_and_token_shapes(Sq, H):
     w = synth.make_workload("s", 3, Sq, H, [200, 77, 513], seed=300 + 10 * Sq + H)
     check_full(w)
+    if Sq * H > 128:
+        # (384 rows are three full blocks of 128, or two of 256 of which one is half empty: always the former)
+        check_full(wide_table(w), kernel=128 if Sq * H == 384 else 256)
 
 
 @pytest.mark.parametrize("lens", [[1], [64], [65], [128], [129], [191], [192], [193], [1000, 3, 0, 257, 64]])
 def test_256_row_kernel_tile_tails(lens):
     # more than 128 query rows per sequence: 256-row items, 128-key tiles whose second page may be absent or partial
     w = synth.make_workload("q", len(lens), 2, 128, lens, seed=400 + sum(lens))
-    check_full(w)
-    check_full(w, binding.RESCALE_ALG2 | binding.lazy(0))
+    check_full(w, kernel=128)
+    check_full(wide_table(w), kernel=256)
+    check_full(w, binding.RESCALE_ALG2 | binding.lazy(0), kernel=256)
 
 
 def test_256_row_kernel_against_128_row_blocks():
     # the same problem through both kernels (256-row items vs independent 128-row blocks): both meet the oracle
-    w = synth.make_workload("ab", 3, 2, 128, [5000, 777, 2049], seed=431)
-    for flags in (binding.DEFAULT_FLAGS, binding.DEFAULT_FLAGS | binding.FLAG_KERNEL_ROWS128):
-        check_full(w, flags)
-    w = synth.make_workload("ab4", 2, 4, 128, [3000, 130], seed=432)
-    for flags in (binding.DEFAULT_FLAGS, binding.DEFAULT_FLAGS | binding.FLAG_KERNEL_ROWS128):
-        check_full(w, flags)
+    for w in (synth.make_workload("ab", 3, 2, 128, [5000, 777, 2049], seed=431), synth.make_workload("ab4", 2, 4, 128, [3000, 130], seed=432)):
+        wide_table(w)
+        check_full(w, binding.DEFAULT_FLAGS, kernel=256)
+        check_full(w, binding.DEFAULT_FLAGS | binding.FLAG_KERNEL_ROWS128, kernel=128)
+
+
+# 400 and 500 rows: the second block of a sequence is half full, or nearly full; 1024 rows: four full blocks.  Some sequences
+# are split over clusters, one begins with rows that see nothing.
+@pytest.mark.parametrize("Sq,H,lens", [(4, 100, [3000, 2, 700]), (5, 100, [2000, 129, 4, 300]), (8, 128, [1500, 64, 333])])
+def test_several_256_row_items_per_sequence_all_rescale_modes(Sq, H, lens):
+    w = wide_table(synth.make_workload("rb", len(lens), Sq, H, lens, seed=460 + Sq))
+    synth.apply_logit_offsets(w, [synth.staircase_offsets(n) if n >= 32 else np.zeros(n) for n in lens])
+    ref = R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)
+    for mode in MODES:
+        check_full(w, mode, kernel=256, ref=ref)
+    # the literal add, on inputs that leave no accumulator at zero
+    w = wide_table(synth.make_workload("rbu", len(lens), Sq, H, lens, seed=465 + Sq))
+    ref = R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)
+    for mode in (binding.RESCALE_ALG2, binding.RESCALE_FOLD):
+        check_full(w, mode | binding.lazy(0) | binding.FLAG_UNGUARDED_ADD, kernel=256, ref=ref)
 
 
 def test_unguarded_add_on_zero_free_inputs():
     # the literal single integer add of Algorithm 2 line 14 (no guard for zeros): valid when no accumulator is
     # exactly zero or tiny, which N(0,1) inputs ensure
-    for Sq in (1, 2):
+    for Sq, kernel in ((1, 128), (2, 256)):
         w = synth.make_workload("ung", 2, Sq, 128, [3000, 1500], seed=440 + Sq)
+        if Sq > 1:
+            wide_table(w)
         for mode in (binding.RESCALE_ALG2, binding.RESCALE_FOLD):
-            check_full(w, mode | binding.lazy(0) | binding.FLAG_UNGUARDED_ADD)
+            check_full(w, mode | binding.lazy(0) | binding.FLAG_UNGUARDED_ADD, kernel=kernel)
 
 
 def test_bounded_wait_reports_a_timeout_instead_of_hanging():
@@ -79,11 +99,12 @@ def test_bounded_wait_reports_a_timeout_instead_of_hanging():
     check_full(synth.config_tiny())
 
 
-def _check_fp8(w, kv_scale=1.0 / 64.0, flags=None):
+def _check_fp8(w, kv_scale=1.0 / 64.0, flags=None, kv8=None, ref=None):
     import torch
     from tests._gpu_util import compare
-    kv8 = synth.quantise_cache_e4m3(w, kv_scale)
-    ro, rl = R.decode_fp8(w.q, kv8, kv_scale, w.block_table, w.seqlens, w.scale)
+    if kv8 is None:
+        kv8 = synth.quantise_cache_e4m3(w, kv_scale)
+    ro, rl = ref if ref is not None else R.decode_fp8(w.q, kv8, kv_scale, w.block_table, w.seqlens, w.scale)
     q, _, bt, sl = to_device(w)
     kvd = torch.from_numpy(kv8).to(q.device)
     out = torch.empty((w.B, w.Sq, w.H, 512), dtype=torch.bfloat16, device=q.device)
@@ -98,7 +119,7 @@ def _check_fp8(w, kv_scale=1.0 / 64.0, flags=None):
 
 def test_fp8_cache_small_shapes():
     # E4M3 cache with a per-tensor scale against the FP64 oracle on the same bytes: tiny, ragged with an empty
-    # sequence, two query tokens (256-row kernel), a scale that is not a power of two
+    # sequence, two query tokens (two 128-row blocks), a scale that is not a power of two
     _check_fp8(synth.config_tiny())
     _check_fp8(synth.make_workload("f8r", 5, 1, 128, [700, 0, 64, 129, 1], seed=601))
     _check_fp8(synth.make_workload("f8q", 3, 2, 128, [1000, 65, 300], seed=602), flags=binding.RESCALE_ALG2 | binding.lazy(0))
@@ -153,8 +174,8 @@ def test_hundreds_of_one_page_units_per_cluster():
 
 @pytest.mark.parametrize("B", [128, 129])
 def test_items_around_the_on_chip_schedule_copy(B):
-    # up to 128 items the CTAs keep the schedule prefix and the sequence lengths in shared memory, above they read them
-    # from the workspace
+    # a full and one item more than the schedule's scan takes in four steps (the on-chip copies end at 512 items, at 160 in
+    # the 256-row kernel: the tests of those are below)
     rng = np.random.default_rng(12 + B)
     w = synth.make_workload("edge", B, 1, 16, rng.integers(0, 300, B), seed=13)
     check_full(w)
@@ -179,6 +200,54 @@ def test_few_row_kernel_row_and_page_edges(lens, Sq, H):
         check_full(w, mode | binding.lazy(0))
 
 
+@pytest.mark.parametrize("Sq,H", [(1, 8), (1, 16), (2, 12), (1, 32)])
+def test_few_row_kernel_rescales_within_long_units(Sq, H):
+    # 160 sequences on the pages of eight: every part holds 20 to 30 pages of one or two sequences, so that O is rewritten
+    # between pages.  Rising logits, a jump of 60 in the middle, falling ones; Sq = 2 masks the last page
+    lens = [1500, 1400, 1279, 1344, 1600, 1217, 1000, 1537]
+    w = synth.make_workload("fewr", 8, Sq, H, lens, seed=480 + H)
+    plain = synth.make_workload("fewu", 8, Sq, H, lens, seed=490 + H)
+    synth.apply_logit_offsets(w, [synth.staircase_offsets(n) if b % 3 == 0 else np.where(np.arange(n) < n // 2, -30.0, 30.0) if b % 3 == 1
+                                  else synth.staircase_offsets(n)[::-1].copy() for b, n in enumerate(lens)])
+    cases = [(w, MODES + [binding.RESCALE_ALG2]), (plain, [m | binding.lazy(0) | binding.FLAG_UNGUARDED_ADD for m in (binding.RESCALE_ALG2, binding.RESCALE_FOLD)])]
+    for w, modes in cases:
+        ref = [np.tile(x, (20,) + (1,) * (x.ndim - 1)) for x in R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)]
+        w = repeated(w, 20)
+        for mode in modes:
+            check_full(w, mode, kernel=32, ref=ref)
+
+
+def _unit_pages(w, parts):
+    """Pages of the units (a stretch of one item in one part) that the 128-row kernel's schedule makes of a batch."""
+    return {int(u[3] - u[2]) for u in binding.plan_host(w.seqlens, w.Sq, w.H, parts)}
+
+
+@pytest.mark.parametrize("fp8", [False, True])
+def test_128_row_kernel_rescales_over_tiles_of_every_width(fp8):
+    # units of 3, 4, 5 (3 + 2), 7 (4 + 3), 8 (4 + 4) pages and more, so that O is rewritten between tiles and the keys of a CTA
+    # begin in the middle of a page (tiles of three pages and of one); rising and jumping logits, tau 0 and 8
+    import torch
+    parts = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    lens = [180, 448, 512, 500, 250, 300, 700, 1250, 192, 65]
+    w = synth.make_workload("pairr", len(lens), 1, 100, lens, seed=470)
+    synth.apply_logit_offsets(w, [synth.staircase_offsets(n) if b % 2 else np.where(np.arange(n) < n // 2, -30.0, 30.0) for b, n in enumerate(lens)])
+    kv_scale = 1.0 / 8.0
+    if fp8:
+        kv8 = synth.quantise_cache_e4m3(w, kv_scale)
+        ref = R.decode_fp8(w.q, kv8, kv_scale, w.block_table, w.seqlens, w.scale)
+    else:
+        ref = R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)
+    ref = [np.tile(x, (15,) + (1,) * (x.ndim - 1)) for x in ref]
+    w = repeated(w, 15)
+    assert {3, 4, 5, 7, 8} <= _unit_pages(w, parts)
+    for mode in MODES:
+        if fp8:
+            _check_fp8(w, kv_scale, mode, kv8, ref)
+            assert binding.last_item_rows() == 128
+        else:
+            check_full(w, mode, kernel=128, ref=ref)
+
+
 @pytest.mark.parametrize("B,Sq,H,n", [(1, 1, 128, 400), (1, 1, 40, 4500), (1, 1, 128, 12000), (9, 1, 128, 1500), (11, 1, 128, 1500), (36, 1, 33, 700),
                                       (1, 1, 16, 20000), (36, 2, 16, 900), (75, 1, 16, 700)])
 def test_merges_by_rows_and_by_quarters_of_rows(B, Sq, H, n):
@@ -190,21 +259,14 @@ def test_merges_by_rows_and_by_quarters_of_rows(B, Sq, H, n):
     check_full(w)
 
 
-def _wide_table(w, pages=4096):
-    # a block table of this width may hold sequences long enough for the 256-row kernel, whatever the lengths are
-    pad = np.full((w.B, pages - w.block_table.shape[1]), -1, np.int32)
-    w.block_table = np.ascontiguousarray(np.concatenate([w.block_table, pad], axis=1))
-    return w
-
-
 @pytest.mark.parametrize("lens", [[1], [64], [65], [128], [129], [191], [192], [193], [1000, 3, 0, 257, 64], "64 short", "65 short", "160 short", "161 short", "300 short", "2100 short"])
 def test_256_row_kernel_on_short_sequences_in_a_wide_table(lens):
     # short sequences of more than 128 rows are blocks of 128 rows where the table's width says that they are short, and
     # 256-row items where it does not: tile tails, and items around its on-chip and in-kernel schedules
     if isinstance(lens, str):
         lens = np.random.default_rng(31).integers(0, 130, int(lens.split()[0]))
-    w = _wide_table(synth.make_workload("wide", len(lens), 2, 128 if len(lens) < 100 else 65, lens, seed=500 + int(np.sum(lens))))
-    check_full(w)
+    w = wide_table(synth.make_workload("wide", len(lens), 2, 128 if len(lens) < 100 else 65, lens, seed=500 + int(np.sum(lens))))
+    check_full(w, kernel=256)
     if len(lens) < 100:
         check_full(w, binding.RESCALE_ALG2 | binding.lazy(0))
 
@@ -228,7 +290,9 @@ def test_more_256_row_items_than_the_in_kernel_schedule_handles():
     # the same with two query tokens and 128 heads: 2100 items of 256 rows, schedule prefix from its own kernel
     rng = np.random.default_rng(14)
     w = synth.make_workload("bigq", 2100, 2, 128, rng.integers(0, 200, 2100), seed=15)
-    check_full(w)
+    ref = R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)
+    check_full(w, kernel=128, ref=ref)
+    check_full(wide_table(w), kernel=256, ref=ref)
 
 
 @pytest.mark.parametrize("mode", MODES)
@@ -268,12 +332,16 @@ def test_large_magnitude_inputs():
 
 
 def test_rerun_is_bit_identical():
-    w = synth.make_workload("d", 4, 2, 128, [3000, 1000, 64, 4097], seed=33)
-    dev = to_device(w)
-    _, _, (o1, l1) = run_gpu(w, dev_inputs=dev)
-    _, _, (o2, l2) = run_gpu(w, dev_inputs=dev)
     import torch
-    assert torch.equal(o1.view(torch.int16), o2.view(torch.int16)) and torch.equal(l1, l2)
+    w = synth.make_workload("d", 4, 2, 128, [3000, 1000, 64, 4097], seed=33)
+    for kernel in (128, 256):
+        if kernel == 256:
+            wide_table(w)
+        dev = to_device(w)
+        _, _, (o1, l1) = run_gpu(w, dev_inputs=dev)
+        _, _, (o2, l2) = run_gpu(w, dev_inputs=dev)
+        assert binding.last_item_rows() == kernel
+        assert torch.equal(o1.view(torch.int16), o2.view(torch.int16)) and torch.equal(l1, l2)
 
 
 @pytest.mark.parametrize("fp8", [False, True])
@@ -419,12 +487,14 @@ def test_accuracy_grid_of_tables_3_4(capsys):
                 name, base, amla = line.split()
                 rows.append((name, float(base), float(amla)))
     assert len(rows) == 12
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
     n_seeds, H, N = int(os.environ.get("AMLA_ACCURACY_SEEDS", "10")), 16, 8192   # the paper averages 100 samples
     lines, checks = [], []
     for i, (name, base, amla) in enumerate(rows):
         arg = float(name[name.index(",") + 1:-1])
         dist, sigma = ("normal", math.sqrt(arg)) if name.startswith("N") else ("uniform", arg)
-        e = {"base": [], "alg2": [], "fmul": [], "default": []}
+        e = {"base": [], "alg2": [], "fmul": [], "default": [], "alg2 whole": [], "fmul whole": []}
         for sd in range(n_seeds):
             w = synth.make_workload("acc", 1, 1, H, [N], seed=5000 + 100 * i + sd, scale=1.0 / math.sqrt(576.0), dist=dist, sigma=sigma)
             ro, rl = R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)
@@ -436,9 +506,15 @@ def test_accuracy_grid_of_tables_3_4(capsys):
             for mn, mf in (("alg2", binding.RESCALE_ALG2 | binding.lazy(0)), ("fmul", binding.RESCALE_FMUL | binding.lazy(0)), ("default", None)):
                 out, lse, _ = run_gpu(w, mf, dev_inputs=dev)
                 e[mn].append(S.rel_frobenius(out, ro))
+            # One sequence is cut into parts of a page each at tau = 0, and O is never rescaled; as often over as the GPU has
+            # SMs, each copy is one unit of 128 pages.
+            dev = to_device(repeated(w, sms))
+            for mn, mf in (("alg2 whole", binding.RESCALE_ALG2 | binding.lazy(0)), ("fmul whole", binding.RESCALE_FMUL | binding.lazy(0))):
+                out, lse, _ = run_gpu(w, mf, dev_inputs=dev)
+                e[mn].append(S.rel_frobenius(out[sms // 2], ro[0]))
         m = {k: float(np.mean(v)) for k, v in e.items()}
         lines.append(f"{name:10s} paper base {base:.2e} amla {amla:.2e} | here ({n_seeds} seeds) base-sim {m['base']:.2e} fmul {m['fmul']:.2e} "
-                     f"alg2 {m['alg2']:.2e} default(tau=8) {m['default']:.2e}")
+                     f"alg2 {m['alg2']:.2e} default(tau=8) {m['default']:.2e} whole sequences: fmul {m['fmul whole']:.2e} alg2 {m['alg2 whole']:.2e}")
         checks.append((name, base, amla, m))
     with capsys.disabled():
         print("\n" + "\n".join(lines))
@@ -452,3 +528,5 @@ def test_accuracy_grid_of_tables_3_4(capsys):
         assert m["alg2"] <= 1.05 * m["base"] + 1e-5, name      # AMLA tracks Base (Tables 3-4)
         assert m["alg2"] <= 1.05 * m["fmul"] + 1e-5, name      # and the kernel's own FP32-multiply variant
         assert m["default"] <= 1.10 * m["fmul"] + 1e-5, name
+        assert m["alg2 whole"] <= 1.05 * m["fmul whole"] + 1e-5, name
+        assert m["alg2 whole"] <= amla * 1.12, name

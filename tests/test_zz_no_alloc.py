@@ -14,7 +14,7 @@ import pytest
 
 from oracle import reference as R
 from paper_2509_25224_b200 import binding, synth
-from tests._gpu_util import TOL_ABS, TOL_LSE, TOL_REL_L2, compare, to_device
+from tests._gpu_util import TOL_ABS, TOL_LSE, TOL_REL_L2, compare, to_device, wide_table
 
 pytestmark = pytest.mark.gpu
 
@@ -58,6 +58,12 @@ def test_static_entry_matches_workspace_entry_on_two_calls_in_a_row():
     _check(synth.make_workload("na1", 5, 2, 128, [3000, 0, 65, 1500, 700], seed=4101))
     # a different shape right after it, on the same (now dirty) scratch
     _check(synth.make_workload("na2", 3, 1, 64, [200, 4097, 1], seed=4102))
+    assert binding.last_item_rows() == 128
+    # and the other two kernels: few rows (FP32 partials), 256-row items
+    _check(synth.make_workload("na3", 3, 1, 16, [5000, 77, 1500], seed=4103))
+    assert binding.last_item_rows() == 32
+    _check(wide_table(synth.make_workload("na4", 5, 2, 128, [3000, 0, 65, 1500, 700], seed=4104)))
+    assert binding.last_item_rows() == 256
 
 
 def test_static_entry_rejects_problems_beyond_its_scratch():
