@@ -28,12 +28,11 @@ def needs_build() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def build_trace(level: int = 1) -> str:
-    """Developer aid: libamla_trace.so, the same sources with -DAMLA_TRACE=level (per-role cycle stamps;
-    level 2 adds several stamps per ring slot, which slows the issuer loops it measures)."""
+def build_trace() -> str:
+    """Developer aid: libamla_trace.so, the same sources with -DAMLA_TRACE (per-role cycle stamps)."""
     out = os.path.join(_HERE, "libamla_trace.so")
     nvcc = os.environ.get("NVCC", "nvcc")
-    flags = [f for f in NVCC_FLAGS if not f.startswith("--use_fast_math")] + [f"-DAMLA_TRACE={level}"]
+    flags = [f for f in NVCC_FLAGS if not f.startswith("--use_fast_math")] + ["-DAMLA_TRACE"]
     subprocess.check_call([nvcc] + flags + sources() + ["-o", out])
     return out
 
@@ -54,6 +53,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 if __name__ == "__main__":
     if "--trace" in sys.argv:
-        print(build_trace(2 if "--full" in sys.argv else 1))
+        print(build_trace())
         sys.exit(0)
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))

@@ -142,10 +142,7 @@ decode_few_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_const
       tile.units.start();
       tile.begin();
     }
-    if (blockIdx.x == 0 && wid == 0) {       // the prefix in the workspace is part of what a call leaves behind
-      for (int it = lane; it <= prm.n_items; it += 32) const_cast<int*>(prm.prefix)[it] = plan_smem[it];
-      if (lane == 0) *prm.status = kStatusOk;
-    }
+    if (blockIdx.x == 0 && wid == 0 && lane == 0) *prm.status = kStatusOk;
   }
   if (tid == 0) AMLA_STAMP(prm, part, 20, 4);
   const bool wide = prm.R > 16;              // N of the P~V products: 16 or 32

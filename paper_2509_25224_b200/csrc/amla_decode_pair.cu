@@ -16,7 +16,8 @@
 // warp group = even / odd pages), write P~ = bf16(P * S16) into the P buffer of their own CTA, apply the integer N to
 // the bit patterns of O when the row's reference moved (lines 13-16; Lemma 3.1) and run the epilogue (line 20).  They
 // never hand data to the other CTA.  Warps 8 and 10-12 load (TMA), warp 9 of the even CTA issues the MMAs for both.
-// Order on the tensor pipe: QK^T(i + 1) before P~V(i), across units too (the paper's [C1, C2, V1] order, Section 4.1).
+// Order on the tensor pipe: QK^T(i + 1) before P~V(i) within a unit (the paper's [C1, C2, V1] order, Section 4.1); a unit's
+// last P~V comes before the next unit's first QK^T.
 //
 // Why this split.  The kernel before it gave one CTA of the pair Q K^T and the other P~ V (M = 128 on one SM each): P~
 // crossed to the other SM by remote stores, Q went through shared memory into tensor memory and the score CTA had to be
@@ -207,10 +208,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       tile.units.start();
       tile.begin();
     }
-    if (blockIdx.x == 0 && wid == 0) {       // the combine kernel reads the prefix in the workspace
-      for (int it = lane; it <= prm.n_items; it += 32) const_cast<int*>(prm.prefix)[it] = plan_smem[it];
-      if (lane == 0) *prm.status = kStatusOk;
-    }
+    if (blockIdx.x == 0 && wid == 0 && lane == 0) *prm.status = kStatusOk;
   }
   if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 4);
 

@@ -485,10 +485,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       first.start();
       any = first.next(fu);
     }
-    if (blockIdx.x == 0 && wid == 6) {       // the prefix in the workspace is part of what a call leaves behind
-      for (int it = lane; it <= prm.n_items; it += 32) const_cast<int*>(prm.prefix)[it] = plan_smem[it];
-      if (lane == 0) *prm.status = kStatusOk;
-    }
+    if (blockIdx.x == 0 && wid == 6 && lane == 0) *prm.status = kStatusOk;
   }
   if (tid == 0) QSTAMP_NS(smem_base, 2);
   // the first unit's Q is requested before the roles start: one piece per lane
@@ -637,69 +634,68 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       }
     } else if (wid == 5) {
       // ---- MMA issuer (even CTA only): S[sb] = Q K^T for both CTAs' rows, 36 steps of K = 16 over three slots
-      // The whole warp runs this loop and one lane is elected per instruction: issued by one lane under a branch, the 36
-      // MMAs took 76 clk each of this warp's time against 64 of the tensor pipe's (4 x 65536 keys x 256 rows: 157.1 us
-      // sustained and 134.8 cool; elected: 150.5 and 128.1).  Written out per slot and column block for the same reason:
-      // with a rolled loop over the slots the call takes 188.7 us.
+      // One elected lane runs the loop.  Under `lane == 0` the 36 MMAs took 76 clk each of this warp's time against 64 of the
+      // tensor pipe's (4 x 65536 keys x 256 rows: 157.1 us sustained and 134.8 cool; elected: 150.5 and 128.1).  Written out
+      // per slot and column block for the same reason: with a rolled loop over the slots the call takes 188.7 us.
       if (leader) {
         if (elect_one()) {
-        constexpr uint32_t idesc = make_idesc_bf16(256, 128, false, false);
-        constexpr uint32_t dhi = smem_desc_hi_sw128(kKGroupStride);
-        constexpr uint32_t qhi = smem_desc_hi_sw128(1024);
-        const uint32_t klo0 = smem_desc_lo(smem_base + kOffK, 16);
-        const uint32_t qlo0 = smem_desc_lo(smem_base + kOffQRope, 16);
-        uint32_t slot = 0, kpar = 0;
-        while (ok && iter.next(u)) {
-          ok = mbar_wait<true>(bar(A_QREADY), un & 1);
-          if (!ok) break;
-          tc_fence_after_sync();
-          for (int t = u.t0; t < u.t1 && ok; ++t, ++gs) {
-            const uint32_t sb = gs & 1;
-            ok = mbar_wait(bar(A_SEMPTY + sb), ((gs >> 1) & 1) ^ 1);
+          constexpr uint32_t idesc = make_idesc_bf16(256, 128, false, false);
+          constexpr uint32_t dhi = smem_desc_hi_sw128(kKGroupStride);
+          constexpr uint32_t qhi = smem_desc_hi_sw128(1024);
+          const uint32_t klo0 = smem_desc_lo(smem_base + kOffK, 16);
+          const uint32_t qlo0 = smem_desc_lo(smem_base + kOffQRope, 16);
+          uint32_t slot = 0, kpar = 0;
+          while (ok && iter.next(u)) {
+            ok = mbar_wait<true>(bar(A_QREADY), un & 1);
             if (!ok) break;
             tc_fence_after_sync();
-            QSTAMP(smem_base, 0, gs);
-            const uint32_t d = tbase + kSCol + 128 * sb;
-            // the three slots of the tile are probed together (their latencies overlap); the blocking wait runs
-            // only for one that is not there yet
-            bool have[3];
-            {
-              uint32_t s2 = slot, p2 = kpar;
+            for (int t = u.t0; t < u.t1 && ok; ++t, ++gs) {
+              const uint32_t sb = gs & 1;
+              ok = mbar_wait(bar(A_SEMPTY + sb), ((gs >> 1) & 1) ^ 1);
+              if (!ok) break;
+              tc_fence_after_sync();
+              QSTAMP(smem_base, 0, gs);
+              const uint32_t d = tbase + kSCol + 128 * sb;
+              // the three slots of the tile are probed together (their latencies overlap); the blocking wait runs
+              // only for one that is not there yet
+              bool have[3];
+              {
+                uint32_t s2 = slot, p2 = kpar;
+#pragma unroll
+                for (int gg = 0; gg < 3; ++gg) {
+                  have[gg] = mbar_probe(bar(A_KFULL) + 8 * s2, p2);
+                  if (++s2 == kNumKSlots) { s2 = 0; p2 ^= 1; }
+                }
+              }
 #pragma unroll
               for (int gg = 0; gg < 3; ++gg) {
-                have[gg] = mbar_probe(bar(A_KFULL) + 8 * s2, p2);
-                if (++s2 == kNumKSlots) { s2 = 0; p2 ^= 1; }
-              }
-            }
+                ok = ok && (have[gg] || mbar_wait(bar(A_KFULL) + 8 * slot, kpar));
+                if (ok) {
+                  if (gg == 0) QSTAMP(smem_base, 12, gs);
+                  const uint32_t klo = klo0 + slot * (kKSlotBytes >> 4);
 #pragma unroll
-            for (int gg = 0; gg < 3; ++gg) {
-              ok = ok && (have[gg] || mbar_wait(bar(A_KFULL) + 8 * slot, kpar));
-              if (ok) {
-                if (gg == 0) QSTAMP(smem_base, 12, gs);
-                const uint32_t klo = klo0 + slot * (kKSlotBytes >> 4);
+                  for (int cl = 0; cl < 3; ++cl) {
+                    const int cb = 3 * gg + cl;
 #pragma unroll
-                for (int cl = 0; cl < 3; ++cl) {
-                  const int cb = 3 * gg + cl;
-#pragma unroll
-                  for (int kk = 0; kk < 4; ++kk) {
-                    const uint64_t bd = smem_desc_join(klo + 64 * cl + 2 * kk, dhi);
-                    if (cb < 8) mma_ts_pair(d, tbase + kQCol + 32 * cb + 8 * kk, bd, idesc, (cb | kk) != 0 ? 1u : 0u);
-                    else mma_ss_pair(d, smem_desc_join(qlo0 + 2 * kk, qhi), bd, idesc, 1u);   // RoPE columns: Q from shared memory
+                    for (int kk = 0; kk < 4; ++kk) {
+                      const uint64_t bd = smem_desc_join(klo + 64 * cl + 2 * kk, dhi);
+                      if (cb < 8) mma_ts_pair(d, tbase + kQCol + 32 * cb + 8 * kk, bd, idesc, (cb | kk) != 0 ? 1u : 0u);
+                      else mma_ss_pair(d, smem_desc_join(qlo0 + 2 * kk, qhi), bd, idesc, 1u);   // RoPE columns: Q from shared memory
+                    }
                   }
+                  mma_commit_pair_multicast(bar(A_KEMPTY) + 8 * slot, kMaskScore);
                 }
-                mma_commit_pair_multicast(bar(A_KEMPTY) + 8 * slot, kMaskScore);
+                if (++slot == kNumKSlots) { slot = 0; kpar ^= 1; }
               }
-              if (++slot == kNumKSlots) { slot = 0; kpar ^= 1; }
+              if (!ok) break;
+              mma_commit_pair_multicast(bar(A_SFULL + sb), kMaskScore);
+              QSTAMP(smem_base, 1, gs);
             }
             if (!ok) break;
-            mma_commit_pair_multicast(bar(A_SFULL + sb), kMaskScore);
-            QSTAMP(smem_base, 1, gs);
+            mma_commit_pair_multicast(bar(A_QFREE), kMaskScore);
+            ++un;
           }
-          if (!ok) break;
-          mma_commit_pair_multicast(bar(A_QFREE), kMaskScore);
-          ++un;
-        }
-        if (!ok) report_timeout(prm.status);
+          if (!ok) report_timeout(prm.status);
         }
         __syncwarp();
       } else if (!leader) {
@@ -898,44 +894,44 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       // K = 16 steps
       if (leader) {
         if (elect_one()) {
-        constexpr uint32_t idesc = make_idesc_bf16(256, 256, false, true);
-        constexpr uint32_t dhi = smem_desc_hi_sw128(1024);
-        const uint32_t vlo0 = smem_desc_lo(smem_base + kOffV, kBoxBytes);
-        const uint32_t plo0 = smem_desc_lo(smem_base + kOffP, 16);
-        uint32_t slot = 0, vpar = 0;
-        while (ok && iter.next(u)) {
-          const int npages = 2 * (u.t1 - u.t0);
-          for (int pi = 0; pi < npages && ok; ++pi, ++gt) {
-            const uint32_t s = gt % kNumP, k = gt / kNumP;
-            ok = mbar_wait<true>(bar(B_PFULL + s), k & 1);
-            if (!ok) break;
-            QSTAMP(smem_base, 10, gt);
-            ok = mbar_wait<true>(bar(B_OREADY + s), k & 1);
-            if (!ok) break;
-            QSTAMP(smem_base, 11, gt);
-            tc_fence_after_sync();
-            fence_proxy_async_smem();
-            ok = mbar_wait(bar(B_VFULL) + 8 * slot, vpar);
-            if (!ok) break;
-            QSTAMP(smem_base, 8, gt);
-            const uint32_t plo = plo0 + s * (kPStride >> 4);
-            const uint32_t vlo = vlo0 + slot * (kVSlotBytes >> 4);
-            const uint32_t acc0 = pi > 0 ? 1u : 0u;
+          constexpr uint32_t idesc = make_idesc_bf16(256, 256, false, true);
+          constexpr uint32_t dhi = smem_desc_hi_sw128(1024);
+          const uint32_t vlo0 = smem_desc_lo(smem_base + kOffV, kBoxBytes);
+          const uint32_t plo0 = smem_desc_lo(smem_base + kOffP, 16);
+          uint32_t slot = 0, vpar = 0;
+          while (ok && iter.next(u)) {
+            const int npages = 2 * (u.t1 - u.t0);
+            for (int pi = 0; pi < npages && ok; ++pi, ++gt) {
+              const uint32_t s = gt % kNumP, k = gt / kNumP;
+              ok = mbar_wait<true>(bar(B_PFULL + s), k & 1);
+              if (!ok) break;
+              QSTAMP(smem_base, 10, gt);
+              ok = mbar_wait<true>(bar(B_OREADY + s), k & 1);
+              if (!ok) break;
+              QSTAMP(smem_base, 11, gt);
+              tc_fence_after_sync();
+              fence_proxy_async_smem();
+              ok = mbar_wait(bar(B_VFULL) + 8 * slot, vpar);
+              if (!ok) break;
+              QSTAMP(smem_base, 8, gt);
+              const uint32_t plo = plo0 + s * (kPStride >> 4);
+              const uint32_t vlo = vlo0 + slot * (kVSlotBytes >> 4);
+              const uint32_t acc0 = pi > 0 ? 1u : 0u;
 #pragma unroll
-            for (int nh = 0; nh < 2; ++nh) {
+              for (int nh = 0; nh < 2; ++nh) {
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                mma_ss_pair(tbase + nh * 256, smem_desc_join(plo + 2 * kk, dhi), smem_desc_join(vlo + nh * (kVHalfBytes >> 4) + 128 * kk, dhi),
-                            idesc, kk == 0 ? acc0 : 1u);
+                for (int kk = 0; kk < 4; ++kk)
+                  mma_ss_pair(tbase + nh * 256, smem_desc_join(plo + 2 * kk, dhi), smem_desc_join(vlo + nh * (kVHalfBytes >> 4) + 128 * kk, dhi),
+                              idesc, kk == 0 ? acc0 : 1u);
+              }
+              mma_commit_pair_multicast(bar(B_VEMPTY) + 8 * slot, kMaskValue);
+              if (++slot == kNumVSlots) { slot = 0; vpar ^= 1; }
+              mma_commit_pair_multicast(bar(X_PV + s), kMaskAll);   // PVDONE in the value CTAs, "P buffer free" in the score CTAs
+              QSTAMP(smem_base, 9, gt);
             }
-            mma_commit_pair_multicast(bar(B_VEMPTY) + 8 * slot, kMaskValue);
-            if (++slot == kNumVSlots) { slot = 0; vpar ^= 1; }
-            mma_commit_pair_multicast(bar(X_PV + s), kMaskAll);   // PVDONE in the value CTAs, "P buffer free" in the score CTAs
-            QSTAMP(smem_base, 9, gt);
+            if (!ok) break;
           }
-          if (!ok) break;
-        }
-        if (!ok) report_timeout(prm.status);
+          if (!ok) report_timeout(prm.status);
         }
         __syncwarp();
       } else if (!leader) {

@@ -164,13 +164,6 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst_smem, const void* tmap,
       ::"r"(dst_smem), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z), "r"(bar)
       : "memory");
 }
-// 4-D tiled load.
-__device__ __forceinline__ void tma_load_4d(uint32_t dst_smem, const void* tmap, int c0, int c1, int c2, int c3, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-      ::"r"(dst_smem), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-      : "memory");
-}
 // The same loads issued by one CTA of an MMA pair (cluster ranks 2k, 2k+1): the data lands in this CTA's shared
 // memory, the bytes are counted on `cluster_bar`, which may be a barrier of the other CTA of the pair (an address
 // from map_to_cta) -- the pair's MMA issuer waits on one barrier for both halves of an operand.  No multicast.
@@ -217,10 +210,6 @@ __device__ __forceinline__ void bulk_copy_to_cluster(uint32_t dst_cluster, uint3
 __device__ __forceinline__ void stg_256(void* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f, uint32_t g, uint32_t h) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e), "r"(f), "r"(g), "r"(h) : "memory");
-}
-// Brings a line into this SM's L1 without a destination register: a later load of it does not wait on the memory system.
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p) : "memory");
 }
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
@@ -362,13 +351,6 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// Like mma_commit, but the arrival is delivered to the barrier at the same shared-memory offset in every
-// CTA of the cluster named in cta_mask (bit i = CTA rank i).
-__device__ __forceinline__ void mma_commit_multicast(uint32_t bar, uint16_t cta_mask) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(bar), "h"(cta_mask) : "memory");
-}
-
 // ---- MMAs over a pair of CTAs (cluster ranks 2k and 2k+1), issued by one thread of the even one.  M = 256: each
 // CTA contributes its own 128 rows of A (same tensor-memory address / same shared-memory offset in both) and
 // receives its 128 rows of D in its own tensor memory; B (N x 16) is split, the even CTA holding rows 0..N/2-1 of
@@ -399,10 +381,6 @@ __device__ __forceinline__ void mma_commit_pair_multicast(uint32_t bar, uint16_t
 // Asynchronous stores into the shared memory of a CTA of the cluster; each adds its size to the transaction
 // count of a barrier of that CTA.  Generic-proxy writes: a consumer that reads them through the async proxy
 // (TMA, tcgen05.mma) fences with fence.proxy.async after its wait.
-__device__ __forceinline__ void st_async_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t cluster_bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-               ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(cluster_bar) : "memory");
-}
 __device__ __forceinline__ void st_async_b32(uint32_t cluster_addr, uint32_t a, uint32_t cluster_bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
                ::"r"(cluster_addr), "r"(a), "r"(cluster_bar) : "memory");
