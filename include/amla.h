@@ -213,14 +213,16 @@ int amla_profile_enable(int on);
 int amla_profile_last_ms(float* ms3);
 
 /*
- * Host mirror of the device-side split-KV schedule (the plan is not in the paper; it exists because
- * B * ceil(Sq*H/128) work items are far fewer than the SMs).  For Sq*H <= 128 the items are (sequence, 128-row
- * block) pairs, their tiles 64-key pages, and every non-empty item but the first is preceded by 6 overhead
- * positions that stand for the cost of starting an item; for Sq*H > 128 the items are (sequence, 256-row block)
- * pairs, the tiles 128 keys (two pages) and the overhead 5 positions.  Items in order form one linear range
- * that is cut into parts of ceil(length / num_parts) positions.  (On the device a part also holds at least 128 keys
- * unless tau is 0, sequences of up to 32 rows have a schedule of their own, with 32-row items and 3 overhead
- * positions, and short sequences of more than 128 rows may run as 128-row items.)
+ * Host mirror of the device-side split-KV schedule (the plan is not in the paper; it exists because a decode batch
+ * has far fewer (sequence, row block) items than the GPU has SMs).  It cuts as the kernel for the row count does with
+ * the default flags:
+ *   Sq*H <= 32    items of 32 rows, tiles of 64 keys (a page), 3 overhead positions (a part is one SM)
+ *   Sq*H <= 128   items of 128 rows, tiles of 64 keys, 6 overhead positions (a part is two SMs)
+ *   above         items of 256 rows, tiles of 128 keys, 5 overhead positions (a part is four SMs)
+ * Every non-empty item but the first is preceded by the overhead positions, which stand for the cost of starting an
+ * item.  Items in order form one linear range that is cut into parts of ceil(length / num_parts) positions, and of at
+ * least 128 keys (with tau = 0: of at least one tile).  (The device runs an E4M3 cache, and more than 128 rows where
+ * that is faster, as 128-row items, and a single sequence of at most 256 keys as one part.)
  * For every (part, item) intersection ("unit") one record of 6 int32 is written:
  *   part, item, tile_begin, tile_end (within the item), slot (-1 = writes out/lse directly,
  *   otherwise index of its fp32 partial), n_split of the item.

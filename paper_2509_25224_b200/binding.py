@@ -110,8 +110,8 @@ def workspace_size(B: int, Sq: int, H: int, max_blocks_per_seq: int, device: int
 
 def plan_host(seqlens, Sq: int, H: int, num_parts: int) -> np.ndarray:
     """Host mirror of the split-KV schedule: int32 [n_units, 6] rows of
-    (part, item, tile_begin, tile_end, slot, n_split).  Items are 128-row blocks with 64-key tiles for
-    Sq*H <= 128, 256-row blocks with 128-key tiles above."""
+    (part, item, tile_begin, tile_end, slot, n_split).  Items are blocks of 32, 128 or 256 rows (Sq*H up to 32, up
+    to 128, above), tiles 64 keys, above 128 rows 128."""
     sl = np.ascontiguousarray(seqlens, dtype=np.int32)
     B = sl.shape[0]
     nrb = (Sq * H + 127) // 128

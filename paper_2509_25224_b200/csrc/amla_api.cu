@@ -426,9 +426,9 @@ extern "C" int amla_plan_host(const int32_t* seqlens, int B, int Sq, int H, int 
   if (!seqlens || !units || num_parts <= 0 || max_units < 0) return AMLA_ERR_INVALID_ARG;
   int rc = check_shape(B, Sq, H, 1);
   if (rc != AMLA_OK) return rc;
-  const bool quad = Sq * H > kRowBlock;
-  const int item_rows = quad ? 2 * kRowBlock : kRowBlock, tile_keys = quad ? 2 * kPage : kPage;
-  const int ovh = quad ? kQuadOverheadTiles : kUnitOverheadTiles;
+  const bool quad = Sq * H > kRowBlock, few = Sq * H <= kFewRows;
+  const int item_rows = quad ? 2 * kRowBlock : few ? kFewRows : kRowBlock, tile_keys = quad ? 2 * kPage : kPage;
+  const int ovh = quad ? kQuadOverheadTiles : few ? kFewOverheadTiles : kUnitOverheadTiles;
   const int nrb = (Sq * H + item_rows - 1) / item_rows;
   const int n_items = B * nrb;
   int* prefix = new (std::nothrow) int[n_items + 1];
@@ -439,7 +439,7 @@ extern "C" int amla_plan_host(const int32_t* seqlens, int B, int Sq, int H, int 
     acc += schedule_length(seqlens[it / nrb], it, tile_keys, ovh);
   }
   prefix[n_items] = acc;
-  const Plan plan = Plan::make(prefix, n_items, num_parts, ovh);
+  const Plan plan = Plan::make(prefix, n_items, num_parts, ovh, kMinPartKeys / tile_keys);
   int n_units = 0;
   bool overflow = false;
   if (acc > 0) {

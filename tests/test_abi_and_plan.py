@@ -13,9 +13,9 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _variant(Sq, H):
-    """(rows per item, keys per tile, overhead positions) of the schedule for a shape: up to 128 query rows per
-    sequence the items are 128-row blocks with one-page tiles, above that 256-row blocks with two-page tiles."""
-    return (256, 128, 5) if Sq * H > 128 else (128, 64, 6)
+    """(rows per item, keys per tile, overhead positions) of the schedule for a shape: up to 32 query rows per sequence
+    are one item, up to 128 one 128-row block, with one-page tiles; above that 256-row blocks with two-page tiles."""
+    return (256, 128, 5) if Sq * H > 128 else (128, 64, 6) if Sq * H > 32 else (32, 64, 3)
 
 
 @pytest.fixture(scope="module")
@@ -94,14 +94,15 @@ def _check_plan(seqlens, Sq, H, P):
             ps = [p for p, _, _ in parts]
             assert ps == list(range(ps[0], ps[0] + len(ps)))   # consecutive parts
     # balance: the schedule cuts a range in which every non-empty item but the first is preceded by UNIT_OVERHEAD positions
-    # (the cost of starting an item) into equal parts, so no part holds more tiles than one such share
+    # (the cost of starting an item) into equal parts of at least 128 keys, so no part holds more tiles than one such share
     Lv = sum(t + (UNIT_OVERHEAD if it else 0) for it, t in enumerate(tiles) if t)
     if Lv:
-        assert per_part.max() <= -(-Lv // min(P, Lv))
+        share = max(-(-Lv // min(P, Lv)), 128 // tile_keys)
+        assert per_part.max() <= share
         starts = np.zeros(P, dtype=np.int64)            # items whose first tile a part holds
         for p, it, t0, t1, slot, ns in units:
             starts[p] += t0 == 0
-        assert (per_part + UNIT_OVERHEAD * starts).max() <= -(-Lv // min(P, Lv)) + UNIT_OVERHEAD
+        assert (per_part + UNIT_OVERHEAD * starts).max() <= share + UNIT_OVERHEAD
     return units
 
 
@@ -116,7 +117,7 @@ def test_plan_covers_every_tile_once_and_balances(lib, P):
     _check_plan(np.array([0, 0, 0]), 1, 128, P)
     for _ in range(10):
         B = int(rng.integers(1, 40))
-        _check_plan(rng.integers(0, 3000, B), int(rng.integers(1, 4)), int(rng.choice([16, 64, 128])), P)
+        _check_plan(rng.integers(0, 3000, B), int(rng.integers(1, 4)), int(rng.choice([8, 16, 64, 128])), P)
 
 
 def test_plan_small_case_by_hand(lib):
@@ -124,6 +125,13 @@ def test_plan_small_case_by_hand(lib):
     # the first item, part 1 = [5,10) the second
     u = binding.plan_host(np.array([129, 10]), 1, 128, 2)
     assert u.tolist() == [[0, 0, 0, 3, -1, 1], [1, 1, 0, 1, -1, 1]]
+
+
+def test_plan_small_case_by_hand_few_rows_and_shortest_parts(lib):
+    # 16 rows: one 32-row item per sequence, 3 overhead positions.  5 and 1 pages: positions [tiles 0-4 | 3 overhead, tile 0]
+    # = 9; 148 parts would be a position each, but no part is shorter than two pages: parts own [0,2), [2,4), [4,6), [6,8), [8,9)
+    u = binding.plan_host(np.array([320, 10]), 1, 16, 148)
+    assert u.tolist() == [[0, 0, 0, 2, 0, 3], [1, 0, 2, 4, 2, 3], [2, 0, 4, 5, 4, 3], [4, 1, 0, 1, -1, 1]]
 
 
 def test_plan_small_case_by_hand_256_row_items(lib):
