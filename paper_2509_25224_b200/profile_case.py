@@ -1,10 +1,11 @@
 """Runs a few decode calls of one (possibly cut-down) workload: the command that profiler captures wrap.
 
     python -m paper_2509_25224_b200.profile_case --config mtp [--batch 32] [--calls 3] [--mode alg2|fold|fmul]
-                                                 [--tau T] [--rows128] [--n N]
+                                                 [--tau T] [--rows128] [--n N] [--heads H]
 
 --batch keeps the first B sequences of the named configuration (its seeded lengths and values), --n overrides the
-sequence length of the fixed-length configurations (stress: the staircase of logit offsets spans the new length).
+sequence length of the fixed-length configurations (stress: the staircase of logit offsets spans the new length), --heads
+the number of heads of dsv3 (16: the kernel for few rows).
 One warm-up call, then --calls calls; the status word is checked and a checksum of the output printed, so that a
 capture can be told from a run that did nothing.
 """
@@ -18,10 +19,10 @@ import numpy as np
 from . import binding, synth
 
 
-def build_workload(name: str, batch: int | None, n: int | None) -> synth.Workload:
+def build_workload(name: str, batch: int | None, n: int | None, heads: int = 128) -> synth.Workload:
     if name == "dsv3":
         B = batch or 32
-        return synth.make_workload("dsv3", B, 1, 128, [n or 4096] * B, synth.SEEDS["dsv3"])
+        return synth.make_workload("dsv3", B, 1, heads, [n or 4096] * B, synth.SEEDS["dsv3"])
     if name == "mtp":
         sl = synth.mtp_seqlens()
         B = batch or len(sl)
@@ -43,12 +44,13 @@ def main() -> int:
     ap.add_argument("--config", default="dsv3", choices=["tiny", "dsv3", "mtp", "stress", "long"])
     ap.add_argument("--batch", type=int, default=None)
     ap.add_argument("--n", type=int, default=None)
+    ap.add_argument("--heads", type=int, default=128)
     ap.add_argument("--calls", type=int, default=3)
     ap.add_argument("--mode", default=None, choices=["alg2", "fold", "fmul"])
     ap.add_argument("--tau", type=int, default=None)
     ap.add_argument("--rows128", action="store_true")
     a = ap.parse_args()
-    w = build_workload(a.config, a.batch, a.n)
+    w = build_workload(a.config, a.batch, a.n, a.heads)
     flags = None
     if a.mode is not None or a.tau is not None or a.rows128:
         flags = ({"alg2": 0, "fold": 1, "fmul": 2}[a.mode or "alg2"] | binding.lazy(binding.DEFAULT_TAU if a.tau is None else a.tau)
@@ -66,7 +68,7 @@ def main() -> int:
         binding.mla_decode(q, kv, bt, sl, w.scale, out, lse, ws, flags)
     binding.check_status(ws)
     torch.cuda.synchronize()
-    print(f"{a.config}: B={w.B} Sq={w.Sq} keys={int(w.seqlens.astype(np.int64).sum())} KV={w.kv.nbytes / 1e6:.0f} MB "
+    print(f"{a.config}: B={w.B} Sq={w.Sq} H={w.H} keys={int(w.seqlens.astype(np.int64).sum())} KV={w.kv.nbytes / 1e6:.0f} MB "
           f"flops/call={w.flops():.4g} algorithmic_bytes/call={w.algorithmic_bytes():.4g} checksum={float(out.float().abs().sum()):.6g}")
     return 0
 
