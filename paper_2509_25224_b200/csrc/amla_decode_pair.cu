@@ -23,11 +23,11 @@
 // crossed to the other SM by remote stores, Q went through shared memory into tensor memory and the score CTA had to be
 // drained before the next unit's Q could follow.  Here nothing but MMA operands crosses, Q is an operand as it lands, and
 // the tile is 256 keys.  Calls with it, from that kernel to this one as it stands (sustained): 192 sequences of 1-512 keys
-// 62.8 -> 43.9 us; one of 2531 33.8 -> 12.2; 16 x 16384 with rising logits 105.2 -> 93.0; 96 x 2048 88.4 -> 80.2; 32 x 4096
-// 59.3 -> 55.1; E4M3 32 x 4096 101.0 -> 61.8.
+// 62.8 -> 45.2 us; one of 2531 33.8 -> 12.8; 16 x 16384 with rising logits 106.0 -> 93.4; 96 x 2048 88.7 -> 81.0; 32 x 4096
+// 59.1 -> 55.5; 96 x 16384 540 -> 447; E4M3 32 x 4096 100.4 -> 62.1.
 // What bounds it: a tile of 256 keys takes ~7500 clk (E4M3 10.4 K) against 4350 of MMAs and 5900 of HBM at its full rate: a
 // CTA takes 278 KB per tile through a ring of 112 KB, whose slots turn around in ~2700 clk (load 1500-2000, MMA, commit,
-// next load), and every slot has to be issued.  Long calls run at the power limit: 32 x 4096 takes 50.2 us cool.
+// next load), and every slot has to be issued.  Long calls run at the power limit: 32 x 4096 takes 51 us cool.
 //
 // All waits are bounded; on expiry the kernel records kStatusTimeout and unwinds.
 #include "amla_common.cuh"
