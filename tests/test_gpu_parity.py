@@ -449,12 +449,16 @@ def test_rescale_mode_accuracy_table(capsys):
     # Accuracy of the three ways to rescale O (Algorithm 2's integer add, Eq. 3's exact fold, Algorithm 1's FP32
     # multiply), each with the reference moved at every new maximum (tau = 0) and lazily (tau = 8), against the FP64
     # oracle: the paper's claim (Tables 3-4) is that the integer add costs no accuracy against the multiply.
-    cases = [("staircase B=2 N=4096", synth.config_stress(B=2, N=4096)),
-             ("normal    B=2 N=8192", synth.make_workload("n", 2, 1, 128, [8192, 8192], seed=77))]
+    # Two sequences alone are cut into parts of one tile, and O is never rescaled; forty times over (on the same pages) they
+    # are more items than the schedule has parts, and every unit is most of a sequence.
+    cases = [(f"{name} {'x 40' if times > 1 else 'cut '}", make(), times) for times in (1, 40) for name, make in
+             (("staircase B=2 N=4096", lambda: synth.config_stress(B=2, N=4096)),
+              ("normal    B=2 N=8192", lambda: synth.make_workload("n", 2, 1, 128, [8192, 8192], seed=77)))]
     modes = [("alg2", binding.RESCALE_ALG2), ("fold", binding.RESCALE_FOLD), ("fmul", binding.RESCALE_FMUL)]
     lines = []
-    for name, w in cases:
-        ro, rl = R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale)
+    for name, w, times in cases:
+        ro, rl = (np.tile(x, (times,) + (1,) * (x.ndim - 1)) for x in R.decode(w.q, w.kv, w.block_table, w.seqlens, w.scale))
+        w = repeated(w, times)
         dev = to_device(w)
         rel = {}
         for mn, mf in modes:
