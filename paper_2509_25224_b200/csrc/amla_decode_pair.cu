@@ -16,8 +16,10 @@
 // warp group = even / odd pages), write P~ = bf16(P * S16) into the P buffer of their own CTA, apply the integer N to
 // the bit patterns of O when the row's reference moved (lines 13-16; Lemma 3.1) and run the epilogue (line 20).  They
 // never hand data to the other CTA.  Warps 8 and 10-12 load (TMA), warp 9 of the even CTA issues the MMAs for both.
-// Order on the tensor pipe: QK^T(i + 1) before P~V(i) within a unit (the paper's [C1, C2, V1] order, Section 4.1); a unit's
-// last P~V comes before the next unit's first QK^T.
+// Order on the tensor pipe: QK^T(i + 1) before P~V(i) (the paper's [C1, C2, V1] order, Section 4.1), whether or not the two
+// tiles belong to one unit: the next unit's Q is asked for as soon as the scores of a unit's last tile are there, and its first
+// scores are made while those are worked on.  (Each unit a chain by itself: 1 x 2531 keys 13.09 -> 12.78 us, 29 x 238-661
+// 18.95 -> 18.69, 32 x 4096 55.75 -> 55.21, E4M3 61.8 -> 60.5; outputs the same bits.)
 //
 // Why this split.  The kernel before it gave one CTA of the pair Q K^T and the other P~ V (M = 128 on one SM each): P~
 // crossed to the other SM by remote stores, Q went through shared memory into tensor memory and the score CTA had to be
@@ -93,7 +95,7 @@ constexpr uint32_t kSCol = 256;          // 2 x 128 columns
 
 // Barriers.  (L): the copy in the even CTA is the one that counts; both CTAs arrive there.  The others exist in both
 // CTAs and complete by multicast commits of the even CTA's MMA warp, except X_XCHG and the raw ring's, which are local.
-enum { X_FULL = 0 /*L*/, X_EMPTY = X_FULL + 7, X_QFULL = X_EMPTY + 7 /*L*/, X_QFREE, X_SFULL, X_SEMPTY = X_SFULL + 2 /*L*/,
+enum { X_FULL = 0 /*L*/, X_EMPTY = X_FULL + 7, X_QFULL = X_EMPTY + 7 /*L*/, X_SFULL, X_SEMPTY = X_SFULL + 2 /*L*/,
        X_PREADY = X_SEMPTY + 2 /*L*/, X_PVDONE, X_XCHG, X_RAWFULL = X_XCHG + 2, X_RAWEMPTY = X_RAWFULL + kRawSlots,
        X_FULLODD = X_RAWEMPTY + kRawSlots /* odd CTA, E4M3: its half of FULL, passed on */, X_NUM = X_FULLODD + kSlots<true> };
 static_assert(X_NUM * 8 + 8 <= kBarBytes, "barrier area too small");
@@ -107,14 +109,24 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
   return __all_sync(0xffffffffu, mbar_wait<kClusterAcquire>(bar, parity));
 }
 
-// What the loader keeps of a score tile: where its pages stand in the block table, how many, the Q row of its unit.
+// What the loader keeps of a score tile: where its pages stand in the block table, how many.
 struct TileRef {
   const int32_t* bt;
-  int np, qrow;
-  bool first, last, valid;
+  int np;
+  bool valid;
 };
 
 using Tiles = TileIter<kTilePages>;
+
+// This CTA's 64 rows of a unit's Q, by one thread of either CTA.  The bytes of both are counted in the even one.
+__device__ __forceinline__ int q_row_of(const DecodeParams& prm, const Unit& u, int rank) { return u.b * prm.R + u.r0 + rank * kCtaRows; }
+__device__ __forceinline__ void request_q(const CUtensorMap& q_map, uint32_t smem_base, uint32_t bars, uint32_t lead_bars, bool leader, int qrow) {
+  if (leader) mbar_arrive_expect_tx(bars + 8u * X_QFULL, 2 * kQBytes);
+  const uint64_t last_use = l2_policy_evict_first();
+#pragma unroll 1
+  for (int c = 0; c < kQBlocks; c += 3)
+    tma_load_3d_pair_hint(smem_base + kOffQ + c * kQBlockBytes, &q_map, 0, qrow, c, lead_bars + 8u * X_QFULL, last_use);
+}
 
 }  // namespace
 
@@ -155,7 +167,6 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       for (int i = 0; i < kRawSlots; ++i) { mbar_init(bar(X_RAWFULL + i), 1); mbar_init(bar(X_RAWEMPTY + i), kWidenWarps); }
     }
     mbar_init(bar(X_QFULL), 1);
-    mbar_init(bar(X_QFREE), 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar(X_SFULL + i), 1);
       mbar_init(bar(X_SEMPTY + i), 2 * kSoftmaxWarps);
@@ -223,6 +234,17 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     const uint32_t prow_smem = smem_base + kOffP + r * 128;
     const uint32_t o_addr = tbase + lane_base + kOCol + 128 * grp;     // this thread's 128 of the row's 512 columns
     uint32_t gs = 0, xc = 0;                             // score tiles and exchanges so far
+    // Warp 7 asks for the next unit's Q as soon as the scores of a unit's last tile are there: the MMAs have then read Q.
+    // It looks the unit up well before that.
+    constexpr int kAsksForQ = 7;
+    UnitIter ahead = tile.units;
+    uint32_t q_asked = 0;                                // units whose Q this warp has asked for
+    int q_next = -1;
+    auto look_ahead = [&]() {
+      Unit n;
+      q_next = ahead.next(n) ? q_row_of(prm, n, rank) : -1;
+    };
+    if (wid == kAsksForQ && tile.valid) look_ahead();
     // tells the row's other three threads `mine`; v[0..3] = what the four told
     auto exchange = [&](float mine, float (&v)[4]) {
       const uint32_t buf = smem_base + kOffXchg + (xc & 1) * (4 * kCtaRows * 4) + r * 4;
@@ -253,6 +275,10 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         if (!ok) break;
         tc_fence_after_sync();
         if (tid == 0 && leader) AMLA_STAMP(prm, part, 8, gs);
+        if (wid == kAsksForQ && tile.last() && q_next >= 0) {
+          if (lane == 0) request_q(q_map, smem_base, bars, lead_bars, leader, q_next);
+          ++q_asked;
+        }
         // A lane half holds 32 np neighbouring keys; this group takes its 32-key chunks grp and grp + 2.  The scores are
         // read from tensor memory twice, a chunk at a time: for the maximum, and for the exponentials once the P buffer is
         // free.  (Held in registers in between they cost 64 more of them and twice the code.)
@@ -399,6 +425,8 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       int2 info;
       const int slot = tile.units.slot_of(u, &info);
       if (tid == 0 && leader) merge_note(prm, part, u.it, info);
+      tile.next();
+      if (wid == kAsksForQ && tile.valid) look_ahead();
       float l4[4];
       exchange(st.l, l4);
       if (!ok) break;
@@ -439,19 +467,19 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         }
       }
       if (tid == 0 && leader) AMLA_STAMP(prm, part, 14, gs - 1);
-      tile.next();
     }
-    if (!ok && lane == 0) report_timeout(prm.status);
+    if (!ok && lane == 0) {
+      report_timeout(prm.status);
+      if (leader && q_asked > 0) mbar_wait(bar(X_QFULL), q_asked & 1);     // let copies that may still be in flight land
+    }
   } else if (wid == 8 || (!kFp8 && wid >= 10)) {
     // ======================================================== TMA loads, in the order in which the MMAs use them:
-    // Q, K(0), K(1), V(0), K(2), V(1), ..., K(n-1), V(n-2), V(n-1), next unit.
+    // K(0), K(1), V(0), K(2), V(1), ..., K(n-1), V(n-2), V(n-1), the tiles counted over all of the part's units.
     //   bf16: one ring of 16 KB slots carries K (one 64-column block of half the tile's keys) and V (one page x 128 columns).
     //     The loader warps walk the same sequence and issue every fourth load of it: a slot takes ~350 clk to issue, a warp by
     //     itself never waits for a slot.  Two -> four loaders: 16 x 16384 keys, rising 85.7 -> 83.3 us cool, 96 x 16384 488 ->
     //     478, 32 x 4096 50.9 -> 50.2; three or five are no better.
     //   E4M3: the same as raw slots of half the size, all by the first loader.
-    // A unit's Q is requested (by the first loader) as soon as the QK^T of the unit before have let go of the buffer, if
-    // need be between the V loads of that unit's last tile.
     if (elect_one()) {
       const uint32_t mine = wid == 8 ? 0u : wid - 9u;
       constexpr uint32_t kRing = kFp8 ? kRawSlots : kSlots<kFp8>;
@@ -460,15 +488,13 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       const uint32_t lead_full0 = lead_bars + 8u * X_FULL, ring0 = smem_base + (kFp8 ? kOffRaw : kOffRing);
       const uint64_t keep = l2_policy_evict_normal(), last_use = l2_policy_evict_first();   // K: V follows a tile later; V: done with
       uint32_t slot = 0, par = 1, n_issued = 0, turn = 0;
-      uint32_t un = 0;                                      // units whose Q has been requested
       auto take = [&]() -> TileRef {
         TileRef x;
         x.valid = tile.valid;
-        x.np = 0; x.qrow = 0; x.first = x.last = false;
+        x.np = 0;
         x.bt = prm.block_table;
         if (x.valid) {
-          x.np = tile.np; x.first = tile.first; x.last = tile.last();
-          x.qrow = tile.u.b * prm.R + tile.u.r0 + rank * kCtaRows;
+          x.np = tile.np;
           x.bt = prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t;
           tile.next();
         }
@@ -478,20 +504,12 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       auto row_of = [&](int page) { return (kFp8 && (page < 0 || page >= prm.num_blocks) ? prm.num_blocks : page) * kPage; };
       auto advance = [&]() { if (++slot == kRing) { slot = 0; par ^= 1; } ++n_issued; if (++turn == kLoaders<kFp8>) turn = 0; };
       auto my_turn = [&]() { return kLoaders<kFp8> == 1 || turn == mine; };
-      auto issue_q = [&](int qrow) {
-        if (leader) mbar_arrive_expect_tx(bar(X_QFULL), 2 * kQBytes);
-#pragma unroll 1
-        for (int c = 0; c < kQBlocks; c += 3)
-          tma_load_3d_pair_hint(smem_base + kOffQ + c * kQBlockBytes, &q_map, 0, qrow, c, lead_bars + 8u * X_QFULL, last_use);
-        ++un;
-      };
       struct Pages { int a, b, c, d; };                    // of a tile
-      auto issue_v = [&](int np, Pages pg, int nxt_qrow, bool q_wanted, bool& q_out) {
+      auto issue_v = [&](int np, Pages pg) {
 #pragma unroll 1
         for (int i = 0; i < 2 * np; ++i) {
           const int nh = i & 1;
           if (my_turn()) {
-            if (q_wanted && !q_out && mbar_probe(bar(X_QFREE), (un - 1) & 1)) { issue_q(nxt_qrow); q_out = true; }
             const uint32_t dst = ring0 + slot * kBytes;
             const int row = row_of(pg.a);
             ok = mbar_wait(empty0 + 8 * slot, par);
@@ -522,21 +540,14 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         pg.d = x.np > 3 ? __ldg(x.bt + 3) : 0;
         return pg;
       };
+      if (mine == 0 && tile.valid)                          // the first unit's Q; the softmax warps ask for the others
+        request_q(q_map, smem_base, bars, lead_bars, leader, q_row_of(prm, tile.u, rank));
       TileRef cur = take();
-      Pages pg = get_pages(cur), pg_prev = {};              // on its way while Q is requested
+      Pages pg = get_pages(cur), pg_prev = {};
       int np_prev = 0;
       TileRef nxt = take();
-      bool q_out = false;                                   // the Q of the unit that starts next has been requested
       uint32_t pt = 0;
       while (ok && cur.valid) {
-        if (cur.first && mine == 0) {
-          if (!q_out) {
-            if (un > 0) ok = mbar_wait(bar(X_QFREE), (un - 1) & 1);
-            if (!ok) break;
-            issue_q(cur.qrow);
-          }
-          q_out = false;
-        }
         const bool odd = (cur.np * rank) & 1;                               // begins in the middle of a page
         const int chunks0 = odd || cur.np == 1 ? 1 : 2, chunks1 = min(cur.np - chunks0, 2);
         const int row0 = row_of(rank == 0 || cur.np == 1 ? pg.a : cur.np == 4 ? pg.c : pg.b) + (odd ? 32 : 0);
@@ -565,9 +576,8 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         }
         if (!ok) break;
         const TileRef nn = take();
-        // V of the tile before, and behind a unit's last K its own V
-        for (int k = cur.first ? 1 : 0; k < (cur.last ? 2 : 1) && ok; ++k)
-          issue_v(k == 0 ? np_prev : cur.np, k == 0 ? pg_prev : pg, nxt.qrow, k == 1 && mine == 0 && nxt.valid, q_out);
+        // V of the tile before (whatever unit that was in), and behind the part's last K its own V
+        for (int k = 0; k < (nxt.valid ? 1 : 2) && ok; ++k) issue_v(k == 0 ? np_prev : cur.np, k == 0 ? pg_prev : pg);
         np_prev = cur.np;
         pg_prev = pg;
         pg = pg_nxt;
@@ -582,7 +592,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           const uint32_t k = n_issued - 1 - i;
           if (kFp8 || (leader && k % kLoaders<kFp8> == mine)) mbar_wait(full0 + 8 * (k % kRing), (k / kRing) & 1);
         }
-        if (leader && un > 0) mbar_wait(bar(X_QFULL), (un - 1) & 1);
+        if (leader && mine == 0) mbar_wait(bar(X_QFULL), 0);
       }
     }
     __syncwarp();
@@ -594,21 +604,21 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     const int wt = ((wid - 10) % kWidenWarps) * 32 + lane;
     // `n` is the number of the slot, `pos` its place in the present phase (K of a tile: nine slots; V of one: two per page).
     uint32_t n = mine, pos = mine, len = kQBlocks;
-    int np_prev = 0;
-    int what = 0;                                        // 0: K of the tile, 1: V of the tile before, 2: V of the tile (unit's last)
-    while (ok && tile.valid) {
-      while (pos >= len) {                               // next phase
+    int np_prev = 0;                                     // pages of the tile before
+    int what = tile.valid ? 0 : 3;                       // 0: K of the tile, 1: V of the tile before, 2: V of the part's last tile, 3: done
+    while (ok) {
+      while (pos >= len && what != 3) {                  // next phase
         pos -= len;
-        if (what == 0 && !tile.first) { what = 1; len = 2 * np_prev; }
-        else if (what != 2 && tile.last()) { what = 2; len = 2 * tile.np; }
+        if (what == 0 && np_prev > 0) { what = 1; len = 2 * np_prev; }
+        else if (what == 2) what = 3;
         else {
           np_prev = tile.np;
           tile.next();
-          what = 0; len = kQBlocks;
-          if (!tile.valid) break;
+          if (tile.valid) { what = 0; len = kQBlocks; }
+          else { what = 2; len = 2 * np_prev; }
         }
       }
-      if (!tile.valid) break;
+      if (what == 3) break;
       const bool is_k = what == 0;
       const uint32_t rslot = n % kRawSlots, rpar = (n / kRawSlots) & 1;
       const uint32_t slot = n % kSlots<kFp8>, par = ((n / kSlots<kFp8>) & 1) ^ 1;
@@ -683,16 +693,16 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       uint32_t slot = 0, par = 0;
       uint32_t gs = 0, gp = 0, un = 0;                      // score tiles, P~V tiles, units so far
       auto advance = [&]() { if (++slot == kSlots<kFp8>) { slot = 0; par ^= 1; } };
-      int np_prev = 0;
-      bool fresh_prev = false;
+      int np_prev = 0;                                      // pages of the tile before, 0: there was none
+      bool fresh_prev = false;                              // it was its unit's first
       while (ok && tile.valid) {
-        if (tile.first) {
+        const int np = tile.np;
+        const bool first = tile.first;
+        if (first) {
           ok = mbar_wait(bar(X_QFULL), un & 1);
           if (!ok) break;
           ++un;
         }
-        const int np = tile.np;
-        const bool first = tile.first, last = tile.last();
         {
           const uint32_t sb = gs & 1;
           AMLA_STAMP(prm, part, 0, gs);
@@ -717,13 +727,13 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           }
           if (!ok) break;
           mma_commit_pair_multicast(bar(X_SFULL + sb), 3);
-          if (last) mma_commit_pair_multicast(bar(X_QFREE), 3);
           AMLA_STAMP(prm, part, 3, gs);
           ++gs;
         }
-        // O (+)= P~ V of the tile before, and behind a unit's last QK^T its own: per page two N = 256 products (128 columns
-        // from either CTA)
-        for (int k = first ? 1 : 0; k < (last ? 2 : 1) && ok; ++k) {
+        tile.next();
+        // O (+)= P~ V of the tile before, whatever unit that was in, and behind the part's last QK^T its own: per page two
+        // N = 256 products (128 columns from either CTA)
+        for (int k = np_prev == 0 ? 1 : 0; k < (tile.valid ? 1 : 2) && ok; ++k) {
           const int np_v = k == 0 ? np_prev : np;
           uint32_t acc = (k == 0 ? fresh_prev : first) ? 0u : 1u;
           AMLA_STAMP(prm, part, 4, gp);
@@ -751,7 +761,6 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         }
         np_prev = np;
         fresh_prev = first;
-        if (ok) tile.next();
       }
       if (!ok) report_timeout(prm.status);
     }
