@@ -237,10 +237,10 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     // Warp 7 asks for the next unit's Q as soon as the scores of a unit's last tile are there: the MMAs have then read Q.
     // It looks the unit up well before that.
     constexpr int kAsksForQ = 7;
-    UnitIter ahead = tile.units;
     uint32_t q_asked = 0;                                // units whose Q this warp has asked for
-    int q_next = -1;
+    int q_next = -1;                                     // first row of the next unit's Q
     auto look_ahead = [&]() {
+      UnitIter ahead = tile.units;                       // stands behind the unit that tile is in
       Unit n;
       q_next = ahead.next(n) ? q_row_of(prm, n, rank) : -1;
     };
@@ -440,30 +440,46 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       if (tid == 0 && leader) AMLA_STAMP(prm, part, 13, gs - 1);
       const bool valid = row < prm.R;
       const int col0 = 256 * khalf + 128 * grp;
-      const size_t prow = static_cast<size_t>(slot < 0 ? 0 : slot) * kRowBlock + rank * kCtaRows + r;   // row of the partial arrays
-      uint16_t* dst = slot < 0 ? reinterpret_cast<uint16_t*>(prm.out) + (static_cast<size_t>(u.b) * prm.R + (valid ? row : 0)) * kDv + col0
-                               : partial_halves(prm) + prow * kDv + col0;
+      const int prow0 = (slot < 0 ? 0 : slot) * kRowBlock + rank * kCtaRows;   // this CTA's first row of the partial arrays
+      // The warp's 32 rows x 64 columns at a time pass through the rows of the P buffer that belong to this row group (P~V has
+      // read them; the group writes them again only behind the next exchange), so that a store covers 128 bytes of eight rows:
+      // whole lines leave the SM at about twice the rate of 32-byte pieces of 32 rows.
+      const int row0 = u.r0 + rank * kCtaRows + (quarter & 1) * 32;       // this warp's first row within the sequence
+      uint16_t* const base = (slot < 0 ? reinterpret_cast<uint16_t*>(prm.out) + (static_cast<size_t>(u.b) * prm.R + row0) * kDv
+                                       : partial_halves(prm) + static_cast<size_t>(prow0 + (quarter & 1) * 32) * kDv) + col0;
+      const uint32_t stage = smem_base + kOffP + (2 * khalf + grp) * kPPageBytes + (quarter & 1) * 32 * 128;
       uint32_t sc = 0;                                    // this thread's four scale bytes
-      uint32_t o[2][32];
-      tmem_ld_32x32b_x32(o_addr, o[0]);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
+#pragma unroll 1
+      for (int c = 0; c < 4; c += 2) {
+        uint32_t o[2][32];
+        tmem_ld_32x32b_x32(o_addr + 32 * c, o[0]);
+        tmem_ld_32x32b_x32(o_addr + 32 * (c + 1), o[1]);
         tmem_wait_ld();
-        if (c + 1 < 4) tmem_ld_32x32b_x32(o_addr + 32 * (c + 1), o[(c + 1) & 1]);
-        uint32_t w[16];
-        if (slot < 0) epilogue_chunk_bf16(o[c & 1], inv, w);
-        else sc |= epilogue_chunk_partial(o[c & 1], inv, w) << (8 * c);
-        if (valid) {
-          stg_256(dst + 32 * c, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-          stg_256(dst + 32 * c + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          uint32_t w[16];
+          if (slot < 0) epilogue_chunk_bf16(o[e], inv, w);
+          else sc |= epilogue_chunk_partial(o[e], inv, w) << (8 * (c + e));
+#pragma unroll
+          for (int i = 0; i < 4; ++i) st_shared_v4(stage + sw128_offset(lane, 4 * e + i), w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int rr = 8 * i + (lane >> 2), piece = 2 * (lane & 3);
+          uint32_t x[8];
+          ld_shared_v4(stage + sw128_offset(rr, piece), x[0], x[1], x[2], x[3]);
+          ld_shared_v4(stage + sw128_offset(rr, piece + 1), x[4], x[5], x[6], x[7]);
+          if (row0 + rr < prm.R) stg_256(base + rr * kDv + 32 * c + 8 * piece, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+        }
+        __syncwarp();
       }
       tc_fence_before_sync();      // O has been read: this warp's next PREADY arrival lets the next unit overwrite it
       if (valid) {
-        if (slot >= 0) *reinterpret_cast<uint32_t*>(partial_scales(prm) + prow * 16 + col0 / 32) = sc;
+        if (slot >= 0) *reinterpret_cast<uint32_t*>(partial_scales(prm) + static_cast<size_t>(prow0 + r) * 16 + col0 / 32) = sc;
         if (khalf == 0 && grp == 0) {
           if (slot < 0) prm.lse[static_cast<size_t>(u.b) * prm.R + row] = lse;
-          else prm.part_lse[prow] = lse;
+          else prm.part_lse[prow0 + r] = lse;
         }
       }
       if (tid == 0 && leader) AMLA_STAMP(prm, part, 14, gs - 1);

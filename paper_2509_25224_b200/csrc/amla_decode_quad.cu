@@ -61,7 +61,8 @@ constexpr uint32_t kVHalfBytes = 2 * kBoxBytes;      // 64 keys x 128 columns: [
 constexpr uint32_t kVSlotBytes = 2 * kVHalfBytes;    // one page: this CTA's 128 columns of either 256-column half of V
 constexpr uint32_t kOffV = 0;
 constexpr uint32_t kOffP = kNumVSlots * kVSlotBytes;
-constexpr uint32_t kEndB = kOffP + kNumP * kPStride;
+constexpr uint32_t kOffOut = kOffP + kNumP * kPStride;   // [8 correction warps] x 2 KB: 16 rows x 64 columns of the epilogue on their way out
+constexpr uint32_t kEndB = kOffOut + 8 * 2048;
 // ---- all four: barriers at the same offset, so that one multicast commit reaches them
 constexpr uint32_t kOffBars = kEndA > kEndB ? kEndA : kEndB;
 constexpr uint32_t kBarBytes = 320;
@@ -800,37 +801,52 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           if (tid == 0) { QSTAMP(smem_base, 12, un); if (un < 1) QSTAMP_NS(smem_base, 3); };
           const int row = u.r0 + half * kRowBlock + r;               // this thread's row within the sequence
           const bool valid = row < prm.R;
-          __nv_bfloat16* orow = prm.out + (static_cast<size_t>(u.b) * prm.R + (valid ? row : 0)) * kDv;
-          const size_t prow = static_cast<size_t>(slot < 0 ? 0 : slot) * kItemRows + half * kRowBlock + r;   // row of the partial arrays
-          uint16_t* hrow = partial_halves(prm) + prow * kDv;
+          const int row0 = u.r0 + half * kRowBlock + (wid & 3) * 32;     // this warp's first row within the sequence
+          const int prow = (slot < 0 ? 0 : slot) * kItemRows + half * kRowBlock + r;   // row of the partial arrays
+          // 64 columns of 16 rows at a time pass through shared memory, so that a store covers 128 bytes of eight rows: whole
+          // lines leave the SM at about twice the rate of 32-byte pieces of 32 rows.
+          uint16_t* const base = (slot < 0 ? reinterpret_cast<uint16_t*>(prm.out) + (static_cast<size_t>(u.b) * prm.R + row0) * kDv
+                                           : partial_halves(prm) + static_cast<size_t>(prow - lane) * kDv) + 32 * c_first;
+          const uint32_t stage = smem_base + kOffOut + ((partner ? 4 : 0) + (wid & 3)) * 2048;
           uint32_t sc_lo = 0, sc_hi = 0;                                  // this thread's eight scale bytes
           uint32_t o[2][32];
           tmem_ld_32x32b_x32(tbase + lane_base + 32 * c_first, o[0]);
+          tmem_ld_32x32b_x32(tbase + lane_base + 32 * (c_first + 1), o[1]);
 #pragma unroll 1
           for (int cq = 0; cq < 8; cq += 2) {
+            uint32_t w[2][16];
+            tmem_wait_ld();
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-              tmem_wait_ld();
-              if (cq + e + 1 < 8) tmem_ld_32x32b_x32(tbase + lane_base + 32 * (c_first + cq + e + 1), o[e ^ 1]);
-              const int cc = c_first + cq + e;
-              uint32_t w[16];
-              uint16_t* dst;
               if (slot < 0) {
-                epilogue_chunk_bf16(o[e], inv, w);
-                dst = reinterpret_cast<uint16_t*>(orow) + 32 * cc;
+                epilogue_chunk_bf16(o[e], inv, w[e]);
               } else {
-                const uint32_t sb = epilogue_chunk_partial(o[e], inv, w);
+                const uint32_t sb = epilogue_chunk_partial(o[e], inv, w[e]);
                 if (cq + e < 4) sc_lo |= sb << (8 * (cq + e)); else sc_hi |= sb << (8 * (cq + e - 4));
-                dst = hrow + 32 * cc;
               }
-              if (valid) {
-                stg_256(dst, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-                stg_256(dst + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+              if (cq + 2 < 8) tmem_ld_32x32b_x32(tbase + lane_base + 32 * (c_first + cq + 2 + e), o[e]);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              if ((lane >> 4) == h) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                  st_shared_v4(stage + sw128_offset(lane & 15, i), w[i >> 2][4 * (i & 3)], w[i >> 2][4 * (i & 3) + 1], w[i >> 2][4 * (i & 3) + 2], w[i >> 2][4 * (i & 3) + 3]);
               }
+              __syncwarp();
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                const int sr = 8 * i + (lane >> 2), rr = 16 * h + sr, piece = 2 * (lane & 3);
+                uint32_t x[8];
+                ld_shared_v4(stage + sw128_offset(sr, piece), x[0], x[1], x[2], x[3]);
+                ld_shared_v4(stage + sw128_offset(sr, piece + 1), x[4], x[5], x[6], x[7]);
+                if (row0 + rr < prm.R) stg_256(base + rr * kDv + 32 * cq + 8 * piece, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+              }
+              __syncwarp();
             }
           }
           if (valid && slot >= 0)
-            *reinterpret_cast<uint2*>(partial_scales(prm) + prow * 16 + c_first) = make_uint2(sc_lo, sc_hi);
+            *reinterpret_cast<uint2*>(partial_scales(prm) + static_cast<size_t>(prow) * 16 + c_first) = make_uint2(sc_lo, sc_hi);
           if (valid && !partner) {
             if (slot < 0) prm.lse[static_cast<size_t>(u.b) * prm.R + row] = lse;
             else prm.part_lse[prow] = lse;
