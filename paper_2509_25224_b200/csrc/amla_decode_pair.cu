@@ -49,8 +49,8 @@ constexpr int kSoftmaxWarps = 8;
 // widen, three pairs taking turns.
 constexpr int kWidenGroups = 3, kWidenWarps = 2;
 constexpr int kWideners = kWidenGroups * kWidenWarps;
-template <bool kFp8> constexpr int kLoaders = kFp8 ? 1 : 4;
-template <bool kFp8> constexpr int kThreads = 32 * (kFp8 ? kSoftmaxWarps + 2 + kWideners : kSoftmaxWarps + 1 + kLoaders<false>);
+constexpr int kLoaders = 4;
+template <bool kFp8> constexpr int kThreads = 32 * (kFp8 ? kSoftmaxWarps + 2 + kWideners : kSoftmaxWarps + 1 + kLoaders);
 constexpr int kTilePages = 4;                           // pages of a score tile: N = 256, the widest MMA
 constexpr int kCtaRows = kRowBlock / 2;                 // query rows per CTA
 constexpr int kQBlocks = kDqk / 64;                     // 64-column blocks of Q and K
@@ -60,16 +60,16 @@ constexpr uint32_t kPPageBytes = kCtaRows * 128;        // P~ of one page: [64 r
 constexpr uint32_t kKBoxBytes = 32 * 128;               // half a page (32 keys) x one 64-column block
 constexpr uint32_t kSlotBytes = 128 * 128;              // K: half of 4 pages' keys x 64 columns; V: 64 keys x 128 columns
 constexpr uint32_t kVBlockBytes = 64 * 128;             // 64 keys x 64 columns
-// The ring of operand slots, and for an E4M3 cache a ring of raw slots in front of it, one for every operand slot.
+// The ring of operand slots, and for an E4M3 cache a ring of raw slots in front of it, one for every two operand slots.
 // A rule that every user of a ring keeps: a thread waits only for slots that it fills or empties itself, and having waited
 // for number w (counted over the whole run; slots are released in order) next for one of w + 1 ... w + R, R being the number
 // of slots.  The barriers tell two successive phases apart, no more: a thread that asks for a phase further on is let
 // through by an older one, and one that comes to ask after the next phase has passed as well is held for good.  (So the
-// four loaders take every fourth number on a ring of seven slots, and the three pairs that widen step by three through four operand slots,
-// and by three through six raw slots: raw slots fill out of order, and that makes each the business of one pair.)
+// four loaders take every fourth number on a ring of seven slots, and the three pairs that widen step by three through four operand
+// slots, and so by one or two through three raw slots.)
 template <bool kFp8> constexpr int kSlots = kFp8 ? 4 : 7;
-constexpr int kRawSlots = 2 * kWidenGroups;
-constexpr uint32_t kRawBytes = kSlotBytes / 2;
+constexpr int kRawSlots = 3;
+constexpr uint32_t kRawBytes = kSlotBytes;              // the bytes of two operand slots
 
 constexpr uint32_t kOffQ = 0;
 constexpr uint32_t kOffP = kOffQ + kQBytes;
@@ -108,13 +108,6 @@ template <bool kClusterAcquire = false>
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
   return __all_sync(0xffffffffu, mbar_wait<kClusterAcquire>(bar, parity));
 }
-
-// What the loader keeps of a score tile: where its pages stand in the block table, how many.
-struct TileRef {
-  const int32_t* bt;
-  int np;
-  bool valid;
-};
 
 using Tiles = TileIter<kTilePages>;
 
@@ -164,7 +157,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       if (kFp8) mbar_init(bar(X_FULLODD + i), kWidenWarps);
     }
     if (kFp8) {
-      for (int i = 0; i < kRawSlots; ++i) { mbar_init(bar(X_RAWFULL + i), 1); mbar_init(bar(X_RAWEMPTY + i), kWidenWarps); }
+      for (int i = 0; i < kRawSlots; ++i) { mbar_init(bar(X_RAWFULL + i), 1); mbar_init(bar(X_RAWEMPTY + i), 2 * kWidenWarps); }
     }
     mbar_init(bar(X_QFULL), 1);
     for (int i = 0; i < 2; ++i) {
@@ -495,136 +488,160 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     //     The loader warps walk the same sequence and issue every fourth load of it: a slot takes ~350 clk to issue, a warp by
     //     itself never waits for a slot.  Two -> four loaders: 16 x 16384 keys, rising 85.7 -> 83.3 us cool, 96 x 16384 488 ->
     //     478, 32 x 4096 50.9 -> 50.2; three or five are no better.
-    //   E4M3: the same as raw slots of half the size, all by the first loader.
+    //   E4M3: the same by one loader, into the raw ring.
     if (elect_one()) {
-      const uint32_t mine = wid == 8 ? 0u : wid - 9u;
-      constexpr uint32_t kRing = kFp8 ? kRawSlots : kSlots<kFp8>;
-      const uint32_t full0 = kFp8 ? bar(X_RAWFULL) : bar(X_FULL), empty0 = kFp8 ? bar(X_RAWEMPTY) : bar(X_EMPTY);
-      constexpr uint32_t kBytes = kFp8 ? kRawBytes : kSlotBytes;
-      const uint32_t lead_full0 = lead_bars + 8u * X_FULL, ring0 = smem_base + (kFp8 ? kOffRaw : kOffRing);
       const uint64_t keep = l2_policy_evict_normal(), last_use = l2_policy_evict_first();   // K: V follows a tile later; V: done with
-      uint32_t slot = 0, par = 1, n_issued = 0, turn = 0;
-      auto take = [&]() -> TileRef {
-        TileRef x;
-        x.valid = tile.valid;
-        x.np = 0;
-        x.bt = prm.block_table;
-        if (x.valid) {
-          x.np = tile.np;
-          x.bt = prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t;
-          tile.next();
-        }
-        return x;
-      };
       // first key row of a page; E4M3: a page outside the cache reads as zeros (rows behind the end of the tensor do)
       auto row_of = [&](int page) { return (kFp8 && (page < 0 || page >= prm.num_blocks) ? prm.num_blocks : page) * kPage; };
-      auto advance = [&]() { if (++slot == kRing) { slot = 0; par ^= 1; } ++n_issued; if (++turn == kLoaders<kFp8>) turn = 0; };
-      auto my_turn = [&]() { return kLoaders<kFp8> == 1 || turn == mine; };
-      struct Pages { int a, b, c, d; };                    // of a tile
-      auto issue_v = [&](int np, Pages pg) {
-#pragma unroll 1
-        for (int i = 0; i < 2 * np; ++i) {
-          const int nh = i & 1;
-          if (my_turn()) {
-            const uint32_t dst = ring0 + slot * kBytes;
-            const int row = row_of(pg.a);
-            ok = mbar_wait(empty0 + 8 * slot, par);
-            if (!ok) return;
-            if (kFp8) {
-              mbar_arrive_expect_tx(full0 + 8 * slot, kRawBytes);
-              tma_load_2d_hint(dst, &v_map, 256 * rank + 128 * nh, row, full0 + 8 * slot, last_use);            // [64 keys][128 columns]
-            } else {
-              if (leader) mbar_arrive_expect_tx(full0 + 8 * slot, 2 * kSlotBytes);
-              tma_load_3d_pair_hint(dst, &v_map, 0, row, 4 * rank + 2 * nh, lead_full0 + 8 * slot, last_use);
-            }
-          }
-          if (nh) { pg.a = pg.b; pg.b = pg.c; pg.c = pg.d; }
-          advance();
+      // The page numbers of a tile are loaded once, a tile ahead: a load of the block table in front of every slot cost a loader
+      // 500 clk there (a tile of the E4M3 cache took 11.9 K clk instead of 10.4 K).
+      static_assert(kTilePages == 4, "a tile's page numbers");
+      struct Pages { int a, b, c, d; };
+      auto take = [&](Pages& pg) {                          // pages of the next tile, 0: none
+        const int np = tile.valid ? tile.np : 0;
+        if (np > 0) {
+          const int32_t* bt = prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t;
+          pg.a = __ldg(bt);
+          pg.b = np > 1 ? __ldg(bt + 1) : 0;
+          pg.c = np > 2 ? __ldg(bt + 2) : 0;
+          pg.d = np > 3 ? __ldg(bt + 3) : 0;
+          tile.next();
         }
+        return np;
       };
       // This CTA's half of the tile's keys, 32 np of them from key 32 np rank on, is at most two boxes: a page, or the half page
       // in the middle of a tile of three pages or of one.  (With 32 keys of every page it was four boxes: E4M3, one loader:
       // 62.6 -> 61.2 us for 32 x 4096 keys, 120.1 -> 116.4 for 32 x 512-8192, two tokens; bf16 494 -> 481 for 96 x 16384.)
-      // The page numbers of a tile are loaded once, a tile ahead, and kept for its V: a load of the block table in front of
-      // every V slot cost the loaders 500 clk there: a tile of the E4M3 cache took 11.9 K clk instead of 10.4 K.
-      static_assert(kTilePages == 4, "a tile's page numbers");
-      auto get_pages = [&](const TileRef& x) {
-        Pages pg;
-        pg.a = x.np > 0 ? __ldg(x.bt) : 0;
-        pg.b = x.np > 1 ? __ldg(x.bt + 1) : 0;
-        pg.c = x.np > 2 ? __ldg(x.bt + 2) : 0;
-        pg.d = x.np > 3 ? __ldg(x.bt + 3) : 0;
-        return pg;
+      struct KBoxes {
+        const CUtensorMap *map0, *map1;
+        int row0, row1, chunks0, chunks1;                   // in chunks of 32 keys
       };
-      if (mine == 0 && tile.valid)                          // the first unit's Q; the softmax warps ask for the others
+      auto boxes = [&](int np, const Pages& pg) {
+        KBoxes x;
+        const bool odd = (np * rank) & 1;                                 // begins in the middle of a page
+        x.chunks0 = odd || np == 1 ? 1 : 2; x.chunks1 = min(np - x.chunks0, 2);
+        x.row0 = row_of(rank == 0 || np == 1 ? pg.a : np == 4 ? pg.c : pg.b) + (odd ? 32 : 0);
+        x.row1 = row_of(rank == 0 ? pg.b : np == 4 ? pg.d : pg.c);
+        x.map0 = x.chunks0 == 2 ? &k_map : &khalf_map;
+        x.map1 = x.chunks1 == 2 ? &k_map : &khalf_map;
+        return x;
+      };
+      const uint32_t lead_full = lead_bars + 8u * X_FULL;
+      if (wid == 8 && tile.valid)                           // the first unit's Q; the softmax warps ask for the others
         request_q(q_map, smem_base, bars, lead_bars, leader, q_row_of(prm, tile.u, rank));
-      TileRef cur = take();
-      Pages pg = get_pages(cur), pg_prev = {};
-      int np_prev = 0;
-      TileRef nxt = take();
-      uint32_t pt = 0;
-      while (ok && cur.valid) {
-        const bool odd = (cur.np * rank) & 1;                               // begins in the middle of a page
-        const int chunks0 = odd || cur.np == 1 ? 1 : 2, chunks1 = min(cur.np - chunks0, 2);
-        const int row0 = row_of(rank == 0 || cur.np == 1 ? pg.a : cur.np == 4 ? pg.c : pg.b) + (odd ? 32 : 0);
-        const int row1 = row_of(rank == 0 ? pg.b : cur.np == 4 ? pg.d : pg.c);
-        const CUtensorMap* const map0 = chunks0 == 2 ? &k_map : &khalf_map;
-        const CUtensorMap* const map1 = chunks1 == 2 ? &k_map : &khalf_map;
-        const Pages pg_nxt = get_pages(nxt);
+      uint32_t n = 0;                                       // slots so far
+      if constexpr (!kFp8) {
+        const uint32_t mine = wid == 8 ? 0 : wid - 9;
+        constexpr uint32_t kRing = kSlots<false>;
+        uint32_t slot = 0, par = 1, turn = 0;
+        auto advance = [&]() { if (++slot == kRing) { slot = 0; par ^= 1; } ++n; if (++turn == kLoaders) turn = 0; };
+        Pages pg = {}, pg_nxt = {}, pg_prev = {};
+        int np = take(pg), np_prev = 0;
+        KBoxes x = boxes(np, pg);
+        while (ok && np > 0) {
+          const int np_nxt = take(pg_nxt);
 #pragma unroll 1
-        for (int c = 0; c < kQBlocks; ++c) {
-          if (my_turn()) {
-            const uint32_t dst = ring0 + slot * kBytes;
-            ok = mbar_wait(empty0 + 8 * slot, par);
-            if (!ok) break;
-            if (leader && (c <= 1 || c >= 7)) AMLA_STAMP(prm, part, c <= 1 ? 16 : 17, pt);
-            if (kFp8) {
-              mbar_arrive_expect_tx(full0 + 8 * slot, cur.np * (kKBoxBytes / 2));
-              tma_load_2d_hint(dst, map0, 64 * c, row0, full0 + 8 * slot, keep);                                          // [64 or 32 keys][64 columns]
-              if (chunks1 > 0) tma_load_2d_hint(dst + chunks0 * (kKBoxBytes / 2), map1, 64 * c, row1, full0 + 8 * slot, keep);
-            } else {
-              if (leader) mbar_arrive_expect_tx(full0 + 8 * slot, 2 * cur.np * kKBoxBytes);
-              tma_load_3d_pair_hint(dst, map0, 0, row0, c, lead_full0 + 8 * slot, keep);
-              if (chunks1 > 0) tma_load_3d_pair_hint(dst + chunks0 * kKBoxBytes, map1, 0, row1, c, lead_full0 + 8 * slot, keep);
+          for (int c = 0; c < kQBlocks; ++c) {
+            if (turn == mine) {
+              ok = mbar_wait(bar(X_EMPTY) + 8 * slot, par);
+              if (!ok) break;
+              const uint32_t dst = smem_base + kOffRing + slot * kSlotBytes;
+              if (leader) mbar_arrive_expect_tx(bar(X_FULL) + 8 * slot, 2 * np * kKBoxBytes);
+              tma_load_3d_pair_hint(dst, x.map0, 0, x.row0, c, lead_full + 8 * slot, keep);
+              if (x.chunks1 > 0) tma_load_3d_pair_hint(dst + x.chunks0 * kKBoxBytes, x.map1, 0, x.row1, c, lead_full + 8 * slot, keep);
+            }
+            advance();
+          }
+          x = boxes(np_nxt, pg_nxt);
+          // V of the tile before (whatever unit that was in), and behind the part's last K its own V
+          for (int k = 0; k < (np_nxt > 0 ? 1 : 2) && ok; ++k) {
+            const int np_v = k == 0 ? np_prev : np;
+            if (k > 0) pg_prev = pg;
+#pragma unroll 1
+            for (int i = 0; i < 2 * np_v; ++i) {
+              if (turn == mine) {
+                ok = mbar_wait(bar(X_EMPTY) + 8 * slot, par);
+                if (!ok) break;
+                if (leader) mbar_arrive_expect_tx(bar(X_FULL) + 8 * slot, 2 * kSlotBytes);
+                tma_load_3d_pair_hint(smem_base + kOffRing + slot * kSlotBytes, &v_map, 0, pg_prev.a * kPage, 4 * rank + 2 * (i & 1), lead_full + 8 * slot, last_use);
+              }
+              if (i & 1) { pg_prev.a = pg_prev.b; pg_prev.b = pg_prev.c; pg_prev.c = pg_prev.d; }
+              advance();
             }
           }
-          advance();
+          np_prev = np; pg_prev = pg;
+          np = np_nxt; pg = pg_nxt;
         }
-        if (!ok) break;
-        const TileRef nn = take();
-        // V of the tile before (whatever unit that was in), and behind the part's last K its own V
-        for (int k = 0; k < (nxt.valid ? 1 : 2) && ok; ++k) issue_v(k == 0 ? np_prev : cur.np, k == 0 ? pg_prev : pg);
-        np_prev = cur.np;
-        pg_prev = pg;
-        pg = pg_nxt;
-        cur = nxt;
-        nxt = nn;
-        ++pt;
-      }
-      if (!ok) {
-        report_timeout(prm.status);
-        // let the copies that may still be in flight land before the CTA exits
-        for (uint32_t i = 0; i < kRing && i < n_issued; ++i) {
-          const uint32_t k = n_issued - 1 - i;
-          if (kFp8 || (leader && k % kLoaders<kFp8> == mine)) mbar_wait(full0 + 8 * (k % kRing), (k / kRing) & 1);
+        if (!ok) {
+          report_timeout(prm.status);
+          // let the copies that may still be in flight land before the CTA exits
+          for (uint32_t i = 0; i < kRing && i < n; ++i) {
+            const uint32_t k = n - 1 - i;
+            if (leader && k % kLoaders == mine) mbar_wait(bar(X_FULL) + 8 * (k % kRing), (k / kRing) & 1);
+          }
         }
-        if (leader && mine == 0) mbar_wait(bar(X_QFULL), 0);
+      } else {
+        uint32_t slot = 0, par = 1;
+        auto advance = [&]() { if (++slot == kRawSlots) { slot = 0; par ^= 1; } ++n; };
+        Pages pg = {}, pg_nxt = {}, pg_prev = {};
+        int np = take(pg), np_prev = 0;
+        while (ok && np > 0) {
+          const int np_nxt = take(pg_nxt);
+          const KBoxes x = boxes(np, pg);
+          // a raw slot is two column blocks of K (the last one by itself: its box reaches past the row's end, where there are zeros
+          // that nothing reads), or a page of V, this CTA's 256 columns of it
+#pragma unroll 1
+          for (int c = 0; c < kQBlocks; c += 2) {
+            const uint32_t full = bar(X_RAWFULL) + 8 * slot, dst = smem_base + kOffRaw + slot * kRawBytes;
+            ok = mbar_wait(bar(X_RAWEMPTY) + 8 * slot, par);
+            if (!ok) break;
+            mbar_arrive_expect_tx(full, np * kKBoxBytes);
+            tma_load_2d_hint(dst, x.map0, 64 * c, x.row0, full, keep);                                          // [64 or 32 keys][128 columns]
+            if (x.chunks1 > 0) tma_load_2d_hint(dst + x.chunks0 * kKBoxBytes, x.map1, 64 * c, x.row1, full, keep);
+            advance();
+          }
+          // V of the tile before (whatever unit that was in), and behind the part's last K its own V
+          for (int k = 0; k < (np_nxt > 0 ? 1 : 2) && ok; ++k) {
+            if (k > 0) pg_prev = pg;
+#pragma unroll 1
+            for (int i = k == 0 ? np_prev : np; i > 0; --i) {
+              const uint32_t full = bar(X_RAWFULL) + 8 * slot;
+              ok = mbar_wait(bar(X_RAWEMPTY) + 8 * slot, par);
+              if (!ok) break;
+              mbar_arrive_expect_tx(full, kRawBytes);
+              tma_load_2d_hint(smem_base + kOffRaw + slot * kRawBytes, &v_map, 256 * rank, row_of(pg_prev.a), full, last_use);   // [64 keys][256 columns]
+              pg_prev.a = pg_prev.b; pg_prev.b = pg_prev.c; pg_prev.c = pg_prev.d;
+              advance();
+            }
+          }
+          np_prev = np; pg_prev = pg;
+          np = np_nxt; pg = pg_nxt;
+        }
+        if (!ok) {
+          report_timeout(prm.status);
+          for (uint32_t i = 0; i < kRawSlots && i < n; ++i) mbar_wait(bar(X_RAWFULL) + 8 * ((n - 1 - i) % kRawSlots), ((n - 1 - i) / kRawSlots) & 1);
+        }
       }
+      if (!ok && leader && wid == 8) mbar_wait(bar(X_QFULL), 0);
     }
     __syncwarp();
   } else if (kFp8 && wid >= 10) {
     // ======================================================== E4M3 cache: raw slot -> operand slots.  The three pairs of
     // warps take every third operand slot each; a thread widens 16 bytes at a time (exact: E4M3 values are bf16 values)
-    // and stores them where the 128-byte swizzle of the operand tiles puts them.
+    // and stores them where the 128-byte swizzle of the operand tiles puts them.  (Raw slots of two operand slots: nine loads
+    // a tile instead of seventeen, of which one loader had its hands full; and no bank conflicts, which V's stores had: 32 x 4096
+    // keys 61.1 -> 60.5 us, 32 x 512-8192 with two tokens 122.2 -> 120.1.  A pair takes ~990 clk for an operand slot.)
     const uint32_t mine = (wid - 10) / kWidenWarps;
     const int wt = ((wid - 10) % kWidenWarps) * 32 + lane;
     // `n` is the number of the slot, `pos` its place in the present phase (K of a tile: nine slots; V of one: two per page).
-    uint32_t n = mine, pos = mine, len = kQBlocks;
+    // Two operand slots come from one raw slot, a tile's last block of K from one of its own.
+    uint32_t n = mine, pos = mine, len = kQBlocks, raw_phase = 0;     // raw_phase: raw slots before this phase
     int np_prev = 0;                                     // pages of the tile before
     int what = tile.valid ? 0 : 3;                       // 0: K of the tile, 1: V of the tile before, 2: V of the part's last tile, 3: done
     while (ok) {
       while (pos >= len && what != 3) {                  // next phase
         pos -= len;
+        raw_phase += (len + 1) >> 1;
         if (what == 0 && np_prev > 0) { what = 1; len = 2 * np_prev; }
         else if (what == 2) what = 3;
         else {
@@ -636,26 +653,33 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       }
       if (what == 3) break;
       const bool is_k = what == 0;
-      const uint32_t rslot = n % kRawSlots, rpar = (n / kRawSlots) & 1;
+      const uint32_t nth = raw_phase + (pos >> 1), second = pos & 1;
+      const uint32_t rslot = nth % kRawSlots, rpar = (nth / kRawSlots) & 1;
       const uint32_t slot = n % kSlots<kFp8>, par = ((n / kSlots<kFp8>) & 1) ^ 1;
       ok = warp_wait(bar(X_RAWFULL + rslot), rpar);
       if (ok) ok = warp_wait(bar(X_EMPTY + slot), par);
       if (!ok) break;
-      // K: row = page * 32 + key, 64 bytes, four threads a row (rows of pages that the tile does not have hold older bytes; the
-      // MMA does not read them).  V: 64 keys x 128 columns -> two blocks of 64 columns, eight threads a row.
+      // Four threads take 64 columns of a row.  The eight that access shared memory together are placed so that no two of them
+      // meet in a bank, neither in the load nor in the stores (whose rows alternate by the 128-byte swizzle):
+      //   K: raw rows of two blocks, 128 bytes, swizzled likewise, row = page * 32 + key (rows of pages that the tile does not
+      //      have hold older bytes; the MMA does not read them).  Rows a and a ^ 5: the other half of the banks in the raw
+      //      slot, odd against even in the operand slot.
+      //   V: raw rows of 256 bytes, 128 of them for this operand slot, 64 for each of its two blocks of 64 columns.  Rows a and
+      //      a + 1 and different blocks.
       const uint32_t raw = smem_base + kOffRaw + rslot * kRawBytes, out = smem_base + kOffRing + slot * kSlotBytes;
-      const int r0 = is_k ? wt >> 2 : wt >> 3;
+      const int other = (wt >> 2) & 1, vblock = is_k ? 0 : ((wt >> 3) & 1) ^ other;
+      const int r0 = is_k ? 8 * (wt >> 5) + (((wt >> 3) & 3) ^ (5 * other)) : 2 * (wt >> 4) + other;
       const uint32_t step = is_k ? 16 * 128 : 8 * 128;    // rows of a thread differ by multiples of 8: the same swizzle
-      const uint32_t src = raw + 16 * wt;                 // the pieces of a slot in order, 64 threads wide
+      const uint32_t src = raw + (is_k ? r0 * 128 + (((4 * second + (wt & 3)) ^ (r0 & 7)) << 4) : r0 * 256 + 128 * second + 64 * vblock + 16 * (wt & 3));
       const uint32_t ch = 2 * (wt & 3), sw = r0 & 7;
-      const uint32_t d0 = out + (is_k ? 0 : ((wt & 7) >> 2) * kVBlockBytes) + r0 * 128 + ((ch ^ sw) << 4);
+      const uint32_t d0 = out + vblock * kVBlockBytes + r0 * 128 + ((ch ^ sw) << 4);
       const uint32_t d1 = (((ch + 1) ^ sw) << 4) - ((ch ^ sw) << 4);
 #pragma unroll
       for (uint32_t h = 0; h < 8; h += 4) {               // eight pieces of 16 bytes, four requested at a time
         uint32_t x[4][4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x[k][0]), "=r"(x[k][1]), "=r"(x[k][2]), "=r"(x[k][3]) : "r"(src + (h + k) * 1024));
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x[k][0]), "=r"(x[k][1]), "=r"(x[k][2]), "=r"(x[k][3]) : "r"(src + (h + k) * 2048));
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           uint32_t w[8];
@@ -670,6 +694,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       if (lane == 0) {
         mbar_arrive(bar((leader ? X_FULL : X_FULLODD) + slot));
         mbar_arrive(bar(X_RAWEMPTY + rslot));
+        if (pos + 1 == len && second == 0) mbar_arrive(bar(X_RAWEMPTY + rslot));   // (a raw slot of one block)
       }
       pos += kWidenGroups;
       n += kWidenGroups;
@@ -813,13 +838,13 @@ cudaError_t launch_mode(const CUtensorMap& kmap, const CUtensorMap& khalf, const
 }
 
 // An E4M3 cache: rows of 576 bytes.
-bool encode_bytes(EncodeTiledFn encode, CUtensorMap* map, const void* base, cuuint64_t rows, cuuint32_t box_rows, cuuint32_t box_cols) {
+bool encode_bytes(EncodeTiledFn encode, CUtensorMap* map, const void* base, cuuint64_t rows, cuuint32_t box_rows, cuuint32_t box_cols, bool swizzle) {
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(kDqk), rows};
   const cuuint64_t strides[1] = {static_cast<cuuint64_t>(kDqk)};
   const cuuint32_t box[2] = {box_cols, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+                swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace
@@ -837,7 +862,9 @@ cudaError_t launch_decode_pair(const DecodeParams& prm, cudaStream_t stream, int
   const cuuint64_t keys = static_cast<cuuint64_t>(prm.num_blocks) * kPage;
   if (!encode_rows(encode, &qmap, prm.q, static_cast<cuuint64_t>(prm.B) * prm.R, kCtaRows, 3)) return cudaErrorInvalidValue;
   if (prm.kv8 != nullptr) {
-    if (!encode_bytes(encode, &kmap, prm.kv8, keys, 64, 64) || !encode_bytes(encode, &khalf, prm.kv8, keys, 32, 64) || !encode_bytes(encode, &vmap, prm.kv8, keys, 64, 128)) return cudaErrorInvalidValue;
+    if (!encode_bytes(encode, &kmap, prm.kv8, keys, 64, 128, true) || !encode_bytes(encode, &khalf, prm.kv8, keys, 32, 128, true) ||
+        !encode_bytes(encode, &vmap, prm.kv8, keys, 64, 256, false))
+      return cudaErrorInvalidValue;
     return launch_mode<true>(kmap, khalf, vmap, qmap, prm, stream);
   }
   if (!encode_rows(encode, &kmap, prm.kv, keys, 64, 1) || !encode_rows(encode, &khalf, prm.kv, keys, 32, 1) || !encode_rows(encode, &vmap, prm.kv, keys, 64, 2)) return cudaErrorInvalidValue;
