@@ -15,7 +15,7 @@
 // Warps 0-7 run Algorithm 2's recurrence (lines 5-12; four threads share a query row: lane half = half of a tile's keys,
 // warp group = even / odd pages), write P~ = bf16(P * S16) into the P buffer of their own CTA, apply the integer N to
 // the bit patterns of O when the row's reference moved (lines 13-16; Lemma 3.1) and run the epilogue (line 20).  They
-// never hand data to the other CTA.  Warps 8 and 10-12 load (TMA), warp 9 of the even CTA issues the MMAs for both.
+// never hand data to the other CTA.  Warps 8, 10 and 11 load (TMA), warp 9 of the even CTA issues the MMAs for both.
 // Order on the tensor pipe: QK^T(i + 1) before P~V(i) (the paper's [C1, C2, V1] order, Section 4.1), whether or not the two
 // tiles belong to one unit: the next unit's Q is asked for as soon as the scores of a unit's last tile are there, and its first
 // scores are made while those are worked on.  (Each unit a chain by itself: 1 x 2531 keys 13.09 -> 12.78 us, 29 x 238-661
@@ -45,11 +45,11 @@ using namespace sm100;
 namespace {
 
 constexpr int kSoftmaxWarps = 8;
-// bf16 cache: warps 8 and 10-12 load.  E4M3 cache: warp 8 loads (more warps would leave too few registers), warps 10-15
+// bf16 cache: warps 8, 10 and 11 load.  E4M3 cache: warp 8 loads (more warps would leave too few registers), warps 10-15
 // widen, three pairs taking turns.
 constexpr int kWidenGroups = 3, kWidenWarps = 2;
 constexpr int kWideners = kWidenGroups * kWidenWarps;
-constexpr int kLoaders = 4;
+constexpr int kLoaders = 3;
 template <bool kFp8> constexpr int kThreads = 32 * (kFp8 ? kSoftmaxWarps + 2 + kWideners : kSoftmaxWarps + 1 + kLoaders);
 constexpr int kTilePages = 4;                           // pages of a score tile: N = 256, the widest MMA
 constexpr int kCtaRows = kRowBlock / 2;                 // query rows per CTA
@@ -65,7 +65,7 @@ constexpr uint32_t kVBlockBytes = 64 * 128;             // 64 keys x 64 columns
 // for number w (counted over the whole run; slots are released in order) next for one of w + 1 ... w + R, R being the number
 // of slots.  The barriers tell two successive phases apart, no more: a thread that asks for a phase further on is let
 // through by an older one, and one that comes to ask after the next phase has passed as well is held for good.  (So the
-// four loaders take every fourth number on a ring of seven slots, and the three pairs that widen step by three through four operand
+// three loaders take every third number on a ring of seven slots, and the three pairs that widen step by three through four operand
 // slots, and so by one or two through three raw slots.)
 template <bool kFp8> constexpr int kSlots = kFp8 ? 4 : 7;
 constexpr int kRawSlots = 3;
@@ -485,10 +485,16 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     // ======================================================== TMA loads, in the order in which the MMAs use them:
     // K(0), K(1), V(0), K(2), V(1), ..., K(n-1), V(n-2), V(n-1), the tiles counted over all of the part's units.
     //   bf16: one ring of 16 KB slots carries K (one 64-column block of half the tile's keys) and V (one page x 128 columns).
-    //     The loader warps walk the same sequence and issue every fourth load of it: a slot takes ~350 clk to issue, a warp by
-    //     itself never waits for a slot.  Two -> four loaders: 16 x 16384 keys, rising 85.7 -> 83.3 us cool, 96 x 16384 488 ->
-    //     478, 32 x 4096 50.9 -> 50.2; three or five are no better.
-    //   E4M3: the same by one loader, into the raw ring.
+    //     The loader warps walk the same sequence and issue every third load of it: a slot takes ~350 clk to issue.
+    //     With each V load goes a request to bring an eighth of the next tile's K into L2.  A slot that waits for HBM turns
+    //     around in ~3000 clk, and while the ring is full of V, which L2 has, nothing is under way from HBM: the next K comes
+    //     from L2 by the time its turn in the ring is there.  32 x 4096 keys 56.3 -> 54.6 us, 96 x 2048 82.7 -> 81.0.  (The
+    //     contiguous form: asked for by the tensor map's boxes 55.8.  A tile earlier: 55.9, 96 x 2048 82.5: V is gone from L2
+    //     by the time it is wanted.  Rings for K and for V by themselves: 63-67, as either is too short for its latency.  V of
+    //     a tile between the K blocks of the one two after it: 57.0, rising logits 93 -> 100, the last tiles' V comes later.)
+    //     Four loaders -> three, which leaves merge blocks room beside a decode CTA: 53.9 -> 53.7, 1 x 2531 12.65 -> 12.55,
+    //     1 x 1500 12.08 -> 11.89.
+    //   E4M3: the same, by one loader into the raw ring.
     if (elect_one()) {
       const uint64_t keep = l2_policy_evict_normal(), last_use = l2_policy_evict_first();   // K: V follows a tile later; V: done with
       // first key row of a page; E4M3: a page outside the cache reads as zeros (rows behind the end of the tensor do)
@@ -564,6 +570,10 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
                 if (!ok) break;
                 if (leader) mbar_arrive_expect_tx(bar(X_FULL) + 8 * slot, 2 * kSlotBytes);
                 tma_load_3d_pair_hint(smem_base + kOffRing + slot * kSlotBytes, &v_map, 0, pg_prev.a * kPage, 4 * rank + 2 * (i & 1), lead_full + 8 * slot, last_use);
+                if (i < 2 * np_nxt) {                       // 16 rows of this CTA's half of the next tile's keys
+                  const int row = (i < 2 * x.chunks0 ? x.row0 : x.row1 - 32 * x.chunks0) + 16 * i;
+                  if (static_cast<uint32_t>(row) < static_cast<uint32_t>(prm.num_blocks * kPage)) bulk_prefetch_l2(prm.kv + static_cast<size_t>(row) * kDqk, 16 * kDqk * 2);
+                }
               }
               if (i & 1) { pg_prev.a = pg_prev.b; pg_prev.b = pg_prev.c; pg_prev.c = pg_prev.d; }
               advance();
