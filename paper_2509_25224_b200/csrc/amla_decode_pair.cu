@@ -66,7 +66,8 @@ constexpr uint32_t kVBlockBytes = 64 * 128;             // 64 keys x 64 columns
 // of slots.  The barriers tell two successive phases apart, no more: a thread that asks for a phase further on is let
 // through by an older one, and one that comes to ask after the next phase has passed as well is held for good.  (So the
 // three loaders take every third number on a ring of seven slots, and the three pairs that widen step by three through four operand
-// slots, and so by one or two through three raw slots.)
+// slots, and so by one or two through three raw slots.  Raw slots are filled in any order, since V comes from L2 and K from HBM, so
+// a pair waits for its operand slot first: that it is free says which raw slots had been full.)
 template <bool kFp8> constexpr int kSlots = kFp8 ? 4 : 7;
 constexpr int kRawSlots = 3;
 constexpr uint32_t kRawBytes = kSlotBytes;              // the bytes of two operand slots
@@ -666,8 +667,11 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       const uint32_t nth = raw_phase + (pos >> 1), second = pos & 1;
       const uint32_t rslot = nth % kRawSlots, rpar = (nth / kRawSlots) & 1;
       const uint32_t slot = n % kSlots<kFp8>, par = ((n / kSlots<kFp8>) & 1) ^ 1;
-      ok = warp_wait(bar(X_RAWFULL + rslot), rpar);
-      if (ok) ok = warp_wait(bar(X_EMPTY + slot), par);
+      // In this order.  Operand slot n is free: the MMAs have read number n - 4, and the raw slot in whose place this one stands
+      // held numbers up to n - 4 at most, so it had been full.  (The other way round the wait for the raw slot could be let through
+      // by the phase before that one's, when V has overtaken K.)
+      ok = warp_wait(bar(X_EMPTY + slot), par);
+      if (ok) ok = warp_wait(bar(X_RAWFULL + rslot), rpar);
       if (!ok) break;
       // Four threads take 64 columns of a row.  The eight that access shared memory together are placed so that no two of them
       // meet in a bank, neither in the load nor in the stores (whose rows alternate by the 128-byte swizzle):
