@@ -641,7 +641,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     // warps take every third operand slot each; a thread widens 16 bytes at a time (exact: E4M3 values are bf16 values)
     // and stores them where the 128-byte swizzle of the operand tiles puts them.  (Raw slots of two operand slots: nine loads
     // a tile instead of seventeen, of which one loader had its hands full; and no bank conflicts, which V's stores had: 32 x 4096
-    // keys 61.1 -> 60.5 us, 32 x 512-8192 with two tokens 122.2 -> 120.1.  A pair takes ~990 clk for an operand slot.)
+    // keys 61.1 -> 60.5 us, 32 x 512-8192 with two tokens 122.2 -> 120.1.)
     const uint32_t mine = (wid - 10) / kWidenWarps;
     const int wt = ((wid - 10) % kWidenWarps) * 32 + lane;
     // `n` is the number of the slot, `pos` its place in the present phase (K of a tile: nine slots; V of one: two per page).
@@ -688,20 +688,19 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       const uint32_t ch = 2 * (wt & 3), sw = r0 & 7;
       const uint32_t d0 = out + vblock * kVBlockBytes + r0 * 128 + ((ch ^ sw) << 4);
       const uint32_t d1 = (((ch + 1) ^ sw) << 4) - ((ch ^ sw) << 4);
+      // Eight pieces of 16 bytes, all requested before the first is widened (four at a time: 32 x 4096 keys 58.0 us, so 56.9; 32 x
+      // 512-8192 with two tokens 113.5 -> 111.3).  The raw slot is handed back at the end and not here: an arrival does not wait
+      // for loads whose data nobody has used yet, and the next load by TMA then overtook them.
+      uint32_t x[8][4];
 #pragma unroll
-      for (uint32_t h = 0; h < 8; h += 4) {               // eight pieces of 16 bytes, four requested at a time
-        uint32_t x[4][4];
+      for (int k = 0; k < 8; ++k) ld_shared_v4(src + k * 2048, x[k][0], x[k][1], x[k][2], x[k][3]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x[k][0]), "=r"(x[k][1]), "=r"(x[k][2]), "=r"(x[k][3]) : "r"(src + (h + k) * 2048));
+      for (int k = 0; k < 8; ++k) {
+        uint32_t w[8];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          uint32_t w[8];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) { w[2 * q] = e4m3x2_to_bf16x2(x[k][q]); w[2 * q + 1] = e4m3x2_to_bf16x2(x[k][q] >> 16); }
-          st_shared_v4(d0 + (h + k) * step, w[0], w[1], w[2], w[3]);
-          st_shared_v4(d0 + d1 + (h + k) * step, w[4], w[5], w[6], w[7]);
-        }
+        for (int q = 0; q < 4; ++q) { w[2 * q] = e4m3x2_to_bf16x2(x[k][q]); w[2 * q + 1] = e4m3x2_to_bf16x2(x[k][q] >> 16); }
+        st_shared_v4(d0 + k * step, w[0], w[1], w[2], w[3]);
+        st_shared_v4(d0 + d1 + k * step, w[4], w[5], w[6], w[7]);
       }
       fence_proxy_async_smem();
       __syncwarp();
