@@ -415,7 +415,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       }
       if (!ok) break;
       // ---- epilogue (line 20): out = O / (l * S16), lse = m + ln l.  Thread = row; the four threads of a row take 128
-      // of its 512 columns each and store them from registers with 256-bit stores (a full 32-byte sector per lane).
+      // of its 512 columns each.
       int2 info;
       const int slot = tile.units.slot_of(u, &info);
       if (tid == 0 && leader) merge_note(prm, part, u.it, info);
@@ -436,8 +436,9 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       const int col0 = 256 * khalf + 128 * grp;
       const int prow0 = (slot < 0 ? 0 : slot) * kRowBlock + rank * kCtaRows;   // this CTA's first row of the partial arrays
       // The warp's 32 rows x 64 columns at a time pass through the rows of the P buffer that belong to this row group (P~V has
-      // read them; the group writes them again only behind the next exchange), so that a store covers 128 bytes of eight rows:
-      // whole lines leave the SM at about twice the rate of 32-byte pieces of 32 rows.
+      // read them; the group writes them again only behind the next exchange), so that a store covers 128 bytes of four rows:
+      // whole lines leave the SM at about twice the rate of 32-byte pieces of 32 rows.  A lane stores 16 bytes, which is what `out`
+      // is aligned to (32 bytes of eight rows are no faster: 192 x 1-512 keys 43.98 us, so 44.00; 60 x 55, five tokens 48.2, 48.2).
       const int row0 = u.r0 + rank * kCtaRows + (quarter & 1) * 32;       // this warp's first row within the sequence
       uint16_t* const base = (slot < 0 ? reinterpret_cast<uint16_t*>(prm.out) + (static_cast<size_t>(u.b) * prm.R + row0) * kDv
                                        : partial_halves(prm) + static_cast<size_t>(prow0 + (quarter & 1) * 32) * kDv) + col0;
@@ -459,12 +460,11 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         }
         __syncwarp();
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int rr = 8 * i + (lane >> 2), piece = 2 * (lane & 3);
-          uint32_t x[8];
+        for (int i = 0; i < 8; ++i) {
+          const int rr = 4 * i + (lane >> 3), piece = lane & 7;
+          uint32_t x[4];
           ld_shared_v4(stage + sw128_offset(rr, piece), x[0], x[1], x[2], x[3]);
-          ld_shared_v4(stage + sw128_offset(rr, piece + 1), x[4], x[5], x[6], x[7]);
-          if (row0 + rr < prm.R) stg_256(base + rr * kDv + 32 * c + 8 * piece, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+          if (row0 + rr < prm.R) stg_128(base + rr * kDv + 32 * c + 8 * piece, x[0], x[1], x[2], x[3]);
         }
         __syncwarp();
       }

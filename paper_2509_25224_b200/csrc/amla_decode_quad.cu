@@ -791,7 +791,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         }
         if (!ok) break;
         // ---- epilogue (line 20): out = O / (l * S16).  Thread = row; a warp and its partner take eight 32-column
-        // chunks each, scale them and store them from registers with 256-bit stores (a full 32-byte sector per lane).
+        // chunks each.
         {
           const uint32_t gl = gt - 1;
           if (tid == 0) QSTAMP(smem_base, 14, un);
@@ -803,8 +803,10 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           const bool valid = row < prm.R;
           const int row0 = u.r0 + half * kRowBlock + (wid & 3) * 32;     // this warp's first row within the sequence
           const int prow = (slot < 0 ? 0 : slot) * kItemRows + half * kRowBlock + r;   // row of the partial arrays
-          // 64 columns of 16 rows at a time pass through shared memory, so that a store covers 128 bytes of eight rows: whole
-          // lines leave the SM at about twice the rate of 32-byte pieces of 32 rows.
+          // 64 columns of 16 rows at a time pass through shared memory, so that a store covers 128 bytes of four rows: whole
+          // lines leave the SM at about twice the rate of 32-byte pieces of 32 rows.  A lane stores 16 bytes, which is what `out` is
+          // aligned to (32 bytes of eight rows are no faster: 64 x 1-8 K keys, two tokens 194.3 us, so 194.9, runs of one side
+          // differing by 1.5).
           uint16_t* const base = (slot < 0 ? reinterpret_cast<uint16_t*>(prm.out) + (static_cast<size_t>(u.b) * prm.R + row0) * kDv
                                            : partial_halves(prm) + static_cast<size_t>(prow - lane) * kDv) + 32 * c_first;
           const uint32_t stage = smem_base + kOffOut + ((partner ? 4 : 0) + (wid & 3)) * 2048;
@@ -835,12 +837,11 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
               }
               __syncwarp();
 #pragma unroll
-              for (int i = 0; i < 2; ++i) {
-                const int sr = 8 * i + (lane >> 2), rr = 16 * h + sr, piece = 2 * (lane & 3);
-                uint32_t x[8];
+              for (int i = 0; i < 4; ++i) {
+                const int sr = 4 * i + (lane >> 3), rr = 16 * h + sr, piece = lane & 7;
+                uint32_t x[4];
                 ld_shared_v4(stage + sw128_offset(sr, piece), x[0], x[1], x[2], x[3]);
-                ld_shared_v4(stage + sw128_offset(sr, piece + 1), x[4], x[5], x[6], x[7]);
-                if (row0 + rr < prm.R) stg_256(base + rr * kDv + 32 * cq + 8 * piece, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+                if (row0 + rr < prm.R) stg_128(base + rr * kDv + 32 * cq + 8 * piece, x[0], x[1], x[2], x[3]);
               }
               __syncwarp();
             }

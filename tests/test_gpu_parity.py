@@ -408,6 +408,40 @@ def test_error_codes_on_device():
     assert e.value.code == -1
 
 
+# rows that end inside a staged block of the epilogue; 128 heads x 3 tokens are three full blocks
+@pytest.mark.parametrize("entry,Sq,H,kernel", [("workspace", 1, 100, 128), ("workspace", 1, 65, 128), ("workspace", 3, 128, 128), ("workspace", 2, 75, 256),
+                                               ("workspace", 2, 128, 256), ("workspace", 1, 16, 32), ("static", 1, 127, 128), ("static", 2, 100, 256),
+                                               ("fp8", 1, 100, 128), ("fp8", 2, 128, 128)])
+def test_outputs_that_begin_at_16_bytes(entry, Sq, H, kernel):
+    # `out` need not be aligned to more than 16 bytes: a view that begins 8 elements into its buffer gets the bits that an
+    # allocation of its own gets, from whole items and from merged ones, and nothing is written in front of it or behind it
+    import torch
+    lens = np.concatenate([np.random.default_rng(Sq * H).integers(0, 500, 90), [3000, 1, 64]])
+    w = synth.make_workload("o16", len(lens), Sq, H, lens, seed=640 + Sq * H)
+    if kernel == 256:
+        wide_table(w, 64)
+    q, kv, bt, sl = to_device(w)
+    if entry == "fp8":
+        kv = torch.from_numpy(synth.quantise_cache_e4m3(w, 1.0 / 64.0)).to(q.device)
+    numel = w.B * Sq * H * 512
+    results = []
+    for first in (16, 8):
+        buf = torch.full((numel + 64,), 7.0, dtype=torch.bfloat16, device=q.device)
+        out = buf[first:first + numel].view(w.B, Sq, H, 512)
+        lse = torch.full((w.B, Sq, H), float("nan"), dtype=torch.float32, device=q.device)
+        assert out.data_ptr() % 32 == 2 * first % 32
+        if entry == "fp8":
+            binding.mla_decode_fp8(q, kv, 1.0 / 64.0, bt, sl, w.scale, out, lse)
+        elif entry == "static":
+            binding.mla_decode_static(q, kv, bt, sl, w.scale, out, lse)
+        else:
+            binding.mla_decode(q, kv, bt, sl, w.scale, out, lse)
+        assert binding.last_item_rows() == kernel
+        assert bool((buf[:first] == 7.0).all()) and bool((buf[first + numel:] == 7.0).all())
+        results.append((out.clone().view(torch.int16), lse))
+    assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
+
+
 # ----------------------------------------------------------------- the five named configurations, at full size,
 # every output element against the oracle (the launch configuration bench.py times)
 
