@@ -271,6 +271,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         if (tid == 0 && leader) AMLA_STAMP(prm, part, 8, gs);
         if (wid == kAsksForQ && tile.last() && q_next >= 0) {
           if (lane == 0) request_q(q_map, smem_base, bars, lead_bars, leader, q_next);
+          __syncwarp();                                    // the loads from tensor memory below are the whole warp's
           ++q_asked;
         }
         // A lane half holds 32 np neighbouring keys; this group takes its 32-key chunks grp and grp + 2.  The scores are
