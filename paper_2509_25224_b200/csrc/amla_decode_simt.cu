@@ -70,10 +70,11 @@ __global__ void __launch_bounds__(kWarps * 32) decode_simt_kernel(DecodeParams p
       for (int t = t0; t < t1; ++t) {
         __syncthreads();
         const int page = bt[t];
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(prm.kv + static_cast<size_t>(page) * kPage * kDqk);
+        const bool in_cache = page >= 0 && page < prm.num_blocks;          // else a page of zeros, as the TMA loads give it
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(prm.kv + static_cast<size_t>(in_cache ? page : 0) * kPage * kDqk);
         for (int i = tid; i < kPage * kQStrideW; i += blockDim.x) {
           const int j = i / kQStrideW, w = i % kQStrideW;
-          Ksm[j * kKStrideW + w] = src[i];
+          Ksm[j * kKStrideW + w] = in_cache ? src[i] : 0u;
         }
         __syncthreads();
 #pragma unroll

@@ -1,6 +1,8 @@
 """Helpers for the GPU parity tests: run a synth.Workload through the C-ABI and compare with the
 FP64 oracle under the three tolerances (max |err| <= 2e-2 and relative L2 <= 5e-3 on the bf16
 output, |lse err| <= 1e-3)."""
+import dataclasses
+
 import numpy as np
 
 from oracle import reference as R
@@ -54,6 +56,24 @@ def repeated(w, times):
     w.block_table = np.ascontiguousarray(np.tile(w.block_table, (times, 1)))
     w.seqlens = np.ascontiguousarray(np.tile(w.seqlens, times))
     return w
+
+
+def outside_the_cache(w, beyond):
+    """(w with every second page that its sequences use outside the cache: the page `beyond` the last one, None: page -1; the same
+    with those pages inside a cache that ends with a page of zeros, for the oracle)."""
+    n = w.num_blocks
+    bad, ref = w.block_table.copy(), w.block_table.copy()
+    for b, length in enumerate(w.seqlens):
+        bad[b, 0:(length + 63) // 64:2] = -1 if beyond is None else n + beyond
+        ref[b, 0:(length + 63) // 64:2] = n
+    zeros = np.zeros((1,) + w.kv.shape[1:], w.kv.dtype)
+    return dataclasses.replace(w, block_table=bad), dataclasses.replace(w, block_table=ref, kv=np.concatenate([w.kv, zeros]))
+
+
+def check_pages_outside_the_cache(w, beyond, flags=None, kernel=None):
+    """A page outside the cache reads as a page of zeros, and nothing faults."""
+    bad, ref = outside_the_cache(w, beyond)
+    check_full(bad, flags, kernel=kernel, ref=R.decode(ref.q, ref.kv, ref.block_table, ref.seqlens, ref.scale))
 
 
 def compare(out, lse, ref_out, ref_lse, what="", tol_abs=TOL_ABS):

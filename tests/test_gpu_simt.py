@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 from paper_2509_25224_b200 import binding, synth
-from tests._gpu_util import check_full
+from tests._gpu_util import check_full, check_pages_outside_the_cache
 
 pytestmark = pytest.mark.gpu
 SIMT = binding.FLAG_KERNEL_SIMT
@@ -26,3 +26,8 @@ def test_simt_ragged_and_split(mode):
 def test_simt_staircase_rescale():
     w = synth.config_stress(B=1, N=2048)
     check_full(w, SIMT)
+
+
+@pytest.mark.parametrize("beyond", [0, 100000, None])
+def test_simt_pages_outside_the_cache(beyond):
+    check_pages_outside_the_cache(synth.make_workload("oob", 3, 1, 40, [300, 65, 64], seed=105), beyond, SIMT)
