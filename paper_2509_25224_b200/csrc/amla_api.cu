@@ -209,21 +209,29 @@ extern "C" int amla_mla_decode_workspace_size(int B, int Sq, int H, int max_bloc
 
 namespace {
 
+// What can be said about a call's arguments without a device.
+int check_arguments(const void* q, const void* cache, const int32_t* block_table, const int32_t* seqlens, float softmax_scale, int B, int Sq, int H,
+                    int num_blocks, int max_blocks_per_seq, const void* out, const float* lse, const void* workspace, int flags) {
+  if (!q || !cache || !block_table || !seqlens || !out || !lse || !workspace) return AMLA_ERR_INVALID_ARG;
+  if (num_blocks <= 0 || !(softmax_scale == softmax_scale)) return AMLA_ERR_INVALID_ARG;
+  const int rc = check_shape(B, Sq, H, max_blocks_per_seq);
+  if (rc != AMLA_OK) return rc;
+  if ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(cache) | reinterpret_cast<uintptr_t>(out)) & 15) return AMLA_ERR_INVALID_ARG;
+  if ((reinterpret_cast<uintptr_t>(block_table) | reinterpret_cast<uintptr_t>(seqlens) | reinterpret_cast<uintptr_t>(lse)) & 3)
+    return AMLA_ERR_INVALID_ARG;
+  if (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) return AMLA_ERR_INVALID_ARG;
+  if ((flags & AMLA_RESCALE_MASK) == 3) return AMLA_ERR_INVALID_ARG;
+  return AMLA_OK;
+}
+
 // The decode call on a bf16 cache (kv_cache) or an E4M3 cache (kv8).  out_scale multiplies the normalised output (1 unless the cache was widened from
 // FP8 with a dequantisation scale); launches are added to g_last_launches.
 int decode_impl(const void* q, const void* kv_cache, const uint8_t* kv8, const int32_t* block_table, const int32_t* seqlens,
                 float softmax_scale, float out_scale, int B, int Sq, int H, int num_blocks, int max_blocks_per_seq,
                 void* out, float* lse, void* workspace, size_t workspace_bytes, void* cuda_stream, int flags) {
-  if (!q || (!kv_cache && !kv8) || !block_table || !seqlens || !out || !lse || !workspace) return AMLA_ERR_INVALID_ARG;
-  if (num_blocks <= 0 || !(softmax_scale == softmax_scale)) return AMLA_ERR_INVALID_ARG;
-  int rc = check_shape(B, Sq, H, max_blocks_per_seq);
+  int rc = check_arguments(q, kv8 ? static_cast<const void*>(kv8) : kv_cache, block_table, seqlens, softmax_scale, B, Sq, H, num_blocks, max_blocks_per_seq,
+                           out, lse, workspace, flags);
   if (rc != AMLA_OK) return rc;
-  if ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(kv_cache) | reinterpret_cast<uintptr_t>(out)) & 15)
-    return AMLA_ERR_INVALID_ARG;
-  if ((reinterpret_cast<uintptr_t>(block_table) | reinterpret_cast<uintptr_t>(seqlens) | reinterpret_cast<uintptr_t>(lse)) & 3)
-    return AMLA_ERR_INVALID_ARG;
-  if (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) return AMLA_ERR_INVALID_ARG;
-  if ((flags & AMLA_RESCALE_MASK) == 3) return AMLA_ERR_INVALID_ARG;
 
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) { cudaGetLastError(); return AMLA_ERR_CUDA; }
@@ -310,12 +318,10 @@ extern "C" int amla_mla_decode_fp8(const void* q, const void* kv_cache_e4m3, flo
                                    int max_blocks_per_seq, void* out, float* lse, void* workspace, size_t workspace_bytes,
                                    void* cuda_stream, int flags) {
   g_last_launches = 0;
-  if (!q || !kv_cache_e4m3 || !block_table || !seqlens || !out || !lse || !workspace) return AMLA_ERR_INVALID_ARG;
-  if (num_blocks <= 0 || !(kv_scale == kv_scale) || !(softmax_scale == softmax_scale)) return AMLA_ERR_INVALID_ARG;
-  if (reinterpret_cast<uintptr_t>(kv_cache_e4m3) & 15) return AMLA_ERR_INVALID_ARG;
-  if (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) return AMLA_ERR_INVALID_ARG;
-  int rc = check_shape(B, Sq, H, max_blocks_per_seq);
+  // (all of it here: the widening kernel is launched ahead of decode_impl)
+  int rc = check_arguments(q, kv_cache_e4m3, block_table, seqlens, softmax_scale, B, Sq, H, num_blocks, max_blocks_per_seq, out, lse, workspace, flags);
   if (rc != AMLA_OK) return rc;
+  if (!(kv_scale == kv_scale) || !(softmax_scale * kv_scale == softmax_scale * kv_scale)) return AMLA_ERR_INVALID_ARG;
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) { cudaGetLastError(); return AMLA_ERR_CUDA; }
   size_t base = 0;

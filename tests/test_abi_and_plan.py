@@ -60,6 +60,21 @@ def test_null_and_bad_arguments_are_rejected_before_any_cuda_call(lib):
     assert lib.amla_mla_decode_workspace_size(1, 1, 16, 4, 0, None) == -1
 
 
+def test_e4m3_arguments_are_rejected_before_any_cuda_call(lib):
+    # also those that only the decode behind the widening of the pages looks at
+    ok = {"q": 256, "kv": 256, "bt": 256, "sl": 256, "out": 256, "lse": 256, "ws": 256, "flags": 0}
+
+    def call(kv_scale=1.0, scale=0.1, **change):
+        a = dict(ok, **change)
+        return lib.amla_mla_decode_fp8(a["q"], a["kv"], kv_scale, a["bt"], a["sl"], scale, 4, 8, 128, 4096, 2048, a["out"], a["lse"], a["ws"], 1 << 40, None, a["flags"])
+
+    for name, bad in (("q", 264), ("kv", 264), ("out", 264), ("bt", 258), ("sl", 258), ("lse", 258), ("ws", 384), ("flags", 3)):
+        assert call(**{name: bad}) == -1, name
+        if name != "flags":
+            assert call(**{name: None}) == -1, name
+    assert call(kv_scale=float("nan")) == -1 and call(scale=float("nan")) == -1
+
+
 def _check_plan(seqlens, Sq, H, P):
     units = binding.plan_host(seqlens, Sq, H, P)
     item_rows, tile_keys, UNIT_OVERHEAD = _variant(Sq, H)
