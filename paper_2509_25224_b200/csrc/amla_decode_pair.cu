@@ -229,14 +229,23 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     const uint32_t o_addr = tbase + lane_base + kOCol + 128 * grp;     // this thread's 128 of the row's 512 columns
     uint32_t gs = 0, xc = 0;                             // score tiles and exchanges so far
     // Warp 7 asks for the next unit's Q as soon as the scores of a unit's last tile are there: the MMAs have then read Q.
-    // It looks the unit up well before that.
+    // It looks the unit up well before that.  A unit of one tile has its scores while this warp is still at the unit before:
+    // then it asks ahead of that one's epilogue, since that unit's P~V is followed by the Q K^T that the Q is for and the last
+    // P~V of the one-tile unit stands behind that.  (With inputs that are not in L2, asked for behind the epilogue and so: 60 x 55
+    // keys, five tokens 48.2 -> 43.8 us, E4M3 53.6 -> 48.3; 150 x 1-128, two tokens 50.0 -> 46.0; 192 x 1-512 43.8 -> 42.2.)
     constexpr int kAsksForQ = 7;
     uint32_t q_asked = 0;                                // units whose Q this warp has asked for
-    int q_next = -1;                                     // first row of the next unit's Q
+    int q_next = -1;                                     // first row of the next unit's Q, -1: there is none, or it has been asked for
     auto look_ahead = [&]() {
       UnitIter ahead = tile.units;                       // stands behind the unit that tile is in
       Unit n;
       q_next = ahead.next(n) ? q_row_of(prm, n, rank) : -1;
+    };
+    auto ask_for_q = [&]() {                             // the scores of the last tile before that unit are there
+      if (lane == 0) request_q(q_map, smem_base, bars, lead_bars, leader, q_next);
+      __syncwarp();                                      // what follows is the whole warp's
+      ++q_asked;
+      q_next = -1;
     };
     if (wid == kAsksForQ && tile.valid) look_ahead();
     // tells the row's other three threads `mine`; v[0..3] = what the four told
@@ -269,11 +278,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         if (!ok) break;
         tc_fence_after_sync();
         if (tid == 0 && leader) AMLA_STAMP(prm, part, 8, gs);
-        if (wid == kAsksForQ && tile.last() && q_next >= 0) {
-          if (lane == 0) request_q(q_map, smem_base, bars, lead_bars, leader, q_next);
-          __syncwarp();                                    // the loads from tensor memory below are the whole warp's
-          ++q_asked;
-        }
+        if (wid == kAsksForQ && tile.last() && q_next >= 0) ask_for_q();
         // A lane half holds 32 np neighbouring keys; this group takes its 32-key chunks grp and grp + 2.  The scores are
         // read from tensor memory twice, a chunk at a time: for the maximum, and for the exponentials once the P buffer is
         // free.  (Held in registers in between they cost 64 more of them and twice the code.)
@@ -425,6 +430,11 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       float l4[4];
       exchange(st.l, l4);
       if (!ok) break;
+      if (wid == kAsksForQ && tile.valid && tile.last() && q_next >= 0) {      // (its Q K^T is in front of the P~V that is waited for next)
+        ok = warp_wait(bar(X_SFULL + (gs & 1)), (gs >> 1) & 1);
+        if (!ok) break;
+        ask_for_q();
+      }
       const float l_all = (l4[0] + l4[1]) + (l4[2] + l4[3]);
       const bool live = l_all > 0.f;
       const float inv = live ? prm.out_scale / (l_all * st.s_out) : 0.f;

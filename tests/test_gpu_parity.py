@@ -248,6 +248,23 @@ def test_128_row_kernel_rescales_over_tiles_of_every_width(fp8):
             check_full(w, mode, kernel=128, ref=ref)
 
 
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("pages", [(1, 1, 1), (4, 1, 5), (1, 9, 1, 1), (5, 6, 1, 4, 1)])
+def test_128_row_kernel_units_of_one_tile_and_of_more_behind_one_another(pages, fp8):
+    # the Q of a unit is asked for ahead of the epilogue of the unit two before it where one tile is all that lies between, and
+    # within the unit before it else; 300 sequences, several units in every part; the last key of a page's first or second half
+    import torch
+    parts = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    lens = [64 * (pages[i % len(pages)] - 1) + (33, 64, 1, 32)[i % 4] for i in range(300)]
+    w = synth.make_workload("tiles", 300, 1, 100, lens, seed=495 + len(pages))
+    units = binding.plan_host(w.seqlens, 1, 100, parts)
+    assert np.bincount(units[:, 0]).max() >= 4 and min(_unit_pages(w, parts)) == 1
+    if fp8:
+        _check_fp8(w)
+    else:
+        check_full(w, kernel=128)
+
+
 @pytest.mark.parametrize("B,Sq,H,n", [(1, 1, 128, 400), (1, 1, 40, 4500), (1, 1, 128, 12000), (9, 1, 128, 1500), (11, 1, 128, 1500), (36, 1, 33, 700),
                                       (1, 1, 16, 20000), (36, 2, 16, 900), (75, 1, 16, 700)])
 def test_merges_by_rows_and_by_quarters_of_rows(B, Sq, H, n):
