@@ -7,6 +7,7 @@ from oracle import amla_sim as S
 from oracle import reference as R
 from paper_2509_25224_b200 import binding, synth
 from tests._gpu_util import check_full, check_sampled, repeated, run_gpu, to_device, wide_table
+from tests._gpu_util import check_pages_outside_the_cache, outside_the_cache
 
 pytestmark = pytest.mark.gpu
 
@@ -133,6 +134,26 @@ def test_fp8_cache_widened_ahead_of_large_calls_of_many_rows(Sq, width, launches
     lens = [300, 0, 65, 1000]
     w = synth.make_workload("f8w", 4, Sq, 128, lens, seed=610 + Sq, spare_blocks=2 * width, max_blocks_per_seq=width)
     _check_fp8(w)
+    assert binding.last_launch_count() == launches
+
+
+@pytest.mark.parametrize("beyond", [0, 100000, None])
+@pytest.mark.parametrize("Sq,H,kernel", [(1, 16, 32), (1, 100, 128), (2, 128, 256)])
+def test_pages_outside_a_bf16_cache_are_pages_of_zeros(Sq, H, kernel, beyond):
+    # the first, the last and every second page between (the 128-row kernel also asks for the next tile's pages ahead of their loads)
+    w = synth.make_workload("oob", 4, Sq, H, [1500, 65, 64, 900], seed=620 + H)
+    check_pages_outside_the_cache(wide_table(w) if kernel == 256 else w, beyond, kernel=kernel)
+
+
+@pytest.mark.parametrize("beyond", [0, 100000, None])
+@pytest.mark.parametrize("Sq,width,launches", [(1, 24, 2), (6, 342, 3)])
+def test_pages_outside_an_e4m3_cache_are_pages_of_zeros(Sq, width, launches, beyond):
+    # widened on their way in, and into a copy ahead of the call
+    w = synth.make_workload("oob8", 4, Sq, 128, [1500, 65, 64, 900], seed=625, spare_blocks=2 * width, max_blocks_per_seq=width)
+    kv8 = synth.quantise_cache_e4m3(w, 1.0 / 64.0)
+    bad, ref = outside_the_cache(w, beyond)
+    ref8 = np.concatenate([kv8, np.zeros((1, 64, 576), np.uint8)])
+    _check_fp8(bad, kv8=kv8, ref=R.decode_fp8(ref.q, ref8, 1.0 / 64.0, ref.block_table, ref.seqlens, ref.scale))
     assert binding.last_launch_count() == launches
 
 

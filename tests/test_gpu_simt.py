@@ -4,7 +4,8 @@ import numpy as np
 import pytest
 
 from paper_2509_25224_b200 import binding, synth
-from tests._gpu_util import check_full, check_pages_outside_the_cache
+from tests._gpu_util import check_full
+from tests._gpu_util import check_pages_outside_the_cache
 
 pytestmark = pytest.mark.gpu
 SIMT = binding.FLAG_KERNEL_SIMT
