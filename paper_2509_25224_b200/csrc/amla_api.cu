@@ -96,6 +96,9 @@ void profile_mark(int i, cudaStream_t stream) {
 // further item that a part begins.  What either takes was measured over 1-200 sequences of 64-60000 keys and 2-8 tokens:
 //   256 rows: 21.5 us + 2.08 us per 128-key tile of a part + 11 us per item of a part beyond the first
 //   128 rows: 13 us + 1.41 us per page of a part + 6 us per item of a part
+// (The figures are from before units of the 128-row kernel ran into one another and the next tile's K came by way of L2.  70 shapes
+// in short bursts since: 21.0 + 1.99 + 10.4 and 13.5 + 1.11 + 5.8.  Which calls take which kernel has not been gone over with that:
+// long calls run at the power limit, where reading the cache once counts for more than a burst shows.)
 // e.g. (two tokens, 128 heads) 1 x 3000 keys 22.0 against 15.7 us, 32 x 256 23.4 / 21.8, 32 x 2000 49 / 57, 1 x 60000 47.9 / 48.8.
 // Lengths are not known here: the block table's width bounds them.
 static bool blocks_of_256(const DecodeParams& prm, int pair_parts, int quad_parts) {
@@ -283,7 +286,7 @@ int decode_impl(const void* q, const void* kv_cache, const uint8_t* kv8, const i
 // 566 / 488; but five and less differ by little or the other way (1 x 4096 20.6 / 21.0, two tokens 32 x 4096 98 / 130), and so
 // do small calls (1 x 100, six tokens 12.1 / 13.6; 20 x 375-3000 79.7 / 81.0).  Lengths are not known here: the table's width
 // stands for them, unless the cache could not fill half of such a table (100 sequences of 300 keys, six tokens, a table of
-// 512 pages: 141 / 184).  (The scalar bring-up kernel reads bf16 only.)
+// 512 pages: 141 / 184).  (All with raw slots of half their present size: 3-5 % off the times on the way in since.)  (The scalar bring-up kernel reads bf16 only.)
 bool widen_first(int B, int rows, int num_blocks, int max_blocks_per_seq, int flags) {
   if (flags & AMLA_FLAG_KERNEL_SIMT) return true;
   const long long row_blocks = (rows + kRowBlock - 1) / kRowBlock, slots = static_cast<long long>(B) * max_blocks_per_seq;

@@ -80,7 +80,7 @@ constexpr int kTraceTiles = 96;
 // tiles whose positions it owns; overhead positions carry no work.
 // ---------------------------------------------------------------------------------------------
 #ifndef AMLA_UNIT_OVERHEAD_TILES
-#define AMLA_UNIT_OVERHEAD_TILES 6            // 128-row kernel: in 64-key pages (a build-time knob for tuning runs)
+#define AMLA_UNIT_OVERHEAD_TILES 6            // 128-row kernel: in 64-key pages (a build-time knob; swept when units still were chains of their own)
 #endif
 constexpr int kUnitOverheadTiles = AMLA_UNIT_OVERHEAD_TILES;
 #ifndef AMLA_QUAD_OVERHEAD_TILES

@@ -25,11 +25,15 @@
 // crossed to the other SM by remote stores, Q went through shared memory into tensor memory and the score CTA had to be
 // drained before the next unit's Q could follow.  Here nothing but MMA operands crosses, Q is an operand as it lands, and
 // the tile is 256 keys.  Calls with it, from that kernel to this one as it stands (sustained): 192 sequences of 1-512 keys
-// 62.8 -> 45.2 us; one of 2531 33.8 -> 12.8; 16 x 16384 with rising logits 106.0 -> 93.4; 96 x 2048 88.7 -> 81.0; 32 x 4096
-// 59.1 -> 55.5; 96 x 16384 540 -> 447; E4M3 32 x 4096 100.4 -> 62.1.
-// What bounds it: a tile of 256 keys takes ~7500 clk (E4M3 10.4 K) against 4350 of MMAs and 5900 of HBM at its full rate: a
-// CTA takes 278 KB per tile through a ring of 112 KB, whose slots turn around in ~2700 clk (load 1500-2000, MMA, commit,
-// next load), and every slot has to be issued.  Long calls run at the power limit: 32 x 4096 takes 51 us cool.
+// 62.8 -> 42.2 us; one of 2531 33.8 -> 12.4; 16 x 16384 with rising logits 106.0 -> 92.7; 96 x 2048 88.7 -> 79.2; 32 x 4096
+// 59.1 -> 53.7; E4M3 32 x 4096 100.4 -> 60.6.
+// What bounds it (trace): a tile of 256 keys takes 7100 clk in long units, 7600 on average over the eight of a 32 x 4096 call,
+// against 4350 of MMAs and 5900 of HBM at its full rate.  The issuer finds every slot full that it comes to, and takes 350 clk
+// for a slot of K and 390 for one of V, 17 of them a tile; what is left are its waits for the softmax warps.  A slot is full
+// 2200 clk (K, most of it from L2) or 2400 clk (V) after it has been asked for, and is asked for again 630 or 690 clk later: a
+// ring of 112 KB for the 278 KB of a tile just about keeps up.  E4M3: 9800 clk; a pair of widening warps takes 700 clk for a
+// slot and has waited 540 for its place, 150 for the raw slot; the issuer waits for one slot in ten.  Long calls run at the
+// power limit: 32 x 4096 takes 50 us cool.
 //
 // All waits are bounded; on expiry the kernel records kStatusTimeout and unwinds.
 #include "amla_common.cuh"
@@ -504,8 +508,8 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     //     contiguous form: asked for by the tensor map's boxes 55.8.  A tile earlier: 55.9, 96 x 2048 82.5: V is gone from L2
     //     by the time it is wanted.  Rings for K and for V by themselves: 63-67, as either is too short for its latency.  V of
     //     a tile between the K blocks of the one two after it: 57.0, rising logits 93 -> 100, the last tiles' V comes later.)
-    //     Four loaders -> three, which leaves merge blocks room beside a decode CTA: 53.9 -> 53.7, 1 x 2531 12.65 -> 12.55,
-    //     1 x 1500 12.08 -> 11.89.
+    //     Four loaders -> three: 53.9 -> 53.7, 1 x 2531 12.65 -> 12.55, 1 x 1500 12.08 -> 11.89.  (Room for a merge block beside a
+    //     decode CTA is not why: twelve warps of 152 registers leave 7168, and the smallest merge block takes 8192.)
     //   E4M3: the same, by one loader into the raw ring.
     if (elect_one()) {
       const uint64_t keep = l2_policy_evict_normal(), last_use = l2_policy_evict_first();   // K: V follows a tile later; V: done with
