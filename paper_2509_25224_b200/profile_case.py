@@ -1,11 +1,11 @@
 """Runs a few decode calls of one (possibly cut-down) workload: the command that profiler captures wrap.
 
     python -m paper_2509_25224_b200.profile_case --config mtp [--batch 32] [--calls 3] [--mode alg2|fold|fmul]
-                                                 [--tau T] [--rows128] [--n N] [--heads H]
+                                                 [--tau T] [--rows128] [--n N] [--heads H] [--fp8]
 
 --batch keeps the first B sequences of the named configuration (its seeded lengths and values), --n overrides the
 sequence length of the fixed-length configurations (stress: the staircase of logit offsets spans the new length), --heads
-the number of heads of dsv3 (16: the kernel for few rows).
+the number of heads of dsv3 (16: the kernel for few rows).  --fp8 rounds the cache to E4M3 (scale 1/64).
 One warm-up call, then --calls calls; the status word is checked and a checksum of the output printed, so that a
 capture can be told from a run that did nothing.
 """
@@ -49,6 +49,7 @@ def main() -> int:
     ap.add_argument("--mode", default=None, choices=["alg2", "fold", "fmul"])
     ap.add_argument("--tau", type=int, default=None)
     ap.add_argument("--rows128", action="store_true")
+    ap.add_argument("--fp8", action="store_true")
     a = ap.parse_args()
     w = build_workload(a.config, a.batch, a.n, a.heads)
     flags = None
@@ -58,14 +59,21 @@ def main() -> int:
     dev = torch.device("cuda", 0)
     torch.cuda.set_device(dev)
     q = torch.from_numpy(w.q.view(np.int16)).to(dev).view(torch.bfloat16)
-    kv = torch.from_numpy(w.kv.view(np.int16)).to(dev).view(torch.bfloat16)
+    if a.fp8:
+        kv = torch.from_numpy(synth.quantise_cache_e4m3(w, 1.0 / 64.0)).to(dev)
+    else:
+        kv = torch.from_numpy(w.kv.view(np.int16)).to(dev).view(torch.bfloat16)
     bt = torch.from_numpy(w.block_table).to(dev)
     sl = torch.from_numpy(w.seqlens).to(dev)
     out = torch.empty((w.B, w.Sq, w.H, 512), dtype=torch.bfloat16, device=dev)
     lse = torch.empty((w.B, w.Sq, w.H), dtype=torch.float32, device=dev)
-    ws = torch.empty(binding.workspace_size(w.B, w.Sq, w.H, w.max_blocks_per_seq, 0), dtype=torch.uint8, device=dev)
+    size = binding.fp8_workspace_size if a.fp8 else binding.workspace_size
+    ws = torch.empty(size(w.B, w.Sq, w.H, w.max_blocks_per_seq, 0), dtype=torch.uint8, device=dev)
     for _ in range(1 + a.calls):
-        binding.mla_decode(q, kv, bt, sl, w.scale, out, lse, ws, flags)
+        if a.fp8:
+            binding.mla_decode_fp8(q, kv, 1.0 / 64.0, bt, sl, w.scale, out, lse, ws, flags)
+        else:
+            binding.mla_decode(q, kv, bt, sl, w.scale, out, lse, ws, flags)
     binding.check_status(ws)
     torch.cuda.synchronize()
     print(f"{a.config}: B={w.B} Sq={w.Sq} H={w.H} keys={int(w.seqlens.astype(np.int64).sum())} KV={w.kv.nbytes / 1e6:.0f} MB "
