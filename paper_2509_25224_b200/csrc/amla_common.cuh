@@ -115,11 +115,16 @@ struct Plan {
   int share;     // positions per part (the last part may have fewer)
 
   __host__ __device__ static Plan make(const int* prefix, int n_items, int max_parts, int ovh, int min_share = 1) {
-    Plan pl;
+    Plan pl = make(prefix[n_items], max_parts, min_share);
     pl.prefix = prefix;
     pl.ovh = ovh;
     pl.n_items = n_items;
-    pl.L = prefix[n_items];
+    return pl;
+  }
+  // the parts alone, for a schedule of L positions
+  __host__ __device__ static Plan make(int L, int max_parts, int min_share) {
+    Plan pl = {};
+    pl.L = L;
     pl.share = pl.L > max_parts ? static_cast<int>((static_cast<unsigned>(pl.L) + max_parts - 1) / static_cast<unsigned>(max_parts)) : 1;
     if (pl.share < min_share) pl.share = min_share;
     pl.P = pl.L > 0 ? static_cast<int>((static_cast<unsigned>(pl.L) + pl.share - 1) / static_cast<unsigned>(pl.share)) : 1;

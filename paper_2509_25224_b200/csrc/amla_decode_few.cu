@@ -54,7 +54,8 @@ constexpr uint32_t kBarBytes = 256;
 constexpr int kSmemPlanItems = 512;
 constexpr uint32_t kOffPlan = kOffBars + kBarBytes;
 constexpr uint32_t kOffSeqlens = kOffPlan + ((kSmemPlanItems + 1) * 4 + 15) / 16 * 16;
-constexpr uint32_t kSmemBytes = kOffSeqlens + kSmemPlanItems * 4;
+constexpr uint32_t kOffFirst = kOffSeqlens + kSmemPlanItems * 4;
+constexpr uint32_t kSmemBytes = kOffFirst + sizeof(FirstUnit);
 static_assert(kSmemBytes <= 232448, "exceeds the shared memory a block can opt in to");
 static_assert(kPageBytes % 1024 == 0 && kOffP % 1024 == 0, "swizzled tiles need 1024-byte alignment");
 
@@ -90,13 +91,14 @@ decode_few_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_const
   auto bar = [&](int i) { return bars + 8u * i; };
   const uint32_t tmem_slot = bars + kBarBytes - 8;
 
-  // Set-up, three things side by side: the load warp works out the schedule from the sequence lengths as they are found
-  // (held against the final ones after the wait below), the MMA warp allocates tensor memory, one thread of a softmax warp
-  // initialises the barriers.
+  // Set-up.  The schedule is worked out from the sequence lengths as they are found (held against the final ones after the
+  // wait below): all threads bring them, then the load warp adds up.  Beside that the MMA warp allocates tensor memory and one
+  // thread of a softmax warp initialises the barriers.
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = reinterpret_cast<int*>(smem_raw + kOffSeqlens);
-  if (wid == kLoadWarp && plan_here) plan_on_chip(prm, plan_smem, lens_smem, lane);
+  FirstUnit* first_smem = reinterpret_cast<FirstUnit*>(smem_raw + kOffFirst);
+  if (plan_here) plan_lengths(prm, plan_smem, lens_smem, tid, kThreads);
   if (tid == 0) {
     for (int i = 0; i < kSlots * kPieces; ++i) mbar_init(bar(X_FULL + i), 1);
     for (int i = 0; i < kSlots; ++i) mbar_init(bar(X_EMPTY + i), 1);
@@ -109,6 +111,10 @@ decode_few_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_const
     prefetch_tensormap(&q_map);
   }
   if (wid == kQkWarp) { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
+  if (plan_here) {
+    __syncthreads();
+    if (wid == kLoadWarp) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
+  }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -129,18 +135,24 @@ decode_few_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_const
     }
   }
   bool ok = true;
-  Tiles tile(UnitIter(prm, prefix, seqlens, part));
-  if (plan_here) {
+  Tiles tile(UnitIter(prm, prefix, seqlens, part), plan_here ? first_smem : nullptr);
+  int first_page = 0;                                        // the load warp's first page: on its way while the lengths are
+  auto load_page = [&]() { if (wid == kLoadWarp && tile.valid) first_page = ldg_here(prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t); };
+  if (!plan_here) {
+    load_page();
+  } else {
     // Launched with programmatic stream serialization: everything above ran while the kernel before this one on the stream
     // was still going; its results (the previous call's reads of the workspace among them) are complete after this wait.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    if (wid == kLoadWarp && lane == 0 && tile.valid) prefetch_pages(prm, tile.u.b, tile.t);
-    if (plan_is_stale(prm, plan_smem, lens_smem, tid, kThreads)) {
-      if (wid == kLoadWarp) plan_on_chip(prm, plan_smem, lens_smem, lane);
+    load_page();                                             // (the guess's place in the table is inside the table)
+    if (plan_is_stale(prm, plan_smem, lens_smem, first_smem, tid, kThreads)) {
+      plan_lengths(prm, plan_smem, lens_smem, tid, kThreads);
       __syncthreads();
-      tile.units.start();
-      tile.begin();
+      if (wid == kLoadWarp) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
+      __syncthreads();
+      tile.start(first_smem);
+      load_page();
     }
     if (blockIdx.x == 0 && wid == 0 && lane == 0) *prm.status = kStatusOk;
   }
@@ -379,7 +391,7 @@ decode_few_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_const
     if (elect_one()) {
       uint32_t slot = 0, par = 1, n_issued = 0;
       auto entry = [&]() { return prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t; };
-      int page = tile.valid ? __ldg(entry()) : 0;
+      int page = first_page;
       auto load = [&](const CUtensorMap* map, int row, uint32_t piece_bytes) {
         ok = mbar_wait(bar(X_EMPTY) + 8 * slot, par);
         if (!ok) return;

@@ -89,7 +89,8 @@ constexpr uint32_t kBarBytes = 384;
 constexpr int kSmemPlanItems = 512;
 constexpr uint32_t kOffPlan = kOffBars + kBarBytes;
 constexpr uint32_t kOffSeqlens = kOffPlan + ((kSmemPlanItems + 1) * 4 + 15) / 16 * 16;
-constexpr uint32_t kSmemBytes = kOffSeqlens + kSmemPlanItems * 4;
+constexpr uint32_t kOffFirst = kOffSeqlens + kSmemPlanItems * 4;
+constexpr uint32_t kSmemBytes = kOffFirst + sizeof(FirstUnit);
 static_assert(kSmemBytes <= 232448, "exceeds the shared memory a block can opt in to");
 static_assert(kOffP % 1024 == 0 && kOffRing % 1024 == 0, "swizzled tiles need 1024-byte alignment");
 
@@ -115,6 +116,21 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
 }
 
 using Tiles = TileIter<kTilePages>;
+
+// The page numbers of a tile.
+static_assert(kTilePages == 4, "a tile's page numbers");
+struct Pages { int a, b, c, d; };
+__device__ __forceinline__ Pages load_pages(const DecodeParams& prm, const Tiles& tile) {
+  Pages pg = {};
+  if (tile.valid) {
+    const int32_t* bt = prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t;
+    pg.a = ldg_here(bt);
+    if (tile.np > 1) pg.b = ldg_here(bt + 1);
+    if (tile.np > 2) pg.c = ldg_here(bt + 2);
+    if (tile.np > 3) pg.d = ldg_here(bt + 3);
+  }
+  return pg;
+}
 
 // This CTA's 64 rows of a unit's Q, by one thread of either CTA.  The bytes of both are counted in the even one.
 __device__ __forceinline__ int q_row_of(const DecodeParams& prm, const Unit& u, int rank) { return u.b * prm.R + u.r0 + rank * kCtaRows; }
@@ -148,13 +164,14 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   const uint32_t tmem_slot = bars + kBarBytes - 8;
   const uint32_t lead_bars = map_to_cta(bars, 0);
 
-  // Set-up, three things side by side: warp 8 works out the schedule of a batch of up to kSmemPlanItems items from the
-  // sequence lengths as they are found (held against the final ones after the wait below), warp 9 allocates tensor memory,
-  // one thread of warp 10 initialises the barriers.
+  // Set-up.  The schedule of a batch of up to kSmemPlanItems items is worked out from the sequence lengths as they are found
+  // (held against the final ones after the wait below): all threads bring them, then warp 8 adds up.  Beside that warp 9
+  // allocates tensor memory and one thread of warp 10 initialises the barriers.
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = reinterpret_cast<int*>(smem_raw + kOffSeqlens);
-  if (wid == 8 && plan_here) plan_on_chip(prm, plan_smem, lens_smem, lane);
+  FirstUnit* first_smem = reinterpret_cast<FirstUnit*>(smem_raw + kOffFirst);
+  if (plan_here) plan_lengths(prm, plan_smem, lens_smem, tid, kThreads<kFp8>);
   if (tid == 32 * 10) {
     for (int i = 0; i < kSlots<kFp8>; ++i) {
       mbar_init(bar(X_FULL + i), kFp8 ? kWidenWarps + 1 : 1);          // E4M3: the warps that fill the slot, and word from the odd CTA
@@ -180,9 +197,13 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   }
   if (wid == 9) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
   if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 6);
+  if (plan_here) {
+    __syncthreads();
+    if (wid == 8) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
+  }
   tc_fence_before_sync();
   __syncthreads();
-  cluster_arrive();        // the peer's barriers are initialised before anyone signals them (waited for below)
+  cluster_arrive_relaxed();        // the peer's barriers are initialised before anyone signals them (waited for below)
   tc_fence_after_sync();
   const uint32_t tbase = ld_shared_b32(tmem_slot);
   if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 3);
@@ -202,20 +223,25 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     }
   }
   bool ok = true;
-  Tiles tile(UnitIter(prm, prefix, seqlens, part));
+  Tiles tile(UnitIter(prm, prefix, seqlens, part), plan_here ? first_smem : nullptr);
   if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 5);
   cluster_wait();
-  if (plan_here) {
+  Pages first_pages = {};                                    // the loaders' first tile: on their way while the lengths are
+  if (!plan_here) {
+    if (wid >= kSoftmaxWarps) first_pages = load_pages(prm, tile);
+  } else {
     // Launched with programmatic stream serialization: everything above ran while the kernel before this one on the stream
     // was still going; its results (the previous call's reads of the workspace among them) are complete after this wait.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    if (wid == 8 && lane == 0 && tile.valid) prefetch_pages(prm, tile.u.b, tile.t);
-    if (plan_is_stale(prm, plan_smem, lens_smem, tid, kThreads<kFp8>)) {     // (both CTAs see the same lengths)
-      if (wid == 8) plan_on_chip(prm, plan_smem, lens_smem, lane);
+    if (wid >= kSoftmaxWarps) first_pages = load_pages(prm, tile);     // (the guess's place in the table is inside the table)
+    if (plan_is_stale(prm, plan_smem, lens_smem, first_smem, tid, kThreads<kFp8>)) {     // (both CTAs see the same lengths)
+      plan_lengths(prm, plan_smem, lens_smem, tid, kThreads<kFp8>);
       __syncthreads();
-      tile.units.start();
-      tile.begin();
+      if (wid == 8) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
+      __syncthreads();
+      tile.start(first_smem);
+      if (wid >= kSoftmaxWarps) first_pages = load_pages(prm, tile);
     }
     if (blockIdx.x == 0 && wid == 0 && lane == 0) *prm.status = kStatusOk;
   }
@@ -517,19 +543,10 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       auto row_of = [&](int page) { return (kFp8 && (page < 0 || page >= prm.num_blocks) ? prm.num_blocks : page) * kPage; };
       // The page numbers of a tile are loaded once, a tile ahead: a load of the block table in front of every slot cost a loader
       // 500 clk there (a tile of the E4M3 cache took 11.9 K clk instead of 10.4 K).
-      static_assert(kTilePages == 4, "a tile's page numbers");
-      struct Pages { int a, b, c, d; };
-      auto take = [&](Pages& pg) {                          // pages of the next tile, 0: none
-        const int np = tile.valid ? tile.np : 0;
-        if (np > 0) {
-          const int32_t* bt = prm.block_table + static_cast<size_t>(tile.u.b) * prm.max_blocks_per_seq + tile.t;
-          pg.a = __ldg(bt);
-          pg.b = np > 1 ? __ldg(bt + 1) : 0;
-          pg.c = np > 2 ? __ldg(bt + 2) : 0;
-          pg.d = np > 3 ? __ldg(bt + 3) : 0;
-          tile.next();
-        }
-        return np;
+      auto take = [&](Pages& pg) {                          // on to the next tile: its pages, 0: there is none
+        tile.next();
+        pg = load_pages(prm, tile);
+        return tile.valid ? tile.np : 0;
       };
       // This CTA's half of the tile's keys, 32 np of them from key 32 np rank on, is at most two boxes: a page, or the half page
       // in the middle of a tile of three pages or of one.  (With 32 keys of every page it was four boxes: E4M3, one loader:
@@ -557,13 +574,14 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         constexpr uint32_t kRing = kSlots<false>;
         uint32_t slot = 0, par = 1, turn = 0;
         auto advance = [&]() { if (++slot == kRing) { slot = 0; par ^= 1; } ++n; if (++turn == kLoaders) turn = 0; };
-        Pages pg = {}, pg_nxt = {}, pg_prev = {};
-        int np = take(pg), np_prev = 0;
+        Pages pg = first_pages, pg_nxt = {}, pg_prev = {};
+        int np = tile.valid ? tile.np : 0, np_prev = 0;
         KBoxes x = boxes(np, pg);
         while (ok && np > 0) {
-          const int np_nxt = take(pg_nxt);
+          int np_nxt = 0;
 #pragma unroll 1
           for (int c = 0; c < kQBlocks; ++c) {
+            if (c == kLoaders) np_nxt = take(pg_nxt);       // (behind this loader's first load: at a call's start that one is waited for)
             if (turn == mine) {
               ok = mbar_wait(bar(X_EMPTY) + 8 * slot, par);
               if (!ok) break;
@@ -609,15 +627,16 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       } else {
         uint32_t slot = 0, par = 1;
         auto advance = [&]() { if (++slot == kRawSlots) { slot = 0; par ^= 1; } ++n; };
-        Pages pg = {}, pg_nxt = {}, pg_prev = {};
-        int np = take(pg), np_prev = 0;
+        Pages pg = first_pages, pg_nxt = {}, pg_prev = {};
+        int np = tile.valid ? tile.np : 0, np_prev = 0;
         while (ok && np > 0) {
-          const int np_nxt = take(pg_nxt);
+          int np_nxt = 0;
           const KBoxes x = boxes(np, pg);
           // a raw slot is two column blocks of K (the last one by itself: its box reaches past the row's end, where there are zeros
           // that nothing reads), or a page of V, this CTA's 256 columns of it
 #pragma unroll 1
           for (int c = 0; c < kQBlocks; c += 2) {
+            if (c == 2) np_nxt = take(pg_nxt);
             const uint32_t full = bar(X_RAWFULL) + 8 * slot, dst = smem_base + kOffRaw + slot * kRawBytes;
             ok = mbar_wait(bar(X_RAWEMPTY) + 8 * slot, par);
             if (!ok) break;

@@ -67,14 +67,15 @@ constexpr uint32_t kEndB = kOffOut + 8 * 2048;
 constexpr uint32_t kOffBars = kEndA > kEndB ? kEndA : kEndB;
 constexpr uint32_t kBarBytes = 320;
 #ifdef AMLA_TRACE
-constexpr int kSmemPlanItems = 4, kSmemLens = 4;     // trace builds: the room goes to the stamps
+constexpr int kSmemPlanItems = 1, kSmemLens = 1;     // trace builds: the room goes to the stamps
 #else
 // on-chip copies of the schedule prefix, and behind a short one of the sequence lengths: that is what room there is
 constexpr int kSmemPlanItems = 160, kSmemLens = 64;
 #endif
 constexpr uint32_t kOffPlan = kOffBars + kBarBytes;
 constexpr uint32_t kOffSeqlens = kOffPlan + (kSmemLens + 1) * 4;
-constexpr uint32_t kEndPlan = kOffPlan + 4 * (kSmemPlanItems + 1 > 2 * kSmemLens + 1 ? kSmemPlanItems + 1 : 2 * kSmemLens + 1);
+constexpr uint32_t kOffFirst = kOffPlan + 4 * (kSmemPlanItems + 1 > 2 * kSmemLens + 1 ? kSmemPlanItems + 1 : 2 * kSmemLens + 1);
+constexpr uint32_t kEndPlan = kOffFirst + sizeof(FirstUnit);
 #ifdef AMLA_TRACE
 // trace builds: every CTA keeps its stamps (low 32 bits of its SM's cycle counter) in shared memory, so that taking
 // one does not put a global store in front of the role's next release, and dumps them when it is done
@@ -125,7 +126,7 @@ struct Cursor {
   int base;
   int ord;       // ordinal of the current unit within the part
   bool valid;
-  __device__ Cursor(const DecodeParams& prm, const int* prefix, const int* seqlens, int part) : it(prm, prefix, seqlens, part), base(0), ord(0) { valid = it.next(u); }
+  __device__ Cursor(const UnitIter& behind_first, const Unit& first, bool any) : it(behind_first), u(first), base(0), ord(0), valid(any) {}
   __device__ bool locate(int k, int& local) {
     while (valid && k >= base + (u.t1 - u.t0)) { base += u.t1 - u.t0; valid = it.next(u); ++ord; }
     local = k - base;
@@ -419,12 +420,13 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   const uint32_t myV_base = map_to_cta(smem_base, 2 + half);           // score CTA j -> value CTA j
   const uint32_t myV_bars = map_to_cta(bars, 2 + half);
 
-  // Warp 6 works out the schedule of a batch of up to kSmemPlanItems items during the set-up, from the sequence lengths as they
-  // are found (held against the final ones after the wait below).
+  // The schedule of a batch of up to kSmemPlanItems items is worked out during the set-up, from the sequence lengths as they
+  // are found (held against the final ones after the wait below): all threads bring them, then warp 6 adds up.
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = prm.n_items <= kSmemLens ? reinterpret_cast<int*>(smem_raw + kOffSeqlens) : nullptr;
-  if (wid == 6 && plan_here) plan_on_chip(prm, plan_smem, lens_smem, lane);
+  FirstUnit* first_smem = reinterpret_cast<FirstUnit*>(smem_raw + kOffFirst);
+  if (plan_here) plan_lengths(prm, plan_smem, lens_smem, tid, kThreads);
   if (tid == 0) {
     for (int i = 0; i < kNumP; ++i) mbar_init(bar(X_PV + i), 1);
     if (is_score) {
@@ -449,10 +451,13 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     prefetch_tensormap(&q_map);
   }
   if (wid == 5) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
+  if (plan_here) {
+    __syncthreads();
+    if (wid == 6) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
+  }
   tc_fence_before_sync();
   __syncthreads();
-  cluster_arrive();
-  cluster_wait();
+  cluster_arrive_relaxed();        // the peers' barriers are initialised before anyone signals them (waited for below)
   tc_fence_after_sync();
   const uint32_t tbase = ld_shared_b32(tmem_slot);
 
@@ -471,30 +476,32 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       __syncthreads();
     }
   }
-  UnitIter first(prm, prefix, seqlens, part);
-  Unit fu;
-  bool any = first.next(fu);
+  UnitIter iter(prm, prefix, seqlens, part);
+  Unit fu;                                                   // the part's first unit; iter stands behind it
+  iter.start(plan_here ? first_smem : nullptr, fu);
   if (plan_here) {
     // Launched with programmatic stream serialization: everything above ran while the kernel before this one on the stream
     // was still going; its results (the previous call's reads of the workspace among them) are complete after this wait.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    if (wid == 4 && lane == 0 && any) prefetch_pages(prm, fu.b, fu.t0 * (kTileKeys / kPage));
-    if (plan_is_stale(prm, plan_smem, lens_smem, tid, kThreads)) {           // (all four CTAs see the same lengths)
-      if (wid == 6) plan_on_chip(prm, plan_smem, lens_smem, lane);
+    if (plan_is_stale(prm, plan_smem, lens_smem, first_smem, tid, kThreads)) {           // (all four CTAs see the same lengths)
+      plan_lengths(prm, plan_smem, lens_smem, tid, kThreads);
       __syncthreads();
-      first.start();
-      any = first.next(fu);
+      if (wid == 6) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
+      __syncthreads();
+      iter.start(first_smem, fu);
     }
     if (blockIdx.x == 0 && wid == 6 && lane == 0) *prm.status = kStatusOk;
   }
+  cluster_wait();
   if (tid == 0) QSTAMP_NS(smem_base, 2);
+  const bool any = fu.t1 > fu.t0;
   // the first unit's Q is requested before the roles start: one piece per lane
   if (is_score && tid < kNumKSlots && any) issue_q_piece(&q_map, smem_base, bars, tid, fu.b * prm.R + fu.r0 + half * kRowBlock);
 
   bool ok = true;
-  UnitIter iter(prm, prefix, seqlens, part);
-  Unit u;
+  Unit u = fu;
+  bool more = any;      // u is a unit to be done
   uint32_t gt = 0;      // 64-key pages processed by this cluster so far (two per tile; all roles count identically)
   uint32_t un = 0;      // units processed so far
 
@@ -508,7 +515,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       const int qr = (wid & 3) * 32 + lane;
       const uint32_t q_lane_base = static_cast<uint32_t>((wid & 3) * 32) << 16;
       const RoleCtx ctx{smem_base, bars, tbase, myV_base, myV_bars, half, tid, part};
-      while (ok && iter.next(u)) {
+      for (; ok && more; more = iter.next(u)) {
         ok = warp_wait(bar(A_QFREE), (un & 1) ^ 1);      // the previous unit's QK^T is finished with Q
         if (!ok) break;
         tc_fence_after_sync();
@@ -562,7 +569,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       // At the start of every unit the slot first carries the lane's piece of that unit's Q (see issue_q_piece; lane 0
       // waits for the previous unit's MMAs to let go of the RoPE tile); the first unit's pieces were requested before
       // the roles split.
-      Cursor cur(prm, prefix, seqlens, part);
+      Cursor cur(iter, fu, any);
       bool fin = lane >= kNumKSlots;
       const bool first_out = !fin && cur.valid;
       UnitIter qit = cur.it;                  // walks the units whose Q this lane has not requested (it stands behind the first)
@@ -646,7 +653,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           const uint32_t klo0 = smem_desc_lo(smem_base + kOffK, 16);
           const uint32_t qlo0 = smem_desc_lo(smem_base + kOffQRope, 16);
           uint32_t slot = 0, kpar = 0;
-          while (ok && iter.next(u)) {
+          for (; ok && more; more = iter.next(u)) {
             ok = mbar_wait<true>(bar(A_QREADY), un & 1);
             if (!ok) break;
             tc_fence_after_sync();
@@ -704,7 +711,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         // lane 2 those of QREADY (one per unit)
 
         int n_units = 0, n_tiles = 0;
-        while (iter.next(u)) { ++n_units; n_tiles += u.t1 - u.t0; }
+        for (; more; more = iter.next(u)) { ++n_units; n_tiles += u.t1 - u.t0; }
         const int phases = lane == 2 ? n_units : lane < 2 ? (n_tiles + 1 - lane) / 2 : 0;
         const int first = lane == 2 ? A_QREADY - 2 : A_SEMPTY;     // lane 2 lands on QREADY
         if (!relay_phases<false>(bars, lead_bars, first, lane, phases) && lane == 0) report_timeout(prm.status);
@@ -721,7 +728,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       const int c_first = partner ? 8 : 0;
       if (tid == 0 && leader) merge_begin(prm, part);
       write_empty_items(prm, prefix, part, prm.P, half * kRowBlock, kRowBlock, partner ? r + kRowBlock : r, 2 * kRowBlock);
-      while (ok && iter.next(u)) {
+      for (; ok && more; more = iter.next(u)) {
         const int npages = 2 * (u.t1 - u.t0);
         int2 info;
         const int slot = iter.slot_of(u, &info);
@@ -862,7 +869,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       // ---- TMA producers: V.  One slot per page: this CTA's 128 columns of either 256-column half of V (two
       // boxes of 64 keys x 128 columns); lane l owns ring slot l.  Both pages of every tile are loaded (the
       // second page of a sequence's odd last tile is the first one again; its probabilities are zero).
-      Cursor cur(prm, prefix, seqlens, part);
+      Cursor cur(iter, fu, any);
       int my_gp = lane;                       // next page of the sequence this lane loads (tile = gp / 2)
       uint32_t par = 1;
       bool fin = lane >= kNumVSlots, have = false;
@@ -916,7 +923,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           const uint32_t vlo0 = smem_desc_lo(smem_base + kOffV, kBoxBytes);
           const uint32_t plo0 = smem_desc_lo(smem_base + kOffP, 16);
           uint32_t slot = 0, vpar = 0;
-          while (ok && iter.next(u)) {
+          for (; ok && more; more = iter.next(u)) {
             const int npages = 2 * (u.t1 - u.t0);
             for (int pi = 0; pi < npages && ok; ++pi, ++gt) {
               const uint32_t s = gt % kNumP, k = gt / kNumP;
@@ -955,7 +962,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         // ---- relay (odd CTA): lane s passes on the completed phases of OREADY[s] (the pages in P buffer s).  The
         // page's P~ in this CTA (remote asynchronous stores, generic proxy) is about to be read by the pair MMA.
         int n_pages = 0;
-        while (iter.next(u)) n_pages += 2 * (u.t1 - u.t0);
+        for (; more; more = iter.next(u)) n_pages += 2 * (u.t1 - u.t0);
         const int phases = lane < kNumP ? (n_pages + kNumP - 1 - lane) / kNumP : 0;
         if (!relay_phases<true>(bars, lead_bars, B_OREADY, lane, phases) && lane == 0) report_timeout(prm.status);
       }

@@ -1,7 +1,10 @@
 // How a cluster walks its share of the schedule: units (the part of one item that falls into the cluster's range) and,
 // inside a unit, score tiles of a few 64-key pages.  Every role of a cluster runs the same walk, so no role has to tell
-// another what comes next.  (Include after amla_common.cuh.)
+// another what comes next.
 #pragma once
+
+#include "amla_common.cuh"
+#include "amla_sm100.cuh"
 
 namespace amla {
 
@@ -17,66 +20,16 @@ __device__ __forceinline__ int warp_inclusive_scan(int v, int lane) {
 // A sequence length, clamped to the table's width.  kGuess: as it stands in the GPU's common cache at this moment; the SM's own
 // cache neither answers nor keeps it.  Otherwise an ordinary load, which griddepcontrol.wait is in front of (0.2-0.4 us less on
 // the way to a call's first load than the other kind).
+__device__ __forceinline__ int clamp_length(const DecodeParams& prm, int n) { return min(max(n, 0), prm.max_blocks_per_seq * kPage); }
 template <bool kGuess>
-__device__ __forceinline__ int load_length(const DecodeParams& prm, int b) {
+__device__ __forceinline__ int load_length_raw(const DecodeParams& prm, int b) {
   int n;
   if (kGuess) asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(n) : "l"(prm.seqlens + b) : "memory");
   else asm volatile("ld.global.b32 %0, [%1];" : "=r"(n) : "l"(prm.seqlens + b) : "memory");
-  return min(max(n, 0), prm.max_blocks_per_seq * kPage);
+  return n;
 }
-
-// The schedule prefix of the batch, by one warp: into shared memory together with the sequence lengths (unless lens is null),
-// or into the workspace.
-//
-// plan_on_chip also runs ahead of griddepcontrol.wait, when a kernel in front that produces the lengths may not have written
-// them yet, or not so that this kernel sees it.  What it finds there is a guess, whatever it is: lengths are clamped to the
-// table's width, for which the schedule's positions fit their type (the launch sees to that).  After the wait
-// plan_is_stale() holds the guess against the lengths as they are; where they differ the plan is made again.
-// (The guess is right unless the kernel directly in front writes the lengths.  One sequence of 256 keys with 16 heads: planned
-// wholly behind the wait 8.5 us, guessed and checked 7.7, guessed and not checked 7.2; 32 x 4096 keys 51.7, 50.9 and 50.4,
-// calls replayed back to back.)
-__device__ __forceinline__ void plan_on_chip(const DecodeParams& prm, int* prefix, int* lens, int lane) {
-  int carry = 0;
-  for (int base = 0; base < prm.n_items; base += 32) {
-    const int it = base + lane;
-    const int b = prm.nrb == 1 ? it : it / prm.nrb;
-    const int n_seq = it < prm.n_items ? load_length<true>(prm, b) : 0;
-    const int v = it < prm.n_items ? schedule_length(n_seq, it, prm.tile_keys, prm.ovh) : 0;
-    const int x = warp_inclusive_scan(v, lane);
-    if (it < prm.n_items) {
-      if (lens) lens[b] = n_seq;                         // same value from every row block
-      prefix[it] = carry + x - v;
-    }
-    carry += __shfl_sync(0xffffffffu, x, 31);
-  }
-  if (lane == 0) prefix[prm.n_items] = carry;
-}
-// Page numbers of the first unit, on their way while the lengths are (the guess's place in the table is inside the table).
-__device__ __forceinline__ void prefetch_pages(const DecodeParams& prm, int b, int page) {
-  asm volatile("{\n\t.reg .b32 x;\n\tld.global.b32 x, [%0];\n\t}" ::"l"(prm.block_table + static_cast<size_t>(b) * prm.max_blocks_per_seq + page));
-}
-// By all threads of the CTA, after griddepcontrol.wait: does the plan differ from what the lengths give?
-__device__ __forceinline__ bool plan_is_stale(const DecodeParams& prm, const int* prefix, const int* lens, int tid, int threads) {
-  bool stale = false;
-  for (int it = tid; it < prm.n_items; it += threads) {
-    const int b = prm.nrb == 1 ? it : it / prm.nrb;
-    const int n_seq = load_length<false>(prm, b);
-    stale |= lens ? lens[b] != n_seq : prefix[it + 1] - prefix[it] != schedule_length(n_seq, it, prm.tile_keys, prm.ovh);
-  }
-  return __syncthreads_or(stale);
-}
-__device__ __forceinline__ void plan_in_workspace(const DecodeParams& prm, int lane) {
-  int* pw = const_cast<int*>(prm.prefix);
-  int carry = 0;
-  for (int base = 0; base < prm.n_items; base += 32) {
-    const int it = base + lane;
-    const int v = it < prm.n_items ? schedule_length(prm.seqlens[it / prm.nrb], it, prm.tile_keys, prm.ovh) : 0;
-    const int x = warp_inclusive_scan(v, lane);
-    if (it < prm.n_items) pw[it] = carry + x - v;
-    carry += __shfl_sync(0xffffffffu, x, 31);
-  }
-  if (lane == 0) pw[prm.n_items] = carry;
-}
+template <bool kGuess>
+__device__ __forceinline__ int load_length(const DecodeParams& prm, int b) { return clamp_length(prm, load_length_raw<kGuess>(prm, b)); }
 
 struct Unit {
   int b, r0, n_b, t0, t1, it;      // sequence, first row of the row block, keys, tile range [t0, t1) of the schedule, item
@@ -114,19 +67,115 @@ static __device__ __noinline__ UnitFound find_unit(const int* prefix, const int*
   return f;
 }
 
+// The first unit of a part and where the walk stands behind it: worked out with the plan, kept on chip for all roles.  (Looked
+// up by every thread for itself once the plan was there, it was 0.9-1.3 us of a call's start.)
+struct FirstUnit {
+  Unit u;                          // t0 == t1: the part has none
+  int g, g1, share;
+};
+
+// The schedule prefix of the batch and the part's first unit, on chip.  plan_lengths() by all threads of the CTA, then a barrier,
+// then plan_units() by one warp, then a barrier: all lengths are on their way together, and one scan does.  (By one warp, 32
+// lengths at a time and each 32 a memory round trip and a scan, the plan of 192 items took 6800 clk, of 32 1550; so 2750 and 2100
+// with the first unit in it.  From a CTA's first instruction to its first load: 192 x 1-512 keys 16.0 K clk, so 6.5 K and the call
+// 42.2 -> 39.0 us; 32 x 4096 8.0 K, so 6.0 K and 52.8 -> 52.1, since that one runs at the power limit.)
+//
+// Both also run ahead of griddepcontrol.wait, when a kernel in front that produces the lengths may not have written
+// them yet, or not so that this kernel sees it.  What is found there is a guess, whatever it is: lengths are clamped to the
+// table's width, for which the schedule's positions fit their type (the launch sees to that).  After the wait
+// plan_is_stale() holds the guess against the lengths as they are; where they differ the plan is made again.
+// (The guess is right unless the kernel directly in front writes the lengths.  One sequence of 256 keys with 16 heads: planned
+// wholly behind the wait 8.5 us, guessed and checked 7.7, guessed and not checked 7.2; 32 x 4096 keys 51.7, 50.9 and 50.4,
+// calls replayed back to back.)
+// Leaves every item's schedule length in prefix[], and the lengths in lens[] (unless that is null).
+__device__ __forceinline__ void plan_lengths(const DecodeParams& prm, int* prefix, int* lens, int tid, int threads) {
+  for (int it = tid; it < prm.n_items; it += threads) {
+    const int b = prm.nrb == 1 ? it : it / prm.nrb, n = load_length<true>(prm, b);
+    if (lens) lens[b] = n;                               // same value from every row block
+    prefix[it] = schedule_length(n, it, prm.tile_keys, prm.ovh);
+  }
+}
+__device__ __forceinline__ void plan_units(const DecodeParams& prm, int* prefix, const int* lens, FirstUnit* first, int part, int lane) {
+  const int per = (prm.n_items + 31) >> 5, it0 = lane * per, it1 = min(it0 + per, prm.n_items);     // a lane takes neighbouring items
+  int sum = 0;
+#pragma unroll 1
+  for (int it = it0; it < it1; ++it) sum += prefix[it];
+  const int upto = warp_inclusive_scan(sum, lane), before = upto - sum, total = __shfl_sync(0xffffffffu, upto, 31);
+#pragma unroll 1
+  for (int it = it0, at = before; it < it1; ++it) {
+    const int v = prefix[it];
+    prefix[it] = at;
+    at += v;
+  }
+  if (lane == 0) prefix[prm.n_items] = total;
+  __syncwarp();
+  // the part's range of positions, as Plan has it
+  const unsigned L = total, P = prm.P, share = max(L > P ? (L + P - 1) / P : 1u, static_cast<unsigned>(prm.min_share));
+  unsigned g = part * share;
+  const unsigned g1 = min(g + share, L);
+  // its first unit: of the last lane whose items begin at or before g
+  int it = (31 - __clz(__ballot_sync(0xffffffffu, it0 < it1 && static_cast<unsigned>(before) <= g) | 1)) * per;
+  Unit u = {};
+  while (g < g1) {
+    while (it + 1 < prm.n_items && static_cast<unsigned>(prefix[it + 1]) <= g) ++it;
+    const unsigned a = prefix[it] + item_overhead(it, prm.ovh), e = prefix[it + 1], from = max(g, a), to = min(e, g1);
+    g = to;
+    if (to > from) {                                     // (else only overhead positions of this item are in the range)
+      u.it = it; u.t0 = from - a; u.t1 = to - a;
+      u.b = prm.nrb == 1 ? it : static_cast<int>(static_cast<unsigned>(it) / static_cast<unsigned>(prm.nrb));
+      u.r0 = (it - u.b * prm.nrb) * prm.item_rows;
+      u.n_b = lens ? lens[u.b] : load_length<true>(prm, u.b);
+      break;
+    }
+  }
+  if (lane == 0) {
+    first->u = u;
+    first->g = g; first->g1 = g1; first->share = share;
+  }
+}
+// By all threads of the CTA, after griddepcontrol.wait: does the plan differ from what the lengths give?
+__device__ __forceinline__ bool plan_is_stale(const DecodeParams& prm, const int* prefix, const int* lens, const FirstUnit* first, int tid, int threads) {
+  bool stale = false;
+  for (int it = tid; it < prm.n_items; it += threads) {
+    const int b = prm.nrb == 1 ? it : it / prm.nrb;
+    const int n_seq = load_length<false>(prm, b);
+    if (lens) stale |= lens[b] != n_seq;
+    else stale |= prefix[it + 1] - prefix[it] != schedule_length(n_seq, it, prm.tile_keys, prm.ovh) || (it == first->u.it && n_seq != first->u.n_b);
+  }
+  return __syncthreads_or(stale);
+}
+__device__ __forceinline__ void plan_in_workspace(const DecodeParams& prm, int lane) {
+  int* pw = const_cast<int*>(prm.prefix);
+  int carry = 0;
+  for (int base = 0; base < prm.n_items; base += 32) {
+    const int it = base + lane;
+    const int v = it < prm.n_items ? schedule_length(prm.seqlens[it / prm.nrb], it, prm.tile_keys, prm.ovh) : 0;
+    const int x = warp_inclusive_scan(v, lane);
+    if (it < prm.n_items) pw[it] = carry + x - v;
+    carry += __shfl_sync(0xffffffffu, x, 31);
+  }
+  if (lane == 0) pw[prm.n_items] = carry;
+}
+
 struct UnitIter {
   const DecodeParams& prm;
   const int* prefix;
   const int* seqlens;
-  int p, g, g1, share, parts;
-  __device__ UnitIter(const DecodeParams& prm_, const int* prefix_, const int* seqlens_, int part) : prm(prm_), prefix(prefix_), seqlens(seqlens_), p(part) {
-    start();
-  }
-  __device__ void start() {
-    const Plan plan = Plan::make(prefix, prm.n_items, prm.P, prm.ovh, prm.min_share);
-    share = plan.share; parts = plan.P;
-    if (plan.L <= 0 || p >= plan.P) { g = g1 = 0; }
-    else { g = plan.part_start(p); g1 = plan.part_start(p + 1); }
+  int p, g, g1, share;
+  __device__ UnitIter(const DecodeParams& prm_, const int* prefix_, const int* seqlens_, int part) : prm(prm_), prefix(prefix_), seqlens(seqlens_), p(part) {}
+  // The part's first unit: from what plan_on_chip left, or looked up in the workspace's prefix (first == nullptr).
+  __device__ void start(const FirstUnit* first, Unit& u) {
+    if (first != nullptr) {
+      u = first->u;
+      g = first->g; g1 = first->g1; share = first->share;
+    } else {
+      const Plan plan = Plan::make(prefix, prm.n_items, prm.P, prm.ovh, prm.min_share);
+      share = plan.share;
+      if (plan.L <= 0 || p >= plan.P) { g = g1 = 0; }
+      else { g = plan.part_start(p); g1 = plan.part_start(p + 1); }
+      u.t0 = u.t1 = 0;
+      next(u);
+    }
   }
   __device__ bool next(Unit& u) {
     if (g >= g1) return false;
@@ -186,13 +235,19 @@ struct TileIter {
   int left, base, rem;   // tiles of the unit after this one, pages of the remaining tiles: base + 1 for `rem` of them, else base
   bool first;            // first tile of its unit
   bool valid;
-  __device__ explicit TileIter(const UnitIter& it) : units(it) { begin(); }
+  __device__ TileIter(const UnitIter& it, const FirstUnit* of_part) : units(it) { start(of_part); }
   __device__ bool last() const { return left == 0; }
+  __device__ void start(const FirstUnit* of_part) {
+    units.start(of_part, u);
+    valid = u.t1 > u.t0;
+    if (valid) begin();
+  }
   __device__ void begin() {
-    valid = units.next(u);
-    if (!valid) return;
-    const int n = u.t1 - u.t0, nt = (n + kMaxPages - 1) / kMaxPages;
-    base = static_cast<int>(static_cast<unsigned>(n) / static_cast<unsigned>(nt)); rem = n - base * nt;
+    const int n = u.t1 - u.t0, nt = static_cast<int>(static_cast<unsigned>(n + kMaxPages - 1) / kMaxPages);
+    base = kMaxPages;                                    // n / nt
+#pragma unroll
+    for (int i = 1; i < kMaxPages; ++i) if (base * nt > n) --base;
+    rem = n - base * nt;
     left = nt; first = true;
     t = u.t0; np = 0;
     step();
@@ -203,7 +258,7 @@ struct TileIter {
     --rem; --left;
   }
   __device__ void next() {
-    if (left == 0) begin();
+    if (left == 0) { valid = units.next(u); if (valid) begin(); }
     else { step(); first = false; }
   }
 };

@@ -53,6 +53,18 @@ def test_256_row_kernel_tile_tails(lens):
     check_full(w, binding.RESCALE_ALG2 | binding.lazy(0), kernel=256)
 
 
+@pytest.mark.parametrize("B,Sq,H,wide", [(31, 1, 4, False), (33, 1, 4, False), (512, 1, 2, False), (513, 1, 2, False), (65, 1, 40, False), (33, 3, 43, False), (300, 1, 33, False),
+                                         (32, 2, 65, True), (65, 2, 65, True), (40, 8, 64, True), (160, 2, 65, True), (161, 2, 65, True)])
+def test_schedules_worked_out_on_chip(B, Sq, H, wide):
+    # items per lane of the planning warp at its edges, several row blocks per sequence, runs of empty sequences; up to and
+    # beyond what is kept on chip
+    lens = np.random.default_rng(B + H).integers(0, 200, B)
+    lens[B // 3:B // 2] = 0
+    lens[[0, -1]] = 130, 1
+    w = synth.make_workload("plan", B, Sq, H, lens, seed=3000 + B + H)
+    check_full(wide_table(w) if wide else w, kernel=256 if wide else 32 if Sq * H <= 32 else 128)
+
+
 def test_256_row_kernel_against_128_row_blocks():
     # the same problem through both kernels (256-row items vs independent 128-row blocks): both meet the oracle
     for w in (synth.make_workload("ab", 3, 2, 128, [5000, 777, 2049], seed=431), synth.make_workload("ab4", 2, 4, 128, [3000, 130], seed=432)):
