@@ -259,10 +259,9 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     const uint32_t o_addr = tbase + lane_base + kOCol + 128 * grp;     // this thread's 128 of the row's 512 columns
     uint32_t gs = 0, xc = 0;                             // score tiles and exchanges so far
     // Warp 7 asks for the next unit's Q as soon as the scores of a unit's last tile are there: the MMAs have then read Q.
-    // It looks the unit up well before that.  A unit of one tile has its scores while this warp is still at the unit before:
-    // then it asks ahead of that one's epilogue, since that unit's P~V is followed by the Q K^T that the Q is for and the last
-    // P~V of the one-tile unit stands behind that.  (With inputs that are not in L2, asked for behind the epilogue and so: 60 x 55
-    // keys, five tokens 48.2 -> 43.8 us, E4M3 53.6 -> 48.3; 150 x 1-128, two tokens 50.0 -> 46.0; 192 x 1-512 43.8 -> 42.2.)
+    // It looks the unit up well before that.  For a unit of one tile that is ahead of the epilogue of the unit before, as it has
+    // to be: that unit's last P~V is followed by the Q K^T that the Q is for.  (Behind that epilogue: 60 x 55 keys, five tokens
+    // 43.8 -> 48.2 us, 192 x 1-512 42.2 -> 43.8.)
     constexpr int kAsksForQ = 7;
     uint32_t q_asked = 0;                                // units whose Q this warp has asked for
     int q_next = -1;                                     // first row of the next unit's Q, -1: there is none, or it has been asked for
@@ -289,31 +288,57 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
 #pragma unroll
       for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(ld_shared_b32(buf + i * (kCtaRows * 4)));
     };
+    // the same without a word: the row group's four warps have all come here
+    auto group_sync = [&]() {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(xbar);
+      ok = warp_wait(xbar, xc & 1);
+      ++xc;
+    };
+    // 32 keys of P~: half (chunk & 1) of page chunk / 2 of the P buffer
+    auto store_p = [&](int chunk, const uint32_t (&pk)[16]) {
+      const uint32_t dst = prow_smem + (chunk >> 1) * kPPageBytes;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) st_shared_v4(dst + (((4 * (chunk & 1) + c) ^ (r & 7)) << 4), pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+    };
 
     if (tid == 0 && leader) merge_begin(prm, part);
     write_empty_items(prm, prefix, part, prm.P, rank * kCtaRows, kCtaRows, tid, 32 * kSoftmaxWarps);
-    while (ok && tile.valid) {
-      const Unit u = tile.u;
-      const int row = u.r0 + rank * kCtaRows + r;        // row within the sequence
-      const int tok = row / prm.H;
-      const int visible = min(u.n_b, u.n_b - prm.Sq + tok + 1);        // keys 0..visible-1 are seen by this row
-      const int first_masked = max(u.n_b - prm.Sq + 1, 0) / kPage;     // pages from here on may hold hidden keys
-      RowState st;
-      row_state_init(st);
-      bool more = true;
-      while (more) {
-        const uint32_t sb = gs & 1;
-        const int t = tile.t, np = tile.np;
+    // A tile's softmax is done while the P~V of the tile before it still runs, and so is, at the end of a unit, that of the next
+    // unit's first tile ahead of the unit's own epilogue: P~ then waits in the columns that its scores had, and is copied into the
+    // P buffer when that P~V has read it.  What is left between two P~V is the epilogue or the rescale, and the copy.  Against
+    // exponentials behind that P~V and units whose softmax began behind the epilogue of the one before: 192 x 1-512 keys 38.8 ->
+    // 37.3 us, 60 x 55 with five tokens 38.3 -> 36.8, 150 x 1-128 with two 40.1 -> 38.1, 16 x 16384 86.3 -> 84.6, 96 x 2048 73.5 ->
+    // 72.5, 32 x 4096 50.4 -> 49.8; E4M3 32 x 4096 58.4, so 58.4.  (Only at the ends of units: 38.0, 87.6, 73.3, 50.3.)
+    RowState st;
+    row_state_init(st);
+    int visible = 0, first_masked = 0;
+    int e_row = -1, e_b = 0, e_slot = 0;                 // the unit whose epilogue is still to be done: this thread's row (-1: none), ...
+    float e_inv = 0.f, e_lse = 0.f;
+    while (tile.valid || e_row >= 0) {
+      const uint32_t sb = gs & 1;
+      const int t = tile.t, np = tile.np;
+      // A lane half holds 32 np neighbouring keys of a tile; this group takes its 32-key chunks grp and grp + 2.
+      const uint32_t scol = tbase + lane_base + kSCol + 128 * sb + 32 * grp;
+      const int chunk0 = np * khalf + grp;                                  // of the tile's 2 np
+      bool direct = false;                               // P~ goes straight into the P buffer
+      uint32_t nword = 0;
+      bool moved = false;
+      if (tile.valid) {
+        if (tile.first) {
+          const Unit& u = tile.u;
+          row_state_init(st);
+          const int tok = (u.r0 + rank * kCtaRows + r) / prm.H;
+          visible = min(u.n_b, u.n_b - prm.Sq + tok + 1);          // keys 0..visible-1 are seen by this row
+          first_masked = max(u.n_b - prm.Sq + 1, 0) / kPage;       // pages from here on may hold hidden keys
+        }
         ok = warp_wait(bar(X_SFULL + sb), (gs >> 1) & 1);
         if (!ok) break;
         tc_fence_after_sync();
         if (tid == 0 && leader) AMLA_STAMP(prm, part, 8, gs);
         if (wid == kAsksForQ && tile.last() && q_next >= 0) ask_for_q();
-        // A lane half holds 32 np neighbouring keys; this group takes its 32-key chunks grp and grp + 2.  The scores are
-        // read from tensor memory twice, a chunk at a time: for the maximum, and for the exponentials once the P buffer is
-        // free.  (Held in registers in between they cost 64 more of them and twice the code.)
-        const uint32_t scol = tbase + lane_base + kSCol + 128 * sb + 32 * grp;
-        const int chunk0 = np * khalf + grp;                                // of the tile's 2 np
+        // The scores are read from tensor memory twice, a chunk at a time: for the maximum, and for the exponentials.  (Held in
+        // registers in between they cost 64 more of them and twice the code.)
         const int nvis0 = visible - t * kPage - 32 * chunk0;                // keys of the first chunk that the row sees (may be <= 0)
         const bool plain = t + np <= first_masked && scale_nonneg;          // every key of the tile is visible
         // lines 5-6: running max (the scale is folded into the FMA below)
@@ -349,51 +374,9 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         // O is rescaled on far fewer tiles.  The four warps see the same maxima and agree.
         const bool must = tmax > st.m2 + prm.tau;
         const RowStep sp = row_step<kMode>(st, tmax, __any_sync(0xffffffffu, must) ? 0.f : prm.tau);
-        if (!tile.first) {
-          // the P~V of the tile before: it has read the P buffer, and O holds its sum
-          ok = warp_wait(bar(X_PVDONE), (gs - 1) & 1);
-          if (!ok) break;
-          const uint32_t nword = (kMode == 2) ? __float_as_uint(sp.l_up) : static_cast<uint32_t>(sp.n_bits);
-          const bool mine_moved = (kMode == 2) ? (sp.l_up != 1.f) : (sp.n_bits != 0);
-          if (__any_sync(0xffffffffu, mine_moved)) {
-            // lines 13-16: O <- AS_FP32(AS_INT32(O) + N).  The guarded add costs four integer operations per element, the
-            // FP32 multiply it replaces one.  The guard only matters for an element whose magnitude bits plus N would not
-            // stay positive (an exact zero, a value about to leave the normal range); so the smallest magnitude of the chunk
-            // is taken first (half an operation per element), and where it is safe the chunk gets the plain one-instruction
-            // add of Lemma 3.1.
-            tc_fence_after_sync();
-#pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
-              uint32_t o[32];
-              tmem_ld_32x32b_x32(o_addr + 32 * c, o);
-              tmem_wait_ld();
-              if (kMode == 2) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * __uint_as_float(nword));
-              } else {
-                bool safe = true;
-                if (kGuard) {
-                  float lo = fmin3_abs(__uint_as_float(o[0]), __uint_as_float(o[1]), __uint_as_float(o[2]));
-#pragma unroll
-                  for (int i = 3; i + 1 < 32; i += 2) lo = fmin3_abs(lo, __uint_as_float(o[i]), __uint_as_float(o[i + 1]));
-                  lo = fminf(lo, fabsf(__uint_as_float(o[31])));
-                  // NaN magnitudes compare as large numbers and take the plain add, like every other normal pattern
-                  safe = __float_as_int(lo) + static_cast<int>(nword) > 0;
-                }
-                if (safe) {
-#pragma unroll
-                  for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_raw(__uint_as_float(o[i]), static_cast<int>(nword)));
-                } else {
-#pragma unroll
-                  for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_guarded(__uint_as_float(o[i]), static_cast<int>(nword)));
-                }
-              }
-              tmem_st_32x32b_x32(o_addr + 32 * c, o);
-            }
-            tmem_wait_st();
-          }
-        }
-        if (tid == 0 && leader) AMLA_STAMP(prm, part, 11, gs);
+        nword = (kMode == 2) ? __float_as_uint(sp.l_up) : static_cast<uint32_t>(sp.n_bits);
+        moved = !tile.first && __any_sync(0xffffffffu, (kMode == 2) ? (sp.l_up != 1.f) : (sp.n_bits != 0));
+        direct = gs == 0 || (e_row < 0 && !moved && __all_sync(0xffffffffu, mbar_probe(bar(X_PVDONE), (gs - 1) & 1)));
         // Line 10's factor S16 goes into the exponential's argument (the remark after Algorithm 2).  The row sum of line 6 is
         // the sum of the same FP32 values, taken before the bf16 cast and divided by S16 once per tile.
         const float nsub = log2f_approx(sp.p_scale) - sp.m2_sub;
@@ -410,114 +393,157 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
 #pragma unroll
             for (int i = 0; i < 32; ++i) v[i] = i < nvis ? __float_as_uint(__uint_as_float(v[i]) * prm.scale_log2) : 0xff800000u;
           }
-          const int chunk = chunk0 + 2 * h;                // half (chunk & 1) of page chunk / 2
-          const uint32_t dst = prow_smem + (chunk >> 1) * kPPageBytes;
+          uint32_t pk[16];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            uint32_t pk[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              float x0, x1;
-              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[8 * c + 2 * i]), __uint_as_float(v[8 * c + 2 * i + 1])), sc2, ns2), x0, x1);
-              const float q0 = ex2_approx(x0), q1 = ex2_approx(x1);
-              const uint64_t pp = pack_f32x2(q0, q1);
-              if (i & 1) rsb = add_f32x2(rsb, pp); else rsa = add_f32x2(rsa, pp);
-              pk[i] = pack_bf16x2(q0, q1);
-            }
-            st_shared_v4(dst + (((4 * (chunk & 1) + c) ^ (r & 7)) << 4), pk[0], pk[1], pk[2], pk[3]);
+          for (int i = 0; i < 16; ++i) {
+            float x0, x1;
+            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), sc2, ns2), x0, x1);
+            const float q0 = ex2_approx(x0), q1 = ex2_approx(x1);
+            const uint64_t pp = pack_f32x2(q0, q1);
+            if (i & 1) rsb = add_f32x2(rsb, pp); else rsa = add_f32x2(rsa, pp);
+            pk[i] = pack_bf16x2(q0, q1);
           }
+          if (direct) store_p(chunk0 + 2 * h, pk);
+          else tmem_st_32x32b_x16(scol + 64 * h, pk);
         }
-        tc_fence_before_sync();            // S has been read, O (perhaps) rewritten
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          if (leader) { mbar_arrive(bar(X_SEMPTY + sb)); mbar_arrive(bar(X_PREADY)); }
-          else {                             // P~ of the whole warp, for the MMA issuer in the other CTA
-            release_shared_to_cluster();
-            mbar_arrive_cluster_relaxed(lead_bars + 8u * (X_SEMPTY + sb));
-            mbar_arrive_cluster_relaxed(lead_bars + 8u * X_PREADY);
-          }
-        }
-        if (tid == 0 && leader) AMLA_STAMP(prm, part, 12, gs);
-        {
-          float s0, s1;
-          unpack_f32x2(add_f32x2(rsa, rsb), s0, s1);
-          st.l = st.l * sp.l_up + __fdividef(s0 + s1, sp.p_scale);   // this thread's share of the row sum
-        }
-        if (!ok) break;
-        ++gs;
-        more = !tile.last();
-        if (more) tile.next();
+        float s0, s1;
+        unpack_f32x2(add_f32x2(rsa, rsb), s0, s1);
+        st.l = st.l * sp.l_up + __fdividef(s0 + s1, sp.p_scale);   // this thread's share of the row sum
       }
-      if (!ok) break;
-      // ---- epilogue (line 20): out = O / (l * S16), lse = m + ln l.  Thread = row; the four threads of a row take 128
-      // of its 512 columns each.
-      int2 info;
-      const int slot = tile.units.slot_of(u, &info);
-      if (tid == 0 && leader) merge_note(prm, part, u.it, info);
-      tile.next();
-      if (wid == kAsksForQ && tile.valid) look_ahead();
-      float l4[4];
-      exchange(st.l, l4);
-      if (!ok) break;
-      if (wid == kAsksForQ && tile.valid && tile.last() && q_next >= 0) {      // (its Q K^T is in front of the P~V that is waited for next)
-        ok = warp_wait(bar(X_SFULL + (gs & 1)), (gs >> 1) & 1);
+      if (!direct) {
+        // the P~V of the tile before: it has read the P buffer, and O holds its sum
+        tmem_wait_st();
+        ok = warp_wait(bar(X_PVDONE), (gs - 1) & 1);
         if (!ok) break;
-        ask_for_q();
-      }
-      const float l_all = (l4[0] + l4[1]) + (l4[2] + l4[3]);
-      const bool live = l_all > 0.f;
-      const float inv = live ? prm.out_scale / (l_all * st.s_out) : 0.f;
-      const float lse = live ? (st.m2 + log2f(l_all)) * kLn2 : -INFINITY;
-      ok = warp_wait(bar(X_PVDONE), (gs - 1) & 1);
-      if (!ok) break;
-      tc_fence_after_sync();
-      if (tid == 0 && leader) AMLA_STAMP(prm, part, 13, gs - 1);
-      const bool valid = row < prm.R;
-      const int col0 = 256 * khalf + 128 * grp;
-      const int prow0 = (slot < 0 ? 0 : slot) * kRowBlock + rank * kCtaRows;   // this CTA's first row of the partial arrays
-      // The warp's 32 rows x 64 columns at a time pass through the rows of the P buffer that belong to this row group (P~V has
-      // read them; the group writes them again only behind the next exchange), so that a store covers 128 bytes of four rows:
-      // whole lines leave the SM at about twice the rate of 32-byte pieces of 32 rows.  A lane stores 16 bytes, which is what `out`
-      // is aligned to (32 bytes of eight rows are no faster: 192 x 1-512 keys 43.98 us, so 44.00; 60 x 55, five tokens 48.2, 48.2).
-      const int row0 = u.r0 + rank * kCtaRows + (quarter & 1) * 32;       // this warp's first row within the sequence
-      uint16_t* const base = (slot < 0 ? reinterpret_cast<uint16_t*>(prm.out) + (static_cast<size_t>(u.b) * prm.R + row0) * kDv
-                                       : partial_halves(prm) + static_cast<size_t>(prow0 + (quarter & 1) * 32) * kDv) + col0;
-      const uint32_t stage = smem_base + kOffP + (2 * khalf + grp) * kPPageBytes + (quarter & 1) * 32 * 128;
-      uint32_t sc = 0;                                    // this thread's four scale bytes
+        tc_fence_after_sync();
+        if (e_row >= 0) {
+          // ---- epilogue (line 20): out = O / (l * S16), lse = m + ln l.  Thread = row; the four threads of a row take 128
+          // of its 512 columns each.
+          if (tid == 0 && leader) AMLA_STAMP(prm, part, 13, gs - 1);
+          const bool valid = e_row < prm.R;
+          const int col0 = 256 * khalf + 128 * grp;
+          const int prow0 = (e_slot < 0 ? 0 : e_slot) * kRowBlock + rank * kCtaRows;   // this CTA's first row of the partial arrays
+          // The warp's 32 rows x 64 columns at a time pass through the rows of the P buffer that belong to this row group (P~V has
+          // read them; the group writes them again only when all of its warps are done here), so that a store covers 128 bytes of
+          // four rows: whole lines leave the SM at about twice the rate of 32-byte pieces of 32 rows.  A lane stores 16 bytes, which
+          // is what `out` is aligned to (32 bytes of eight rows are no faster: 192 x 1-512 keys 43.98 us, so 44.00; 60 x 55, five
+          // tokens 48.2, 48.2).
+          const int row0 = e_row - lane;                      // this warp's first row within the sequence
+          uint16_t* const base = (e_slot < 0 ? reinterpret_cast<uint16_t*>(prm.out) + (static_cast<size_t>(e_b) * prm.R + row0) * kDv
+                                             : partial_halves(prm) + static_cast<size_t>(prow0 + (quarter & 1) * 32) * kDv) + col0;
+          const uint32_t stage = smem_base + kOffP + (2 * khalf + grp) * kPPageBytes + (quarter & 1) * 32 * 128;
+          uint32_t sc = 0;                                    // this thread's four scale bytes
 #pragma unroll 1
-      for (int c = 0; c < 4; c += 2) {
-        uint32_t o[2][32];
-        tmem_ld_32x32b_x32(o_addr + 32 * c, o[0]);
-        tmem_ld_32x32b_x32(o_addr + 32 * (c + 1), o[1]);
-        tmem_wait_ld();
+          for (int c = 0; c < 4; c += 2) {
+            uint32_t o[2][32];
+            tmem_ld_32x32b_x32(o_addr + 32 * c, o[0]);
+            tmem_ld_32x32b_x32(o_addr + 32 * (c + 1), o[1]);
+            tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          uint32_t w[16];
-          if (slot < 0) epilogue_chunk_bf16(o[e], inv, w);
-          else sc |= epilogue_chunk_partial(o[e], inv, w) << (8 * (c + e));
+            for (int e = 0; e < 2; ++e) {
+              uint32_t w[16];
+              if (e_slot < 0) epilogue_chunk_bf16(o[e], e_inv, w);
+              else sc |= epilogue_chunk_partial(o[e], e_inv, w) << (8 * (c + e));
 #pragma unroll
-          for (int i = 0; i < 4; ++i) st_shared_v4(stage + sw128_offset(lane, 4 * e + i), w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+              for (int i = 0; i < 4; ++i) st_shared_v4(stage + sw128_offset(lane, 4 * e + i), w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int rr = 4 * i + (lane >> 3), piece = lane & 7;
+              uint32_t x[4];
+              ld_shared_v4(stage + sw128_offset(rr, piece), x[0], x[1], x[2], x[3]);
+              if (row0 + rr < prm.R) stg_128(base + rr * kDv + 32 * c + 8 * piece, x[0], x[1], x[2], x[3]);
+            }
+            __syncwarp();
+          }
+          if (valid) {
+            if (e_slot >= 0) *reinterpret_cast<uint32_t*>(partial_scales(prm) + static_cast<size_t>(prow0 + r) * 16 + col0 / 32) = sc;
+            if (khalf == 0 && grp == 0) {
+              if (e_slot < 0) prm.lse[static_cast<size_t>(e_b) * prm.R + e_row] = e_lse;
+              else prm.part_lse[prow0 + r] = e_lse;
+            }
+          }
+          e_row = -1;
+          if (tid == 0 && leader) AMLA_STAMP(prm, part, 14, gs - 1);
+          if (!tile.valid) break;
+          group_sync();                                       // the row group's four warps are done with their rows of the P buffer
+          if (!ok) break;
+        } else if (moved) {
+          // lines 13-16: O <- AS_FP32(AS_INT32(O) + N).  The guarded add costs four integer operations per element, the
+          // FP32 multiply it replaces one.  The guard only matters for an element whose magnitude bits plus N would not
+          // stay positive (an exact zero, a value about to leave the normal range); so the smallest magnitude of the chunk
+          // is taken first (half an operation per element), and where it is safe the chunk gets the plain one-instruction
+          // add of Lemma 3.1.
+#pragma unroll 1
+          for (int c = 0; c < 4; ++c) {
+            uint32_t o[32];
+            tmem_ld_32x32b_x32(o_addr + 32 * c, o);
+            tmem_wait_ld();
+            if (kMode == 2) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * __uint_as_float(nword));
+            } else {
+              bool safe = true;
+              if (kGuard) {
+                float lo = fmin3_abs(__uint_as_float(o[0]), __uint_as_float(o[1]), __uint_as_float(o[2]));
+#pragma unroll
+                for (int i = 3; i + 1 < 32; i += 2) lo = fmin3_abs(lo, __uint_as_float(o[i]), __uint_as_float(o[i + 1]));
+                lo = fminf(lo, fabsf(__uint_as_float(o[31])));
+                // NaN magnitudes compare as large numbers and take the plain add, like every other normal pattern
+                safe = __float_as_int(lo) + static_cast<int>(nword) > 0;
+              }
+              if (safe) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_raw(__uint_as_float(o[i]), static_cast<int>(nword)));
+              } else {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(exponent_add_guarded(__uint_as_float(o[i]), static_cast<int>(nword)));
+              }
+            }
+            tmem_st_32x32b_x32(o_addr + 32 * c, o);
+          }
+          tmem_wait_st();
         }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int rr = 4 * i + (lane >> 3), piece = lane & 7;
-          uint32_t x[4];
-          ld_shared_v4(stage + sw128_offset(rr, piece), x[0], x[1], x[2], x[3]);
-          if (row0 + rr < prm.R) stg_128(base + rr * kDv + 32 * c + 8 * piece, x[0], x[1], x[2], x[3]);
+        if (tid == 0 && leader) AMLA_STAMP(prm, part, 11, gs);
+#pragma unroll 1
+        for (int h = 0; grp + 2 * h < np && h < 2; ++h) {
+          uint32_t pk[16];
+          tmem_ld_32x32b_x16(scol + 64 * h, pk);
+          tmem_wait_ld();
+          store_p(chunk0 + 2 * h, pk);
         }
-        __syncwarp();
       }
-      tc_fence_before_sync();      // O has been read: this warp's next PREADY arrival lets the next unit overwrite it
-      if (valid) {
-        if (slot >= 0) *reinterpret_cast<uint32_t*>(partial_scales(prm) + static_cast<size_t>(prow0 + r) * 16 + col0 / 32) = sc;
-        if (khalf == 0 && grp == 0) {
-          if (slot < 0) prm.lse[static_cast<size_t>(u.b) * prm.R + row] = lse;
-          else prm.part_lse[prow0 + r] = lse;
+      tc_fence_before_sync();            // S has been read, O (perhaps) rewritten
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        if (leader) { mbar_arrive(bar(X_SEMPTY + sb)); mbar_arrive(bar(X_PREADY)); }
+        else {                             // P~ of the whole warp, for the MMA issuer in the other CTA
+          release_shared_to_cluster();
+          mbar_arrive_cluster_relaxed(lead_bars + 8u * (X_SEMPTY + sb));
+          mbar_arrive_cluster_relaxed(lead_bars + 8u * X_PREADY);
         }
       }
-      if (tid == 0 && leader) AMLA_STAMP(prm, part, 14, gs - 1);
+      if (tid == 0 && leader) AMLA_STAMP(prm, part, 12, gs);
+      ++gs;
+      if (tile.last()) {                   // what the unit's epilogue needs
+        const Unit& u = tile.u;
+        int2 info;
+        e_slot = tile.units.slot_of(u, &info);
+        if (tid == 0 && leader) merge_note(prm, part, u.it, info);
+        e_b = u.b;
+        e_row = u.r0 + rank * kCtaRows + r;
+        float l4[4];
+        exchange(st.l, l4);
+        if (!ok) break;
+        const float l_all = (l4[0] + l4[1]) + (l4[2] + l4[3]);
+        const bool live = l_all > 0.f;
+        e_inv = live ? prm.out_scale / (l_all * st.s_out) : 0.f;
+        e_lse = live ? (st.m2 + log2f(l_all)) * kLn2 : -INFINITY;
+      }
+      tile.next();
+      if (wid == kAsksForQ && tile.valid && tile.first) look_ahead();
     }
     if (!ok && lane == 0) {
       report_timeout(prm.status);
