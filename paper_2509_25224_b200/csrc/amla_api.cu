@@ -108,6 +108,18 @@ static bool blocks_of_256(const DecodeParams& prm, int pair_parts, int quad_part
   return 21.5 + 2.08 * items2 * tiles + 11. * std::max(items2 - 1., 0.) < 13. + 1.41 * items1 * pages + 6. * items1;
 }
 
+// An E4M3 cache in the 128-row kernel: are K's bytes multiplied as they are, with a Q that is split into 8-bit numbers, or is K widened
+// like V?  Splitting Q costs a call 1-1.5 us at its start and every further item of a part ~3 us, and a page takes 0.3 us less.
+// Measured over 1-300 items of 55-20000 keys (widened / split, us): 1 x 4000 keys 15.0 / 16.2, 1 x 20000 21.8 / 21.7, 60 x 256
+// 22.1 / 25.5, 60 x 1000 38.4 / 38.3, 150 x 512 48.1 / 50.0, 150 x 1024 70.9 / 66.8, 200 x 1-2048 95.2 / 87.5; five tokens, 60 x 55
+// 41.9 / 54.9, 60 x 512 77.9 / 81.7, 60 x 1024 124 / 118.5; two, 32 x 512-8192 111 / 94.5.  Lengths are not known here: the table's
+// width stands for them, or the pages that the cache has.
+static bool split_q_pays(const DecodeParams& prm, int parts) {
+  const double slots = std::min(static_cast<double>(prm.B) * prm.max_blocks_per_seq, static_cast<double>(prm.num_blocks));
+  const double pages = slots * prm.nrb / parts, items = static_cast<double>(prm.n_items) / parts;
+  return 0.3 * pages > 1. + 3.2 * items;
+}
+
 // Chooses the kernel for the shape and fills the schedule fields of prm (rows per item, keys per tile, parts):
 //   up to 32 query rows of a bf16 cache      the kernel for few rows
 //   more than 128 rows of a bf16 cache       the 256-row kernel (four-CTA clusters, pair MMAs) where it is the faster one
@@ -135,6 +147,7 @@ int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
   prm.nrb = (prm.R + prm.item_rows - 1) / prm.item_rows;
   prm.n_items = prm.B * prm.nrb;
   prm.P = simt || few ? sms : quad ? quad_parts : decode_pair_parts(sms);
+  prm.split_q = prm.kv8 != nullptr && split_q_pays(prm, prm.P) ? 1 : 0;
   // No more parts than the longest schedule that the block table's width allows can fill.  A schedule of one score tile at
   // most is one part: nothing is split and no combine kernel runs.
   const long long tiles = (static_cast<long long>(prm.max_blocks_per_seq) * kPage + prm.tile_keys - 1) / prm.tile_keys;
