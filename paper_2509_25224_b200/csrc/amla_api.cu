@@ -293,13 +293,15 @@ int decode_impl(const void* q, const void* kv_cache, const uint8_t* kv8, const i
 }
 
 // Are the pages of an E4M3 cache widened into a bf16 copy first, and the bf16 kernels run on that, or does the 128-row kernel
-// widen them on their way in?  On their way in they are widened once more for every 128 query rows, and for K and for V; the
-// copy costs its writing and reading once, and more than 128 rows then are blocks of 256.  Measured (on the way in / copy
-// first, 128 heads): eight tokens 32 x 4096 keys 381 / 326 us, 16 x 16384 734 / 599, 1 x 65536 183 / 150; six tokens 289 / 259,
-// 566 / 488; but five and less differ by little or the other way (1 x 4096 20.6 / 21.0, two tokens 32 x 4096 98 / 130), and so
-// do small calls (1 x 100, six tokens 12.1 / 13.6; 20 x 375-3000 79.7 / 81.0).  Lengths are not known here: the table's width
-// stands for them, unless the cache could not fill half of such a table (100 sequences of 300 keys, six tokens, a table of
-// 512 pages: 141 / 184).  (All with raw slots of half their present size: 3-5 % off the times on the way in since.)  (The scalar bring-up kernel reads bf16 only.)
+// widen them on their way in?  On their way in they are widened once more for every 128 query rows, for V and mostly for K; the
+// copy costs its writing and reading once, and more than 128 rows then are blocks of 256.  Where K's bytes are an operand as
+// they land (a split Q: long parts), only V is widened on its way in.  Measured (on the way in / copy first, 128 heads, us):
+// eight tokens 32 x 4096 keys 332 / 330, 16 x 16384 624 / 597, 64 x 1000 209 / 195; six tokens 253 / 267, 472 / 488.  So the
+// line of six blocks costs such calls 3-6 % at six blocks and gains 1-7 % at eight; it was drawn where K is widened
+// too (six tokens 289 / 259, 566 / 488; five and less differ by little or the other way: 1 x 4096 20.6 / 21.0, two tokens
+// 32 x 4096 98 / 130), and small calls are kept out of it (1 x 100, six tokens 12.1 / 13.6; 20 x 375-3000 79.7 / 81.0).
+// Lengths are not known here: the table's width stands for them, unless the cache could not fill half of such a table
+// (100 sequences of 300 keys, six tokens, a table of 512 pages: 141 / 184).  (The scalar bring-up kernel reads bf16 only.)
 bool widen_first(int B, int rows, int num_blocks, int max_blocks_per_seq, int flags) {
   if (flags & AMLA_FLAG_KERNEL_SIMT) return true;
   const long long row_blocks = (rows + kRowBlock - 1) / kRowBlock, slots = static_cast<long long>(B) * max_blocks_per_seq;
