@@ -147,7 +147,7 @@ int amla_mla_decode_ex(const void* q, const void* kv_cache, const int32_t* block
 
 /*
  * The same decode on an FP8 cache (the remark after Lemma 3.1: the rescaling trick is tied to the accumulator's
- * format, not to the inputs'; the accumulator stays FP32, P~ stays bf16).
+ * format, not to the inputs'; the accumulator stays FP32, Q and P~ stay bf16).
  *
  *   kv_cache_e4m3  device, uint8 [num_blocks, 64, 576], 16-byte aligned: OCP FP8 E4M3 (1 sign, 4 exponent bits with
  *                  bias 7, 3 mantissa bits; no infinities, S.1111.111 is NaN).  The value of an element is
@@ -156,9 +156,7 @@ int amla_mla_decode_ex(const void* q, const void* kv_cache, const int32_t* block
  *   workspace      at least amla_mla_decode_fp8_workspace_size() bytes, 256-byte aligned
  *   flags          as for amla_mla_decode_ex
  *
- * The pages are widened, exactly, on their way into the tensor cores' operand tiles, or, in long calls, V is and K's
- * bytes are multiplied as they are with each element of Q as the sum of an E4M3 and an E5M2 number (exact down to 2^-14
- * of its row's largest magnitude, to 2^-20 of that below); kv_scale is folded into the
+ * The pages are widened, exactly, on their way into the tensor cores' operand tiles; kv_scale is folded into the
  * softmax scale and into the final normalisation.  A call reads half the bytes of a bf16 cache.  (Large calls of more
  * than 640 query rows per sequence, and AMLA_FLAG_KERNEL_SIMT, widen the used pages into a bf16 copy inside the
  * workspace first: B * max_blocks_per_seq pages of 73 728 bytes.)  Everything else (visibility rule,

@@ -108,18 +108,6 @@ static bool blocks_of_256(const DecodeParams& prm, int pair_parts, int quad_part
   return 21.5 + 2.08 * items2 * tiles + 11. * std::max(items2 - 1., 0.) < 13. + 1.41 * items1 * pages + 6. * items1;
 }
 
-// An E4M3 cache in the 128-row kernel: are K's bytes multiplied as they are, with a Q that is split into 8-bit numbers, or is K widened
-// like V?  Splitting Q costs a call 1-1.5 us at its start and every further item of a part ~3 us, and a page takes 0.3 us less.
-// Measured over 1-300 items of 55-20000 keys (widened / split, us): 1 x 4000 keys 15.0 / 16.2, 1 x 20000 21.8 / 21.7, 60 x 256
-// 22.1 / 25.5, 60 x 1000 38.4 / 38.3, 150 x 512 48.1 / 50.0, 150 x 1024 70.9 / 66.8, 200 x 1-2048 95.2 / 87.5; five tokens, 60 x 55
-// 41.9 / 54.9, 60 x 512 77.9 / 81.7, 60 x 1024 124 / 118.5; two, 32 x 512-8192 111 / 94.5.  Lengths are not known here: the table's
-// width stands for them, or the pages that the cache has.
-static bool split_q_pays(const DecodeParams& prm, int parts) {
-  const double slots = std::min(static_cast<double>(prm.B) * prm.max_blocks_per_seq, static_cast<double>(prm.num_blocks));
-  const double pages = slots * prm.nrb / parts, items = static_cast<double>(prm.n_items) / parts;
-  return 0.3 * pages > 1. + 3.2 * items;
-}
-
 // Chooses the kernel for the shape and fills the schedule fields of prm (rows per item, keys per tile, parts):
 //   up to 32 query rows of a bf16 cache      the kernel for few rows
 //   more than 128 rows of a bf16 cache       the 256-row kernel (four-CTA clusters, pair MMAs) where it is the faster one
@@ -147,7 +135,6 @@ int configure_schedule(DecodeParams& prm, int device, int sms, int flags) {
   prm.nrb = (prm.R + prm.item_rows - 1) / prm.item_rows;
   prm.n_items = prm.B * prm.nrb;
   prm.P = simt || few ? sms : quad ? quad_parts : decode_pair_parts(sms);
-  prm.split_q = prm.kv8 != nullptr && split_q_pays(prm, prm.P) ? 1 : 0;
   // No more parts than the longest schedule that the block table's width allows can fill.  A schedule of one score tile at
   // most is one part: nothing is split and no combine kernel runs.
   const long long tiles = (static_cast<long long>(prm.max_blocks_per_seq) * kPage + prm.tile_keys - 1) / prm.tile_keys;
@@ -293,15 +280,13 @@ int decode_impl(const void* q, const void* kv_cache, const uint8_t* kv8, const i
 }
 
 // Are the pages of an E4M3 cache widened into a bf16 copy first, and the bf16 kernels run on that, or does the 128-row kernel
-// widen them on their way in?  On their way in they are widened once more for every 128 query rows, for V and mostly for K; the
-// copy costs its writing and reading once, and more than 128 rows then are blocks of 256.  Where K's bytes are an operand as
-// they land (a split Q: long parts), only V is widened on its way in.  Measured (on the way in / copy first, 128 heads, us):
-// eight tokens 32 x 4096 keys 332 / 330, 16 x 16384 624 / 597, 64 x 1000 209 / 195; six tokens 253 / 267, 472 / 488.  So the
-// line of six blocks costs such calls 3-6 % at six blocks and gains 1-7 % at eight; it was drawn where K is widened
-// too (six tokens 289 / 259, 566 / 488; five and less differ by little or the other way: 1 x 4096 20.6 / 21.0, two tokens
-// 32 x 4096 98 / 130), and small calls are kept out of it (1 x 100, six tokens 12.1 / 13.6; 20 x 375-3000 79.7 / 81.0).
-// Lengths are not known here: the table's width stands for them, unless the cache could not fill half of such a table
-// (100 sequences of 300 keys, six tokens, a table of 512 pages: 141 / 184).  (The scalar bring-up kernel reads bf16 only.)
+// widen them on their way in?  On their way in they are widened once more for every 128 query rows, and for K and for V; the
+// copy costs its writing and reading once, and more than 128 rows then are blocks of 256.  Measured (on the way in / copy
+// first, 128 heads, us): eight tokens 32 x 4096 keys 387 / 325, 16 x 16384 744 / 561, 64 x 1000 227 / 182; six tokens 275 / 253,
+// 551 / 452; but five and less differ by little or the other way (32 x 4096 220, 1 x 4096 20.6 / 21.0, two tokens 32 x 4096
+// 98 / 130), and so do small calls (1 x 100, six tokens 12.1 / 13.6; 20 x 375-3000 79.7 / 81.0).  Lengths are not known here: the
+// table's width stands for them, unless the cache could not fill half of such a table (100 sequences of 300 keys, six tokens, a
+// table of 512 pages: 141 / 184).  (The scalar bring-up kernel reads bf16 only.)
 bool widen_first(int B, int rows, int num_blocks, int max_blocks_per_seq, int flags) {
   if (flags & AMLA_FLAG_KERNEL_SIMT) return true;
   const long long row_blocks = (rows + kRowBlock - 1) / kRowBlock, slots = static_cast<long long>(B) * max_blocks_per_seq;

@@ -52,7 +52,6 @@ struct DecodeParams {
   int item_rows;                 // query rows per work item: 32, 128 or 256, after the kernel (nrb counts these)
   int ovh;                       // schedule positions that stand for the cost of starting an item
   int min_share;                 // a part is given at least this many positions
-  int split_q;                   // an E4M3 cache: the 128-row kernel multiplies K's bytes with a split Q instead of widening K
   unsigned long long* trace;     // timeline buffer of a -DAMLA_TRACE build, else unused (nullptr)
 };
 
@@ -211,20 +210,6 @@ __device__ __forceinline__ uint32_t e4m3x2_to_bf16x2(uint32_t pair) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
-}
-
-// Two FP32 values as the sum of an E4M3 and an E5M2 each (lower value in the low byte): the nearest E4M3, then the nearest
-// E5M2 to what that leaves.
-__device__ __forceinline__ void split_f8x2(float lo, float hi, uint32_t& e4m3x2, uint32_t& e5m2x2) {
-  uint16_t a, b;
-  uint32_t h2, back, rest;
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(h2) : "f"(hi), "f"(lo));
-  asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(a) : "r"(h2));
-  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(back) : "h"(a));
-  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(rest) : "r"(h2), "r"(back));
-  asm("cvt.rn.satfinite.e5m2x2.f16x2 %0, %1;" : "=h"(b) : "r"(rest));
-  e4m3x2 = a;
-  e5m2x2 = b;
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -25,15 +25,15 @@
 // crossed to the other SM by remote stores, Q went through shared memory into tensor memory and the score CTA had to be
 // drained before the next unit's Q could follow.  Here nothing but MMA operands crosses, Q is an operand as it lands, and
 // the tile is 256 keys.  Calls with it, from that kernel to this one as it stands (sustained): 192 sequences of 1-512 keys
-// 62.8 -> 37.5 us; one of 2531 33.8 -> 12.4; 16 x 16384 with rising logits 106.0 -> 88; 96 x 2048 88.7 -> 75; 32 x 4096
-// 59.1 -> 51.4; E4M3 32 x 4096 100.4 -> 52.
+// 62.8 -> 42.2 us; one of 2531 33.8 -> 12.4; 16 x 16384 with rising logits 106.0 -> 92.7; 96 x 2048 88.7 -> 79.2; 32 x 4096
+// 59.1 -> 53.7; E4M3 32 x 4096 100.4 -> 60.6.
 // What bounds it (trace): a tile of 256 keys takes 7100 clk in long units, 7600 on average over the eight of a 32 x 4096 call,
-// against 4350 of MMAs, 5600 of shared memory at 128 bytes a clk (MMA operands 408 KB, TMA 278, P~ 32) and 5900-6600 of HBM.  The
-// issuer finds every slot full that it comes to, and takes 350 clk for a slot of K and 390 for one of V, 17 of them a tile: the
-// operands of four MMAs and the 16 KB that TMA writes meanwhile are 320 clk of shared memory.  E4M3: see split_q_rows.  From a call's
-// first loads to Q K^T of its second tile HBM is what it waits for (6.8 us for two tiles of all clusters: neither asking for
-// the second tile's K ahead of its slots nor for the first one's before griddepcontrol.wait helped).  Long calls run at the power limit, at
-// 1.4-1.7 GHz: 32 x 4096 takes 48.5 us cool, 16 x 16384 77 where it takes 88 sustained.
+// against 4350 of MMAs and 5900 of HBM at its full rate.  The issuer finds every slot full that it comes to, and takes 350 clk
+// for a slot of K and 390 for one of V, 17 of them a tile; what is left are its waits for the softmax warps.  A slot is full
+// 2200 clk (K, most of it from L2) or 2400 clk (V) after it has been asked for, and is asked for again 630 or 690 clk later: a
+// ring of 112 KB for the 278 KB of a tile just about keeps up.  E4M3: 9800 clk; a pair of widening warps takes 700 clk for a
+// slot and has waited 540 for its place, 150 for the raw slot; the issuer waits for one slot in ten.  Long calls run at the
+// power limit: 32 x 4096 takes 50 us cool.
 //
 // All waits are bounded; on expiry the kernel records kStatusTimeout and unwinds.
 #include "amla_common.cuh"
@@ -49,15 +49,12 @@ using namespace sm100;
 namespace {
 
 constexpr int kSoftmaxWarps = 8;
-// What the kernel reads: a bf16 cache; an E4M3 cache whose K and V are both widened to bf16; an E4M3 cache whose K is an operand
-// as it is, against a Q that is split into 8-bit numbers.  (launch_decode_pair's caller chooses between the last two.)
-enum { kBf16 = 0, kWidenAll = 1, kSplitQ = 2 };
 // bf16 cache: warps 8, 10 and 11 load.  E4M3 cache: warp 8 loads (more warps would leave too few registers), warps 10-15
 // widen, three pairs taking turns.
 constexpr int kWidenGroups = 3, kWidenWarps = 2;
 constexpr int kWideners = kWidenGroups * kWidenWarps;
 constexpr int kLoaders = 3;
-template <int kCache> constexpr int kThreads = 32 * (kCache != kBf16 ? kSoftmaxWarps + 2 + kWideners : kSoftmaxWarps + 1 + kLoaders);
+template <bool kFp8> constexpr int kThreads = 32 * (kFp8 ? kSoftmaxWarps + 2 + kWideners : kSoftmaxWarps + 1 + kLoaders);
 constexpr int kTilePages = 4;                           // pages of a score tile: N = 256, the widest MMA
 constexpr int kCtaRows = kRowBlock / 2;                 // query rows per CTA
 constexpr int kQBlocks = kDqk / 64;                     // 64-column blocks of Q and K
@@ -67,32 +64,24 @@ constexpr uint32_t kPPageBytes = kCtaRows * 128;        // P~ of one page: [64 r
 constexpr uint32_t kKBoxBytes = 32 * 128;               // half a page (32 keys) x one 64-column block
 constexpr uint32_t kSlotBytes = 128 * 128;              // K: half of 4 pages' keys x 64 columns; V: 64 keys x 128 columns
 constexpr uint32_t kVBlockBytes = 64 * 128;             // 64 keys x 64 columns
-// The ring of operand slots, and for an E4M3 cache a second ring: of raw slots in front of it, one for every two operand slots
-// (kWidenAll), or of K's bytes beside it (kSplitQ).
+// The ring of operand slots, and for an E4M3 cache a ring of raw slots in front of it, one for every two operand slots.
 // A rule that every user of a ring keeps: a thread waits only for slots that it fills or empties itself, and having waited
 // for number w (counted over the whole run; slots are released in order) next for one of w + 1 ... w + R, R being the number
 // of slots.  The barriers tell two successive phases apart, no more: a thread that asks for a phase further on is let
 // through by an older one, and one that comes to ask after the next phase has passed as well is held for good.  (So the
 // three loaders take every third number on a ring of seven slots, and the three pairs that widen step by three through four operand
 // slots, and so by one or two through three raw slots.  Raw slots are filled in any order, since V comes from L2 and K from HBM, so
-// a pair waits for its operand slot first: that it is free says which raw slots had been full.  With kSplitQ each pair has one
-// of three operand slots.)
-template <int kCache> constexpr int kSlots = kCache == kSplitQ ? 3 : kCache == kWidenAll ? 4 : 7;
+// a pair waits for its operand slot first: that it is free says which raw slots had been full.)
+template <bool kFp8> constexpr int kSlots = kFp8 ? 4 : 7;
 constexpr int kRawSlots = 3;
 constexpr uint32_t kRawBytes = kSlotBytes;              // the bytes of two operand slots
-constexpr int kByteSlots = 4;
-constexpr int kByteSlotsOfTile = (kQBlocks + 1) / 2;    // half of 4 pages' keys x 128 columns of bytes each
-// kSplitQ: Q as two 8-bit numbers for each of bf16's, see split_q_rows: 128 columns of the larger ones in 16 KB steps, 128 of the
-// smaller behind them, and the RoPE columns' of both side by side at the end.
-constexpr uint32_t kQStep = 2 * kQBlockBytes;
 
 constexpr uint32_t kOffQ = 0;
 constexpr uint32_t kOffP = kOffQ + kQBytes;
 constexpr uint32_t kOffRing = kOffP + kTilePages * kPPageBytes;
-constexpr uint32_t kOffRaw = kOffRing + kSlots<kWidenAll> * kSlotBytes;
-constexpr uint32_t kOffBytes = kOffRing + kSlots<kSplitQ> * kSlotBytes;
+constexpr uint32_t kOffRaw = kOffRing + kSlots<true> * kSlotBytes;
 constexpr uint32_t kOffXchg = kOffRing + 7 * kSlotBytes;           // float [2][4 threads of a row][64 rows]
-static_assert(kOffRaw + kRawSlots * kRawBytes <= kOffXchg && kOffBytes + kByteSlots * kSlotBytes <= kOffXchg && kSlots<kBf16> <= 7, "the rings share one area");
+static_assert(kOffRaw + kRawSlots * kRawBytes <= kOffXchg && kSlots<false> <= 7, "the rings share one area");
 constexpr uint32_t kOffBars = kOffXchg + 2 * 4 * kCtaRows * 4;
 constexpr uint32_t kBarBytes = 384;
 // a copy of the schedule prefix and of the sequence lengths for batches of up to kSmemPlanItems items, so that the
@@ -101,12 +90,7 @@ constexpr int kSmemPlanItems = 512;
 constexpr uint32_t kOffPlan = kOffBars + kBarBytes;
 constexpr uint32_t kOffSeqlens = kOffPlan + ((kSmemPlanItems + 1) * 4 + 15) / 16 * 16;
 constexpr uint32_t kOffFirst = kOffSeqlens + kSmemPlanItems * 4;
-// kSplitQ: float [units, the last four][64 rows].  (Q of a unit is converted when Q K^T of all before it is done, whose scores have
-// two buffers: the softmax warps have then begun the unit three before, so that a fourth set can be overwritten, and its barrier
-// reused.)
-constexpr int kRowScales = 4;
-constexpr uint32_t kOffRowScale = (kOffFirst + sizeof(FirstUnit) + 15) / 16 * 16;
-constexpr uint32_t kSmemBytes = kOffRowScale + kRowScales * kCtaRows * 4;
+constexpr uint32_t kSmemBytes = kOffFirst + sizeof(FirstUnit);
 static_assert(kSmemBytes <= 232448, "exceeds the shared memory a block can opt in to");
 static_assert(kOffP % 1024 == 0 && kOffRing % 1024 == 0, "swizzled tiles need 1024-byte alignment");
 
@@ -116,19 +100,10 @@ constexpr uint32_t kOCol = 0;            // 256 columns
 constexpr uint32_t kSCol = 256;          // 2 x 128 columns
 
 // Barriers.  (L): the copy in the even CTA is the one that counts; both CTAs arrive there.  The others exist in both
-// CTAs and complete by multicast commits of the even CTA's MMA warp, except X_XCHG, X_QTHERE, X_QSCALE, the raw
-// ring's and those of the odd CTA's half of FULL, which are local.
+// CTAs and complete by multicast commits of the even CTA's MMA warp, except X_XCHG and the raw ring's, which are local.
 enum { X_FULL = 0 /*L*/, X_EMPTY = X_FULL + 7, X_QFULL = X_EMPTY + 7 /*L*/, X_SFULL, X_SEMPTY = X_SFULL + 2 /*L*/,
-       X_PREADY = X_SEMPTY + 2 /*L*/, X_PVDONE, X_XCHG,
-       X_CACHE = X_XCHG + 2,
-       // kWidenAll: the raw ring; the odd CTA's half of FULL, passed on
-       X_RAWFULL = X_CACHE, X_RAWEMPTY = X_RAWFULL + kRawSlots, X_RAWODD = X_RAWEMPTY + kRawSlots,
-       // kSplitQ: the ring of K's bytes; the odd CTA's half of FULL, passed on; the MMAs have read a unit's Q; the next one's is
-       // there, as bf16; it is split and the scales of its rows are there
-       X_BYTESFULL = X_CACHE /*L*/, X_BYTESEMPTY = X_BYTESFULL + kByteSlots, X_VODD = X_BYTESEMPTY + kByteSlots, X_QFREE = X_VODD + kSlots<kSplitQ>,
-       X_QTHERE, X_QSCALE, X_NUM = X_QSCALE + kRowScales };
-static_assert(X_RAWODD + kSlots<kWidenAll> <= X_NUM, "barriers");
-template <int kCache> constexpr int kFullOdd = kCache == kWidenAll ? X_RAWODD : X_VODD;
+       X_PREADY = X_SEMPTY + 2 /*L*/, X_PVDONE, X_XCHG, X_RAWFULL = X_XCHG + 2, X_RAWEMPTY = X_RAWFULL + kRawSlots,
+       X_FULLODD = X_RAWEMPTY + kRawSlots /* odd CTA, E4M3: its half of FULL, passed on */, X_NUM = X_FULLODD + kSlots<true> };
 static_assert(X_NUM * 8 + 8 <= kBarBytes, "barrier area too small");
 
 __device__ __forceinline__ void report_timeout(int* status) { atomicExch(status, kStatusTimeout); }
@@ -167,77 +142,12 @@ __device__ __forceinline__ void request_q(const CUtensorMap& q_map, uint32_t sme
     tma_load_3d_pair_hint(smem_base + kOffQ + c * kQBlockBytes, &q_map, 0, qrow, c, lead_bars + 8u * X_QFULL, last_use);
 }
 
-// E4M3: four rows of Q (eight threads each), which lie where they landed as bf16, [block of 64 columns][64 rows][128 B], become two
-// 8-bit numbers for each of theirs where they are: two blocks of a row its 128 larger numbers and its 128 smaller ones, the ninth
-// (the RoPE columns) both side by side.  `row`: of the CTA's 64; leaves the factor on the row's scores.
-//
-// Q K^T of an E4M3 cache is made of 8-bit products: K's bytes are an operand as they land, and a row of Q, times the power of
-// two that brings its largest magnitude into [128, 256), is the sum of an E4M3 and an E5M2 number for each of its bf16 numbers
-// (eight significant bits = four and a rest of three): two MMAs of K = 32 at twice the rate of bf16's.  The sum is exact for
-// what is not below 2^-14 of the row's largest magnitude, and off by 2^-20 of that at most below.  The power of two comes
-// off again in the factor on the row's scores.  A row with an infinity or a NaN in it gets NaN scores.
-//
-// Why: what an E4M3 tile spent its time on was not HBM or the tensor pipe but making operands of bytes.  Widened, K and V are 17
-// slots of 16 KB a tile, ~575 clk each: shared memory moves 996 KB for a tile of 256 keys (7.8 K clk at 128 bytes), and two
-// schedulers of the four convert 17 x 352 clk.  K's bytes as they are leave 8 slots and 775 KB.  A tile 10.9 K clk -> 8.4 K; 32 x 4096 keys
-// 58.2 -> 51.2 us, 32 x 512-8192 with two tokens 113 -> 99, 16 x 16384 104.7 -> 88.5.  Errors against 64 bits, from widened K to this
-// (256-20000 keys): out 1.76-1.97e-3 of its norm, to five digits the same; lse 5.4-5.8e-7 -> 4.9-5.3e-7, as the smaller parts are
-// summed first (5.5-5.9e-7 otherwise, 0.3 % faster).  Also with one column of Q a thousand times the others.
-//
-// In loops and not inlined: code that is run once for a unit costs its way into the instruction cache (written out, with the
-// rows in registers: 1.9 us for four rows and six warps; so 0.8).
-static __device__ __noinline__ void split_q_rows(uint32_t q_smem, uint32_t factors, int row, float scale_log2) {
-  const uint32_t ln = threadIdx.x & 7, sw = row & 7, base = q_smem + row * 128, mine = (ln ^ sw) << 4;
-  uint32_t most = 0;
-#pragma unroll 3
-  for (int c = 0; c < kQBlocks; ++c) {
-    uint32_t x[4];
-    ld_shared_v4(base + c * kQBlockBytes + mine, x[0], x[1], x[2], x[3]);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) most = __vmaxu2(most, x[i] & 0x7fff7fffu);
-  }
-#pragma unroll
-  for (int o = 4; o; o >>= 1) most = __vmaxu2(most, __shfl_xor_sync(0xffffffffu, most, o));
-  const uint32_t e = max(most & 0xffffu, most >> 16) >> 7;             // exponent field of the largest magnitude
-  const uint32_t ec = max(e, 14u);                                     // (a row of zeros or of next to nothing)
-  const float up = __uint_as_float((261u - ec) << 23);                 // 2^(134 - ec)
-  if (ln == 0) st_shared_b32(factors + row * 4, e == 255u ? 0x7fffffffu : __float_as_uint(scale_log2 * __uint_as_float((ec - 7u) << 23)));
-#pragma unroll 1
-  for (int c = 0; c < kQBlocks; c += 2) {
-    const uint32_t at = base + c * kQBlockBytes;
-    const bool rope = c == kQBlocks - 1;
-    uint32_t x[2][4];
-    ld_shared_v4(at + mine, x[0][0], x[0][1], x[0][2], x[0][3]);
-    ld_shared_v4(at + (rope ? 0 : kQBlockBytes) + mine, x[1][0], x[1][1], x[1][2], x[1][3]);
-    uint32_t hi[2][4], lo[2][4];
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        split_f8x2(__uint_as_float(x[h][i] << 16) * up, __uint_as_float(x[h][i] & 0xffff0000u) * up, hi[h][i], lo[h][i]);
-    __syncwarp();                                                      // (the row has been read)
-    const uint32_t half = 8 * (ln & 1), p0 = (((ln >> 1) ^ sw) << 4) + half, p1 = (((4 + (ln >> 1)) ^ sw) << 4) + half, rest = rope ? p1 : kQBlockBytes + p0;
-    st_shared_v2(at + p0, hi[0][0] | (hi[0][1] << 16), hi[0][2] | (hi[0][3] << 16));
-    st_shared_v2(at + rest, lo[0][0] | (lo[0][1] << 16), lo[0][2] | (lo[0][3] << 16));
-    if (!rope) {
-      st_shared_v2(at + p1, hi[1][0] | (hi[1][1] << 16), hi[1][2] | (hi[1][3] << 16));
-      st_shared_v2(at + kQBlockBytes + p1, lo[1][0] | (lo[1][1] << 16), lo[1][2] | (lo[1][3] << 16));
-    }
-  }
-  fence_proxy_async_smem();
-}
-constexpr int kRowGroups = kCtaRows / 4;
-// The first unit's Q is split by the softmax warps as well, which have nothing else to do yet: a group each, the widening warps the rest.
-__device__ __forceinline__ void first_q_arrive() { asm volatile("barrier.cta.arrive 1, %0;" ::"n"(32 * (kSoftmaxWarps + kWideners)) : "memory"); }
-__device__ __forceinline__ void first_q_sync() { asm volatile("barrier.cta.sync 1, %0;" ::"n"(32 * (kSoftmaxWarps + kWideners)) : "memory"); }
-
 }  // namespace
 
-template <int kMode, bool kGuard, int kCache>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads<kCache>, 1)
+template <int kMode, bool kGuard, bool kFp8>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads<kFp8>, 1)
 decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap khalf_map, const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap q_map,
                    const DecodeParams prm) {
-  constexpr bool kFp8 = kCache != kBf16, kBytes = kCache == kSplitQ;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t smem_base = smem_u32(smem_raw);
   const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
@@ -261,23 +171,17 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = reinterpret_cast<int*>(smem_raw + kOffSeqlens);
   FirstUnit* first_smem = reinterpret_cast<FirstUnit*>(smem_raw + kOffFirst);
-  if (plan_here) plan_lengths(prm, plan_smem, lens_smem, tid, kThreads<kCache>);
+  if (plan_here) plan_lengths(prm, plan_smem, lens_smem, tid, kThreads<kFp8>);
   if (tid == 32 * 10) {
-    for (int i = 0; i < kSlots<kCache>; ++i) {
+    for (int i = 0; i < kSlots<kFp8>; ++i) {
       mbar_init(bar(X_FULL + i), kFp8 ? kWidenWarps + 1 : 1);          // E4M3: the warps that fill the slot, and word from the odd CTA
       mbar_init(bar(X_EMPTY + i), 1);
-      if (kFp8) mbar_init(bar(kFullOdd<kCache> + i), kWidenWarps);
+      if (kFp8) mbar_init(bar(X_FULLODD + i), kWidenWarps);
     }
-    if (kCache == kWidenAll) {
+    if (kFp8) {
       for (int i = 0; i < kRawSlots; ++i) { mbar_init(bar(X_RAWFULL + i), 1); mbar_init(bar(X_RAWEMPTY + i), 2 * kWidenWarps); }
     }
-    if (kBytes) {
-      for (int i = 0; i < kByteSlots; ++i) { mbar_init(bar(X_BYTESFULL + i), 1); mbar_init(bar(X_BYTESEMPTY + i), 1); }
-      mbar_init(bar(X_QFREE), 1);
-      mbar_init(bar(X_QTHERE), 1);
-      for (int i = 0; i < kRowScales; ++i) mbar_init(bar(X_QSCALE + i), kWideners);
-    }
-    mbar_init(bar(X_QFULL), kBytes ? 2 * kWideners : 1);
+    mbar_init(bar(X_QFULL), 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar(X_SFULL + i), 1);
       mbar_init(bar(X_SEMPTY + i), 2 * kSoftmaxWarps);
@@ -331,8 +235,8 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     if (wid >= kSoftmaxWarps) first_pages = load_pages(prm, tile);     // (the guess's place in the table is inside the table)
-    if (plan_is_stale(prm, plan_smem, lens_smem, first_smem, tid, kThreads<kCache>)) {     // (both CTAs see the same lengths)
-      plan_lengths(prm, plan_smem, lens_smem, tid, kThreads<kCache>);
+    if (plan_is_stale(prm, plan_smem, lens_smem, first_smem, tid, kThreads<kFp8>)) {     // (both CTAs see the same lengths)
+      plan_lengths(prm, plan_smem, lens_smem, tid, kThreads<kFp8>);
       __syncthreads();
       if (wid == 8) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
       __syncthreads();
@@ -372,7 +276,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       ++q_asked;
       q_next = -1;
     };
-    if (!kBytes && wid == kAsksForQ && tile.valid) look_ahead();
+    if (wid == kAsksForQ && tile.valid) look_ahead();
     // tells the row's other three threads `mine`; v[0..3] = what the four told
     auto exchange = [&](float mine, float (&v)[4]) {
       const uint32_t buf = smem_base + kOffXchg + (xc & 1) * (4 * kCtaRows * 4) + r * 4;
@@ -398,11 +302,6 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       for (int c = 0; c < 4; ++c) st_shared_v4(dst + (((4 * (chunk & 1) + c) ^ (r & 7)) << 4), pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
     };
 
-    if (kBytes && tile.valid) {
-      ok = warp_wait(bar(X_QTHERE), 0);
-      if (ok) split_q_rows(smem_base + kOffQ, smem_base + kOffRowScale, 4 * wid + (lane >> 3), prm.scale_log2);
-      first_q_arrive();
-    }
     if (tid == 0 && leader) merge_begin(prm, part);
     write_empty_items(prm, prefix, part, prm.P, rank * kCtaRows, kCtaRows, tid, 32 * kSoftmaxWarps);
     // A tile's softmax is done while the P~V of the tile before it still runs, and so is, at the end of a unit, that of the next
@@ -414,11 +313,9 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
     RowState st;
     row_state_init(st);
     int visible = 0, first_masked = 0;
-    float scale = prm.scale_log2;                        // of this row's scores
-    uint32_t un = 0;                                     // units so far
     int e_row = -1, e_b = 0, e_slot = 0;                 // the unit whose epilogue is still to be done: this thread's row (-1: none), ...
     float e_inv = 0.f, e_lse = 0.f;
-    while (ok && (tile.valid || e_row >= 0)) {
+    while (tile.valid || e_row >= 0) {
       const uint32_t sb = gs & 1;
       const int t = tile.t, np = tile.np;
       // A lane half holds 32 np neighbouring keys of a tile; this group takes its 32-key chunks grp and grp + 2.
@@ -434,18 +331,12 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           const int tok = (u.r0 + rank * kCtaRows + r) / prm.H;
           visible = min(u.n_b, u.n_b - prm.Sq + tok + 1);          // keys 0..visible-1 are seen by this row
           first_masked = max(u.n_b - prm.Sq + 1, 0) / kPage;       // pages from here on may hold hidden keys
-          if (kBytes) {
-            ok = warp_wait(bar(X_QSCALE + un % kRowScales), (un / kRowScales) & 1);
-            if (!ok) break;
-            scale = __uint_as_float(ld_shared_b32(smem_base + kOffRowScale + ((un % kRowScales) * kCtaRows + r) * 4));
-            ++un;
-          }
         }
         ok = warp_wait(bar(X_SFULL + sb), (gs >> 1) & 1);
         if (!ok) break;
         tc_fence_after_sync();
         if (tid == 0 && leader) AMLA_STAMP(prm, part, 8, gs);
-        if (!kBytes && wid == kAsksForQ && tile.last() && q_next >= 0) ask_for_q();
+        if (wid == kAsksForQ && tile.last() && q_next >= 0) ask_for_q();
         // The scores are read from tensor memory twice, a chunk at a time: for the maximum, and for the exponentials.  (Held in
         // registers in between they cost 64 more of them and twice the code.)
         const int nvis0 = visible - t * kPage - 32 * chunk0;                // keys of the first chunk that the row sees (may be <= 0)
@@ -464,11 +355,11 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
               a = fmax3(a, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
               b = fmax3(b, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
             }
-            a = fmaxf(a, b) * scale;
+            a = fmaxf(a, b) * prm.scale_log2;
           } else {
             const int nvis = nvis0 - 64 * h;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) a = fmaxf(a, i < nvis ? __uint_as_float(v[i]) * scale : -INFINITY);
+            for (int i = 0; i < 32; ++i) a = fmaxf(a, i < nvis ? __uint_as_float(v[i]) * prm.scale_log2 : -INFINITY);
           }
           ext = fmaxf(ext, a);
         }
@@ -489,7 +380,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         // Line 10's factor S16 goes into the exponential's argument (the remark after Algorithm 2).  The row sum of line 6 is
         // the sum of the same FP32 values, taken before the bf16 cast and divided by S16 once per tile.
         const float nsub = log2f_approx(sp.p_scale) - sp.m2_sub;
-        const float sc = plain ? scale : 1.f;
+        const float sc = plain ? prm.scale_log2 : 1.f;
         const uint64_t sc2 = pack_f32x2(sc, sc), ns2 = pack_f32x2(nsub, nsub);
         uint64_t rsa = pack_f32x2(0.f, 0.f), rsb = rsa;
 #pragma unroll 1
@@ -500,7 +391,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           if (!plain) {
             const int nvis = nvis0 - 64 * h;        // scaled here; hidden keys become 2^-inf = 0
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = i < nvis ? __float_as_uint(__uint_as_float(v[i]) * scale) : 0xff800000u;
+            for (int i = 0; i < 32; ++i) v[i] = i < nvis ? __float_as_uint(__uint_as_float(v[i]) * prm.scale_log2) : 0xff800000u;
           }
           uint32_t pk[16];
 #pragma unroll
@@ -652,11 +543,11 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         e_lse = live ? (st.m2 + log2f(l_all)) * kLn2 : -INFINITY;
       }
       tile.next();
-      if (!kBytes && wid == kAsksForQ && tile.valid && tile.first) look_ahead();
+      if (wid == kAsksForQ && tile.valid && tile.first) look_ahead();
     }
     if (!ok && lane == 0) {
       report_timeout(prm.status);
-      if (!kBytes && leader && q_asked > 0) mbar_wait(bar(X_QFULL), q_asked & 1);     // let copies that may still be in flight land
+      if (leader && q_asked > 0) mbar_wait(bar(X_QFULL), q_asked & 1);     // let copies that may still be in flight land
     }
   } else if (wid == 8 || (!kFp8 && wid >= 10)) {
     // ======================================================== TMA loads, in the order in which the MMAs use them:
@@ -701,21 +592,12 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
         return x;
       };
       const uint32_t lead_full = lead_bars + 8u * X_FULL;
-      if (!kBytes && tile.valid && wid == 8)                // the first unit's Q; the softmax warps ask for the others
+      if (wid == 8 && tile.valid)                           // the first unit's Q; the softmax warps ask for the others
         request_q(q_map, smem_base, bars, lead_bars, leader, q_row_of(prm, tile.u, rank));
-      uint32_t un = 0;                                      // E4M3: units whose Q has been asked for
-      auto ask_for_q = [&](int qrow) {
-        ok = mbar_wait(bar(X_QFREE), (un & 1) ^ 1);         // the MMAs have read the unit before
-        if (!ok) return;
-        mbar_arrive_expect_tx(bar(X_QTHERE), kQBytes);
-#pragma unroll 1
-        for (int c = 0; c < kQBlocks; c += 3) tma_load_3d(smem_base + kOffQ + c * kQBlockBytes, &q_map, 0, qrow, c, bar(X_QTHERE));
-        ++un;
-      };
       uint32_t n = 0;                                       // slots so far
       if constexpr (!kFp8) {
         const uint32_t mine = wid == 8 ? 0 : wid - 9;
-        constexpr uint32_t kRing = kSlots<kBf16>;
+        constexpr uint32_t kRing = kSlots<false>;
         uint32_t slot = 0, par = 1, turn = 0;
         auto advance = [&]() { if (++slot == kRing) { slot = 0; par ^= 1; } ++n; if (++turn == kLoaders) turn = 0; };
         Pages pg = first_pages, pg_nxt = {}, pg_prev = {};
@@ -768,7 +650,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
             if (leader && k % kLoaders == mine) mbar_wait(bar(X_FULL) + 8 * (k % kRing), (k / kRing) & 1);
           }
         }
-      } else if constexpr (kCache == kWidenAll) {
+      } else {
         uint32_t slot = 0, par = 1;
         auto advance = [&]() { if (++slot == kRawSlots) { slot = 0; par ^= 1; } ++n; };
         Pages pg = first_pages, pg_nxt = {}, pg_prev = {};
@@ -810,46 +692,11 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           report_timeout(prm.status);
           for (uint32_t i = 0; i < kRawSlots && i < n; ++i) mbar_wait(bar(X_RAWFULL) + 8 * ((n - 1 - i) % kRawSlots), ((n - 1 - i) / kRawSlots) & 1);
         }
-      } else {
-        uint32_t slot = 0, par = 1;
-        const uint32_t lead_bytes = lead_bars + 8u * X_BYTESFULL;
-        Pages pg = first_pages;
-        int np = tile.valid ? tile.np : 0;
-        if (np > 0) ask_for_q(q_row_of(prm, tile.u, rank));
-        while (ok && np > 0) {
-          int np_nxt = 0;
-          const int q_row = n > 0 && tile.first ? q_row_of(prm, tile.u, rank) : -1;
-          const KBoxes x = boxes(np, pg);
-          // two column blocks of K a slot (the last one by itself: its box reaches past the row's end, where there are zeros that
-          // nothing reads)
-#pragma unroll 1
-          for (int c = 0; c < kQBlocks; c += 2) {
-            // (the ring has room for one slot less than a tile: when the last one finds its place, the tile before has been used up)
-            if (c == kQBlocks - 1 && q_row >= 0) { ask_for_q(q_row); if (!ok) break; }
-            if (c == 2) np_nxt = take(pg);
-            ok = mbar_wait(bar(X_BYTESEMPTY) + 8 * slot, par);
-            if (!ok) break;
-            const uint32_t full = lead_bytes + 8 * slot, dst = smem_base + kOffBytes + slot * kSlotBytes;
-            if (leader) mbar_arrive_expect_tx(bar(X_BYTESFULL) + 8 * slot, 2 * np * kKBoxBytes);
-            tma_load_2d_pair_hint(dst, x.map0, 64 * c, x.row0, full, keep);                                     // [64 or 32 keys][128 columns]
-            if (x.chunks1 > 0) tma_load_2d_pair_hint(dst + x.chunks0 * kKBoxBytes, x.map1, 64 * c, x.row1, full, keep);
-            if (++slot == kByteSlots) { slot = 0; par ^= 1; }
-            ++n;
-          }
-          np = np_nxt;
-        }
-        if (!ok) {
-          report_timeout(prm.status);
-          // let the copies that may still be in flight land before the CTA exits
-          if (un > 0) mbar_wait(bar(X_QTHERE), (un - 1) & 1);
-          for (uint32_t i = 0; leader && i < kByteSlots && i < n; ++i)
-            mbar_wait(bar(X_BYTESFULL) + 8 * ((n - 1 - i) % kByteSlots), ((n - 1 - i) / kByteSlots) & 1);
-        }
       }
-      if (!kBytes && !ok && leader && wid == 8) mbar_wait(bar(X_QFULL), 0);
+      if (!ok && leader && wid == 8) mbar_wait(bar(X_QFULL), 0);
     }
     __syncwarp();
-  } else if (kCache == kWidenAll && wid >= 10) {
+  } else if (kFp8 && wid >= 10) {
     // ======================================================== E4M3 cache: raw slot -> operand slots.  The three pairs of
     // warps take every third operand slot each; a thread widens 16 bytes at a time (exact: E4M3 values are bf16 values)
     // and stores them where the 128-byte swizzle of the operand tiles puts them.  (Raw slots of two operand slots: nine loads
@@ -879,7 +726,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       const bool is_k = what == 0;
       const uint32_t nth = raw_phase + (pos >> 1), second = pos & 1;
       const uint32_t rslot = nth % kRawSlots, rpar = (nth / kRawSlots) & 1;
-      const uint32_t slot = n % kSlots<kCache>, par = ((n / kSlots<kCache>) & 1) ^ 1;
+      const uint32_t slot = n % kSlots<kFp8>, par = ((n / kSlots<kFp8>) & 1) ^ 1;
       // In this order.  Operand slot n is free: the MMAs have read number n - 4, and the raw slot in whose place this one stands
       // held numbers up to n - 4 at most, so it had been full.  (The other way round the wait for the raw slot could be let through
       // by the phase before that one's, when V has overtaken K.)
@@ -918,7 +765,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(bar((leader ? X_FULL : X_RAWODD) + slot));
+        mbar_arrive(bar((leader ? X_FULL : X_FULLODD) + slot));
         mbar_arrive(bar(X_RAWEMPTY + rslot));
         if (pos + 1 == len && second == 0) mbar_arrive(bar(X_RAWEMPTY + rslot));   // (a raw slot of one block)
       }
@@ -926,123 +773,20 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       n += kWidenGroups;
     }
     if (!ok && lane == 0) report_timeout(prm.status);
-  } else if (kBytes && wid >= 10) {
-    // ======================================================== E4M3 cache, kSplitQ: Q is split, V widened.  The three pairs of warps take
-    // every third operand slot of V each, half of this CTA's columns of a page, which they load from global memory (L2 has it: K's
-    // load was before) into registers one slot ahead: no raw slots, whose room K's ring has.  (V through raw slots of the same ring as
-    // K, four in all: 54.3 us for 32 x 4096 where this took 51.3.)
-    const uint32_t mine = (wid - 10) / kWidenWarps;
-    uint32_t un = 0;
-    // Q of a unit, four rows (a group) at a time, between the slots of V.
-    const int w = wid - 10;
-    int group = kRowGroups;                              // this warp's next group of the Q at hand
-    auto split = [&](int g) { split_q_rows(smem_base + kOffQ, smem_base + kOffRowScale + (un % kRowScales) * (kCtaRows * 4), 4 * g + (lane >> 3), prm.scale_log2); };
-    auto q_is_split = [&]() {
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(bar(X_QSCALE + un % kRowScales));
-        if (leader) mbar_arrive(bar(X_QFULL));
-        else { release_shared_to_cluster(); mbar_arrive_cluster_relaxed(lead_bars + 8u * X_QFULL); }
-      }
-      ++un;
-    };
-    auto split_some = [&](bool all) {                    // what there is left, or a group if Q is there
-      while (group < kRowGroups) {
-        if (!all && !__all_sync(0xffffffffu, mbar_probe(bar(X_QTHERE), un & 1))) return;
-        ok = warp_wait(bar(X_QTHERE), un & 1);
-        if (!ok) return;
-        split(group);
-        group += kWideners;
-        if (group >= kRowGroups) q_is_split();
-        if (!all) return;
-      }
-    };
-    uint32_t n = 0;                                      // operand slots before the present tile
-    uint32_t par = 1;                                    // of this pair's slot
-    // Four threads take 64 columns of a row, 16 bytes at a time (exact: E4M3 values are bf16 values), and store them where the
-    // 128-byte swizzle of the operand tiles puts them.  The eight threads that store together take rows a and a + 1 and different
-    // blocks of 64 columns, so that no two of them meet in a bank.
-    auto widen = [&](const int32_t* pages, int np) {     // the np page numbers of the tile
-      const int wt = ((wid - 10) % kWidenWarps) * 32 + lane;
-      const int other = (wt >> 2) & 1, vblock = ((wt >> 3) & 1) ^ other, r0 = 2 * (wt >> 4) + other;    // rows r0, r0 + 8, ...: the same swizzle
-      const uint8_t* const src0 = prm.kv8 + static_cast<size_t>(r0) * kDqk + 256 * rank + 64 * vblock + 16 * (wt & 3);
-      const uint32_t ch = 2 * (wt & 3), sw = r0 & 7;
-      const uint32_t d0 = smem_base + kOffRing + mine * kSlotBytes + vblock * kVBlockBytes + r0 * 128 + ((ch ^ sw) << 4);
-      const uint32_t d1 = (((ch + 1) ^ sw) << 4) - ((ch ^ sw) << 4);
-      uint32_t x[8][4];
-      auto load = [&](int pos) {                         // half (pos & 1) of page pos / 2; zeros behind the last
-        const int page = pos < 2 * np ? __ldg(pages + (pos >> 1)) : -1;
-        const bool inside = static_cast<uint32_t>(page) < static_cast<uint32_t>(prm.num_blocks);      // a page outside the cache reads as zeros
-        const uint8_t* src = src0 + static_cast<size_t>(inside ? page : 0) * (kPage * kDqk) + 128 * (pos & 1);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) ldg_bytes16(src + k * 8 * kDqk, inside, x[k]);
-      };
-      int pos = static_cast<int>((mine + 2 * n) % kWidenGroups);     // (n + pos = mine modulo 3)
-      load(pos);
-#pragma unroll 1
-      do {
-        if (pos < 2 * np) {
-          ok = warp_wait(bar(X_EMPTY + mine), par);
-          if (!ok) return;
-          par ^= 1;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            uint32_t w[8];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) { w[2 * q] = e4m3x2_to_bf16x2(x[k][q]); w[2 * q + 1] = e4m3x2_to_bf16x2(x[k][q] >> 16); }
-            st_shared_v4(d0 + k * 8 * 128, w[0], w[1], w[2], w[3]);
-            st_shared_v4(d0 + d1 + k * 8 * 128, w[4], w[5], w[6], w[7]);
-          }
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar((leader ? X_FULL : X_VODD) + mine));
-          pos += kWidenGroups;
-        }
-        split_some(pos >= 2 * np);
-        if (!ok) return;
-        load(pos);                                       // (in every case: nothing is kept over split_some())
-      } while (pos < 2 * np);
-      n += 2 * np;
-    };
-    // `tile` is two tiles ahead of the one whose V is widened: that one's P~V stands in front of the Q K^T of a unit's first tile.
-    if (tile.valid) {
-      ok = warp_wait(bar(X_QTHERE), 0);
-      if (ok) {
-        split(kSoftmaxWarps + w);
-        if ((w >> 1) == 1) split(kSoftmaxWarps + kWideners + w - 2);
-      }
-      static_assert(kRowGroups == kSoftmaxWarps + kWideners + 2, "the groups of the first unit's Q");
-      first_q_sync();
-      q_is_split();
-    }
-    int np0 = 0, at0 = 0, np1 = 0, at1 = 0;              // of the two tiles before `tile`: pages, and where their numbers are (less than 2^30)
-    auto on = [&]() {
-      np0 = np1; at0 = at1;
-      np1 = tile.valid ? tile.np : 0;
-      at1 = tile.u.b * prm.max_blocks_per_seq + tile.t;
-      if (tile.valid) tile.next();
-    };
-    on();
-    while (ok && (tile.valid || np0 > 0 || np1 > 0)) {
-      if (tile.valid && tile.first) group = w;
-      widen(prm.block_table + at0, np0);
-      on();
-    }
-    if (!ok && lane == 0) report_timeout(prm.status);
   } else if (kFp8 && wid == 9 && !leader) {
-    // ======================================================== E4M3 cache, odd CTA: passes on to the MMA issuer that a widened slot is
+    // ======================================================== E4M3 cache, odd CTA: passes on to the MMA issuer that a slot is
     // full.  (By the widening warps themselves, behind a fence for every slot, 32 x 4096 keys took 58.1 us instead of 57.3, 32
     // x 4000 with two tokens 101.4 instead of 99.8; 8 x 1000 17.4 instead of 17.6.  With arrivals that published nothing: 56.9,
     // 98.9 and 17.1.)  A slot is filled again when the MMAs have read it, so no phase can pass unseen.
     if (elect_one()) {
       uint32_t slot = 0, par = 0;
       while (ok && tile.valid) {
-        for (int i = (kBytes ? 0 : kQBlocks) + 2 * tile.np; i > 0 && ok; --i) {
-          ok = mbar_wait(bar(kFullOdd<kCache>) + 8 * slot, par);
+        for (int i = kQBlocks + 2 * tile.np; i > 0 && ok; --i) {
+          ok = mbar_wait(bar(X_FULLODD) + 8 * slot, par);
           if (!ok) break;
           release_shared_to_cluster();
           mbar_arrive_cluster_relaxed(lead_bars + 8u * (X_FULL + slot));
-          if (++slot == kSlots<kCache>) { slot = 0; par ^= 1; }
+          if (++slot == kSlots<kFp8>) { slot = 0; par ^= 1; }
         }
         if (ok) tile.next();
       }
@@ -1055,169 +799,82 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       constexpr uint32_t idesc_pv = make_idesc_bf16(128, 256, false, true);
       constexpr uint32_t idesc_qk1 = make_idesc_bf16(128, 64, false, false);     // N = 64 per page
       constexpr uint32_t idesc_step = make_idesc_bf16(128, 128, false, false) - idesc_qk1;
-      constexpr uint32_t idesc_hi1 = make_idesc_f8(128, 64, 0, 0), idesc_lo1 = make_idesc_f8(128, 64, 1, 0);   // E4M3 K, Q's larger and smaller numbers
       constexpr uint32_t dhi = smem_desc_hi_sw128(1024);
       const uint32_t qlo = smem_desc_lo(smem_base + kOffQ, 16);
       const uint32_t plo = smem_desc_lo(smem_base + kOffP, 16);
-      const uint32_t klo = smem_desc_lo(smem_base + (kBytes ? kOffBytes : kOffRing), 16);
+      const uint32_t klo = smem_desc_lo(smem_base + kOffRing, 16);
       const uint32_t vlo = smem_desc_lo(smem_base + kOffRing, kVBlockBytes);
       uint32_t slot = 0, par = 0;
       uint32_t gs = 0, gp = 0, un = 0;                      // score tiles, P~V tiles, units so far
-      uint32_t bslot = 0, bpar = 0;                         // E4M3: K's ring
-      auto advance = [&]() { if (++slot == kSlots<kCache>) { slot = 0; par ^= 1; } };
-      if constexpr (!kBytes) {
-        int np_prev = 0;                                      // pages of the tile before, 0: there was none
-        bool fresh_prev = false;                              // it was its unit's first
-        while (ok && tile.valid) {
-          const int np = tile.np;
-          const bool first = tile.first;
-          if (first) {
-            ok = mbar_wait(bar(X_QFULL), un & 1);
-            if (!ok) break;
-            ++un;
-          }
-          {
-            const uint32_t sb = gs & 1;
-            AMLA_STAMP(prm, part, 0, gs);
-            ok = mbar_wait<true>(bar(X_SEMPTY + sb), ((gs >> 1) & 1) ^ 1);
-            if (!ok) break;
-            tc_fence_after_sync();
-            AMLA_STAMP(prm, part, 1, gs);
-            const uint32_t d = tbase + kSCol + 128 * sb;
-            const uint32_t idesc = idesc_qk1 + (np - 1) * idesc_step;
-#pragma unroll 1
-            for (int c = 0; c < kQBlocks; ++c) {
-              ok = mbar_wait<kFp8>(bar(X_FULL) + 8 * slot, par);     // bf16: TMA data -> MMA operand, both async proxy, no fence needed; E4M3: the widening threads have fenced
-              if (!ok) break;
-              if (c == 0) AMLA_STAMP(prm, part, 2, gs);
-              const uint32_t kl = klo + slot * (kSlotBytes >> 4), ql = qlo + c * (kQBlockBytes >> 4);
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                mma_ss_pair(d, smem_desc_join(ql + 2 * kk, dhi), smem_desc_join(kl + 2 * kk, dhi), idesc, (c | kk) != 0 ? 1u : 0u);
-              mma_commit_pair_multicast(bar(X_EMPTY) + 8 * slot, 3);
-              advance();
-            }
-            if (!ok) break;
-            mma_commit_pair_multicast(bar(X_SFULL + sb), 3);
-            AMLA_STAMP(prm, part, 3, gs);
-            ++gs;
-          }
-          tile.next();
-          // O (+)= P~ V of the tile before, whatever unit that was in, and behind the part's last QK^T its own: per page two
-          // N = 256 products (128 columns from either CTA)
-          for (int k = np_prev == 0 ? 1 : 0; k < (tile.valid ? 1 : 2) && ok; ++k) {
-            const int np_v = k == 0 ? np_prev : np;
-            uint32_t acc = (k == 0 ? fresh_prev : first) ? 0u : 1u;
-            AMLA_STAMP(prm, part, 4, gp);
-            ok = mbar_wait<true>(bar(X_PREADY), gp & 1);
-            if (!ok) break;
-            AMLA_STAMP(prm, part, 5, gp);
-            tc_fence_after_sync();               // the softmax warps may have rewritten O (tcgen05.st) before arriving
-#pragma unroll 1
-            for (int i = 0; i < 2 * np_v; ++i) {
-              ok = mbar_wait<kFp8>(bar(X_FULL) + 8 * slot, par);
-              if (!ok) break;
-              if (i == 0) AMLA_STAMP(prm, part, 6, gp);
-              const uint32_t pl = plo + (i >> 1) * (kPPageBytes >> 4), vl = vlo + slot * (kSlotBytes >> 4), d = tbase + kOCol + 128 * (i & 1);
-              if (i >= 2) acc = 1u;
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                mma_ss_pair(d, smem_desc_join(pl + 2 * kk, dhi), smem_desc_join(vl + 128 * kk, dhi), idesc_pv, kk == 0 ? acc : 1u);
-              mma_commit_pair_multicast(bar(X_EMPTY) + 8 * slot, 3);
-              advance();
-            }
-            if (!ok) break;
-            mma_commit_pair_multicast(bar(X_PVDONE), 3);
-            AMLA_STAMP(prm, part, 7, gp);
-            ++gp;
-          }
-          np_prev = np;
-          fresh_prev = first;
+      auto advance = [&]() { if (++slot == kSlots<kFp8>) { slot = 0; par ^= 1; } };
+      int np_prev = 0;                                      // pages of the tile before, 0: there was none
+      bool fresh_prev = false;                              // it was its unit's first
+      while (ok && tile.valid) {
+        const int np = tile.np;
+        const bool first = tile.first;
+        if (first) {
+          ok = mbar_wait(bar(X_QFULL), un & 1);
+          if (!ok) break;
+          ++un;
         }
-      } else {
-        // Q K^T of the tile two ahead goes between the slots of P~V, a slot of K behind a page of V, since the slots of V are
-        // made while the tensor pipe is at K's, two of the five so that three are left to hide the hand-over of the next P~ (none
-        // between / two / four: 32 x 512-8192 keys, two tokens 99.9 / 98.5 / 98.9 us; 32 x 4096 51.3 / 51.0 / 51.0).  A unit's first
-        // tile comes behind P~V, as its Q has to be split first.
-        auto begin_scores = [&]() {                         // of `tile`: may its scores' place be written, is its Q there?
-          if (tile.first) {
-            ok = mbar_wait<true>(bar(X_QFULL), un & 1);
-            if (!ok) return;
-            ++un;
-          }
+        {
+          const uint32_t sb = gs & 1;
           AMLA_STAMP(prm, part, 0, gs);
-          ok = mbar_wait<true>(bar(X_SEMPTY + (gs & 1)), ((gs >> 1) & 1) ^ 1);
+          ok = mbar_wait<true>(bar(X_SEMPTY + sb), ((gs >> 1) & 1) ^ 1);
+          if (!ok) break;
           tc_fence_after_sync();
           AMLA_STAMP(prm, part, 1, gs);
-        };
-        auto scores = [&](int c) {                          // column blocks 2 c and 2 c + 1
-          ok = mbar_wait(bar(X_BYTESFULL) + 8 * bslot, bpar);
-          if (!ok) return;
-          if (c == 0) AMLA_STAMP(prm, part, 2, gs);
-          const uint32_t d = tbase + kSCol + 128 * (gs & 1), more_n = (tile.np - 1) * idesc_step;
-          const uint32_t kl = klo + bslot * (kSlotBytes >> 4), ql = qlo + c * (kQStep >> 4);
-          const bool rope = c == kByteSlotsOfTile - 1;
-          const uint32_t ll = ql + (rope ? 64 >> 4 : kQBlockBytes >> 4);
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {                   // the smaller parts first (see split_q_rows)
-            if (kk >= 2 && rope) break;
-            mma_f8_ss_pair(d, smem_desc_join(ll + 2 * kk, dhi), smem_desc_join(kl + 2 * kk, dhi), idesc_lo1 + more_n, (c | kk) != 0 ? 1u : 0u);
-          }
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            if (kk >= 2 && rope) break;
-            mma_f8_ss_pair(d, smem_desc_join(ql + 2 * kk, dhi), smem_desc_join(kl + 2 * kk, dhi), idesc_hi1 + more_n, 1u);
-          }
-          mma_commit_pair_multicast(bar(X_BYTESEMPTY) + 8 * bslot, 3);
-          if (++bslot == kByteSlots) { bslot = 0; bpar ^= 1; }
-          if (rope) {
-            mma_commit_pair_multicast(bar(X_SFULL + (gs & 1)), 3);
-            if (tile.last()) mma_commit_pair_multicast(bar(X_QFREE), 3);
-            AMLA_STAMP(prm, part, 3, gs);
-            ++gs;
-          }
-        };
-        constexpr int kMixed = 2;
-        int np0 = 0, np1 = 0;                               // pages of the two tiles before `tile`
-        bool fresh0 = false, fresh1 = false;                // were they their units' first?
-        while (ok && (tile.valid || np0 > 0 || np1 > 0)) {
-          const bool mixed = tile.valid && !tile.first && np0 > 0;
-          int c = 0;
-          if (mixed || (tile.valid && np0 == 0)) { begin_scores(); if (!ok) break; }
-          if (np0 > 0) {
-            AMLA_STAMP(prm, part, 4, gp);
-            ok = mbar_wait<true>(bar(X_PREADY), gp & 1);
-            if (!ok) break;
-            AMLA_STAMP(prm, part, 5, gp);
-            tc_fence_after_sync();               // the softmax warps may have rewritten O (tcgen05.st) before arriving
+          const uint32_t d = tbase + kSCol + 128 * sb;
+          const uint32_t idesc = idesc_qk1 + (np - 1) * idesc_step;
 #pragma unroll 1
-            for (int i = 0; i < 2 * np0; ++i) {
-              ok = mbar_wait<true>(bar(X_FULL) + 8 * slot, par);          // (the widening threads have fenced)
-              if (!ok) break;
-              if (i == 0) AMLA_STAMP(prm, part, 6, gp);
-              const uint32_t pl = plo + (i >> 1) * (kPPageBytes >> 4), vl = vlo + slot * (kSlotBytes >> 4), d = tbase + kOCol + 128 * (i & 1);
-              const uint32_t on = fresh0 && i < 2 ? 0u : 1u;
+          for (int c = 0; c < kQBlocks; ++c) {
+            // bf16: TMA data -> MMA operand, both async proxy, no fence needed; E4M3: the widening threads have fenced
+            ok = mbar_wait<kFp8>(bar(X_FULL) + 8 * slot, par);
+            if (!ok) break;
+            if (c == 0) AMLA_STAMP(prm, part, 2, gs);
+            const uint32_t kl = klo + slot * (kSlotBytes >> 4), ql = qlo + c * (kQBlockBytes >> 4);
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                mma_ss_pair(d, smem_desc_join(pl + 2 * kk, dhi), smem_desc_join(vl + 128 * kk, dhi), idesc_pv, kk == 0 ? on : 1u);
-              mma_commit_pair_multicast(bar(X_EMPTY) + 8 * slot, 3);
-              advance();
-              if (i + 1 == 2 * np0) { mma_commit_pair_multicast(bar(X_PVDONE), 3); AMLA_STAMP(prm, part, 7, gp); }
-              if (mixed && (i & 1) && c < kMixed) { scores(c++); if (!ok) break; }
-            }
-            if (!ok) break;
-            ++gp;
-            if (tile.valid && !mixed) { begin_scores(); if (!ok) break; }
+            for (int kk = 0; kk < 4; ++kk)
+              mma_ss_pair(d, smem_desc_join(ql + 2 * kk, dhi), smem_desc_join(kl + 2 * kk, dhi), idesc, (c | kk) != 0 ? 1u : 0u);
+            mma_commit_pair_multicast(bar(X_EMPTY) + 8 * slot, 3);
+            advance();
           }
-          if (tile.valid) {
-#pragma unroll 1
-            for (; c < kByteSlotsOfTile && ok; ++c) scores(c);
-            if (!ok) break;
-          }
-          np0 = np1; fresh0 = fresh1;
-          np1 = tile.valid ? tile.np : 0; fresh1 = tile.first;
-          if (tile.valid) tile.next();
+          if (!ok) break;
+          mma_commit_pair_multicast(bar(X_SFULL + sb), 3);
+          AMLA_STAMP(prm, part, 3, gs);
+          ++gs;
         }
+        tile.next();
+        // O (+)= P~ V of the tile before, whatever unit that was in, and behind the part's last QK^T its own: per page two
+        // N = 256 products (128 columns from either CTA)
+        for (int k = np_prev == 0 ? 1 : 0; k < (tile.valid ? 1 : 2) && ok; ++k) {
+          const int np_v = k == 0 ? np_prev : np;
+          uint32_t acc = (k == 0 ? fresh_prev : first) ? 0u : 1u;
+          AMLA_STAMP(prm, part, 4, gp);
+          ok = mbar_wait<true>(bar(X_PREADY), gp & 1);
+          if (!ok) break;
+          AMLA_STAMP(prm, part, 5, gp);
+          tc_fence_after_sync();               // the softmax warps may have rewritten O (tcgen05.st) before arriving
+#pragma unroll 1
+          for (int i = 0; i < 2 * np_v; ++i) {
+            ok = mbar_wait<kFp8>(bar(X_FULL) + 8 * slot, par);
+            if (!ok) break;
+            if (i == 0) AMLA_STAMP(prm, part, 6, gp);
+            const uint32_t pl = plo + (i >> 1) * (kPPageBytes >> 4), vl = vlo + slot * (kSlotBytes >> 4), d = tbase + kOCol + 128 * (i & 1);
+            if (i >= 2) acc = 1u;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              mma_ss_pair(d, smem_desc_join(pl + 2 * kk, dhi), smem_desc_join(vl + 128 * kk, dhi), idesc_pv, kk == 0 ? acc : 1u);
+            mma_commit_pair_multicast(bar(X_EMPTY) + 8 * slot, 3);
+            advance();
+          }
+          if (!ok) break;
+          mma_commit_pair_multicast(bar(X_PVDONE), 3);
+          AMLA_STAMP(prm, part, 7, gp);
+          ++gp;
+        }
+        np_prev = np;
+        fresh_prev = first;
       }
       if (!ok) report_timeout(prm.status);
     }
@@ -1238,19 +895,19 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
 // ---------------------------------------------------------------------------------------------------
 namespace {
 
-template <int kMode, bool kGuard, int kCache>
+template <int kMode, bool kGuard, bool kFp8>
 cudaError_t launch_variant(const CUtensorMap& kmap, const CUtensorMap& khalf, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
   static std::atomic<uint64_t> done{0};
-  return launch_serialized(decode_pair_kernel<kMode, kGuard, kCache>, done, 2 * prm.P, kThreads<kCache>, kSmemBytes, stream, kmap, khalf, vmap, qmap, prm);
+  return launch_serialized(decode_pair_kernel<kMode, kGuard, kFp8>, done, 2 * prm.P, kThreads<kFp8>, kSmemBytes, stream, kmap, khalf, vmap, qmap, prm);
 }
 
-template <int kCache>
+template <bool kFp8>
 cudaError_t launch_mode(const CUtensorMap& kmap, const CUtensorMap& khalf, const CUtensorMap& vmap, const CUtensorMap& qmap, const DecodeParams& prm, cudaStream_t stream) {
   const int mode = prm.flags & 3;
   const bool guard = !(prm.flags & 4);
-  if (mode == 0) return guard ? launch_variant<0, true, kCache>(kmap, khalf, vmap, qmap, prm, stream) : launch_variant<0, false, kCache>(kmap, khalf, vmap, qmap, prm, stream);
-  if (mode == 1) return guard ? launch_variant<1, true, kCache>(kmap, khalf, vmap, qmap, prm, stream) : launch_variant<1, false, kCache>(kmap, khalf, vmap, qmap, prm, stream);
-  return launch_variant<2, true, kCache>(kmap, khalf, vmap, qmap, prm, stream);
+  if (mode == 0) return guard ? launch_variant<0, true, kFp8>(kmap, khalf, vmap, qmap, prm, stream) : launch_variant<0, false, kFp8>(kmap, khalf, vmap, qmap, prm, stream);
+  if (mode == 1) return guard ? launch_variant<1, true, kFp8>(kmap, khalf, vmap, qmap, prm, stream) : launch_variant<1, false, kFp8>(kmap, khalf, vmap, qmap, prm, stream);
+  return launch_variant<2, true, kFp8>(kmap, khalf, vmap, qmap, prm, stream);
 }
 
 // An E4M3 cache: rows of 576 bytes.
@@ -1281,10 +938,10 @@ cudaError_t launch_decode_pair(const DecodeParams& prm, cudaStream_t stream, int
     if (!encode_bytes(encode, &kmap, prm.kv8, keys, 64, 128, true) || !encode_bytes(encode, &khalf, prm.kv8, keys, 32, 128, true) ||
         !encode_bytes(encode, &vmap, prm.kv8, keys, 64, 256, false))
       return cudaErrorInvalidValue;
-    return prm.split_q ? launch_mode<kSplitQ>(kmap, khalf, vmap, qmap, prm, stream) : launch_mode<kWidenAll>(kmap, khalf, vmap, qmap, prm, stream);
+    return launch_mode<true>(kmap, khalf, vmap, qmap, prm, stream);
   }
   if (!encode_rows(encode, &kmap, prm.kv, keys, 64, 1) || !encode_rows(encode, &khalf, prm.kv, keys, 32, 1) || !encode_rows(encode, &vmap, prm.kv, keys, 64, 2)) return cudaErrorInvalidValue;
-  return launch_mode<kBf16>(kmap, khalf, vmap, qmap, prm, stream);
+  return launch_mode<false>(kmap, khalf, vmap, qmap, prm, stream);
 }
 
 }  // namespace amla
