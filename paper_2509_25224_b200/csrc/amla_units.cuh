@@ -91,7 +91,7 @@ struct FirstUnit {
 __device__ __forceinline__ void plan_lengths(const DecodeParams& prm, int* prefix, int* lens, int tid, int threads) {
   for (int it = tid; it < prm.n_items; it += threads) {
     const int b = prm.nrb == 1 ? it : it / prm.nrb, n = load_length<true>(prm, b);
-    if (lens) lens[b] = n;                               // same value from every row block
+    if (lens) lens[b] = n;                               // (row blocks of a sequence may differ in a guess: see item_is_stale)
     prefix[it] = schedule_length(n, it, prm.tile_keys, prm.ovh);
   }
 }
@@ -133,15 +133,22 @@ __device__ __forceinline__ void plan_units(const DecodeParams& prm, int* prefix,
     first->g = g; first->g1 = g1; first->share = share;
   }
 }
+// Does a plan's item `it` differ from what the n_seq keys of its sequence give?
+// The length that is on chip says it all where a sequence is one item.  Where it is several, each of them has loaded the length for
+// itself: while a kernel in front is writing it, prefix[] may have got the old one from one row block and the new one, which
+// lens[] then holds, from another.  So what prefix[] has of the item is looked at too.
+__host__ __device__ inline bool item_is_stale(const DecodeParams& prm, const int* prefix, const int* lens, const FirstUnit* first, int it, int n_seq) {
+  if (lens != nullptr) {
+    if (lens[prm.nrb == 1 ? it : it / prm.nrb] != n_seq) return true;
+    if (prm.nrb == 1) return false;
+  }
+  return prefix[it + 1] - prefix[it] != schedule_length(n_seq, it, prm.tile_keys, prm.ovh) || (lens == nullptr && it == first->u.it && n_seq != first->u.n_b);
+}
 // By all threads of the CTA, after griddepcontrol.wait: does the plan differ from what the lengths give?
 __device__ __forceinline__ bool plan_is_stale(const DecodeParams& prm, const int* prefix, const int* lens, const FirstUnit* first, int tid, int threads) {
   bool stale = false;
-  for (int it = tid; it < prm.n_items; it += threads) {
-    const int b = prm.nrb == 1 ? it : it / prm.nrb;
-    const int n_seq = load_length<false>(prm, b);
-    if (lens) stale |= lens[b] != n_seq;
-    else stale |= prefix[it + 1] - prefix[it] != schedule_length(n_seq, it, prm.tile_keys, prm.ovh) || (it == first->u.it && n_seq != first->u.n_b);
-  }
+  for (int it = tid; it < prm.n_items; it += threads)
+    stale |= item_is_stale(prm, prefix, lens, first, it, load_length<false>(prm, prm.nrb == 1 ? it : it / prm.nrb));
   return __syncthreads_or(stale);
 }
 __device__ __forceinline__ void plan_in_workspace(const DecodeParams& prm, int lane) {

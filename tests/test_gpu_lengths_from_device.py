@@ -110,3 +110,45 @@ def test_lengths_written_directly_in_front_of_the_call(late, B, Sq, H, longest, 
         binding.static_check_status()
     else:
         binding.check_status(ws)
+
+
+@pytest.mark.parametrize("B,Sq,H,longest,fp8,width", [(40, 3, 128, 600, True, 0), (25, 3, 128, 900, False, 4096), (70, 3, 43, 500, True, 0), (60, 5, 128, 400, False, 4096)])
+def test_lengths_written_while_a_call_of_several_row_blocks_starts(late, B, Sq, H, longest, fp8, width):
+    # the items of a sequence load its length one by one: the write falls before, among and behind these loads
+    import torch
+    rng = np.random.default_rng(B)
+    w = synth.make_workload("blocks", B, Sq, H, [longest] * B, seed=950 + B)
+    if width:
+        pad = np.full((B, width - w.block_table.shape[1]), -1, np.int32)
+        w.block_table = np.ascontiguousarray(np.concatenate([w.block_table, pad], axis=1))
+    q, kv, bt, _ = to_device(w)
+    dev = q.device
+    if fp8:
+        kv = torch.from_numpy(synth.quantise_cache_e4m3(w, 1.0 / 64.0)).to(dev)
+    size = binding.fp8_workspace_size if fp8 else binding.workspace_size
+    ws = torch.empty(size(B, Sq, H, bt.shape[1], 0), dtype=torch.uint8, device=dev)
+    dlens = [torch.from_numpy(rng.integers(0, longest + 1, B).astype(np.int32)).to(dev) for _ in range(2)]
+    seqlens = torch.empty(B, dtype=torch.int32, device=dev)
+    out = torch.empty((B, Sq, H, 512), dtype=torch.bfloat16, device=dev)
+    lse = torch.empty((B, Sq, H), dtype=torch.float32, device=dev)
+    stream = torch.cuda.current_stream().cuda_stream
+
+    def call_behind(write):
+        out.fill_(float("nan"))
+        lse.fill_(float("nan"))
+        write()
+        if fp8:
+            binding.mla_decode_fp8(q, kv, 1.0 / 64.0, bt, seqlens, w.scale, out, lse, ws)
+        else:
+            binding.mla_decode(q, kv, bt, seqlens, w.scale, out, lse, ws)
+        torch.cuda.synchronize()
+        return out.view(torch.int16).clone(), lse.clone()
+
+    want = [call_behind(lambda x=x: seqlens.copy_(x)) for x in dlens]
+    for i, delay in enumerate(range(0, 16000, 400)):
+        seqlens.copy_(dlens[1 - i % 2])
+        code = []
+        got = call_behind(lambda: code.append(late(dlens[i % 2].data_ptr(), seqlens.data_ptr(), B, delay, stream)))
+        assert code == [0]
+        assert torch.equal(got[0], want[i % 2][0]) and torch.equal(got[1], want[i % 2][1]), (i, delay)
+    binding.check_status(ws)
