@@ -142,7 +142,8 @@ __host__ __device__ inline bool item_is_stale(const DecodeParams& prm, const int
     if (lens[prm.nrb == 1 ? it : it / prm.nrb] != n_seq) return true;
     if (prm.nrb == 1) return false;
   }
-  return prefix[it + 1] - prefix[it] != schedule_length(n_seq, it, prm.tile_keys, prm.ovh) || (lens == nullptr && it == first->u.it && n_seq != first->u.n_b);
+  const bool of_first = lens == nullptr && it == first->u.it && first->u.t1 > first->u.t0;      // (a part without a unit has no length to be wrong)
+  return prefix[it + 1] - prefix[it] != schedule_length(n_seq, it, prm.tile_keys, prm.ovh) || (of_first && n_seq != first->u.n_b);
 }
 // By all threads of the CTA, after griddepcontrol.wait: does the plan differ from what the lengths give?
 __device__ __forceinline__ bool plan_is_stale(const DecodeParams& prm, const int* prefix, const int* lens, const FirstUnit* first, int tid, int threads) {

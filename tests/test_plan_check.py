@@ -53,3 +53,15 @@ def test_a_length_that_changes_no_tile_is_found_on_chip(item_is_stale, tile_keys
     for nrb in (1, 2):
         assert _stale(item_is_stale, nrb, tile_keys, ovh, [65] * nrb + [130] * nrb, [65, 130], [66, 130])
         assert not _stale(item_is_stale, nrb, tile_keys, ovh, [65] * nrb + [130] * nrb, [65, 130], [65, 130])
+
+
+def test_a_part_without_a_unit_keeps_a_right_schedule(item_is_stale):
+    # the prefix alone is on chip: the length that the part's first unit was given is looked at, if it has one
+    lens = [300, 0, 700]
+    for nrb in (1, 2):
+        per_item = np.repeat(lens, nrb).tolist()
+        assert not _stale(item_is_stale, nrb, 128, 5, per_item, None, lens)
+        for it in (0, 2 * nrb):
+            assert not _stale(item_is_stale, nrb, 128, 5, per_item, None, lens, (it, 0, 2, lens[it // nrb]))
+            assert _stale(item_is_stale, nrb, 128, 5, per_item, None, lens, (it, 0, 2, lens[it // nrb] - 1))
+        assert _stale(item_is_stale, nrb, 128, 5, per_item, None, [300, 0, 900])
