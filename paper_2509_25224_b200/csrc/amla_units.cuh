@@ -87,8 +87,11 @@ struct FirstUnit {
 // (The guess is right unless the kernel directly in front writes the lengths.  One sequence of 256 keys with 16 heads: planned
 // wholly behind the wait 8.5 us, guessed and checked 7.7, guessed and not checked 7.2; 32 x 4096 keys 51.7, 50.9 and 50.4,
 // calls replayed back to back.)
+// The loops over items stay rolled: written out four times they were code that a short call runs through once, cold (one sequence
+// of 256 keys with 16 heads 8.05 us, rolled 7.99; the check behind the wait 1195 clk, rolled 1040).
 // Leaves every item's schedule length in prefix[], and the lengths in lens[] (unless that is null).
 __device__ __forceinline__ void plan_lengths(const DecodeParams& prm, int* prefix, int* lens, int tid, int threads) {
+#pragma unroll 1
   for (int it = tid; it < prm.n_items; it += threads) {
     const int b = prm.nrb == 1 ? it : it / prm.nrb, n = load_length<true>(prm, b);
     if (lens) lens[b] = n;                               // (row blocks of a sequence may differ in a guess: see item_is_stale)
@@ -148,6 +151,7 @@ __host__ __device__ inline bool item_is_stale(const DecodeParams& prm, const int
 // By all threads of the CTA, after griddepcontrol.wait: does the plan differ from what the lengths give?
 __device__ __forceinline__ bool plan_is_stale(const DecodeParams& prm, const int* prefix, const int* lens, const FirstUnit* first, int tid, int threads) {
   bool stale = false;
+#pragma unroll 1
   for (int it = tid; it < prm.n_items; it += threads)
     stale |= item_is_stale(prm, prefix, lens, first, it, load_length<false>(prm, prm.nrb == 1 ? it : it / prm.nrb));
   return __syncthreads_or(stale);
@@ -171,7 +175,7 @@ struct UnitIter {
   const int* seqlens;
   int p, g, g1, share;
   __device__ UnitIter(const DecodeParams& prm_, const int* prefix_, const int* seqlens_, int part) : prm(prm_), prefix(prefix_), seqlens(seqlens_), p(part) {}
-  // The part's first unit: from what plan_on_chip left, or looked up in the workspace's prefix (first == nullptr).
+  // The part's first unit: from what plan_units() left, or looked up in the workspace's prefix (first == nullptr).
   __device__ void start(const FirstUnit* first, Unit& u) {
     if (first != nullptr) {
       u = first->u;
