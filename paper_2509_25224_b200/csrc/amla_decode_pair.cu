@@ -295,11 +295,9 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       ok = warp_wait(xbar, xc & 1);
       ++xc;
     };
-    // 32 keys of P~: half (chunk & 1) of page chunk / 2 of the P buffer
-    auto store_p = [&](int chunk, const uint32_t (&pk)[16]) {
-      const uint32_t dst = prow_smem + (chunk >> 1) * kPPageBytes;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) st_shared_v4(dst + (((4 * (chunk & 1) + c) ^ (r & 7)) << 4), pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+    // 32 keys of P~: half (chunk & 1) of page chunk / 2 of the P buffer, in pieces of 8
+    auto store_p_piece = [&](int chunk, int c, const uint32_t (&pk)[16]) {
+      st_shared_v4(prow_smem + (chunk >> 1) * kPPageBytes + (((4 * (chunk & 1) + c) ^ (r & 7)) << 4), pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
     };
 
     if (tid == 0 && leader) merge_begin(prm, part);
@@ -321,7 +319,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       // A lane half holds 32 np neighbouring keys of a tile; this group takes its 32-key chunks grp and grp + 2.
       const uint32_t scol = tbase + lane_base + kSCol + 128 * sb + 32 * grp;
       const int chunk0 = np * khalf + grp;                                  // of the tile's 2 np
-      bool direct = false;                               // P~ goes straight into the P buffer
+      bool direct = false;                               // P~ goes straight into the P buffer, 8 keys at a time as they are ready
       uint32_t nword = 0;
       bool moved = false;
       if (tile.valid) {
@@ -402,9 +400,9 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
             const uint64_t pp = pack_f32x2(q0, q1);
             if (i & 1) rsb = add_f32x2(rsb, pp); else rsa = add_f32x2(rsa, pp);
             pk[i] = pack_bf16x2(q0, q1);
+            if ((i & 3) == 3 && direct) store_p_piece(chunk0 + 2 * h, i >> 2, pk);
           }
-          if (direct) store_p(chunk0 + 2 * h, pk);
-          else tmem_st_32x32b_x16(scol + 64 * h, pk);
+          if (!direct) tmem_st_32x32b_x16(scol + 64 * h, pk);
         }
         float s0, s1;
         unpack_f32x2(add_f32x2(rsa, rsb), s0, s1);
@@ -511,7 +509,8 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           uint32_t pk[16];
           tmem_ld_32x32b_x16(scol + 64 * h, pk);
           tmem_wait_ld();
-          store_p(chunk0 + 2 * h, pk);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) store_p_piece(chunk0 + 2 * h, c, pk);
         }
       }
       tc_fence_before_sync();            // S has been read, O (perhaps) rewritten

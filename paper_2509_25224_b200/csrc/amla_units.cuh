@@ -88,7 +88,7 @@ struct FirstUnit {
 // wholly behind the wait 8.5 us, guessed and checked 7.7, guessed and not checked 7.2; 32 x 4096 keys 51.7, 50.9 and 50.4,
 // calls replayed back to back.)
 // The loops over items stay rolled: written out four times they were code that a short call runs through once, cold (one sequence
-// of 256 keys with 16 heads 8.05 us, rolled 7.99; the check behind the wait 1195 clk, rolled 1040).
+// of 256 keys with 16 heads 8.16 us, rolled 8.04; the check behind the wait 1113 clk, rolled 990).
 // Leaves every item's schedule length in prefix[], and the lengths in lens[] (unless that is null).
 __device__ __forceinline__ void plan_lengths(const DecodeParams& prm, int* prefix, int* lens, int tid, int threads) {
 #pragma unroll 1
