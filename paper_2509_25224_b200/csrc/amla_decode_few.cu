@@ -92,13 +92,14 @@ decode_few_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_const
   const uint32_t tmem_slot = bars + kBarBytes - 8;
 
   // Set-up.  The schedule is worked out from the sequence lengths as they are found (held against the final ones after the
-  // wait below): all threads bring them, then the load warp adds up.  Beside that the MMA warp allocates tensor memory and one
-  // thread of a softmax warp initialises the barriers.
+  // wait below): all threads bring them, or the load warp where they are few, and the load warp adds up.  Beside that the MMA warp
+  // allocates tensor memory and one thread of a softmax warp initialises the barriers.
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = reinterpret_cast<int*>(smem_raw + kOffSeqlens);
   FirstUnit* first_smem = reinterpret_cast<FirstUnit*>(smem_raw + kOffFirst);
-  if (plan_here) plan_lengths(prm, plan_smem, lens_smem, tid, kThreads);
+  const bool by_warp = prm.n_items <= kWarpPlanItems;
+  if (plan_here && (!by_warp || wid == kLoadWarp)) plan_lengths(prm, plan_smem, lens_smem, by_warp ? lane : tid, by_warp ? 32 : kThreads);
   if (tid == 0) {
     for (int i = 0; i < kSlots * kPieces; ++i) mbar_init(bar(X_FULL + i), 1);
     for (int i = 0; i < kSlots; ++i) mbar_init(bar(X_EMPTY + i), 1);
@@ -112,7 +113,7 @@ decode_few_kernel(const __grid_constant__ CUtensorMap kv_map, const __grid_const
   }
   if (wid == kQkWarp) { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
   if (plan_here) {
-    __syncthreads();
+    if (by_warp) __syncwarp(); else __syncthreads();
     if (wid == kLoadWarp) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
   }
   tc_fence_before_sync();

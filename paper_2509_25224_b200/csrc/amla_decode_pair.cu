@@ -165,13 +165,14 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   const uint32_t lead_bars = map_to_cta(bars, 0);
 
   // Set-up.  The schedule of a batch of up to kSmemPlanItems items is worked out from the sequence lengths as they are found
-  // (held against the final ones after the wait below): all threads bring them, then warp 8 adds up.  Beside that warp 9
-  // allocates tensor memory and one thread of warp 10 initialises the barriers.
+  // (held against the final ones after the wait below): all threads bring them, or warp 8 where they are few, and warp 8 adds up.
+  // Beside that warp 9 allocates tensor memory and one thread of warp 10 initialises the barriers.
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = reinterpret_cast<int*>(smem_raw + kOffSeqlens);
   FirstUnit* first_smem = reinterpret_cast<FirstUnit*>(smem_raw + kOffFirst);
-  if (plan_here) plan_lengths(prm, plan_smem, lens_smem, tid, kThreads<kFp8>);
+  const bool by_warp = prm.n_items <= kWarpPlanItems;
+  if (plan_here && (!by_warp || wid == 8)) plan_lengths(prm, plan_smem, lens_smem, by_warp ? lane : tid, by_warp ? 32 : kThreads<kFp8>);
   if (tid == 32 * 10) {
     for (int i = 0; i < kSlots<kFp8>; ++i) {
       mbar_init(bar(X_FULL + i), kFp8 ? kWidenWarps + 1 : 1);          // E4M3: the warps that fill the slot, and word from the odd CTA
@@ -198,7 +199,7 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   if (wid == 9) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
   if (tid == 0 && leader) AMLA_STAMP(prm, part, 20, 6);
   if (plan_here) {
-    __syncthreads();
+    if (by_warp) __syncwarp(); else __syncthreads();
     if (wid == 8) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
   }
   tc_fence_before_sync();

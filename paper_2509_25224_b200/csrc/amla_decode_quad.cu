@@ -421,12 +421,14 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   const uint32_t myV_bars = map_to_cta(bars, 2 + half);
 
   // The schedule of a batch of up to kSmemPlanItems items is worked out during the set-up, from the sequence lengths as they
-  // are found (held against the final ones after the wait below): all threads bring them, then warp 6 adds up.
+  // are found (held against the final ones after the wait below): all threads bring them, or warp 6 where they are few, and
+  // warp 6 adds up.
   const bool plan_here = prm.fused_plan && prm.n_items <= kSmemPlanItems;
   int* plan_smem = reinterpret_cast<int*>(smem_raw + kOffPlan);
   int* lens_smem = prm.n_items <= kSmemLens ? reinterpret_cast<int*>(smem_raw + kOffSeqlens) : nullptr;
   FirstUnit* first_smem = reinterpret_cast<FirstUnit*>(smem_raw + kOffFirst);
-  if (plan_here) plan_lengths(prm, plan_smem, lens_smem, tid, kThreads);
+  const bool by_warp = prm.n_items <= kWarpPlanItems;
+  if (plan_here && (!by_warp || wid == 6)) plan_lengths(prm, plan_smem, lens_smem, by_warp ? lane : tid, by_warp ? 32 : kThreads);
   if (tid == 0) {
     for (int i = 0; i < kNumP; ++i) mbar_init(bar(X_PV + i), 1);
     if (is_score) {
@@ -452,7 +454,7 @@ decode_quad_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
   }
   if (wid == 5) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
   if (plan_here) {
-    __syncthreads();
+    if (by_warp) __syncwarp(); else __syncthreads();
     if (wid == 6) plan_units(prm, plan_smem, lens_smem, first_smem, part, lane);
   }
   tc_fence_before_sync();

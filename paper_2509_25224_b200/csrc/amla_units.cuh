@@ -89,6 +89,10 @@ struct FirstUnit {
 // calls replayed back to back.)
 // The loops over items stay rolled: written out four times they were code that a short call runs through once, cold (one sequence
 // of 256 keys with 16 heads 8.16 us, rolled 8.04; the check behind the wait 1113 clk, rolled 990).
+// Up to kWarpPlanItems items the one warp brings the lengths too, beside the other warps' set-up and without a barrier in between:
+// 32 lengths are one load of a warp.  (By all threads / by one warp, us: one sequence of 256 keys with 16 heads 7.97 / 7.94, two
+// tokens 1 x 256 10.59 / 10.54, 16 x 1-300 14.81 / 14.77.)
+constexpr int kWarpPlanItems = 32;
 // Leaves every item's schedule length in prefix[], and the lengths in lens[] (unless that is null).
 __device__ __forceinline__ void plan_lengths(const DecodeParams& prm, int* prefix, int* lens, int tid, int threads) {
 #pragma unroll 1
