@@ -115,20 +115,19 @@ struct Plan {
   int share;     // positions per part (the last part may have fewer)
 
   __host__ __device__ static Plan make(const int* prefix, int n_items, int max_parts, int ovh, int min_share = 1) {
-    Plan pl = make(prefix[n_items], max_parts, min_share);
+    Plan pl;
     pl.prefix = prefix;
     pl.ovh = ovh;
     pl.n_items = n_items;
-    return pl;
-  }
-  // the parts alone, for a schedule of L positions
-  __host__ __device__ static Plan make(int L, int max_parts, int min_share) {
-    Plan pl = {};
-    pl.L = L;
-    pl.share = pl.L > max_parts ? static_cast<int>((static_cast<unsigned>(pl.L) + max_parts - 1) / static_cast<unsigned>(max_parts)) : 1;
-    if (pl.share < min_share) pl.share = min_share;
+    pl.L = prefix[n_items];
+    pl.share = share_of(pl.L, max_parts, min_share);
     pl.P = pl.L > 0 ? static_cast<int>((static_cast<unsigned>(pl.L) + pl.share - 1) / static_cast<unsigned>(pl.share)) : 1;
     return pl;
+  }
+  // Positions per part of a schedule of L positions.
+  __host__ __device__ static int share_of(int L, int max_parts, int min_share) {
+    const int share = L > max_parts ? static_cast<int>((static_cast<unsigned>(L) + max_parts - 1) / static_cast<unsigned>(max_parts)) : 1;
+    return share < min_share ? min_share : share;
   }
   __host__ __device__ int part_start(int p) const { return p >= P ? L : p * share; }
   __host__ __device__ int part_of_tile(int g) const { return static_cast<int>(static_cast<unsigned>(g) / static_cast<unsigned>(share)); }

@@ -117,7 +117,7 @@ __device__ __forceinline__ void plan_units(const DecodeParams& prm, int* prefix,
   if (lane == 0) prefix[prm.n_items] = total;
   __syncwarp();
   // the part's range of positions, as Plan has it
-  const unsigned L = total, P = prm.P, share = max(L > P ? (L + P - 1) / P : 1u, static_cast<unsigned>(prm.min_share));
+  const unsigned L = total, share = Plan::share_of(total, prm.P, prm.min_share);
   unsigned g = part * share;
   const unsigned g1 = min(g + share, L);
   // its first unit: of the last lane whose items begin at or before g
