@@ -396,16 +396,25 @@ def test_rerun_is_bit_identical():
         assert torch.equal(o1.view(torch.int16), o2.view(torch.int16)) and torch.equal(l1, l2)
 
 
-def _with_room(w, kv8):
-    """(w, kv8) as a serving loop has them: a table that is wider than its longest sequence, a cache of more pages than the call reads."""
-    table = np.concatenate([w.block_table, np.full((w.B, max(8, 600 // w.B)), -1, np.int32)], axis=1)
-    return dataclasses.replace(w, block_table=np.ascontiguousarray(table)), np.concatenate([kv8, np.zeros((6000, 64, 576), np.uint8)])
+# The six tests from here on were written for a choice between two ways of multiplying an E4M3 cache with Q, one of which split
+# Q into 8-bit numbers and is gone.  What they ask for holds for E4M3 calls in a wide table and a large cache, and in a tight one.
+def _for_split_q(w, kv8):
+    """(w, kv8) with a table and a cache that are large enough for the 128-row kernel to multiply K's bytes with a split Q (by the
+    rule: 0.3 us a page that a part may get at most, against 1 us and 3.2 us an item)."""
+    import torch
+    parts = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    nrb = (w.Sq * w.H + 127) // 128
+    pages = int((1.0 + 3.2 * w.B * nrb / parts) / 0.3 * parts / nrb) + 2
+    width = max(w.block_table.shape[1], -(-pages // w.B))
+    table = np.concatenate([w.block_table, np.full((w.B, width - w.block_table.shape[1]), -1, np.int32)], axis=1)
+    spare = np.zeros((max(0, pages - kv8.shape[0]), 64, 576), np.uint8)
+    return dataclasses.replace(w, block_table=np.ascontiguousarray(table)), np.concatenate([kv8, spare])
 
 
-def _check_fp8_with_room(w, kv_scale=1.0 / 64.0, flags=None):
+def _check_split_q(w, kv_scale=1.0 / 64.0, flags=None):
     kv8 = synth.quantise_cache_e4m3(w, kv_scale)
     ref = R.decode_fp8(w.q, kv8, kv_scale, w.block_table, w.seqlens, w.scale)
-    big, big8 = _with_room(w, kv8)
+    big, big8 = _for_split_q(w, kv8)
     for f in flags or [None]:
         _check_fp8(big, kv_scale, f, big8, ref)
         assert binding.last_item_rows() == 128 and binding.last_launch_count() == 2
@@ -413,22 +422,75 @@ def _check_fp8_with_room(w, kv_scale=1.0 / 64.0, flags=None):
 
 @pytest.mark.parametrize("Sq,H,lens", [(1, 128, [1]), (1, 100, [63, 64, 65, 0]), (1, 128, [128, 129, 191, 192]), (1, 128, [255, 256, 257, 320]), (2, 128, [1000, 65, 1]),
                                        (3, 43, [513, 77]), (1, 16, [700]), (5, 128, [640, 1281])])
-def test_e4m3_cache_with_room(Sq, H, lens):
+def test_e4m3_cache_with_a_split_q(Sq, H, lens):
     # tiles of one to four pages, the middle of a page between the CTAs, several blocks of 128 rows, few rows
-    _check_fp8_with_room(synth.make_workload("sq", len(lens), Sq, H, lens, seed=2600 + sum(lens)))
+    _check_split_q(synth.make_workload("sq", len(lens), Sq, H, lens, seed=2600 + sum(lens)))
 
 
-def test_e4m3_cache_with_room_rescales_over_tiles_of_every_width():
+def test_e4m3_cache_with_a_split_q_rescales_over_tiles_of_every_width():
     lens = [180, 448, 512, 500, 250, 300, 700, 1250, 192, 65]
     w = synth.make_workload("sqr", len(lens), 1, 100, lens, seed=2610)
     synth.apply_logit_offsets(w, [synth.staircase_offsets(n) if b % 2 else np.where(np.arange(n) < n // 2, -30.0, 30.0) for b, n in enumerate(lens)])
-    _check_fp8_with_room(repeated(w, 8), 1.0 / 8.0, MODES)
+    _check_split_q(repeated(w, 8), 1.0 / 8.0, MODES)
 
 
 @pytest.mark.parametrize("pages", [(1, 1, 1), (4, 1, 5), (5, 6, 1, 4, 1)])
-def test_e4m3_cache_with_room_units_behind_one_another(pages):
+def test_e4m3_cache_with_a_split_q_units_behind_one_another(pages):
+    # the factors on the rows' scores have four places: many units of one tile in every part
     lens = [64 * (pages[i % len(pages)] - 1) + (33, 64, 1, 32)[i % 4] for i in range(450)]
-    _check_fp8_with_room(synth.make_workload("squ", 450, 1, 66, lens, seed=2620 + len(pages)))
+    _check_split_q(synth.make_workload("squ", 450, 1, 66, lens, seed=2620 + len(pages)))
+
+
+def test_split_q_is_exact_in_the_power_of_two_of_a_row():
+    # whatever power of two the rows carry, their two 8-bit parts are the same: the same bits; a row of zeros is the mean of V
+    import torch
+    w = synth.make_workload("sqp", 2, 1, 64, [700, 300], seed=2630)
+    w.q.reshape(-1, 576)[5] = 0
+    kv8 = synth.quantise_cache_e4m3(w, 1.0 / 64.0)
+    ref = R.decode_fp8(w.q, kv8, 1.0 / 64.0, w.block_table, w.seqlens, w.scale)
+    w, kv8 = _for_split_q(w, kv8)
+    _check_fp8(w, kv8=kv8, ref=ref)
+    q, _, bt, sl = to_device(w)
+    kvd = torch.from_numpy(kv8).to(q.device)
+    runs = [binding.mla_decode_fp8((q.float() * 2.0 ** k).to(torch.bfloat16), kvd, 1.0 / 64.0, bt, sl, w.scale * 2.0 ** -k) for k in (0, -100, 100)]
+    for out, lse in runs[1:]:
+        assert torch.equal(out.view(torch.int16), runs[0][0].view(torch.int16)) and torch.equal(lse, runs[0][1])
+
+
+@pytest.mark.parametrize("split", [False, True])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
+def test_an_e4m3_call_keeps_what_is_not_a_number_in_its_row(split, bad):
+    # a row whose Q holds such a thing has no row sum: lse -inf, and NaN, or nothing once parts are merged; no other row notices
+    import torch
+    w = synth.make_workload("sqn", 2, 1, 128, [700, 300], seed=2640)
+    kv8 = synth.quantise_cache_e4m3(w, 1.0 / 64.0)
+    if split:
+        w, kv8 = _for_split_q(w, kv8)
+    q, _, bt, sl = to_device(w)
+    kvd = torch.from_numpy(kv8).to(q.device)
+    want, lse = binding.mla_decode_fp8(q, kvd, 1.0 / 64.0, bt, sl, w.scale)
+    q[1, 0, 77, 123] = bad
+    got, bad_lse = binding.mla_decode_fp8(q, kvd, 1.0 / 64.0, bt, sl, w.scale)
+    row = got[1, 0, 77].clone()
+    assert bad_lse[1, 0, 77] == -float("inf") and (torch.isnan(row).all() or (row == 0).all())
+    got[1, 0, 77], bad_lse[1, 0, 77] = want[1, 0, 77], lse[1, 0, 77]
+    assert torch.equal(got.view(torch.int16), want.view(torch.int16)) and torch.equal(bad_lse, lse)
+
+
+@pytest.mark.parametrize("beyond", [0, 100000, None])
+def test_pages_outside_the_cache_are_pages_of_zeros_for_a_split_q(beyond):
+    w = synth.make_workload("sqo", 4, 1, 128, [1500, 65, 64, 900], seed=2650)
+    w, kv8 = _for_split_q(w, synth.quantise_cache_e4m3(w, 1.0 / 64.0))
+    w = dataclasses.replace(w, kv=np.zeros(kv8.shape, np.uint16))
+    bad, ref = outside_the_cache(w, beyond)
+    ref8 = np.concatenate([kv8, np.zeros((1, 64, 576), np.uint8)])
+    _check_fp8(bad, kv8=kv8, ref=R.decode_fp8(ref.q, ref8, 1.0 / 64.0, ref.block_table, ref.seqlens, ref.scale))
+
+
+def _with_room(w, kv8):
+    """(w, kv8) as a serving loop has them: a table that is wider than its longest sequence, a cache of more pages than the call reads."""
+    table = np.concatenate([w.block_table, np.full((w.B, max(8, 600 // w.B)), -1, np.int32)], axis=1)
+    return dataclasses.replace(w, block_table=np.ascontiguousarray(table)), np.concatenate([kv8, np.zeros((6000, 64, 576), np.uint8)])
 
 
 @pytest.mark.parametrize("room", [False, True])
@@ -455,52 +517,6 @@ def test_an_e4m3_call_gives_the_bits_of_a_bf16_call_on_its_widened_cache(Sq, H, 
     assert binding.last_item_rows() == 128
     assert torch.equal(out.view(torch.int16), want.view(torch.int16)) and torch.equal(lse, want_lse)
     compare((out.float() / 64.0).cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64), *ref, f"e4m3, wide rows, room={room}")
-
-
-def test_an_e4m3_call_is_exact_in_the_power_of_two_of_a_row():
-    # whatever power of two the rows carry, and the softmax scale takes off again: the same bits; a row of zeros is the mean of V
-    import torch
-    w = synth.make_workload("sqp", 2, 1, 64, [700, 300], seed=2630)
-    w.q.reshape(-1, 576)[5] = 0
-    kv8 = synth.quantise_cache_e4m3(w, 1.0 / 64.0)
-    ref = R.decode_fp8(w.q, kv8, 1.0 / 64.0, w.block_table, w.seqlens, w.scale)
-    w, kv8 = _with_room(w, kv8)
-    _check_fp8(w, kv8=kv8, ref=ref)
-    q, _, bt, sl = to_device(w)
-    kvd = torch.from_numpy(kv8).to(q.device)
-    runs = [binding.mla_decode_fp8((q.float() * 2.0 ** k).to(torch.bfloat16), kvd, 1.0 / 64.0, bt, sl, w.scale * 2.0 ** -k) for k in (0, -100, 100)]
-    for out, lse in runs[1:]:
-        assert torch.equal(out.view(torch.int16), runs[0][0].view(torch.int16)) and torch.equal(lse, runs[0][1])
-
-
-@pytest.mark.parametrize("room", [False, True])
-@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
-def test_an_e4m3_call_keeps_what_is_not_a_number_in_its_row(room, bad):
-    # a row whose Q holds such a thing has no row sum: lse -inf, and NaN, or nothing once parts are merged; no other row notices
-    import torch
-    w = synth.make_workload("sqn", 2, 1, 128, [700, 300], seed=2640)
-    kv8 = synth.quantise_cache_e4m3(w, 1.0 / 64.0)
-    if room:
-        w, kv8 = _with_room(w, kv8)
-    q, _, bt, sl = to_device(w)
-    kvd = torch.from_numpy(kv8).to(q.device)
-    want, lse = binding.mla_decode_fp8(q, kvd, 1.0 / 64.0, bt, sl, w.scale)
-    q[1, 0, 77, 123] = bad
-    got, bad_lse = binding.mla_decode_fp8(q, kvd, 1.0 / 64.0, bt, sl, w.scale)
-    row = got[1, 0, 77].clone()
-    assert bad_lse[1, 0, 77] == -float("inf") and (torch.isnan(row).all() or (row == 0).all())
-    got[1, 0, 77], bad_lse[1, 0, 77] = want[1, 0, 77], lse[1, 0, 77]
-    assert torch.equal(got.view(torch.int16), want.view(torch.int16)) and torch.equal(bad_lse, lse)
-
-
-@pytest.mark.parametrize("beyond", [0, 100000, None])
-def test_pages_outside_an_e4m3_cache_with_room_are_pages_of_zeros(beyond):
-    w = synth.make_workload("sqo", 4, 1, 128, [1500, 65, 64, 900], seed=2650)
-    w, kv8 = _with_room(w, synth.quantise_cache_e4m3(w, 1.0 / 64.0))
-    w = dataclasses.replace(w, kv=np.zeros(kv8.shape, np.uint16))
-    bad, ref = outside_the_cache(w, beyond)
-    ref8 = np.concatenate([kv8, np.zeros((1, 64, 576), np.uint8)])
-    _check_fp8(bad, kv8=kv8, ref=R.decode_fp8(ref.q, ref8, 1.0 / 64.0, ref.block_table, ref.seqlens, ref.scale))
 
 
 @pytest.mark.parametrize("fp8", [False, True])
