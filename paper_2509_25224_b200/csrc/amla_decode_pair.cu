@@ -25,15 +25,14 @@
 // crossed to the other SM by remote stores, Q went through shared memory into tensor memory and the score CTA had to be
 // drained before the next unit's Q could follow.  Here nothing but MMA operands crosses, Q is an operand as it lands, and
 // the tile is 256 keys.  Calls with it, from that kernel to this one as it stands (sustained): 192 sequences of 1-512 keys
-// 62.8 -> 42.2 us; one of 2531 33.8 -> 12.4; 16 x 16384 with rising logits 106.0 -> 92.7; 96 x 2048 88.7 -> 79.2; 32 x 4096
-// 59.1 -> 53.7; E4M3 32 x 4096 100.4 -> 60.6.
+// 62.8 -> 38.1 us; one of 2531 33.8 -> 12.3; 16 x 16384 with rising logits 106.0 -> 93.7; 96 x 2048 88.7 -> 78.4; 32 x 4096
+// 59.1 -> 53.2; E4M3 32 x 4096 100.4 -> 60.4.  (The last of each pair from one GPU; others are up to 3 % faster.)
 // What bounds it (trace): a tile of 256 keys takes 7100 clk in long units, 7600 on average over the eight of a 32 x 4096 call,
-// against 4350 of MMAs and 5900 of HBM at its full rate.  The issuer finds every slot full that it comes to, and takes 350 clk
-// for a slot of K and 390 for one of V, 17 of them a tile; what is left are its waits for the softmax warps.  A slot is full
-// 2200 clk (K, most of it from L2) or 2400 clk (V) after it has been asked for, and is asked for again 630 or 690 clk later: a
-// ring of 112 KB for the 278 KB of a tile just about keeps up.  E4M3: 9800 clk; a pair of widening warps takes 700 clk for a
-// slot and has waited 540 for its place, 150 for the raw slot; the issuer waits for one slot in ten.  Long calls run at the
-// power limit: 32 x 4096 takes 50 us cool.
+// against 4350 of MMAs, 5600 of shared memory at 128 bytes a clk (MMA operands 408 KB, TMA 278, P~ 32) and 5900-6600 of HBM.  The
+// issuer finds every slot full that it comes to, and takes 350 clk for a slot of K and 390 for one of V, 17 of them a tile: the
+// operands of four MMAs and the 16 KB that TMA writes meanwhile are 320 clk of shared memory.  E4M3: a tile is 17 slots of ~575 clk,
+// 996 KB through shared memory (7800 clk), and two of the four schedulers convert 17 x 352 clk beside the softmax.  Long calls run
+// at the power limit, at 1.4-1.75 GHz: 32 x 4096 takes 48.5 us cool.
 //
 // All waits are bounded; on expiry the kernel records kStatusTimeout and unwinds.
 #include "amla_common.cuh"
@@ -320,7 +319,10 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
       // A lane half holds 32 np neighbouring keys of a tile; this group takes its 32-key chunks grp and grp + 2.
       const uint32_t scol = tbase + lane_base + kSCol + 128 * sb + 32 * grp;
       const int chunk0 = np * khalf + grp;                                  // of the tile's 2 np
-      bool direct = false;                               // P~ goes straight into the P buffer, 8 keys at a time as they are ready
+      // P~ goes straight into the P buffer, 8 keys at a time as they are ready; into tensor memory 32 at a time, with an E4M3 cache,
+      // where registers are few, 8.  (32 / 8: E4M3, 1 x 130 keys 10.73 / 10.62 us, 1 x 256 10.99 / 10.90, 8 x 1000 with 16 heads 14.38 /
+      // 14.23; bf16, 8 at a time: 1 x 256 with 16 heads 7.87 / 7.95, 192 x 1-512 32.6 / 32.8.)
+      bool direct = false;
       uint32_t nword = 0;
       bool moved = false;
       if (tile.valid) {
@@ -394,16 +396,20 @@ decode_pair_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_const
           }
           uint32_t pk[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            float x0, x1;
-            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), sc2, ns2), x0, x1);
-            const float q0 = ex2_approx(x0), q1 = ex2_approx(x1);
-            const uint64_t pp = pack_f32x2(q0, q1);
-            if (i & 1) rsb = add_f32x2(rsb, pp); else rsa = add_f32x2(rsa, pp);
-            pk[i] = pack_bf16x2(q0, q1);
-            if ((i & 3) == 3 && direct) store_p_piece(chunk0 + 2 * h, i >> 2, pk);
+          for (int c = 0; c < 4; ++c) {
+#pragma unroll
+            for (int i = 4 * c; i < 4 * c + 4; ++i) {
+              float x0, x1;
+              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), sc2, ns2), x0, x1);
+              const float q0 = ex2_approx(x0), q1 = ex2_approx(x1);
+              const uint64_t pp = pack_f32x2(q0, q1);
+              if (i & 1) rsb = add_f32x2(rsb, pp); else rsa = add_f32x2(rsa, pp);
+              pk[i] = pack_bf16x2(q0, q1);
+            }
+            if (direct) store_p_piece(chunk0 + 2 * h, c, pk);
+            else if (kFp8) tmem_st_32x32b_x4(scol + 64 * h + 4 * c, pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
           }
-          if (!direct) tmem_st_32x32b_x16(scol + 64 * h, pk);
+          if (!kFp8 && !direct) tmem_st_32x32b_x16(scol + 64 * h, pk);
         }
         float s0, s1;
         unpack_f32x2(add_f32x2(rsa, rsb), s0, s1);
